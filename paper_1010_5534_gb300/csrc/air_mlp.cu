@@ -7,7 +7,7 @@
 //
 // Tensor cores: every layer of the forward pass and both data-gradient
 // products of the backward pass are mma.sync m16n8k16 (BF16 in, FP32 out). A
-// warp owns 32 samples (two 16-row tiles); the FP32 accumulator fragments of
+// warp owns 16 samples (one 16-row tile); the FP32 accumulator fragments of
 // two adjacent 8-column tiles are exactly the BF16 A-operand fragment of the
 // next 16-wide K slice, so layers chain in registers. The weight gradients
 // dW = act^T d over the block's 128 samples are mma.sync products as well:
@@ -32,17 +32,26 @@ constexpr int kIn = 16, kH = 64, kOut = 5, kOutP = 8;
 constexpr int oW1 = 0, ob1 = oW1 + kIn * kH, oW2 = ob1 + kH, ob2 = oW2 + kH * kH, oW3 = ob2 + kH,
               ob3 = oW3 + kH * kOut, kNP = ob3 + kOut;
 static_assert(kNP == AIR_MLP_NPARAMS, "parameter count");
-constexpr int kTile = 128;  // samples per block (4 warps x 32)
+constexpr int kTile = 128;             // samples of a tile: 8 warps x 16 rows
+constexpr int kThreads = kTile * 2;
+
+// Row strides in shared memory, in 32-bit words: rows of 8 (features) and 32
+// (hidden units) words are padded by 4, so that the eight rows a fragment load
+// or an ldmatrix touches start in different banks (with unpadded rows of 128
+// bytes every such access was an eight-way conflict, which bound the kernel:
+// the minibatch of 8192 samples took 33 us).
+constexpr int kRowIn = kIn / 2 + 4, kRowH = kH / 2 + 4, kRowOut = kOutP / 2;
 
 // BF16 copies of the weights in the layouts the fragments read, as 32-bit
-// words (two BF16 along K per word):
+// words (two BF16 along K per word), rows padded as above:
 //   W1T [64][16]  forward layer 1, B[k][n] = W1[k][n] stored n-major
 //   W2T [64][64]  forward layer 2, n-major
 //   W3T [8][64]   forward layer 3 (outputs 5..7 zero), n-major
 //   W3P [64][8]   backward d3 W3^T: B[k=out][n=hidden] = W3[n][k], row-major W3 padded
 //   W2R [64][64]  backward d2 W2^T: B[k][n] = W2[n][k], row-major W2
-constexpr int kW1T = 0, kW2T = kW1T + kH * kIn / 2, kW3T = kW2T + kH * kH / 2,
-              kW3P = kW3T + kOutP * kH / 2, kW2R = kW3P + kH * kOutP / 2, kWords = kW2R + kH * kH / 2;
+constexpr int kW1T = 0, kW2T = kW1T + kH * kRowIn, kW3T = kW2T + kH * kRowH,
+              kW3P = kW3T + kOutP * kRowH, kW2R = kW3P + kH * kRowOut, kWords = kW2R + kH * kRowH;
+static_assert(kWords % 4 == 0, "copied in 16-byte pieces");
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -87,28 +96,28 @@ __device__ __forceinline__ void stage_hi_lo(uint32_t *h, uint32_t *l, int w, flo
   l[w] = pack_bf16(v0 - bf16_lo(hw), v1 - bf16_hi(hw));
 }
 
-__global__ void k_pack_weights(const float *__restrict__ th, uint32_t *__restrict__ w) {
+// Parameter j (flat index) into the packed layouts. The padding of the rows
+// and of W3's missing outputs is zeroed once (air_mlp_create).
+__device__ __forceinline__ void pack_weight(uint32_t *__restrict__ w, int j, float v) {
   uint16_t *h = reinterpret_cast<uint16_t *>(w);
-  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < kWords * 2; x += gridDim.x * blockDim.x) {
-    float v = 0.f;
-    if (x < kW2T * 2) {  // W1T[n][k]
-      const int n = x / kIn, k = x % kIn;
-      v = th[oW1 + k * kH + n];
-    } else if (x < kW3T * 2) {  // W2T[n][k]
-      const int y = x - kW2T * 2, n = y / kH, k = y % kH;
-      v = th[oW2 + k * kH + n];
-    } else if (x < kW3P * 2) {  // W3T[n][k], n < 8
-      const int y = x - kW3T * 2, n = y / kH, k = y % kH;
-      v = n < kOut ? th[oW3 + k * kOut + n] : 0.f;
-    } else if (x < kW2R * 2) {  // W3P[n][k], k < 8
-      const int y = x - kW3P * 2, n = y / kOutP, k = y % kOutP;
-      v = k < kOut ? th[oW3 + n * kOut + k] : 0.f;
-    } else {  // W2R[n][k] = W2[n][k]
-      const int y = x - kW2R * 2;
-      v = th[oW2 + y];
-    }
-    h[x] = bf16_bits(v);
+  const uint16_t b = bf16_bits(v);
+  if (j < ob1) {
+    const int k = (j - oW1) / kH, n = (j - oW1) % kH;
+    h[2 * (kW1T + n * kRowIn) + k] = b;
+  } else if (j >= oW2 && j < ob2) {
+    const int k = (j - oW2) / kH, n = (j - oW2) % kH;
+    h[2 * (kW2T + n * kRowH) + k] = b;
+    h[2 * (kW2R + k * kRowH) + n] = b;
+  } else if (j >= oW3 && j < ob3) {
+    const int k = (j - oW3) / kOut, n = (j - oW3) % kOut;
+    h[2 * (kW3T + n * kRowH) + k] = b;
+    h[2 * (kW3P + k * kRowOut) + n] = b;
   }
+}
+
+__global__ void k_pack_weights(const float *__restrict__ th, uint32_t *__restrict__ w) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < kNP; j += gridDim.x * blockDim.x)
+    pack_weight(w, j, th[j]);
 }
 
 struct MlpArgs {
@@ -124,30 +133,34 @@ struct MlpArgs {
 
 // Shared memory of a training block (bytes): weights + staged tile.
 constexpr size_t kSmW = sizeof(uint32_t) * kWords;
-constexpr size_t kSmTrain = kSmW + sizeof(uint32_t) * kTile * (kIn / 2 + kH / 2 + kH / 2) +
-                            sizeof(float) * kTile * (kH + kH + kOutP) + sizeof(float) * 4;
+constexpr size_t kSmTrain = kSmW + sizeof(uint32_t) * kTile * (kRowIn + 6 * kRowH + 2 * kRowOut) +
+                            sizeof(float) * 2 * kThreads;
 
+// One warp carries 16 samples through the network. Training: one tile per
+// block. Inference: blocks loop over tiles, so the weights are staged once per
+// block and not once per tile.
+//
+// Launched as a dependent of the optimiser step before it: a tile's features
+// are fetched before the wait, the weights after it.
 template <bool TRAIN>
-__global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
+__global__ void __launch_bounds__(kThreads) k_mlp(MlpArgs a) {
   extern __shared__ __align__(16) uint32_t sm[];
   uint32_t *sw = sm;
-  for (int x = threadIdx.x; x < kWords; x += blockDim.x) sw[x] = a.w[x];
-  uint32_t *xs = sm + kWords;                 // [128][8]
-  uint32_t *h1s = xs + kTile * (kIn / 2);     // [128][32]
-  uint32_t *h2s = h1s + kTile * (kH / 2);     // [128][32]
+  uint32_t *xs = sm + kWords;            // [128] rows of kRowIn
+  uint32_t *h1s = xs + kTile * kRowIn;   // [128] rows of kRowH
+  uint32_t *h2s = h1s + kTile * kRowH;
   // back-propagated errors, two BF16 parts each (hi, lo), two per word along
-  // the output unit: d1 and d2 [128][64], d3 [128][8]
-  uint32_t *d1h = h2s + kTile * (kH / 2), *d1l = d1h + kTile * (kH / 2);
-  uint32_t *d2h = d1l + kTile * (kH / 2), *d2l = d2h + kTile * (kH / 2);
-  uint32_t *d3h = d2l + kTile * (kH / 2), *d3l = d3h + kTile * (kOutP / 2);
-  float *lsum = reinterpret_cast<float *>(d3l + kTile * (kOutP / 2));  // [4] per-warp loss
-  __syncthreads();
+  // the output unit: d1 and d2 [128] rows of kRowH, d3 [128] rows of kRowOut
+  uint32_t *d1h = h2s + kTile * kRowH, *d1l = d1h + kTile * kRowH;
+  uint32_t *d2h = d1l + kTile * kRowH, *d2l = d2h + kTile * kRowH;
+  uint32_t *d3h = d2l + kTile * kRowH, *d3l = d3h + kTile * kRowOut;
+  float *lsum = reinterpret_cast<float *>(d3l + kTile * kRowOut);  // [8 warps][32 lanes][2]: loss terms
   const uint32_t *W1T = sw + kW1T, *W2T = sw + kW2T, *W3T = sw + kW3T, *W3P = sw + kW3P, *W2R = sw + kW2R;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-  float wloss = 0.f;
-  for (int mt = 0; mt < 2; ++mt) {
-    const int r0 = warp * 32 + mt * 16;                 // row in the tile
-    const int64_t gr0 = (int64_t)blockIdx.x * kTile + r0;  // global sample
+  const int64_t tiles = (a.n + kTile - 1) / kTile;
+  const int r0 = warp * 16;  // the warp's first row in the tile
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int64_t gr0 = tile * kTile + r0;  // global sample
     const int64_t ra = gr0 + g, rb = gr0 + g + 8;
     const bool va = ra < a.n, vb = rb < a.n;
     uint32_t ax[4];
@@ -155,13 +168,19 @@ __global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
     ax[1] = vb ? a.x[rb * 8 + t] : 0u;
     ax[2] = va ? a.x[ra * 8 + t + 4] : 0u;
     ax[3] = vb ? a.x[rb * 8 + t + 4] : 0u;
+    if (tile == blockIdx.x) {
+      wait_prior_grid();
+      for (int x = threadIdx.x; x < kWords / 4; x += blockDim.x)
+        reinterpret_cast<uint4 *>(sw)[x] = reinterpret_cast<const uint4 *>(a.w)[x];
+      __syncthreads();
+    }
     // layer 1
     float acc[8][4];
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
       const float b0 = a.th[ob1 + nt * 8 + 2 * t], b1 = a.th[ob1 + nt * 8 + 2 * t + 1];
       acc[nt][0] = b0; acc[nt][1] = b1; acc[nt][2] = b0; acc[nt][3] = b1;
-      const uint32_t *wr = W1T + (nt * 8 + g) * (kIn / 2);
+      const uint32_t *wr = W1T + (nt * 8 + g) * kRowIn;
       mma16816(acc[nt], ax, wr[t], wr[t + 4]);
     }
     uint32_t a2[4][4];
@@ -177,7 +196,7 @@ __global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
     for (int nt = 0; nt < 8; ++nt) {
       const float b0 = a.th[ob2 + nt * 8 + 2 * t], b1 = a.th[ob2 + nt * 8 + 2 * t + 1];
       acc[nt][0] = b0; acc[nt][1] = b1; acc[nt][2] = b0; acc[nt][3] = b1;
-      const uint32_t *wr = W2T + (nt * 8 + g) * (kH / 2);
+      const uint32_t *wr = W2T + (nt * 8 + g) * kRowH;
 #pragma unroll
       for (int kt = 0; kt < 4; ++kt) mma16816(acc[nt], a2[kt], wr[kt * 8 + t], wr[kt * 8 + t + 4]);
     }
@@ -195,7 +214,7 @@ __global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
       const int c0 = 2 * t, c1 = 2 * t + 1;
       const float b0 = c0 < kOut ? a.th[ob3 + c0] : 0.f, b1 = c1 < kOut ? a.th[ob3 + c1] : 0.f;
       lg[0] = b0; lg[1] = b1; lg[2] = b0; lg[3] = b1;
-      const uint32_t *wr = W3T + g * (kH / 2);
+      const uint32_t *wr = W3T + g * kRowH;
 #pragma unroll
       for (int kt = 0; kt < 4; ++kt) mma16816(lg, a3[kt], wr[kt * 8 + t], wr[kt * 8 + t + 4]);
     }
@@ -215,20 +234,20 @@ __global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
     }
     // ---- training: stage activations (BF16, as used in the products)
     const int la = r0 + g, lb = r0 + g + 8;
-    xs[la * 8 + t] = ax[0];
-    xs[lb * 8 + t] = ax[1];
-    xs[la * 8 + t + 4] = ax[2];
-    xs[lb * 8 + t + 4] = ax[3];
+    xs[la * kRowIn + t] = ax[0];
+    xs[lb * kRowIn + t] = ax[1];
+    xs[la * kRowIn + t + 4] = ax[2];
+    xs[lb * kRowIn + t + 4] = ax[3];
 #pragma unroll
     for (int kt = 0; kt < 4; ++kt) {
-      h1s[la * 32 + kt * 8 + t] = a2[kt][0];
-      h1s[lb * 32 + kt * 8 + t] = a2[kt][1];
-      h1s[la * 32 + kt * 8 + 4 + t] = a2[kt][2];
-      h1s[lb * 32 + kt * 8 + 4 + t] = a2[kt][3];
-      h2s[la * 32 + kt * 8 + t] = a3[kt][0];
-      h2s[lb * 32 + kt * 8 + t] = a3[kt][1];
-      h2s[la * 32 + kt * 8 + 4 + t] = a3[kt][2];
-      h2s[lb * 32 + kt * 8 + 4 + t] = a3[kt][3];
+      h1s[la * kRowH + kt * 8 + t] = a2[kt][0];
+      h1s[lb * kRowH + kt * 8 + t] = a2[kt][1];
+      h1s[la * kRowH + kt * 8 + 4 + t] = a2[kt][2];
+      h1s[lb * kRowH + kt * 8 + 4 + t] = a2[kt][3];
+      h2s[la * kRowH + kt * 8 + t] = a3[kt][0];
+      h2s[lb * kRowH + kt * 8 + t] = a3[kt][1];
+      h2s[la * kRowH + kt * 8 + 4 + t] = a3[kt][2];
+      h2s[lb * kRowH + kt * 8 + 4 + t] = a3[kt][3];
     }
     // softmax cross-entropy on rows g and g+8 (a quad holds one row's 8 columns)
     float d3[4];
@@ -248,24 +267,28 @@ __global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
       const float p0 = e0 / s, p1 = e1 / s;
       d3[2 * half] = (vr && v0) ? (p0 - (yr == 2 * t ? 1.f : 0.f)) * a.inv_count : 0.f;
       d3[2 * half + 1] = (vr && v1) ? (p1 - (yr == 2 * t + 1 ? 1.f : 0.f)) * a.inv_count : 0.f;
-      if (vr && yr == 2 * t) wloss -= logf(p0);
-      if (vr && yr == 2 * t + 1) wloss -= logf(p1);
+      // this lane's loss term of the row (at most one of its two outputs is
+      // the label)
+      float x = 0.f;
+      if (vr && yr == 2 * t) x = logf(p0);
+      if (vr && yr == 2 * t + 1) x = logf(p1);
+      lsum[(warp * 32 + lane) * 2 + half] = x;
     }
-    stage_hi_lo(d3h, d3l, la * (kOutP / 2) + t, d3[0], d3[1]);
-    stage_hi_lo(d3h, d3l, lb * (kOutP / 2) + t, d3[2], d3[3]);
+    stage_hi_lo(d3h, d3l, la * kRowOut + t, d3[0], d3[1]);
+    stage_hi_lo(d3h, d3l, lb * kRowOut + t, d3[2], d3[3]);
     // d2 = (d3 W3^T) * [z2 > 0]
     const uint32_t ad3[4] = {pack_bf16(d3[0], d3[1]), pack_bf16(d3[2], d3[3]), 0u, 0u};
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
       acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-      mma16816(acc[nt], ad3, W3P[(nt * 8 + g) * (kOutP / 2) + t], 0u);
+      mma16816(acc[nt], ad3, W3P[(nt * 8 + g) * kRowOut + t], 0u);
       const uint32_t hg = a3[nt >> 1][(nt & 1) * 2], hg8 = a3[nt >> 1][(nt & 1) * 2 + 1];
       if (bf16_lo(hg) == 0.f) acc[nt][0] = 0.f;
       if (bf16_hi(hg) == 0.f) acc[nt][1] = 0.f;
       if (bf16_lo(hg8) == 0.f) acc[nt][2] = 0.f;
       if (bf16_hi(hg8) == 0.f) acc[nt][3] = 0.f;
-      stage_hi_lo(d2h, d2l, la * (kH / 2) + nt * 4 + t, acc[nt][0], acc[nt][1]);
-      stage_hi_lo(d2h, d2l, lb * (kH / 2) + nt * 4 + t, acc[nt][2], acc[nt][3]);
+      stage_hi_lo(d2h, d2l, la * kRowH + nt * 4 + t, acc[nt][0], acc[nt][1]);
+      stage_hi_lo(d2h, d2l, lb * kRowH + nt * 4 + t, acc[nt][2], acc[nt][3]);
     }
     uint32_t ad2[4][4];
 #pragma unroll
@@ -279,7 +302,7 @@ __global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
       acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-      const uint32_t *wr = W2R + (nt * 8 + g) * (kH / 2);
+      const uint32_t *wr = W2R + (nt * 8 + g) * kRowH;
 #pragma unroll
       for (int kt = 0; kt < 4; ++kt) mma16816(acc[nt], ad2[kt], wr[kt * 8 + t], wr[kt * 8 + t + 4]);
       const uint32_t hg = a2[nt >> 1][(nt & 1) * 2], hg8 = a2[nt >> 1][(nt & 1) * 2 + 1];
@@ -287,30 +310,27 @@ __global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
       if (bf16_hi(hg) == 0.f) acc[nt][1] = 0.f;
       if (bf16_lo(hg8) == 0.f) acc[nt][2] = 0.f;
       if (bf16_hi(hg8) == 0.f) acc[nt][3] = 0.f;
-      stage_hi_lo(d1h, d1l, la * (kH / 2) + nt * 4 + t, acc[nt][0], acc[nt][1]);
-      stage_hi_lo(d1h, d1l, lb * (kH / 2) + nt * 4 + t, acc[nt][2], acc[nt][3]);
+      stage_hi_lo(d1h, d1l, la * kRowH + nt * 4 + t, acc[nt][0], acc[nt][1]);
+      stage_hi_lo(d1h, d1l, lb * kRowH + nt * 4 + t, acc[nt][2], acc[nt][3]);
     }
   }
   if (!TRAIN) return;
-  // per-warp loss
-  for (int off = 16; off > 0; off >>= 1) wloss += __shfl_xor_sync(0xffffffffu, wloss, off);
-  if (lane == 0) lsum[warp] = wloss;
   __syncthreads();
   // weight gradients: 44 output tiles of 16 x 8 (dW1: 1 x 8, dW2: 4 x 8,
-  // dW3: 4 x 1), a warp taking every fourth; each sums the 128 samples in 8
+  // dW3: 4 x 1), a warp taking every eighth; each sums the 128 samples in 8
   // K steps of 16, hi and lo parts of d in turn (fixed order)
   float *out = a.partial + (int64_t)blockIdx.x * (kNP + 1);
-  for (int tile = warp; tile < 44; tile += 4) {
+  for (int tile = warp; tile < 44; tile += kThreads / 32) {
     const uint32_t *act, *dh, *dl;
     int lda, ldd, m0, n0, ow, ncols;
     if (tile < 8) {
-      act = xs; lda = kIn; dh = d1h; dl = d1l; ldd = kH; m0 = 0; n0 = tile * 8; ow = oW1; ncols = kH;
+      act = xs; lda = 2 * kRowIn; dh = d1h; dl = d1l; ldd = 2 * kRowH; m0 = 0; n0 = tile * 8; ow = oW1; ncols = kH;
     } else if (tile < 40) {
       const int u = tile - 8;
-      act = h1s; lda = kH; dh = d2h; dl = d2l; ldd = kH; m0 = (u >> 3) * 16; n0 = (u & 7) * 8;
+      act = h1s; lda = 2 * kRowH; dh = d2h; dl = d2l; ldd = 2 * kRowH; m0 = (u >> 3) * 16; n0 = (u & 7) * 8;
       ow = oW2; ncols = kH;
     } else {
-      act = h2s; lda = kH; dh = d3h; dl = d3l; ldd = kOutP; m0 = (tile - 40) * 16; n0 = 0;
+      act = h2s; lda = 2 * kRowH; dh = d3h; dl = d3l; ldd = 2 * kRowOut; m0 = (tile - 40) * 16; n0 = 0;
       ow = oW3; ncols = kOut;
     }
     const uint16_t *ah = reinterpret_cast<const uint16_t *>(act);
@@ -318,7 +338,7 @@ __global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
     const uint16_t *bl = reinterpret_cast<const uint16_t *>(dl);
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     const int mi = lane >> 3, j = lane & 7;
-#pragma unroll 2
+#pragma unroll 4
     for (int r0 = 0; r0 < kTile; r0 += 16) {
       // A = act^T: 8 x 8 blocks (samples r0 + 8 (mi >> 1) .., features m0 + 8 (mi & 1) ..)
       uint32_t fa[4], fb[2], fl[2];
@@ -337,49 +357,95 @@ __global__ void __launch_bounds__(kTile) k_mlp(MlpArgs a) {
       if (n < ncols) out[ow + m * ncols + n] = acc[e];
     }
   }
-  // bias gradients: column sums of hi + lo over the 128 samples (fixed order)
+  // bias gradients: column sums of hi + lo over the 128 samples (in order)
   for (int c = threadIdx.x; c < 2 * kH + kOut; c += blockDim.x) {
     const uint16_t *bh, *bl;
     int ldd, n, ob;
     if (c < kH) {
       bh = reinterpret_cast<const uint16_t *>(d1h); bl = reinterpret_cast<const uint16_t *>(d1l);
-      ldd = kH; n = c; ob = ob1;
+      ldd = 2 * kRowH; n = c; ob = ob1;
     } else if (c < 2 * kH) {
       bh = reinterpret_cast<const uint16_t *>(d2h); bl = reinterpret_cast<const uint16_t *>(d2l);
-      ldd = kH; n = c - kH; ob = ob2;
+      ldd = 2 * kRowH; n = c - kH; ob = ob2;
     } else {
       bh = reinterpret_cast<const uint16_t *>(d3h); bl = reinterpret_cast<const uint16_t *>(d3l);
-      ldd = kOutP; n = c - 2 * kH; ob = ob3;
+      ldd = 2 * kRowOut; n = c - 2 * kH; ob = ob3;
     }
     float sum = 0.f;
+#pragma unroll 16
     for (int r = 0; r < kTile; ++r)
       sum += __uint_as_float((uint32_t)bh[r * ldd + n] << 16) + __uint_as_float((uint32_t)bl[r * ldd + n] << 16);
     out[ob + n] = sum;
   }
-  if (threadIdx.x == 0) out[kNP] = lsum[0] + lsum[1] + lsum[2] + lsum[3];
+  // loss: a lane's four rows (of two neighbouring warps' tiles) in order, then
+  // the lanes, then the four 32-sample groups
+  if (warp == kThreads / 32 - 1) {
+    float l4[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float wl = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) wl -= lsum[((2 * q + (e >> 1)) * 32 + lane) * 2 + (e & 1)];
+      for (int off = 16; off > 0; off >>= 1) wl += __shfl_xor_sync(0xffffffffu, wl, off);
+      l4[q] = wl;
+    }
+    if (lane == 0) out[kNP] = l4[0] + l4[1] + l4[2] + l4[3];
+  }
 }
 
-// grad[j] = sum over blocks of partial[b][j] (block order); loss likewise.
+// Sum over blocks of partial[b][j] in FP64, in block order (loads 8 at a
+// time).
+__device__ __forceinline__ double sum_partials(const float *__restrict__ partial, int64_t nblocks,
+                                               int j) {
+  double s = 0.0;
+  int64_t b = 0;
+  for (; b + 8 <= nblocks; b += 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = partial[(b + u) * (kNP + 1) + j];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += (double)v[u];
+  }
+  for (; b < nblocks; ++b) s += (double)partial[b * (kNP + 1) + j];
+  return s;
+}
+
+// grad[j] = the sum over blocks; loss likewise.
 __global__ void k_reduce_partials(const float *__restrict__ partial, int64_t nblocks,
                                   float *__restrict__ grad, double *__restrict__ loss) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j > kNP) return;
-  double s = 0.0;
-  for (int64_t b = 0; b < nblocks; ++b) s += (double)partial[b * (kNP + 1) + j];
+  const double s = sum_partials(partial, nblocks, j);
   if (j < kNP) grad[j] = (float)s;
   else *loss = s;
 }
 
-__global__ void k_adam(float *__restrict__ th, float *__restrict__ m, float *__restrict__ v,
-                       const float *__restrict__ g, float lr, float c1, float c2) {
+// One optimiser step in one launch: the gradient (as k_reduce_partials), Adam
+// and the packed BF16 copies of parameter j by one thread; the minibatch's
+// loss to *loss. (Three launches before: reduction, Adam, packing.) Blocks of
+// 64 spread the FP64 sums over 88 SMs.
+__global__ void __launch_bounds__(64) k_step(const float *__restrict__ partial, int64_t nblocks,
+                                             float *__restrict__ th, float *__restrict__ m,
+                                             float *__restrict__ v, float *__restrict__ grad,
+                                             uint32_t *__restrict__ w, double *__restrict__ loss,
+                                             float lr, float c1, float c2) {
+  wait_prior_grid();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= kNP) return;
-  const float gj = g[j];
+  if (j > kNP) return;
+  const double s = sum_partials(partial, nblocks, j);
+  if (j == kNP) {
+    *loss = s;
+    return;
+  }
+  const float gj = (float)s;
+  grad[j] = gj;
   const float mj = 0.9f * m[j] + 0.1f * gj;
   const float vj = 0.999f * v[j] + 0.001f * gj * gj;
   m[j] = mj;
   v[j] = vj;
-  th[j] -= lr * (mj / c1) / (sqrtf(vj / c2) + 1e-8f);
+  const float x = th[j] - lr * (mj / c1) / (sqrtf(vj / c2) + 1e-8f);
+  th[j] = x;
+  pack_weight(w, j, x);
 }
 
 }  // namespace air
@@ -389,7 +455,8 @@ struct air_mlp {
   float *th = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr, *partial = nullptr;
   uint32_t *w = nullptr;
   double *d_loss = nullptr, *h_loss = nullptr;
-  size_t partial_b = 0;
+  double *hist = nullptr;  // loss of every minibatch of an epoch
+  size_t partial_b = 0, hist_b = 0;
   int64_t step = 0;
 };
 
@@ -415,14 +482,16 @@ air_status mlp_forward(air_mlp *m, const uint16_t *x, int64_t n, float *logits, 
   a.w = m->w;
   a.th = m->th;
   a.logits = logits;
-  const int64_t blocks = (n + kTile - 1) / kTile;
-  k_mlp<false><<<(unsigned)blocks, kTile, kSmW, st>>>(a);
+  // up to 8 blocks of 8 warps per SM (24 KB of weights each) share the tiles
+  const int64_t blocks = std::min<int64_t>((n + kTile - 1) / kTile, (int64_t)sm_count() * 8);
+  k_mlp<false><<<(unsigned)blocks, kThreads, kSmW, st>>>(a);
   CU_TRY(cudaGetLastError());
   return AIR_OK;
 }
 
-// Mean cross-entropy gradient over x[0..n) into m->grad (device), loss to m->d_loss.
-static air_status mlp_grad(air_mlp *m, const uint16_t *x, const int32_t *y, int64_t n) {
+// Per-block sums of the mean cross-entropy's gradient over x[0..n) and of the
+// loss into m->partial.
+static air_status mlp_partials(air_mlp *m, const uint16_t *x, const int32_t *y, int64_t n) {
   const int64_t blocks = (n + kTile - 1) / kTile;
   CU_TRY(ensure((void **)&m->partial, &m->partial_b, sizeof(float) * (size_t)blocks * (kNP + 1)));
   MlpArgs a{};
@@ -438,19 +507,30 @@ static air_status mlp_grad(air_mlp *m, const uint16_t *x, const int32_t *y, int6
     CU_TRY(cudaFuncSetAttribute(k_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmTrain));
     attr = true;
   }
-  k_mlp<true><<<(unsigned)blocks, kTile, kSmTrain, m->stream>>>(a);
-  CU_TRY(cudaGetLastError());
+  CU_TRY(launch_pdl(k_mlp<true>, dim3((unsigned)blocks), dim3(kThreads), kSmTrain, m->stream, a));
+  return AIR_OK;
+}
+
+// The gradient itself into m->grad (device), the loss to m->d_loss.
+static air_status mlp_grad(air_mlp *m, const uint16_t *x, const int32_t *y, int64_t n) {
+  const air_status s = mlp_partials(m, x, y, n);
+  if (s) return s;
+  const int64_t blocks = (n + kTile - 1) / kTile;
   k_reduce_partials<<<(kNP + 1 + 255) / 256, 256, 0, m->stream>>>(m->partial, blocks, m->grad, m->d_loss);
   CU_TRY(cudaGetLastError());
   return AIR_OK;
 }
 
-static air_status mlp_adam(air_mlp *m, float lr) {
+// One minibatch of training; its loss to *loss (device).
+static air_status mlp_step(air_mlp *m, const uint16_t *x, const int32_t *y, int64_t n, float lr,
+                           double *loss) {
+  const air_status s = mlp_partials(m, x, y, n);
+  if (s) return s;
   m->step += 1;
   const float c1 = 1.0f - powf(0.9f, (float)m->step), c2 = 1.0f - powf(0.999f, (float)m->step);
-  k_adam<<<(kNP + 255) / 256, 256, 0, m->stream>>>(m->th, m->m, m->v, m->grad, lr, c1, c2);
-  CU_TRY(cudaGetLastError());
-  return mlp_pack(m);
+  CU_TRY(launch_pdl(k_step, dim3((kNP + 1 + 63) / 64), dim3(64), 0, m->stream, (const float *)m->partial,
+                    (int64_t)((n + kTile - 1) / kTile), m->th, m->m, m->v, m->grad, m->w, loss, lr, c1, c2));
+  return AIR_OK;
 }
 
 }  // namespace air
@@ -472,6 +552,7 @@ air_status air_mlp_create(const float *params, void *stream, air_mlp **out) {
   if (e == cudaSuccess) e = cudaMalloc((void **)&m->w, sizeof(uint32_t) * kWords);
   if (e == cudaSuccess) e = cudaMalloc((void **)&m->d_loss, sizeof(double));
   if (e == cudaSuccess) e = cudaMallocHost((void **)&m->h_loss, sizeof(double));
+  if (e == cudaSuccess) e = cudaMemsetAsync(m->w, 0, sizeof(uint32_t) * kWords, m->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(m->th, 0, sizeof(float) * kNP, m->stream);
   if (e == cudaSuccess && params)
     e = cudaMemcpyAsync(m->th, params, sizeof(float) * kNP, cudaMemcpyHostToDevice, m->stream);
@@ -557,22 +638,26 @@ air_status air_mlp_train(air_mlp *m, const uint16_t *x, const int32_t *y, int64_
     while (b) { const int64_t r = a % b; a = b; b = r; }
     if (a == 1) { stride = c % (nb > 0 ? nb : 1); if (stride == 0) stride = 1; break; }
   }
+  // the minibatches' losses stay on the device until the epoch ends, so the
+  // host queues one minibatch behind the other without waiting
+  CU_TRY(ensure((void **)&m->hist, &m->hist_b, sizeof(double) * (size_t)nb));
+  std::vector<double> losses;
   for (int e = 0; e < epochs; ++e) {
-    double ep = 0.0;
     for (int64_t q = 0; q < nb; ++q) {
       const int64_t bi = (q * stride + (int64_t)e * 7) % nb;
       const int64_t s0 = bi * batch, cnt = std::min<int64_t>(batch, n - s0);
-      air_status s = mlp_grad(m, x + s0 * kIn, y + s0, cnt);
+      const air_status s = mlp_step(m, x + s0 * kIn, y + s0, cnt, lr, m->hist + q);
       if (s) return s;
-      s = mlp_adam(m, lr);
-      if (s) return s;
-      if (loss_history) {
-        CU_TRY(cudaMemcpyAsync(m->h_loss, m->d_loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-        CU_TRY(cudaStreamSynchronize(m->stream));
-        ep += *m->h_loss;
-      }
     }
-    if (loss_history) loss_history[e] = ep / (double)n;
+    if (loss_history) {
+      losses.resize((size_t)nb);
+      CU_TRY(cudaMemcpyAsync(losses.data(), m->hist, sizeof(double) * (size_t)nb, cudaMemcpyDeviceToHost,
+                             m->stream));
+      CU_TRY(cudaStreamSynchronize(m->stream));
+      double ep = 0.0;
+      for (const double l : losses) ep += l;
+      loss_history[e] = ep / (double)n;
+    }
   }
   CU_TRY(cudaStreamSynchronize(m->stream));
   return AIR_OK;
@@ -583,7 +668,7 @@ void air_mlp_free(air_mlp *m) {
   if (m->stream) cudaStreamSynchronize(m->stream);
   else cudaDeviceSynchronize();
   cudaFree(m->th); cudaFree(m->m); cudaFree(m->v); cudaFree(m->grad); cudaFree(m->partial);
-  cudaFree(m->w); cudaFree(m->d_loss);
+  cudaFree(m->w); cudaFree(m->d_loss); cudaFree(m->hist);
   if (m->h_loss) cudaFreeHost(m->h_loss);
   delete m;
 }
