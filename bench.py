@@ -134,7 +134,8 @@ def oracle_sample_rate(sc, view, n0, budget_s=15.0, chunk=65536, max_rays=1 << 2
     return steps / t_used, done, t_used
 
 
-MARCH_SOURCES = ("air_march.cuh", "air_march.cu", "air_internal.cuh", "air_refine.cuh")
+MARCH_SOURCES = ("air_march.cuh", "air_march_kernel.cuh", "air_march.cu", "air_internal.cuh",
+                 "air_refine.cuh")
 
 
 def march_source_hash():

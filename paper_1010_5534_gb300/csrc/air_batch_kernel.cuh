@@ -1,0 +1,400 @@
+// air_batch_kernel.cuh -- the batched persistent kernel and its launch, as
+// templates over the bands one thread carries; each width is compiled in a
+// translation unit of its own (air_batch_<width>.cu). See air_batch.cu.
+#pragma once
+#include "air_handle.cuh"
+#include "air_march.cuh"
+#include "air_tree.cuh"
+
+namespace air {
+
+typedef cudaError_t (*BatchOccFn)(int *, size_t);
+typedef cudaError_t (*BatchLaunchFn)(const BatchArgs &, int, size_t, cudaStream_t);
+
+constexpr int kBatchBlock = 128;
+constexpr int kBatchMaxViews = 256;
+constexpr uint32_t kErrBalance = 1u, kErrTimeout = 2u, kErrCapacity = 4u;
+
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// Grid barrier with a time limit. `expected` arrivals release it.
+static __device__ bool grid_sync(BatchCtl *ctl, unsigned expected, long long timeout_ns) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ok = 1;
+    volatile unsigned *genp = &ctl->bar_gen;
+    const unsigned gen = *genp;
+    __threadfence();
+    const unsigned arrived = atomicAdd(&ctl->bar_count, 1u) + 1u;
+    if (arrived == expected) {
+      atomicExch(&ctl->bar_count, 0u);
+      __threadfence();
+      atomicAdd(&ctl->bar_gen, 1u);
+    } else {
+      const unsigned long long t0 = global_ns();
+      while (*genp == gen) {
+        if ((long long)(global_ns() - t0) > timeout_ns) {
+          atomicOr(&ctl->err, kErrTimeout);
+          ok = 0;
+          break;
+        }
+        __nanosleep(128);
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+// Items [s0, s1) of one block, in rounds of blockDim. For every selected item
+// k of view v: emit(k, v, run[v] + rank), rank = selected items of view v
+// before k in the block's range. run[] (shared, V entries) advances per round.
+template <class Pred, class Emit>
+__device__ void block_emit_by_view(const Pred &pred, const int16_t *__restrict__ view, Emit &emit,
+                                   int64_t s0, int64_t s1, int V, int64_t *run, int32_t *wcnt) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int64_t r0 = s0; r0 < s1; r0 += blockDim.x) {
+    for (int x = threadIdx.x; x < nw * V; x += blockDim.x) wcnt[x] = 0;
+    __syncthreads();
+    const int64_t k = r0 + threadIdx.x;
+    const bool sel = k < s1 && pred(k);
+    const int v = sel ? (int)view[k] : -1;
+    const unsigned m = __match_any_sync(0xffffffffu, v);
+    const int rank_w = __popc(m & ((1u << lane) - 1u));
+    if (sel && rank_w == 0) wcnt[warp * V + v] = __popc(m);
+    __syncthreads();
+    if (sel) {
+      int64_t before = 0;
+      for (int w = 0; w < warp; ++w) before += wcnt[w * V + v];
+      emit(k, v, run[v] + before + rank_w);
+    }
+    __syncthreads();
+    for (int vv = threadIdx.x; vv < V; vv += blockDim.x) {
+      int64_t s = 0;
+      for (int w = 0; w < nw; ++w) s += wcnt[w * V + vv];
+      run[vv] += s;
+    }
+    __syncthreads();
+  }
+}
+
+struct FlagPred {
+  const uint32_t *flag;
+  __device__ bool operator()(int64_t k) const { return flag[k] != 0; }
+};
+
+struct EmitChildrenV {
+  TreeView t;
+  int16_t *view;
+  const int64_t *vbase;  // shared: first child slot of each view this sweep
+  __device__ void operator()(int64_t k, int v, int64_t rank) {
+    const int64_t c0 = vbase[v] + 4 * rank;
+    const int L = t.lvl[k] + 1, i = t.pi[k], j = t.pj[k];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      t.lvl[c0 + c] = (int8_t)L;
+      t.pi[c0 + c] = 2 * i + (c & 1);
+      t.pj[c0 + c] = 2 * j + (c >> 1);
+      t.child[c0 + c] = -1;
+      view[c0 + c] = (int16_t)v;
+    }
+    t.child[k] = (int32_t)c0;
+  }
+};
+
+// Shared memory of a block: the emission tables of every band chunk, and the
+// per-view counters.
+template <int NBT>
+static size_t batch_smem(const GridView &g, int V) {
+  const size_t tab = g.cell_fmt == kCellXq ? ((g.n_bands + NBT - 1) / NBT) * tab_bytes<NBT>(g.n_tbins) : 0;
+  return tab + 3 * sizeof(int64_t) * V + sizeof(int32_t) * V + sizeof(int32_t) * (kBatchBlock / 32) * V;
+}
+
+// No minimum-blocks bound: with one, the compiler takes more registers (198
+// instead of 152 at 8 bands per thread) and the batch runs slower; bounds of 4
+// and more blocks per SM spill in the refinement phases and run 2.5x slower.
+template <int NBT, bool AMR, int FMT>
+__global__ void __launch_bounds__(kBatchBlock) k_air_batch(BatchArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const GridView &g = a.g;
+  const int V = a.V, nb = g.n_bands;
+  float *tab = (float *)smem_raw;
+  int64_t *run = (int64_t *)(smem_raw + (FMT == kCellXq ? a.chunks * tab_bytes<NBT>(g.n_tbins) : 0));
+  int64_t *tot = run + V;
+  int64_t *vbase = tot + V;
+  int32_t *cnt = (int32_t *)(vbase + V);
+  int32_t *wcnt = cnt + V;
+  __shared__ int64_t s_total;
+  if (FMT == kCellXq)
+    for (int c = 0; c < a.chunks; ++c)
+      tab_fill<NBT>(tab + c * (tab_bytes<NBT>(g.n_tbins) / sizeof(float)), g, c * NBT);
+  __syncthreads();
+
+  const TreeView t = a.t;
+  const int n0 = t.n0;
+  const int64_t nn0 = (int64_t)n0 * n0;
+  const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
+  const unsigned nblk = gridDim.x;
+  const int lane = threadIdx.x & 31;
+
+  // step i: the base image of every view, view-major, row-major within a view
+  // (mode 2 continues from the base images a mode-1 launch traced)
+  const int64_t nbase = (int64_t)V * nn0;
+  if (a.mode != 2) {
+    for (int64_t k = gtid; k < nbase; k += gstride) {
+      const int v = (int)(k / nn0);
+      const int64_t r = k - (int64_t)v * nn0;
+      t.lvl[k] = 0;
+      t.pi[k] = (int32_t)(r % n0);
+      t.pj[k] = (int32_t)(r / n0);
+      t.child[k] = -1;
+      a.view[k] = (int16_t)v;
+    }
+    if (!grid_sync(a.ctl, nblk + (a.stall ? 1u : 0u), a.timeout_ns)) return;
+  }
+
+  int64_t first = a.mode == 2 ? nbase : 0, n = nbase;
+  if (a.mode == 2 && a.P > 0) {
+    // the proposal wave of every view: (ray, band chunk) items from the queue
+    const unsigned long long items = (unsigned long long)a.P * (unsigned long long)a.chunks;
+    for (;;) {
+      unsigned long long b = 0;
+      if (lane == 0) b = atomicAdd(&a.ctl->q_head, 32ull);
+      b = __shfl_sync(0xffffffffu, b, 0);
+      if (b >= items) break;
+      const unsigned long long it = b + lane;
+      if (it < items) {
+        const int chunk = (int)(it / (unsigned long long)a.P);
+        const int64_t q = (int64_t)(it - (unsigned long long)chunk * a.P);
+        const int b0 = chunk * NBT;
+        BandCtx bc;
+        bc.tab = tab + chunk * (tab_bytes<NBT>(g.n_tbins) / sizeof(float));
+        bc.nbh = min(NBT, nb - b0);
+        BandRegs<NBT> br;
+        band_regs<NBT>(br, g.bands, b0, bc.nbh);
+        const RayGeom &rg = a.geoms[a.pview[q]];
+        RTState<NBT> st;
+        trace_ray<NBT, AMR, FMT>(st, g, rg, a.plvl[q], a.ppi[q], a.ppj[q], a.fp64_level, bc, br);
+        if (chunk == 0) {
+          a.pN[q] = st.N;
+          a.psteps[q] = st.steps;
+        }
+#pragma unroll
+        for (int c = 0; c < NBT; ++c)
+          if (c < bc.nbh) a.pI[(int64_t)(b0 + c) * a.P + q] = st.I[c];
+        if (a.chunks == 1) {
+          float p = 0.f;
+#pragma unroll
+          for (int c = 0; c < NBT; ++c)
+            if (c < bc.nbh) p += st.I[c];
+          a.pp[q] = p;
+        }
+      }
+    }
+    if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->q_head = 0ull;
+  }
+  int sweep = 0;
+  for (;; ++sweep) {
+    // step ii: trace the rays added last sweep, all views and band chunks
+    const int64_t cnt_r = n - first;
+    const unsigned long long items = (unsigned long long)cnt_r * (unsigned long long)a.chunks;
+    for (;;) {
+      unsigned long long b = 0;
+      if (lane == 0) b = atomicAdd(&a.ctl->q_head, 32ull);
+      b = __shfl_sync(0xffffffffu, b, 0);
+      if (b >= items) break;
+      const unsigned long long it = b + lane;
+      bool todo = it < items;
+      int chunk = 0, v = 0, b0 = 0;
+      int64_t k = 0;
+      if (todo) {
+        chunk = (int)(it / (unsigned long long)cnt_r);
+        k = first + (int64_t)(it - (unsigned long long)chunk * cnt_r);
+        v = a.view[k];
+        b0 = chunk * NBT;
+      }
+      if (todo && a.mode == 2) {
+        // the pixel's values from its view's proposal wave when the wave
+        // traced it (the same trace, so the same bits); else trace it
+        const int L = t.lvl[k], i = t.pi[k], j = t.pj[k];
+        const int64_t pb = (int64_t)v * nn0 + (int64_t)(j >> L) * n0 + (i >> L);
+        const int64_t q = prop_index(a.pdepth + 4 * pb, a.poff[pb], L, i, j);
+        if (q >= 0) {
+          if (chunk == 0) {
+            t.N[k] = a.pN[q];
+            t.steps[k] = a.psteps[q];
+          }
+          const int nbh = min(NBT, nb - b0);
+          for (int c = 0; c < nbh; ++c) t.I[(int64_t)(b0 + c) * t.cap + k] = a.pI[(int64_t)(b0 + c) * a.P + q];
+          if (a.chunks == 1) t.p[k] = a.pp[q];
+          todo = false;
+        } else if (chunk == 0) {
+          atomicAdd(&a.ctl->fb_rays, 1ull);
+        }
+      }
+      if (todo) {
+        BandCtx bc;
+        bc.tab = tab + chunk * (tab_bytes<NBT>(g.n_tbins) / sizeof(float));
+        bc.nbh = min(NBT, nb - b0);
+        BandRegs<NBT> br;
+        band_regs<NBT>(br, g.bands, b0, bc.nbh);
+        const RayGeom &rg = a.geoms[v];
+        RTState<NBT> st;
+        trace_ray<NBT, AMR, FMT>(st, g, rg, t.lvl[k], t.pi[k], t.pj[k], a.fp64_level, bc, br);
+        if (chunk == 0) {
+          t.N[k] = st.N;
+          t.steps[k] = st.steps;
+          if (a.mode == 1) a.maxlev[k] = (uint8_t)st.maxlev;
+        }
+#pragma unroll
+        for (int q = 0; q < NBT; ++q)
+          if (q < bc.nbh) t.I[(int64_t)(b0 + q) * t.cap + k] = st.I[q];
+        if (a.chunks == 1) {
+          float p = 0.f;
+#pragma unroll
+          for (int q = 0; q < NBT; ++q)
+            if (q < bc.nbh) p += st.I[q];
+          t.p[k] = p;
+        }
+      }
+    }
+    if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->q_head = 0ull;  // next sweep's queue
+    if (a.chunks > 1) {
+      for (int64_t k = first + gtid; k < n; k += gstride) {
+        float s = 0.f;
+        for (int q = 0; q < nb; ++q) s += t.I[(int64_t)q * t.cap + k];
+        t.p[k] = s;
+      }
+      if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
+    }
+    if (a.mode == 1) {
+      // the base images are traced (and their band sums): the host computes
+      // the features and the proposal, then launches mode 2
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctl->n_nodes = n;
+        a.ctl->sweeps = 0;
+      }
+      return;
+    }
+    // step iii: scan, then balance
+    for (int64_t k = gtid; k < n; k += gstride)
+      a.flag[k] = xi_flag(t, NodeLookup{(int)(a.view[k] * nn0), nullptr}, k, a.xi_crit, a.xi_norm, a.refine_on);
+    if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
+    for (int64_t k = gtid; k < n; k += gstride)
+      if (a.flag[k]) balance_from(t, NodeLookup{(int)(a.view[k] * nn0), nullptr}, (int)k, a.flag, &a.ctl->err);
+    if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
+    // step iv: per-view prefix sum over static node ranges
+    const int64_t per = (n + nblk - 1) / nblk;
+    const int64_t s0 = min(n, (int64_t)blockIdx.x * per), s1 = min(n, s0 + per);
+    for (int v = threadIdx.x; v < V; v += blockDim.x) cnt[v] = 0;
+    __syncthreads();
+    for (int64_t k = s0 + threadIdx.x; k < s1; k += blockDim.x)
+      if (a.flag[k]) atomicAdd(&cnt[a.view[k]], 1);
+    __syncthreads();
+    for (int v = threadIdx.x; v < V; v += blockDim.x) a.bcnt[(int64_t)blockIdx.x * V + v] = cnt[v];
+    if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
+    for (int v = threadIdx.x; v < V; v += blockDim.x) {
+      int64_t off = 0, all = 0;
+      for (unsigned b2 = 0; b2 < nblk; ++b2) {
+        const int64_t c = a.bcnt[(int64_t)b2 * V + v];
+        if (b2 < blockIdx.x) off += c;
+        all += c;
+      }
+      run[v] = off;
+      tot[v] = all;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int64_t acc = 0;
+      for (int v = 0; v < V; ++v) {
+        vbase[v] = n + 4 * acc;
+        acc += tot[v];
+      }
+      s_total = acc;
+    }
+    __syncthreads();
+    const int64_t total = s_total;
+    if (total == 0) break;
+    if (n + 4 * total > t.cap) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctl->need = n + 4 * total;
+        atomicOr(&a.ctl->err, kErrCapacity);
+      }
+      break;
+    }
+    EmitChildrenV em{t, a.view, vbase};
+    block_emit_by_view(FlagPred{a.flag}, a.view, em, s0, s1, V, run, wcnt);
+    if (blockIdx.x == 0)
+      for (int v = threadIdx.x; v < V; v += blockDim.x)
+        if (tot[v] > 0) {
+          a.refined[v] += tot[v];
+          a.vsweeps[v] += 1;
+        }
+    if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
+    first = n;
+    n += 4 * total;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    a.ctl->n_nodes = n;
+    a.ctl->sweeps = sweep;
+  }
+}
+
+template <int NBT, bool AMR, int FMT>
+static cudaError_t batch_occupancy(int *blocks_per_sm, size_t smem) {
+  cudaError_t e = cudaFuncSetAttribute(k_air_batch<NBT, AMR, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_air_batch<NBT, AMR, FMT>, kBatchBlock, smem);
+}
+
+template <int NBT, bool AMR, int FMT>
+static cudaError_t batch_launch(const BatchArgs &a, int grid, size_t smem, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kBatchBlock);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_air_batch<NBT, AMR, FMT>, a);
+}
+
+// Occupancy and launch functions and shared memory of the kernel for a grid
+// and V views with NBT bands per thread; false where there is no such form.
+template <int NBT>
+bool batch_fns(const GridView &g, int V, BatchOccFn *occ, BatchLaunchFn *launch, size_t *smem) {
+  const bool amr = g.kind == AIR_GRID_AMR;
+  const int fmt = g.cell_fmt;
+  *smem = batch_smem<NBT>(g, V);
+  if (fmt == kCellLam) {
+    // per-cell Lambda exists for one-band grids only
+    if constexpr (NBT == 1) {
+      *occ = amr ? batch_occupancy<1, true, kCellLam> : batch_occupancy<1, false, kCellLam>;
+      *launch = amr ? batch_launch<1, true, kCellLam> : batch_launch<1, false, kCellLam>;
+      return true;
+    }
+    return false;
+  }
+  if (fmt == kCellXq) {
+    *occ = amr ? batch_occupancy<NBT, true, kCellXq> : batch_occupancy<NBT, false, kCellXq>;
+    *launch = amr ? batch_launch<NBT, true, kCellXq> : batch_launch<NBT, false, kCellXq>;
+  } else {
+    *occ = amr ? batch_occupancy<NBT, true, kCellRho> : batch_occupancy<NBT, false, kCellRho>;
+    *launch = amr ? batch_launch<NBT, true, kCellRho> : batch_launch<NBT, false, kCellRho>;
+  }
+  return true;
+}
+
+}  // namespace air

@@ -173,7 +173,7 @@ void dfree(T *&p) {
 
 void free_grid_impl(air_grid *g) {
   dfree(g->d_cells); dfree(g->d_base); dfree(g->d_oct); dfree(g->d_bmap);
-  dfree(g->d_table); dfree(g->d_kappa); dfree(g->d_invkappa);
+  dfree(g->d_table); dfree(g->d_kappa); dfree(g->d_bands);
   dfree(g->raster.scratch);
   g->raster.ok = false;
   {
@@ -281,7 +281,8 @@ air_status load_grid_impl(const air_grid_desc *d, air_grid *g) {
   // ---- device copies: emission table first (the upload of one-band grids uses it)
   {
     const int ts = v.n_tbins + 1;
-    std::vector<float> tab((size_t)d->n_bands * ts, 0.f), kap(d->n_bands), ik(d->n_bands);
+    std::vector<float> tab((size_t)d->n_bands * ts, 0.f), kap(d->n_bands);
+    std::vector<BandConst> bands(d->n_bands);
     if (d->emis_mode == 1)
       for (int b = 0; b < d->n_bands; ++b) {
         for (int x = 0; x < d->n_tbins; ++x) tab[(size_t)b * ts + x] = d->lambda_table[(size_t)b * d->n_tbins + x];
@@ -289,17 +290,25 @@ air_status load_grid_impl(const air_grid_desc *d, air_grid *g) {
       }
     for (int b = 0; b < d->n_bands; ++b) {
       kap[b] = (float)d->kappa[b];
-      ik[b] = d->kappa[b] > 0.0 ? (float)(1.0 / d->kappa[b]) : 0.f;
+      BandConst &c = bands[b];
+      c.kap = kap[b];
+      c.ik = d->kappa[b] > 0.0 ? (float)(1.0 / d->kappa[b]) : 0.f;
+      c.nk = (float)(-(double)kap[b] * 1.4426950408889634);
+      // the leading bins whose table values are all zero: the interpolated
+      // value is zero up to (and at) the last of them
+      int z = 0;
+      while (d->emis_mode == 1 && z < d->n_tbins && tab[(size_t)b * ts + z] == 0.f) ++z;
+      c.xz = z == 0 ? 0u : ((uint32_t)(z - 1) << kXqFracBits) + 1u;
     }
     CU_TRY(cudaMalloc((void **)&g->d_table, sizeof(float) * tab.size()));
     CU_TRY(cudaMemcpy(g->d_table, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice));
     CU_TRY(cudaMalloc((void **)&g->d_kappa, sizeof(float) * kap.size()));
     CU_TRY(cudaMemcpy(g->d_kappa, kap.data(), sizeof(float) * kap.size(), cudaMemcpyHostToDevice));
-    CU_TRY(cudaMalloc((void **)&g->d_invkappa, sizeof(float) * ik.size()));
-    CU_TRY(cudaMemcpy(g->d_invkappa, ik.data(), sizeof(float) * ik.size(), cudaMemcpyHostToDevice));
+    CU_TRY(cudaMalloc((void **)&g->d_bands, sizeof(BandConst) * bands.size()));
+    CU_TRY(cudaMemcpy(g->d_bands, bands.data(), sizeof(BandConst) * bands.size(), cudaMemcpyHostToDevice));
     v.table = g->d_table;
     v.kappa = g->d_kappa;
-    v.invkappa = g->d_invkappa;
+    v.bands = g->d_bands;
   }
   cudaStream_t st = g->stream;
   v.cell_fmt = d->emis_mode == 0 ? kCellRho : (d->n_bands == 1 ? kCellLam : kCellXq);

@@ -202,7 +202,8 @@ struct air_grid {
   void *d_cells = nullptr;
   int32_t *d_base = nullptr, *d_oct = nullptr;
   int32_t *d_bmap = nullptr;
-  float *d_table = nullptr, *d_kappa = nullptr, *d_invkappa = nullptr;
+  float *d_table = nullptr, *d_kappa = nullptr;
+  air::BandConst *d_bands = nullptr;
   int64_t n_cells = 0;
   air::Workspace ws;
   air::LastRender last;

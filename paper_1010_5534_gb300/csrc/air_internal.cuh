@@ -15,6 +15,14 @@ constexpr int kMapLevelShift = 27;  // brick map entry: id | level << 27
 constexpr int32_t kMapIdMask = (1 << kMapLevelShift) - 1;
 enum { kCellRho = 0, kCellLam = 1, kCellXq = 2 };
 
+// Per-band constants of the march (one 16-byte load).
+struct __align__(16) BandConst {
+  float kap;     // kappa_b
+  float ik;      // 1 / kappa_b (0 where kappa_b = 0)
+  float nk;      // -kappa_b log2(e)
+  uint32_t xz;   // Lambda_b is zero at every table coordinate below xz
+};
+
 // Grid as the kernels see it. Positions are in units of the finest cell
 // (uniform: the cell), F = (x - lo) / h per axis.
 struct GridView {
@@ -41,7 +49,7 @@ struct GridView {
   int emis_mode, n_bands, n_tbins;
   const float *table;   // [n_bands][n_tbins + 1] (last entry repeated)
   const float *kappa;   // [n_bands]
-  const float *invkappa;// [n_bands] (0 where kappa == 0)
+  const BandConst *bands;  // [n_bands]
 };
 
 // Orthographic camera resolved on the host in FP64.

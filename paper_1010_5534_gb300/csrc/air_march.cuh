@@ -32,6 +32,7 @@
 // a Taylor polynomial for dtau < 1/4, and (j/alpha)(T_prev - T_next) above.
 #pragma once
 #include <cfloat>
+#include <cmath>
 
 #include "air_internal.cuh"
 
@@ -43,11 +44,45 @@ struct RTState {
   float T[NBT], I[NBT], cI[NBT];
   uint32_t steps;
   int maxlev;  // deepest brick level crossed
+  // T[] is not that of the current N: cells that emit nothing left it behind.
+  // It is then 2^(nk (tN + tp)), formed as fma(nk, tp, nk tN).
+  bool stale;
+  float tN, tp;
 };
 
+// Emission table of a band chunk in shared memory (kCellXq): per table bin
+// the pairs {Lambda_b, next bin's Lambda_b - Lambda_b} of the chunk's NBT bands
+// side by side, so a cell's look-up is one 16-byte load per two bands and one
+// fused multiply-add per band. (Before: two 4-byte loads from two places and a
+// subtraction per band.) Rows of four and more bands are padded by 16 bytes,
+// so that rows of neighbouring bins start in different banks.
+template <int NBT>
+__host__ __device__ constexpr int tab_row() {  // floats per bin
+  return 2 * NBT + (NBT >= 4 ? 4 : 0);
+}
+template <int NBT>
+__host__ __device__ constexpr size_t tab_bytes(int n_tbins) {
+  return (sizeof(float) * (size_t)(tab_row<NBT>() * n_tbins) + 15) & ~(size_t)15;
+}
+// Fill the table of bands [b0, b0 + NBT) (zero beyond n_bands) by one block.
+template <int NBT>
+__device__ __forceinline__ void tab_fill(float *tab, const GridView &g, int b0) {
+  const int ts = g.n_tbins + 1;
+  for (int x = threadIdx.x; x < NBT * g.n_tbins; x += blockDim.x) {
+    const int k = x / NBT, b = x - k * NBT;
+    float v = 0.f, d = 0.f;
+    if (b0 + b < g.n_bands) {
+      v = g.table[(b0 + b) * ts + k];
+      d = g.table[(b0 + b) * ts + k + 1] - v;
+    }
+    tab[k * tab_row<NBT>() + 2 * b] = v;
+    tab[k * tab_row<NBT>() + 2 * b + 1] = d;
+  }
+}
+
 struct BandCtx {
-  const float *tab;  // shared: [NBT][tstride] (kCellXq)
-  int tstride, nbh;
+  const float *tab;  // shared: the chunk's table (tab_fill)
+  int nbh;
 };
 
 // Per-band constants held in registers for the whole ray.
@@ -57,21 +92,36 @@ struct BandRegs {
   float ik[NBT];   // 1 / kappa_b (0 where kappa_b = 0)
   float nk[NBT];   // -kappa_b log2(e): T_b = 2^(nk_b N)
   float kmax;      // largest kappa_b of the chunk
+  uint32_t xz;     // table coordinates below xz emit nothing in any band (kCellXq)
 };
 
 // Per-band registers of bands [b0, b0 + nbh) (zero beyond).
 template <int NBT>
-__device__ __forceinline__ void band_regs(BandRegs<NBT> &br, const float *kappa,
-                                          const float *invkappa, int b0, int nbh) {
+__device__ __forceinline__ void band_regs(BandRegs<NBT> &br, const BandConst *bands, int b0,
+                                          int nbh) {
+  br.kmax = 0.f;
+  br.xz = 0xffffffffu;
 #pragma unroll
   for (int b = 0; b < NBT; ++b) {
-    br.kap[b] = b < nbh ? __ldg(kappa + b0 + b) : 0.f;
-    br.ik[b] = b < nbh ? __ldg(invkappa + b0 + b) : 0.f;
-    br.nk[b] = (float)(-(double)br.kap[b] * 1.4426950408889634);
+    float4 c = make_float4(0.f, 0.f, -0.f, __uint_as_float(0xffffffffu));
+    if (b < nbh) c = __ldg(reinterpret_cast<const float4 *>(bands + b0 + b));
+    br.kap[b] = c.x;
+    br.ik[b] = c.y;
+    br.nk[b] = c.z;
+    br.xz = min(br.xz, __float_as_uint(c.w));
+    br.kmax = fmaxf(br.kmax, br.kap[b]);
   }
-  br.kmax = 0.f;
-#pragma unroll
-  for (int b = 0; b < NBT; ++b) br.kmax = fmaxf(br.kmax, br.kap[b]);
+}
+
+// Whether a cell emits nothing in any band of the chunk, from its auxiliary
+// word: rho Lambda = 0 (kCellLam), or a table coordinate below which every
+// band's table is zero (kCellXq). Cool gas has no X-ray emission, and most of
+// a grid's volume is cool. Such a cell adds zero to every I_b and only its
+// rho ds to N, so the march leaves the band arithmetic out where the sums'
+// bits allow it (rt_term, march_column).
+template <int FMT>
+__device__ __forceinline__ bool cell_dark(uint32_t aux, uint32_t xz) {
+  return FMT == kCellLam ? aux == 0u : (FMT == kCellXq ? aux < xz : false);
 }
 
 // 2^x by the hardware approximation (PTX ex2.approx.ftz.f32).
@@ -87,6 +137,9 @@ __device__ __forceinline__ void rt_init(RTState<NBT> &r) {
   r.cN = 0.f;
   r.steps = 0;
   r.maxlev = 0;
+  r.stale = false;
+  r.tN = 0.f;
+  r.tp = 0.f;
 #pragma unroll
   for (int b = 0; b < NBT; ++b) {
     r.T[b] = 1.f;
@@ -95,46 +148,100 @@ __device__ __forceinline__ void rt_init(RTState<NBT> &r) {
   }
 }
 
+// T[] brought up to the current N after cells that emit nothing.
+template <int NBT>
+__device__ __forceinline__ void rt_refresh(RTState<NBT> &r, const BandRegs<NBT> &br) {
+#pragma unroll
+  for (int b = 0; b < NBT; ++b)
+    r.T[b] = ex2_approx(fmaf(br.nk[b], r.tp, __fmul_rn(br.nk[b], r.tN)));
+  r.stale = false;
+}
+
+// After dark cells up to N = tN + tp.
+template <int NBT>
+__device__ __forceinline__ void rt_dark(RTState<NBT> &r, float tN, float tp) {
+  if (!r.stale) {
+#pragma unroll
+    for (int b = 0; b < NBT; ++b) kahan_add(r.I[b], r.cI[b], 0.f);
+    r.stale = true;
+  }
+  r.tN = tN;
+  r.tp = tp;
+}
+
+// Lambda of bands 2 q and 2 q + 1 at table row `row` (tab_fill) and weight w.
+template <int NBT>
+__device__ __forceinline__ void tab_pair(const float *row, int q, float w, float &l0, float &l1) {
+  if (NBT == 1) {
+    const float2 t = *reinterpret_cast<const float2 *>(row);
+    l0 = fmaf(w, t.y, t.x);
+  } else {
+    const float4 t = *reinterpret_cast<const float4 *>(row + 4 * q);
+    l0 = fmaf(w, t.y, t.x);
+    l1 = fmaf(w, t.w, t.z);
+  }
+}
+
 // Transfer step of one cell chord of length ds: density rho, and aux =
 // rho Lambda (kCellLam, as float bits) or the table coordinate of T (kCellXq).
 // With dtau = 0 (kappa_b = 0 or rho = 0) the series form gives the optically
 // thin term j ds T exactly, so no separate case is needed.
 // Both forms of the cell term are evaluated and the one for the cell's dtau
-// is selected, which keeps the loop free of divergent branches.
+// is selected, which keeps the band loop free of divergent branches.
+//
+// A cell that emits nothing (cell_dark) leaves I_b and T_b out. Adding its
+// zero term can change a compensated sum once (it moves a residue that is
+// not yet below half an ulp into the sum) and never again, so the zero is
+// added at the first dark cell after an emitting one and skipped at the rest;
+// T_b is formed at the next emitting cell from N, as it would have been. (One
+// band: the zero is added and T formed each time, six operations.)
+// Where N overflows, every cell takes the full path. All bits are those of
+// the full path.
 //
 // The products that feed the compensated sums (rho ds, and each form's final
 // product) are rounded explicitly (__fmul_rn), so the compiler cannot fuse
 // them into the sums' subtractions: every instantiation (band chunking, form)
 // rounds alike and gives the same bits.
-template <int NBT, int FMT>
+// DARK = false: without the test (for one-band callers that have made it).
+template <int NBT, int FMT, bool DARK = true>
 __device__ __forceinline__ void rt_term(RTState<NBT> &r, float rho, uint32_t aux, float ds,
                                         const BandCtx &bc, const BandRegs<NBT> &br) {
   const float rds = __fmul_rn(rho, ds);
   kahan_add(r.N, r.cN, rds);
-  int k = 0;
-  float w = 0.f, lam1 = 1.f;
+  if (DARK && FMT != kCellRho && cell_dark<FMT>(aux, br.xz) && r.N <= FLT_MAX) {
+    if (NBT == 1) {
+      kahan_add(r.I[0], r.cI[0], 0.f);
+      r.T[0] = ex2_approx(br.nk[0] * r.N);
+    } else {
+      rt_dark<NBT>(r, r.N, 0.f);
+    }
+    return;
+  }
+  if (FMT != kCellRho && NBT > 1 && r.stale) rt_refresh<NBT>(r, br);
+  float w = 0.f;
+  const float *row = bc.tab;
   if (FMT == kCellXq) {
-    k = (int)(aux >> kXqFracBits);
+    row += (int)(aux >> kXqFracBits) * tab_row<NBT>();
     w = (float)(aux & ((1u << kXqFracBits) - 1u)) * (1.0f / (float)(1u << kXqFracBits));
-  } else if (FMT == kCellLam) {
-    lam1 = __uint_as_float(aux);
   }
 #pragma unroll
-  for (int b = 0; b < NBT; ++b) {
-    if (NBT == 1 || b < bc.nbh) {
-      float lam = lam1;
-      if (FMT == kCellXq) {
-        const float *t = bc.tab + b * bc.tstride + k;
-        lam = fmaf(w, t[1] - t[0], t[0]);
+  for (int q = 0; q < (NBT + 1) / 2; ++q) {
+    if (NBT <= 2 || 2 * q < bc.nbh) {
+      float lam[2] = {1.f, 1.f};
+      if (FMT == kCellXq) tab_pair<NBT>(row, q, w, lam[0], lam[1]);
+#pragma unroll
+      for (int e = 0; e < (NBT == 1 ? 1 : 2); ++e) {
+        const int b = 2 * q + e;
+        const float dtau = br.kap[b] * rds;
+        const float Tn = ex2_approx(br.nk[b] * r.N);
+        // rho Lambda_b
+        const float rl = FMT == kCellLam ? __uint_as_float(aux) : (FMT == kCellXq ? rho * lam[e] : rho);
+        const float t_small = __fmul_rn(rl * rds, r.T[b] * one_minus_exp_over_x(dtau));
+        const float t_large = __fmul_rn(rl * br.ik[b], r.T[b] - Tn);
+        const float term = dtau < 0.25f ? t_small : t_large;
+        r.T[b] = Tn;
+        kahan_add(r.I[b], r.cI[b], term);
       }
-      const float dtau = br.kap[b] * rds;
-      const float Tn = ex2_approx(br.nk[b] * r.N);
-      const float rl = FMT == kCellLam ? lam1 : rho * lam;  // rho Lambda_b
-      const float t_small = __fmul_rn(rl * rds, r.T[b] * one_minus_exp_over_x(dtau));
-      const float t_large = __fmul_rn(rl * br.ik[b], r.T[b] - Tn);
-      const float term = dtau < 0.25f ? t_small : t_large;
-      r.T[b] = Tn;
-      kahan_add(r.I[b], r.cI[b], term);
     }
   }
 }
@@ -151,8 +258,12 @@ __device__ __forceinline__ void rt_cell(RTState<NBT> &r, float rho, uint32_t aux
   rt_term<NBT, FMT>(r, rho, aux, ds, bc, br);
 }
 
-// Cells of a block requested ahead of the march along its dominant axis.
-constexpr int kPrefetchAhead = 3;
+// Cells that the DDA steps through, and requests, before it sums the first of
+// them (march_block).
+template <int NBT>
+struct DdaChunk {
+  static constexpr int value = 4;
+};
 
 // Fields of cell idx: rho and the auxiliary word of the format.
 template <int FMT, typename Idx>
@@ -201,6 +312,7 @@ __device__ __forceinline__ float one_minus_exp_over_x_short(float x) {
 // instantiations are few enough to afford another form;
 // FORM 2: below 1/64 (the short series); FORM 1: below 1/4 (the full series);
 // FORM 0: the form is selected per cell and band.
+// rh: the cells' rho, or their rho ds already formed (kCellLam).
 template <int NBT, int FMT, int FORM, int U>
 __device__ __forceinline__ void column_group(RTState<NBT> &r, const float (&rh)[U],
                                              const uint32_t (&xv)[U], float ds, const BandCtx &bc,
@@ -216,26 +328,22 @@ __device__ __forceinline__ void column_group(RTState<NBT> &r, const float (&rh)[
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const float rho = rh[u];
-    const float rds = __fmul_rn(rho, ds);
+    const float rds = FMT == kCellLam ? rho : __fmul_rn(rho, ds);
     pN = __fadd_rn(pN, rds);
-    int k = 0;
-    float w = 0.f, lam1 = 1.f;
+    float w = 0.f;
+    const float *row = bc.tab;
     if (FMT == kCellXq) {
-      k = (int)(xv[u] >> kXqFracBits);
+      row += (int)(xv[u] >> kXqFracBits) * tab_row<NBT>();
       w = (float)(xv[u] & ((1u << kXqFracBits) - 1u)) * (1.0f / (float)(1u << kXqFracBits));
-    } else if (FMT == kCellLam) {
-      lam1 = __uint_as_float(xv[u]);
     }
+    float lam[2] = {1.f, 1.f};
 #pragma unroll
     for (int b = 0; b < NBT; ++b) {
-      if (NBT == 1 || b < bc.nbh) {
-        float lam = lam1;
-        if (FMT == kCellXq) {
-          const float *t = bc.tab + b * bc.tstride + k;
-          lam = fmaf(w, t[1] - t[0], t[0]);
-        }
+      if (NBT <= 2 || (b & ~1) < bc.nbh) {
+        if (FMT == kCellXq && (b & 1) == 0) tab_pair<NBT>(row, b >> 1, w, lam[0], lam[1]);
         const float Tn = ex2_approx(fmaf(br.nk[b], pN, nN0[b]));
-        const float rl = FMT == kCellLam ? lam1 : __fmul_rn(rho, lam);  // rho Lambda_b
+        // rho Lambda_b
+        const float rl = FMT == kCellLam ? __uint_as_float(xv[u]) : __fmul_rn(rho, lam[b & 1]);
         float P, Q;
         if (FORM == 3) {
           // T (1 - dtau / 2) with dtau = kappa_b (rho ds)
@@ -266,17 +374,77 @@ __device__ __forceinline__ void column_group(RTState<NBT> &r, const float (&rh)[
   kahan_add(r.N, r.cN, pN);
 #pragma unroll
   for (int b = 0; b < NBT; ++b)
-    if (NBT == 1 || b < bc.nbh) kahan_add(r.I[b], r.cI[b], pI[b]);
+    if (NBT <= 2 || (b & ~1) < bc.nbh) kahan_add(r.I[b], r.cI[b], pI[b]);
+}
+
+// A group whose cells all emit nothing: N alone, summed as column_group sums
+// it; its zero partial sums change I_b as theirs do (once after an emitting
+// group or cell, see rt_term), and T_b waits for the next emitting group.
+// False where N overflows: the caller then takes the full path.
+template <int NBT, int FMT, int U>
+__device__ __forceinline__ bool column_group_dark(RTState<NBT> &r, const float (&rh)[U], float ds,
+                                                  const BandRegs<NBT> &br) {
+  float pN = 0.f;
+#pragma unroll
+  for (int u = 0; u < U; ++u) pN = __fadd_rn(pN, FMT == kCellLam ? rh[u] : __fmul_rn(rh[u], ds));
+  // N + pN plus the compensation is finite if twice the larger sum is
+  if (!(r.N + pN <= 0.5f * FLT_MAX)) return false;
+  if (NBT == 1) {
+    kahan_add(r.I[0], r.cI[0], 0.f);
+    r.T[0] = ex2_approx(fmaf(br.nk[0], pN, __fmul_rn(br.nk[0], r.N)));
+  } else {
+    rt_dark<NBT>(r, r.N, pN);
+  }
+  kahan_add(r.N, r.cN, pN);
+  return true;
+}
+
+// Largest of U non-negative floats (their bits compare as integers; three
+// operands per instruction).
+template <int U>
+__device__ __forceinline__ float max_of(const float (&v)[U]) {
+  int m = __float_as_int(v[0]);
+#pragma unroll
+  for (int u = 1; u + 1 < U; u += 2) m = __vimax3_s32(m, __float_as_int(v[u]), __float_as_int(v[u + 1]));
+  if (U % 2 == 0) m = max(m, __float_as_int(v[U - 1]));
+  return __int_as_float(m);
+}
+
+// One group of U column cells, fetched into rh and xv: the dark path, or the
+// transfer form chosen from kmax (rho_max ds) for the group's largest rho,
+// which bounds every cell's dtau = kappa_b (rho ds) (FP32 rounding is
+// monotonic).
+template <int NBT, int FMT, int U>
+__device__ __forceinline__ void column_cells(RTState<NBT> &r, float (&rh)[U],
+                                             const uint32_t (&xv)[U], float ds, const BandCtx &bc,
+                                             const BandRegs<NBT> &br) {
+  if (FMT == kCellLam) {
+    // only rho ds is used from here on (the record holds rho Lambda)
+#pragma unroll
+    for (int u = 0; u < U; ++u) rh[u] = __fmul_rn(rh[u], ds);
+  }
+  if (FMT != kCellRho) {
+    uint32_t x = xv[0];
+#pragma unroll
+    for (int u = 1; u < U; ++u) x = FMT == kCellLam ? x | xv[u] : max(x, xv[u]);
+    if (cell_dark<FMT>(x, br.xz) && column_group_dark<NBT, FMT, U>(r, rh, ds, br)) return;
+    if (NBT > 1 && r.stale) rt_refresh<NBT>(r, br);
+  }
+  const float m = max_of<U>(rh);
+  const float dmax = br.kmax * (FMT == kCellLam ? m : __fmul_rn(m, ds));
+  if (FMT == kCellLam && dmax < 0x1p-12f) column_group<NBT, FMT, 3, U>(r, rh, xv, ds, bc, br);
+  else if (dmax < 0.015625f) column_group<NBT, FMT, 2, U>(r, rh, xv, ds, bc, br);
+  else if (dmax < 0.25f) column_group<NBT, FMT, 1, U>(r, rh, xv, ds, bc, br);
+  else column_group<NBT, FMT, 0, U>(r, rh, xv, ds, bc, br);
 }
 
 // n cells of one column (cell idx, idx + d, ...), every one crossed whole
 // with the same chord ds: the path of a ray parallel to a grid axis, which
 // enters each block of cells through a face and leaves through the opposite
 // one. No DDA is needed. Cells are fetched U at a time (U loads in flight per
-// thread) and summed as a group (column_group); the transfer form is chosen
-// per group from kmax (rho_max ds) for the group's largest rho, which bounds
-// every cell's dtau = kappa_b (rho ds) (FP32 rounding is monotonic).
-template <int NBT, int FMT, int U, typename Idx>
+// thread) and summed as a group (column_cells).
+// TAIL = false: n is known to be a multiple of U.
+template <int NBT, int FMT, int U, bool TAIL, typename Idx>
 __device__ __forceinline__ void march_column(RTState<NBT> &r, const void *__restrict__ cells, Idx idx,
                                              Idx d, int n, float ds, const BandCtx &bc,
                                              const BandRegs<NBT> &br) {
@@ -288,22 +456,50 @@ __device__ __forceinline__ void march_column(RTState<NBT> &r, const void *__rest
 #pragma unroll
     for (int u = 0; u < U; ++u) load_cell<FMT>(cells, idx + (Idx)u * d, rh[u], xv[u]);
     idx += (Idx)U * d;
-    float m = rh[0];
+    column_cells<NBT, FMT, U>(r, rh, xv, ds, bc, br);
+  }
+  // the rest (all of a brick of fewer than U cells) one by one, fetched 4 at
+  // a time (8 at a time spilled 240 bytes in the one-axis kernels)
+  for (; TAIL && k < n; k += 4) {
+    float rh[4];
+    uint32_t xv[4];
 #pragma unroll
-    for (int u = 1; u < U; ++u) m = fmaxf(m, rh[u]);
-    const float dmax = br.kmax * __fmul_rn(m, ds);
-    if (FMT == kCellLam && dmax < 0x1p-12f) column_group<NBT, FMT, 3, U>(r, rh, xv, ds, bc, br);
-    else if (dmax < 0.015625f) column_group<NBT, FMT, 2, U>(r, rh, xv, ds, bc, br);
-    else if (dmax < 0.25f) column_group<NBT, FMT, 1, U>(r, rh, xv, ds, bc, br);
-    else column_group<NBT, FMT, 0, U>(r, rh, xv, ds, bc, br);
+    for (int u = 0; u < 4; ++u)
+      if (k + u < n) load_cell<FMT>(cells, idx + (Idx)u * d, rh[u], xv[u]);
+    idx += (Idx)4 * d;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (k + u < n) rt_term<NBT, FMT>(r, rh[u], xv[u], ds, bc, br);
   }
-  for (; k < n; ++k) {
-    float rh;
-    uint32_t xv;
-    load_cell<FMT>(cells, idx, rh, xv);
-    idx += d;
-    rt_term<NBT, FMT>(r, rh, xv, ds, bc, br);
+}
+
+// The column of a 16^3 brick along axis A (16 cells, one group), at cells =
+// its lowest cell: strides are constants here, so the 16 loads need no address
+// arithmetic, and along x a load takes two records. Integer instructions issue
+// at half the rate of FP32 ones on this GPU and bound the general form (78% of
+// their peak; 48 of a group's 260 instructions formed addresses).
+template <int NBT, int FMT, int A, bool POS>
+__device__ __forceinline__ void march_column16(RTState<NBT> &r, const void *__restrict__ cells,
+                                               float ds, const BandCtx &bc, const BandRegs<NBT> &br) {
+  constexpr int st = A == 0 ? 1 : (A == 1 ? 16 : 256);
+  float rh[16];
+  uint32_t xv[16];
+  r.steps += 16u;
+  if (A == 0 && FMT != kCellRho) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const uint4 c = __ldg((const uint4 *)cells + u);
+      const int p = POS ? 2 * u : 15 - 2 * u, q = POS ? 2 * u + 1 : 14 - 2 * u;
+      rh[p] = __uint_as_float(c.x);
+      xv[p] = c.y;
+      rh[q] = __uint_as_float(c.z);
+      xv[q] = c.w;
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < 16; ++u) load_cell<FMT>(cells, (POS ? u : 15 - u) * st, rh[u], xv[u]);
   }
+  column_cells<NBT, FMT, 16>(r, rh, xv, ds, bc, br);
 }
 
 // Cells fetched per group in the column march: 16 in the compiled one-axis
@@ -328,20 +524,20 @@ struct ColumnUnroll {
 // parameter does not grow with the number of cells marched. Parameters are
 // measured from the entry cell, so their FP32 rounding scales with the
 // distance marched inside the block, not with the ray's distance from the
-// origin. The fields of the next cell are fetched before the current cell's
-// transfer step, so the load latency overlaps that arithmetic, and the cell
-// kPrefetchAhead steps further along the axis the ray crosses fastest is
-// requested from L1 at every step (clamped into the block), so most loads
-// find their line already on the way. The loop body is straight-line code
-// (the axis to step, the next index and the transfer form are selected, not
-// branched on); its one branch is the exit from the block.
+// origin.
+//
+// Which cells a ray crosses does not depend on their fields, so the walk runs
+// DdaChunk cells ahead of the sums: it steps through a chunk of cells, asking
+// for each record as its index is known, and only then sums the chunk. One
+// load latency is paid per chunk instead of one per cell, and the step's own
+// dependent operations overlap the loads.
 template <int NBT, int FMT, typename Idx>
 __device__ __forceinline__ void march_block(RTState<NBT> &r, const float Q[3], const float Dl[3],
                                             const float inv[3], float tend, int lx, int ly, int lz,
                                             int nx, int ny, int nz, Idx sy, Idx sz,
                                             const void *__restrict__ cells, const BandCtx &bc,
                                             const BandRegs<NBT> &br) {
-  {
+  constexpr int K = DdaChunk<NBT>::value;
   const float INF = FLT_MAX;
   const bool p0 = Dl[0] > 0.f, p1 = Dl[1] > 0.f, p2 = Dl[2] > 0.f;
   const float a0 = fabsf(inv[0]), a1 = fabsf(inv[1]), a2 = fabsf(inv[2]);
@@ -356,49 +552,42 @@ __device__ __forceinline__ void march_block(RTState<NBT> &r, const float Q[3], c
   float k0 = 0.f, k1 = 0.f, k2 = 0.f;
   float tm0 = q0, tm1 = q1, tm2 = q2;
   Idx idx = (Idx)lz * sz + (Idx)ly * sy + (Idx)lx;
-  const float e0 = fabsf(Dl[0]), e1 = fabsf(Dl[1]), e2 = fabsf(Dl[2]);
-  const Idx pstep = (e0 >= e1 && e0 >= e2) ? d0 : (e1 >= e2 ? d1 : d2);
-  const Idx plast = (Idx)nz * sz - 1;
-  float rh;
-  uint32_t xv;
-  load_cell<FMT>(cells, idx, rh, xv);
-#pragma unroll
-  for (int n = 2; n <= kPrefetchAhead; ++n) {
-    const Idx pi = idx + (Idx)n * pstep;
-    prefetch_cell<FMT>(cells, pi < 0 ? (Idx)0 : (pi > plast ? plast : pi));
-  }
   float tl = 0.f;
-  for (;;) {
-    const float tn = fminf(fminf(tm0, tm1), fminf(tm2, tend));
-    const float ds = fmaxf(tn - tl, 0.f);
-    tl = tn;
-    // step the axis whose face comes first (selects, no branches); an axis
-    // that is not stepped keeps its count and so its boundary parameter
-    const bool x0 = tm0 <= tm1 && tm0 <= tm2;
-    const bool x1 = !x0 && tm1 <= tm2;
-    const bool x2 = !x0 && !x1;
-    k0 += x0 ? 1.f : 0.f;
-    k1 += x1 ? 1.f : 0.f;
-    k2 += x2 ? 1.f : 0.f;
-    tm0 = fmaf(k0, a0, q0);
-    tm1 = fmaf(k1, a1, q1);
-    tm2 = fmaf(k2, a2, q2);
-    const bool more = tn < tend && k0 <= km0 && k1 <= km1 && k2 <= km2;
-    const Idx nidx = idx + (x0 ? d0 : (x1 ? d1 : d2));
-    idx = more ? nidx : idx;  // past the block: reload the current cell (no use)
-    float rh_n;
-    uint32_t xv_n;
-    load_cell<FMT>(cells, idx, rh_n, xv_n);
-    if (kPrefetchAhead > 1) {
-      const Idx pi = idx + (Idx)kPrefetchAhead * pstep;
-      prefetch_cell<FMT>(cells, pi < 0 ? (Idx)0 : (pi > plast ? plast : pi));
+  bool more = true;
+  do {
+    float ds[K], rh[K];
+    uint32_t xv[K];
+    bool in[K];  // cell u of the chunk lies in the block
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+      in[u] = more;
+      if (more) load_cell<FMT>(cells, idx, rh[u], xv[u]);
+      const float tn = fminf(fminf(tm0, tm1), fminf(tm2, tend));
+      ds[u] = fmaxf(tn - tl, 0.f);
+      tl = tn;
+      // step the axis whose face comes first; an axis that is not stepped
+      // keeps its count and so its boundary parameter
+      const bool x0 = tm0 <= tm1 && tm0 <= tm2;
+      const bool x1 = !x0 && tm1 <= tm2;
+      if (x0) {
+        k0 += 1.f;
+        tm0 = fmaf(k0, a0, q0);
+        idx += d0;
+      } else if (x1) {
+        k1 += 1.f;
+        tm1 = fmaf(k1, a1, q1);
+        idx += d1;
+      } else {
+        k2 += 1.f;
+        tm2 = fmaf(k2, a2, q2);
+        idx += d2;
+      }
+      more = more && tn < tend && k0 <= km0 && k1 <= km1 && k2 <= km2;
     }
-    rt_cell<NBT, FMT>(r, rh, xv, ds, bc, br);
-    if (!more) break;  // left the block (through its far face, or by rounding)
-    rh = rh_n;
-    xv = xv_n;
-  }
-  }
+#pragma unroll
+    for (int u = 0; u < K; ++u)
+      if (in[u]) rt_cell<NBT, FMT>(r, rh[u], xv[u], ds[u], bc, br);
+  } while (more);  // until the block is left (through its far face, or by rounding)
 }
 
 // Per-launch ray geometry, resolved on the host in FP64: the pixel centre
@@ -412,6 +601,10 @@ struct RayGeom {
   float invDhi[3];       // 1 / Dhi, correctly rounded (0 where D = 0); for a
                          // brick at 2^s finest cells per cell, 1 / (Dhi 2^-s)
                          // is exactly invDhi 2^s
+  // FP32 copies for what FP32 can decide: the grid coordinate of a pixel
+  // centre is fO + uc fU + vc fV to within eO finest cells (eO infinite where
+  // these numbers are too large or too small for FP32)
+  float fO[3], fU[3], fV[3], eO[3], fH, fpix0;
   // Axis views whose u and v are grid axes too: the cell of every pixel
   // column on each fixed axis, from axis_table_entry (exactly the set-up's
   // FP64 operations, once per column instead of once per ray), or NULL.
@@ -435,8 +628,18 @@ __device__ __forceinline__ double exp2_neg(int L) {
 // The grid coordinate x / h is the correctly rounded quotient (a product with
 // 1/h and one residual correction), so a pixel centre that lies exactly on a
 // cell face maps exactly onto it, and the half-open rule picks the higher cell.
-__device__ __forceinline__ bool ray_setup(const GridView &g, const RayGeom &rg, int L, int i,
-                                          int j, double O[3], double &t0, int &eax) {
+//
+// FP64 costs this GPU 16 SM cycles per warp instruction and 67 cycles of
+// latency, conversions to and from FP64 as much as arithmetic, against a
+// quarter of a cycle for FP32 (measured). So FP64 is kept to the values that
+// are used; what only decides is decided in FP32 where a bound on its error
+// allows: whether the ray misses the box, through which face it enters, and
+// that it enters before it leaves. What FP32 leaves open goes to
+// ray_setup_full, so every result has the bits of that path. About 30 FP64
+// instructions instead of 80 for a ray that hits the box, none for most rays
+// that miss it.
+static __device__ __noinline__ bool ray_setup_full(const GridView &g, const RayGeom &rg, int L, int i,
+                                                  int j, double O[3], double &t0, int &eax) {
   const double pix = rg.pix0 * exp2_neg(L);
   const double uc = fma((double)i + 0.5, pix, -rg.H);
   const double vc = fma((double)j + 0.5, pix, -rg.H);
@@ -470,6 +673,103 @@ __device__ __forceinline__ bool ray_setup(const GridView &g, const RayGeom &rg, 
 
 __device__ __forceinline__ int clampi(int x, int lo, int hi) { return x < lo ? lo : (x > hi ? hi : x); }
 
+// Exact FP64 value of a finite float by integer operations (zeros and
+// subnormals by a conversion).
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t u = __float_as_uint(f), m = u & 0x7fffffffu;
+  if (m < 0x00800000u) return (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+}
+// Exact FP64 value of an integer.
+__device__ __forceinline__ double widen_int(int n) {
+  return abs(n) < (1 << 24) ? widen((float)n) : (double)n;
+}
+__device__ __forceinline__ double pick(int a, double x0, double x1, double x2) {
+  return a == 0 ? x0 : (a == 1 ? x1 : x2);
+}
+
+// Double-float values (unevaluated sums of two FP32 numbers).
+struct F2 {
+  float hi, lo;
+};
+__device__ __forceinline__ F2 f2_from(double x) {
+  F2 r;
+  r.hi = (float)x;
+  r.lo = (float)(x - widen(r.hi));
+  return r;
+}
+
+// Of: O as double-floats.
+__device__ __forceinline__ bool ray_setup(const GridView &g, const RayGeom &rg, int L, int i, int j,
+                                          double O[3], F2 Of[3], double &t0, int &eax) {
+  const float ic = (float)i + 0.5f, jc = (float)j + 0.5f;  // exact: i, j < 2^20
+  {
+    // the box widened by the error of the pixel centre's coordinate; 2^-20
+    // relative covers the roundings of each parameter (16 units, 5 occur)
+    const float pix = rg.fpix0 * __int_as_float((127 - L) << 23);
+    const float uc = fmaf(ic, pix, -rg.fH), vc = fmaf(jc, pix, -rg.fH);
+    float tin = -FLT_MAX, tout = FLT_MAX;
+    bool miss = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const float o = fmaf(vc, rg.fV[a], fmaf(uc, rg.fU[a], rg.fO[a]));
+      const float nf = (float)g.nf[a];
+      const float e = fmaf(nf, 0x1p-20f, rg.eO[a]);
+      if (rg.Dhi[a] == 0.f) {
+        miss = miss || o < -e || o > nf + e;
+      } else {
+        const float ta = (-e - o) * rg.invDhi[a], tb = (nf + e - o) * rg.invDhi[a];
+        const float x = fminf(ta, tb), y = fmaxf(ta, tb);
+        tin = fmaxf(tin, x - fabsf(x) * 0x1p-20f);
+        tout = fminf(tout, y + fabsf(y) * 0x1p-20f);
+      }
+    }
+    if (miss || tin > tout) return false;
+  }
+  const double pix = rg.pix0 * exp2_neg(L);
+  const double uc = fma(widen(ic), pix, -rg.H);
+  const double vc = fma(widen(jc), pix, -rg.H);
+  // bounds lo <= entry parameter <= hi per axis, and on the exit
+  float lo[3], hi[3], tout = FLT_MAX;
+  bool clear = true;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const double x = fma(vc, rg.V[a], fma(uc, rg.U[a], rg.C[a]));
+    const double q = x * rg.invh[a];
+    O[a] = fma(fma(-q, rg.h[a], x), rg.invh[a], q);
+    Of[a] = f2_from(O[a]);
+    const float nf = (float)g.nf[a], o = Of[a].hi;
+    lo[a] = hi[a] = -FLT_MAX;
+    if (rg.Dhi[a] == 0.f) {
+      clear = clear && o > nf * 0x1p-20f && o < nf - nf * 0x1p-20f;
+    } else {
+      const float ta = -o * rg.invDhi[a], tb = (nf - o) * rg.invDhi[a];
+      const float err = (nf + fabsf(o)) * fabsf(rg.invDhi[a]) * 0x1p-20f;
+      lo[a] = fminf(ta, tb) - err;
+      hi[a] = fminf(ta, tb) + err;
+      tout = fminf(tout, fmaxf(ta, tb) - err);
+    }
+  }
+  eax = lo[0] > hi[1] && lo[0] > hi[2] ? 0 : (lo[1] > hi[0] && lo[1] > hi[2] ? 1 : 2);
+  const float tlo = eax == 0 ? lo[0] : (eax == 1 ? lo[1] : lo[2]);
+  const float thi = eax == 0 ? hi[0] : (eax == 1 ? hi[1] : hi[2]);
+  const float other = eax == 0 ? fmaxf(hi[1], hi[2]) : (eax == 1 ? fmaxf(hi[0], hi[2]) : fmaxf(hi[0], hi[1]));
+  if (!(clear && tlo > other && thi < tout)) {
+    double Ox[3], tx;  // of their own, so that O stays in registers
+    int ex;
+    const bool hit = ray_setup_full(g, rg, L, i, j, Ox, tx, ex);
+    t0 = tx;
+    eax = ex;
+    return hit;
+  }
+  const float De = eax == 0 ? rg.Dhi[0] : (eax == 1 ? rg.Dhi[1] : rg.Dhi[2]);
+  const int ne = eax == 0 ? g.nf[0] : (eax == 1 ? g.nf[1] : g.nf[2]);
+  const double Oe = pick(eax, O[0], O[1], O[2]);
+  const double dist = De > 0.f ? -Oe : widen_int(ne) - Oe;
+  t0 = dist * pick(eax, rg.invD[0], rg.invD[1], rg.invD[2]);
+  return true;
+}
+
 // ray_setup for a ray along grid axis A: only the two fixed coordinates are
 // needed (the ray enters at the grid face and crosses every cell of its
 // column), computed exactly as ray_setup computes them, so the cells are the
@@ -480,43 +780,41 @@ __device__ __forceinline__ int clampi(int x, int lo, int hi) { return x < lo ? l
 // and v are grid axes, x_a depends on one pixel index only (the other term is
 // an exact zero), and the table holds this function's result for every
 // column (axis_table_entry), so the cells are the same bits.
-template <int A>
-__device__ __noinline__ unsigned long long axis_cells_fp64(const GridView &g, const RayGeom &rg,
-                                                           int L, int i, int j);
+//
+// A is a constant where the kernel is compiled for one axis; the kernels for
+// any direction hold one copy of this code and pass the view's axis.
+static __device__ __noinline__ unsigned long long axis_cells_fp64(const GridView &g, const RayGeom &rg,
+                                                           int A, int L, int i, int j);
 
-template <int A>
-__device__ __forceinline__ bool axis_ray_setup(const GridView &g, const RayGeom &rg, int L, int i,
-                                               int j, int c[3]) {
+// Cells on axes (A + 1) % 3 and (A + 2) % 3; false where the ray misses.
+__device__ __forceinline__ bool axis_ray_setup(const GridView &g, const RayGeom &rg, int A, int L,
+                                               int i, int j, int &c1, int &c2) {
   if (rg.tab) {
     const int o = rg.tab_n0 * ((1 << L) - 1);
-    const int c1 = __ldg(rg.tab + o + ((rg.tab_byj & 1) ? j : i));
-    const int c2 = __ldg(rg.tab + rg.tab_slot + o + ((rg.tab_byj & 2) ? j : i));
-    c[(A + 1) % 3] = c1;
-    c[(A + 2) % 3] = c2;
+    c1 = __ldg(rg.tab + o + ((rg.tab_byj & 1) ? j : i));
+    c2 = __ldg(rg.tab + rg.tab_slot + o + ((rg.tab_byj & 2) ? j : i));
     return c1 >= 0 && c2 >= 0;
   }
   // a separate function, so that none of its FP64 work is executed ahead of
   // the branch on views that have a table
-  const unsigned long long cc = axis_cells_fp64<A>(g, rg, L, i, j);
-  const int c1 = (int)(uint32_t)cc, c2 = (int)(uint32_t)(cc >> 32);
-  c[(A + 1) % 3] = c1;
-  c[(A + 2) % 3] = c2;
+  const unsigned long long cc = axis_cells_fp64(g, rg, A, L, i, j);
+  c1 = (int)(uint32_t)cc;
+  c2 = (int)(uint32_t)(cc >> 32);
   return c1 >= 0 && c2 >= 0;
 }
 
 // The two fixed cells of pixel (L, i, j)'s ray along axis A in FP64: cell on
 // axis (A + 1) % 3 in the low word, on (A + 2) % 3 in the high word, -1 where
 // the ray misses the grid on that axis.
-template <int A>
-__device__ __noinline__ unsigned long long axis_cells_fp64(const GridView &g, const RayGeom &rg,
-                                                           int L, int i, int j) {
+static __device__ __noinline__ unsigned long long axis_cells_fp64(const GridView &g, const RayGeom &rg,
+                                                           int A, int L, int i, int j) {
   const double pix = rg.pix0 * exp2_neg(L);
   const double uc = fma((double)i + 0.5, pix, -rg.H);
   const double vc = fma((double)j + 0.5, pix, -rg.H);
   int c[2];
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
-    const int a = (A + 1 + s) % 3;
+    const int a0 = A + 1 + s, a = a0 >= 3 ? a0 - 3 : a0;
     const double x = fma(vc, rg.V[a], fma(uc, rg.U[a], rg.C[a]));
     const double q = __dmul_rn(x, rg.invh[a]);
     const double o = fma(fma(-q, rg.h[a], x), rg.invh[a], q);
@@ -548,29 +846,26 @@ __device__ void march_uniform(RTState<NBT> &r, const GridView &g, const double O
   int lc[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const double F = O[a] + t0 * rg.D[a];
-    lc[a] = clampi((int)floor(F), 0, g.nf[a] - 1);
-    Q[a] = (float)(F - (double)lc[a]);
+    const double F = fma(t0, rg.D[a], O[a]);
+    lc[a] = clampi(__double2int_rd(F), 0, g.nf[a] - 1);
+    Q[a] = (float)(F - widen_int(lc[a]));
     Dl[a] = rg.Dhi[a];
     inv[a] = rg.invDhi[a];
   }
   // the ray leaves through a face of the grid: no end parameter needed
-  march_block<NBT, FMT, int64_t>(r, Q, Dl, inv, FLT_MAX, lc[0], lc[1], lc[2], g.nf[0], g.nf[1],
-                                 g.nf[2], (int64_t)g.nf[0], (int64_t)g.nf[0] * g.nf[1], g.cells,
-                                 bc, br);
+  // (indices are 32-bit where every cell has one; a step past the block may
+  // lie one row beyond)
+  if ((int64_t)g.nf[0] * g.nf[1] * ((int64_t)g.nf[2] + 2) <= 0x7fffffff)
+    march_block<NBT, FMT, int>(r, Q, Dl, inv, FLT_MAX, lc[0], lc[1], lc[2], g.nf[0], g.nf[1], g.nf[2],
+                               g.nf[0], g.nf[0] * g.nf[1], g.cells, bc, br);
+  else
+    march_block<NBT, FMT, int64_t>(r, Q, Dl, inv, FLT_MAX, lc[0], lc[1], lc[2], g.nf[0], g.nf[1],
+                                   g.nf[2], (int64_t)g.nf[0], (int64_t)g.nf[0] * g.nf[1], g.cells,
+                                   bc, br);
 }
 
-// Double-float helpers (error-free transformations: Knuth's TwoSum and the
-// fused-multiply-add form of Dekker's TwoProduct).
-struct F2 {
-  float hi, lo;
-};
-__device__ __forceinline__ F2 f2_from(double x) {
-  F2 r;
-  r.hi = (float)x;
-  r.lo = (float)(x - (double)r.hi);
-  return r;
-}
+// Error-free transformations (Knuth's TwoSum and the fused-multiply-add form
+// of Dekker's TwoProduct).
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
   s = a + b;
   const float bb = s - a;
@@ -629,20 +924,21 @@ __device__ __forceinline__ int brick_of(const GridView &g, int e, const int c[3]
 // (direction, its inverse and its double-float split) are read from the
 // kernel-parameter bank, not held per thread.
 template <int NBT, int FMT>
-__device__ void march_amr(RTState<NBT> &r, const GridView &g, const double O[3],
+__device__ void march_amr(RTState<NBT> &r, const GridView &g, const double O[3], const F2 Of[3],
                           const RayGeom &rg, double t0, int eax, int fp64_level,
                           const BandCtx &bc, const BandRegs<NBT> &br) {
   const int B = g.B, lb = g.log2B, Lm = g.Lm;
-  const double *D = rg.D, *invD = rg.invD;
-  F2 Of[3];
   int c[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    Of[a] = f2_from(O[a]);
-    c[a] = clampi((int)floor(O[a] + t0 * D[a]), 0, g.nf[a] - 1);
+    // the entry face's coordinate is 0 or nf to within rounding: its cell is
+    // the first or the last
+    if (a == eax) c[a] = rg.Dhi[a] > 0.f ? 0 : g.nf[a] - 1;
+    else c[a] = clampi(__double2int_rd(rg.Dhi[a] == 0.f ? O[a] : fma(t0, rg.D[a], O[a])), 0, g.nf[a] - 1);
   }
   F2 t = f2_from(t0);
   const int max_iter = 4 * (g.nf[0] + g.nf[1] + g.nf[2]);
+  const float ulp = fmaf((float)max(g.nf[0], max(g.nf[1], g.nf[2])), 0x1p-44f, (float)B * 0x1p-20f);
   int e = map_entry(g, c[0], c[1], c[2]);
   for (int it = 0; it < max_iter; ++it) {
     int lev;
@@ -675,8 +971,18 @@ __device__ void march_amr(RTState<NBT> &r, const GridView &g, const double O[3],
     // in double-float. Only the other axes need the FP64 (or double-float)
     // position of the entry point.
     if (deep) {
-      const double td = (double)t.hi + (double)t.lo;
-      double tmin = DBL_MAX;
+      const double td = widen(t.hi) + widen(t.lo);
+      // the two axes b1, b2 that are not the entry axis
+      const int b1 = eax == 0 ? 1 : 0, b2 = eax == 2 ? 1 : 2;
+      const double E1 = pick(b1, O[0], O[1], O[2]) - widen_int(b1 == 0 ? anchor[0] : anchor[1]);
+      const double E2 = pick(b2, O[0], O[1], O[2]) - widen_int(b2 == 1 ? anchor[1] : anchor[2]);
+      const float Q1 = (float)fma(td, pick(b1, rg.D[0], rg.D[1], rg.D[2]), E1) * scale;
+      const float Q2 = (float)fma(td, pick(b2, rg.D[0], rg.D[1], rg.D[2]), E2) * scale;
+      // exit parameters from the entry point in FP32, to within 2^-20 of the
+      // brick's edge (5 roundings of 2^-24, and the entry point is within
+      // 2^-24 of a cell) and 2^-44 of the grid's (td has 48 bits): they tell
+      // the exit axis unless two faces are met almost together
+      float x[3], xe[3];
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         if (a == eax)
@@ -684,18 +990,38 @@ __device__ void march_amr(RTState<NBT> &r, const GridView &g, const double O[3],
         else if (Dl[a] == 0.f)
           Q[a] = ((Of[a].hi - (float)anchor[a]) + Of[a].lo) * scale;
         else
-          Q[a] = (float)fma(td, D[a], O[a] - (double)anchor[a]) * scale;
-        if (Dl[a] != 0.f) {
-          const double face = (double)(Dl[a] > 0.f ? bo[a] + S : bo[a]);
-          const double ta = (face - O[a]) * invD[a];
-          if (ta < tmin) {
-            tmin = ta;
-            ax = a;
-          }
-        }
+          Q[a] = a == b1 ? Q1 : Q2;
+        x[a] = Dl[a] == 0.f ? FLT_MAX : ((float)(Dl[a] > 0.f ? B - lc[a] : -lc[a]) - Q[a]) * inv[a];
+        xe[a] = ulp * fabsf(inv[a]);
       }
-      te = tmin < td ? td : tmin;
-      tend = (float)(te - td);
+      ax = x[0] <= x[1] && x[0] <= x[2] ? 0 : (x[1] <= x[2] ? 1 : 2);
+      const float xm = ax == 0 ? x[0] + xe[0] : (ax == 1 ? x[1] + xe[1] : x[2] + xe[2]);
+      const bool clear = (ax == 0 || xm < x[0] - xe[0]) && (ax == 1 || xm < x[1] - xe[1]) &&
+                         (ax == 2 || xm < x[2] - xe[2]);
+      double tmin;
+      if (clear) {
+        const int face = ax == 0 ? (Dl[0] > 0.f ? bo[0] + S : bo[0])
+                                 : (ax == 1 ? (Dl[1] > 0.f ? bo[1] + S : bo[1])
+                                            : (Dl[2] > 0.f ? bo[2] + S : bo[2]));
+        tmin = (widen_int(face) - pick(ax, O[0], O[1], O[2])) * pick(ax, rg.invD[0], rg.invD[1], rg.invD[2]);
+      } else {
+        tmin = DBL_MAX;
+        ax = -1;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+          if (Dl[a] != 0.f) {
+            const double ta = (widen_int(Dl[a] > 0.f ? bo[a] + S : bo[a]) - O[a]) * rg.invD[a];
+            if (ta < tmin) {
+              tmin = ta;
+              ax = a;
+            }
+          }
+      }
+      // te = max(tmin, td); tend = te - td (the difference's sign is exact)
+      const double dt = tmin - td;
+      const bool fwd = __double2hiint(dt) >= 0;
+      te = fwd ? tmin : td;
+      tend = fwd ? (float)dt : 0.f;
     } else {
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -764,73 +1090,196 @@ __device__ void march_amr(RTState<NBT> &r, const GridView &g, const double O[3],
 // form (and the batched kernel) sends such a ray here, so all give the same
 // bits for it. The map entry of the next brick is fetched before the current
 // brick's column is marched, so its latency overlaps the march.
-template <int NBT, int FMT, int A, int U>
-__device__ __forceinline__ void march_amr_axis(RTState<NBT> &r, const GridView &g, int c[3], const RayGeom &rg,
-                               const BandCtx &bc, const BandRegs<NBT> &br) {
-  constexpr int A1 = (A + 1) % 3, A2 = (A + 2) % 3;
-  const int B = g.B, lb = g.log2B, Lm = g.Lm;
-  const bool pos = rg.Dhi[A] > 0.f;
-  const float a1 = fabsf(rg.invDhi[A]);
+// W16 = +1 / -1: bricks of 16^3 cells, rays towards higher / lower cells of
+// the constant axis A (march_column16); 0: any brick and direction.
+template <int NBT, int FMT, int U, bool TAIL, int W16 = 0, int CA = 0>
+__device__ __forceinline__ void march_amr_axis(RTState<NBT> &r, const GridView &g, int A, int c1,
+                                               int c2, const RayGeom &rg, const BandCtx &bc,
+                                               const BandRegs<NBT> &br) {
+  if (W16 != 0) A = CA;
+  const int A1 = A == 2 ? 0 : A + 1, A2 = A == 0 ? 2 : A - 1;
+  const int B = W16 != 0 ? 16 : g.B, lb = W16 != 0 ? 4 : g.log2B, Lm = g.Lm;
+  const int nfA = A == 0 ? g.nf[0] : (A == 1 ? g.nf[1] : g.nf[2]);
+  const bool pos = W16 != 0 ? W16 > 0 : (A == 0 ? rg.Dhi[0] : (A == 1 ? rg.Dhi[1] : rg.Dhi[2])) > 0.f;
+  const float a1 = fabsf(A == 0 ? rg.invDhi[0] : (A == 1 ? rg.invDhi[1] : rg.invDhi[2]));
   // cell strides inside a brick, x fastest
-  const int sA = A == 0 ? 1 : (A == 1 ? B : B * B);
-  const int sA1 = A1 == 0 ? 1 : (A1 == 1 ? B : B * B);
-  const int sA2 = A2 == 0 ? 1 : (A2 == 1 ? B : B * B);
-  const int d = pos ? sA : -sA;
-  c[A] = pos ? 0 : g.nf[A] - 1;  // the ray enters through the grid face
-  const int max_iter = 4 * g.nf[A];
-  int e = map_entry(g, c[0], c[1], c[2]);
+  const int lA = A * lb, l1 = A1 * lb, l2 = A2 * lb;
+  const int d = pos ? (1 << lA) : -(1 << lA);
+  // the brick map along the ray: entry column + (cA >> sm) * step
+  const int sm = lb + Lm - g.mapL;
+  const int m0 = 1, m1 = g.nm[0], m2 = g.nm[0] * g.nm[1];  // at most 2^24 entries
+  const int32_t *column = g.bmap + (c1 >> sm) * (A1 == 0 ? m0 : (A1 == 1 ? m1 : m2)) +
+                          (c2 >> sm) * (A2 == 0 ? m0 : (A2 == 1 ? m1 : m2));
+  const int step = A == 0 ? m0 : (A == 1 ? m1 : m2);
+  int cA = pos ? 0 : nfA - 1;  // the ray enters through the grid face
+  const int max_iter = 4 * nfA;
+  int e = __ldg(column + (cA >> sm) * step);
   for (int it = 0; it < max_iter; ++it) {
     int lev;
-    const int code = brick_of(g, e, c, lev);
+    if (e >= 0) {
+      lev = e >> kMapLevelShift;
+      e &= kMapIdMask;
+    } else {
+      lev = g.mapL;
+      while (e < 0) {
+        ++lev;
+        const int sh = lb + Lm - lev;
+        const int oc = (((cA >> sh) & 1) << A) | (((c1 >> sh) & 1) << A1) | (((c2 >> sh) & 1) << A2);
+        e = __ldg(g.oct + (int64_t)(-e - 1) * 8 + oc);
+      }
+    }
     r.maxlev = max(r.maxlev, lev);
     const int shift = Lm - lev;
     const int S = B << shift;
-    const int cn = pos ? c[A] + S : c[A] - S;
-    const bool out = cn < 0 || cn >= g.nf[A];
-    int nc[3];
-    nc[A] = cn;
-    nc[A1] = c[A1];
-    nc[A2] = c[A2];
-    const int en = out ? 0 : map_entry(g, nc[0], nc[1], nc[2]);
-    const int idx = (pos ? 0 : (B - 1) * sA) + ((c[A1] >> shift) & (B - 1)) * sA1 +
-                    ((c[A2] >> shift) & (B - 1)) * sA2;
+    const int cn = pos ? cA + S : cA - S;
+    const bool out = cn < 0 || cn >= nfA;
+    const int en = out ? 0 : __ldg(column + (cn >> sm) * step);
+    const int idx = (pos ? 0 : (B - 1) << lA) + (((c1 >> shift) & (B - 1)) << l1) +
+                    (((c2 >> shift) & (B - 1)) << l2);
     const float ds = a1 * __int_as_float((127 + shift) << 23);  // a1 2^shift
-    const int64_t boff = (int64_t)code << (3 * lb);
+    const int64_t boff = (int64_t)e << (3 * lb);
     const void *cb = FMT == kCellRho ? (const void *)((const float *)g.cells + boff)
                                      : (const void *)((const uint2 *)g.cells + boff);
-    march_column<NBT, FMT, U, int>(r, cb, idx, d, B, ds, bc, br);
+    if constexpr (W16 != 0) {
+      const int low = (((c1 >> shift) & 15) << l1) + (((c2 >> shift) & 15) << l2);
+      march_column16<NBT, FMT, CA, (W16 > 0)>(
+          r, FMT == kCellRho ? (const void *)((const float *)cb + low) : (const void *)((const uint2 *)cb + low),
+          ds, bc, br);
+    } else {
+      march_column<NBT, FMT, U, TAIL, int>(r, cb, idx, d, B, ds, bc, br);
+    }
     if (out) break;
-    c[A] = cn;
+    cA = cn;
     e = en;
   }
 }
 
-// The uniform grid's version: the whole column of nf[A] cells.
-template <int NBT, int FMT, int A, int U>
-__device__ __forceinline__ void march_uniform_axis(RTState<NBT> &r, const GridView &g, const int c[3],
-                                   const RayGeom &rg, const BandCtx &bc, const BandRegs<NBT> &br) {
-  constexpr int A1 = (A + 1) % 3, A2 = (A + 2) % 3;
-  const bool pos = rg.Dhi[A] > 0.f;
-  const int64_t st[3] = {1, (int64_t)g.nf[0], (int64_t)g.nf[0] * g.nf[1]};
-  const int64_t idx = (pos ? 0 : (int64_t)(g.nf[A] - 1) * st[A]) + (int64_t)c[A1] * st[A1] +
-                      (int64_t)c[A2] * st[A2];
-  march_column<NBT, FMT, U, int64_t>(r, g.cells, idx, pos ? st[A] : -st[A], g.nf[A],
-                                     fabsf(rg.invDhi[A]), bc, br);
+// march_amr_axis for bricks of at most 8 cells, compiled on its own: a brick's
+// cells are too few for a group, so each takes the compensated step, and a ray
+// spends its time waiting for one short column after the other. Here the next
+// brick's records (and the map entry of the one after) are on their way while
+// a brick is summed. (One kernel with both walks spilled registers; the walk
+// that waits for each column took 26 us a sweep on the ring grid, 8^3 bricks.)
+template <int NBT, int FMT>
+__device__ __forceinline__ void march_amr_axis_small(RTState<NBT> &r, const GridView &g, int A,
+                                                     int c1, int c2, const RayGeom &rg,
+                                                     const BandCtx &bc, const BandRegs<NBT> &br) {
+  constexpr int M = 8;  // largest brick edge
+  const int A1 = A == 2 ? 0 : A + 1, A2 = A == 0 ? 2 : A - 1;
+  const int B = g.B, lb = g.log2B, Lm = g.Lm;
+  const int nfA = A == 0 ? g.nf[0] : (A == 1 ? g.nf[1] : g.nf[2]);
+  const bool pos = (A == 0 ? rg.Dhi[0] : (A == 1 ? rg.Dhi[1] : rg.Dhi[2])) > 0.f;
+  const float a1 = fabsf(A == 0 ? rg.invDhi[0] : (A == 1 ? rg.invDhi[1] : rg.invDhi[2]));
+  const int lA = A * lb, l1 = A1 * lb, l2 = A2 * lb;
+  const int d = pos ? (1 << lA) : -(1 << lA);
+  const int sm = lb + Lm - g.mapL;
+  const int m0 = 1, m1 = g.nm[0], m2 = g.nm[0] * g.nm[1];
+  const int32_t *column = g.bmap + (c1 >> sm) * (A1 == 0 ? m0 : (A1 == 1 ? m1 : m2)) +
+                          (c2 >> sm) * (A2 == 0 ? m0 : (A2 == 1 ? m1 : m2));
+  const int step = A == 0 ? m0 : (A == 1 ? m1 : m2);
+  int cA = pos ? 0 : nfA - 1;  // finest cell through which the next brick is entered
+  int e = __ldg(column + (cA >> sm) * step);
+  float rh[M], nrh[M], ds = 0.f, nds = 0.f;
+  uint32_t xv[M], nxv[M];
+  bool have = false, more = true;
+  while (true) {
+    if (more) {  // ask for the brick at cA
+      int lev;
+      if (e >= 0) {
+        lev = e >> kMapLevelShift;
+        e &= kMapIdMask;
+      } else {
+        lev = g.mapL;
+        while (e < 0) {
+          ++lev;
+          const int sh = lb + Lm - lev;
+          const int oc = (((cA >> sh) & 1) << A) | (((c1 >> sh) & 1) << A1) | (((c2 >> sh) & 1) << A2);
+          e = __ldg(g.oct + (int64_t)(-e - 1) * 8 + oc);
+        }
+      }
+      r.maxlev = max(r.maxlev, lev);
+      const int shift = Lm - lev;
+      const int idx = (pos ? 0 : (B - 1) << lA) + (((c1 >> shift) & (B - 1)) << l1) +
+                      (((c2 >> shift) & (B - 1)) << l2);
+      nds = a1 * __int_as_float((127 + shift) << 23);  // a1 2^shift
+      const int64_t at = ((int64_t)e << (3 * lb)) + idx;
+#pragma unroll
+      for (int u = 0; u < M; ++u)
+        if (u < B) load_cell<FMT>(g.cells, at + u * d, nrh[u], nxv[u]);
+      cA = pos ? cA + (B << shift) : cA - (B << shift);
+    }
+    const bool next = more;
+    more = next && cA >= 0 && cA < nfA;
+    if (more) e = __ldg(column + (cA >> sm) * step);
+    if (have) {
+      r.steps += (uint32_t)B;
+      // the whole brick's column dark: N alone (see rt_term; the zero terms
+      // of several dark cells change a sum as one does)
+      uint32_t x = 0u;
+      float tot = 0.f;
+#pragma unroll
+      for (int u = 0; u < M; ++u)
+        if (u < B) {
+          x = FMT == kCellLam ? x | xv[u] : max(x, xv[u]);
+          tot += rh[u];
+        }
+      if (FMT != kCellRho && cell_dark<FMT>(x, br.xz) && fmaf(tot, ds, r.N) <= 0.5f * FLT_MAX) {
+#pragma unroll
+        for (int u = 0; u < M; ++u)
+          if (u < B) kahan_add(r.N, r.cN, __fmul_rn(rh[u], ds));
+        kahan_add(r.I[0], r.cI[0], 0.f);
+        r.T[0] = ex2_approx(br.nk[0] * r.N);
+      } else {
+#pragma unroll
+        for (int u = 0; u < M; ++u)
+          if (u < B) rt_term<NBT, FMT, false>(r, rh[u], xv[u], ds, bc, br);
+      }
+    }
+    if (!next) break;
+#pragma unroll
+    for (int u = 0; u < M; ++u) {
+      rh[u] = nrh[u];
+      xv[u] = nxv[u];
+    }
+    ds = nds;
+    have = true;
+  }
 }
 
-// Pixel (L, i, j)'s ray along grid axis A through either kind of grid.
-template <int NBT, bool AMR, int FMT, int A, int U>
+// The uniform grid's version: the whole column of nf[A] cells.
+template <int NBT, int FMT, int U>
+__device__ __forceinline__ void march_uniform_axis(RTState<NBT> &r, const GridView &g, int A, int c1,
+                                                   int c2, const RayGeom &rg, const BandCtx &bc,
+                                                   const BandRegs<NBT> &br) {
+  const bool pos = (A == 0 ? rg.Dhi[0] : (A == 1 ? rg.Dhi[1] : rg.Dhi[2])) > 0.f;
+  const float ds = fabsf(A == 0 ? rg.invDhi[0] : (A == 1 ? rg.invDhi[1] : rg.invDhi[2]));
+  const int nfA = A == 0 ? g.nf[0] : (A == 1 ? g.nf[1] : g.nf[2]);
+  const int64_t s1 = g.nf[0], s2 = (int64_t)g.nf[0] * g.nf[1];
+  const int64_t stA = A == 0 ? 1 : (A == 1 ? s1 : s2);
+  const int64_t st1 = A == 0 ? s1 : (A == 1 ? s2 : 1), st2 = A == 0 ? s2 : (A == 1 ? 1 : s1);
+  const int64_t idx = (pos ? 0 : (int64_t)(nfA - 1) * stA) + (int64_t)c1 * st1 + (int64_t)c2 * st2;
+  march_column<NBT, FMT, U, true, int64_t>(r, g.cells, idx, pos ? stA : -stA, nfA, ds, bc, br);
+}
+
+// Pixel (L, i, j)'s ray along grid axis A through either kind of grid. DIR: the
+// kernel's form (trace_ray).
+template <int NBT, bool AMR, int FMT, int DIR, int U>
 __device__ __forceinline__ void march_axis(RTState<NBT> &st, const GridView &g, const RayGeom &rg,
-                                           int L, int i, int j, const BandCtx &bc,
+                                           int A, int L, int i, int j, const BandCtx &bc,
                                            const BandRegs<NBT> &br) {
-  int c[3];
-  if (!axis_ray_setup<A>(g, rg, L, i, j, c)) return;
-  if (AMR) march_amr_axis<NBT, FMT, A, U>(st, g, c, rg, bc, br);
-  else march_uniform_axis<NBT, FMT, A, U>(st, g, c, rg, bc, br);
+  int c1, c2;
+  if (!axis_ray_setup(g, rg, A, L, i, j, c1, c2)) return;
+  if constexpr (!AMR) march_uniform_axis<NBT, FMT, U>(st, g, A, c1, c2, rg, bc, br);
+  else if constexpr (DIR >= 7) march_amr_axis<NBT, FMT, U, false, (DIR < 10 ? 1 : -1), (DIR - 1) % 3>(st, g, A, c1, c2, rg, bc, br);
+  else if constexpr (DIR >= 4) march_amr_axis_small<NBT, FMT>(st, g, A, c1, c2, rg, bc, br);
+  else march_amr_axis<NBT, FMT, U, DIR == 0>(st, g, A, c1, c2, rg, bc, br);
 }
 
 // One ray (pixel (L, i, j)) through the grid, bands [b0, b0 + NBT) of bc/br.
-// DIR = 1 + A: every ray of the launch is parallel to grid axis A.
+// DIR = 1 + A: every ray of the launch is parallel to grid axis A (bricks of 16
+// cells and more, or a uniform grid); 4 + A: the same with bricks of at most 8
+// cells; 7 + A and 10 + A: with 16^3 bricks, towards higher and lower cells;
+// 0: any direction.
 template <int NBT, bool AMR, int FMT, int DIR = 0>
 __device__ __forceinline__ void trace_ray(RTState<NBT> &st, const GridView &g, const RayGeom &rg,
                                           int L, int i, int j, int fp64_level, const BandCtx &bc,
@@ -838,19 +1287,18 @@ __device__ __forceinline__ void trace_ray(RTState<NBT> &st, const GridView &g, c
   rt_init<NBT>(st);
   constexpr int U = ColumnUnroll<DIR>::value;
   if constexpr (DIR >= 1) {
-    march_axis<NBT, AMR, FMT, (DIR - 1) % 3, U>(st, g, rg, L, i, j, bc, br);
+    march_axis<NBT, AMR, FMT, DIR, U>(st, g, rg, (DIR - 1) % 3, L, i, j, bc, br);
   } else {
     const bool m0 = rg.Dhi[0] != 0.f, m1 = rg.Dhi[1] != 0.f, m2 = rg.Dhi[2] != 0.f;
     if (m0 + m1 + m2 == 1) {
-      if (m0) march_axis<NBT, AMR, FMT, 0, U>(st, g, rg, L, i, j, bc, br);
-      else if (m1) march_axis<NBT, AMR, FMT, 1, U>(st, g, rg, L, i, j, bc, br);
-      else march_axis<NBT, AMR, FMT, 2, U>(st, g, rg, L, i, j, bc, br);
+      march_axis<NBT, AMR, FMT, DIR, U>(st, g, rg, m0 ? 0 : (m1 ? 1 : 2), L, i, j, bc, br);
       return;
     }
     double O[3], t0;
+    F2 Of[3];
     int eax;
-    if (!ray_setup(g, rg, L, i, j, O, t0, eax)) return;
-    if (AMR) march_amr<NBT, FMT>(st, g, O, rg, t0, eax, fp64_level, bc, br);
+    if (!ray_setup(g, rg, L, i, j, O, Of, t0, eax)) return;
+    if (AMR) march_amr<NBT, FMT>(st, g, O, Of, rg, t0, eax, fp64_level, bc, br);
     else march_uniform<NBT, FMT>(st, g, O, rg, t0, bc, br);
   }
 }
@@ -879,6 +1327,17 @@ static inline RayGeom make_geom(const GridView &g, const Camera &cam, int n0) {
   }
   rg.H = cam.H;
   rg.pix0 = (2.0 * cam.H) / (double)n0;
+  rg.fH = (float)rg.H;
+  rg.fpix0 = (float)rg.pix0;
+  for (int a = 0; a < 3; ++a) {
+    rg.fO[a] = (float)(rg.C[a] * rg.invh[a]);
+    rg.fU[a] = (float)(rg.U[a] * rg.invh[a]);
+    rg.fV[a] = (float)(rg.V[a] * rg.invh[a]);
+    // roundings of FP32: at most 8 units of each product (32 allowed)
+    const double reach = (fabs(rg.C[a]) + 2.0 * rg.H * (fabs(rg.U[a]) + fabs(rg.V[a]))) * rg.invh[a];
+    const bool fits = rg.H < 1e25 && rg.pix0 > 1e-25 && rg.invh[a] < 1e25 && rg.invh[a] > 1e-25 && reach < 1e15;
+    rg.eO[a] = fits ? (float)(reach * 0x1p-20) : HUGE_VALF;
+  }
   rg.tab = nullptr;
   rg.tab_slot = 0;
   rg.tab_n0 = n0;

@@ -1,0 +1,214 @@
+// air_march_kernel.cuh -- the march kernel and its launch, as templates over
+// the bands one thread carries. Each width is compiled in a translation unit
+// of its own (air_march_<width>.cu, air_march_axis.cu), in parallel: one unit
+// with every form took 150 s of a build, the slowest of these takes a quarter.
+#pragma once
+#include "air_march.cuh"
+#include "air_refine.cuh"
+
+namespace air {
+
+// One launch of the march, as launch_march resolved it.
+struct MarchLaunch {
+  const GridView &g;
+  const RayGeom &rg;
+  const RaySource &src;
+  const RayOut &out;
+  int64_t blocks;  // of kMarchBlock rays; with the count on the device, unused
+  int chunks;      // band chunks
+  int fp64_level;
+  cudaStream_t st;
+};
+
+// Resident blocks per SM of the one-band kernels of rays parallel to an axis
+// (DIR = 1 + A). Measured on the cone-shock bench image, one process, each
+// variant twice (AIR / fixed 4096^2 image, ms): 12 blocks with 8-cell groups
+// 5.39 / 4.89, 10 blocks 5.22 / 4.82, 8 blocks 5.02 / 4.30, 8 blocks with
+// 16-cell groups 4.92 / 4.37 (the form kept). A separate form for launches
+// of at most one wave (more registers, deeper load groups) is then the same
+// kernel, so there is one.
+constexpr int kAxisBlocks = 8;
+constexpr int kAxisBlocksSmall = 6;  // bricks of at most 8 cells: two bricks' records in registers
+
+template <int NBT, int DIR>
+struct MinBlocks {
+  static constexpr int value = DIR >= 4 && DIR <= 6 ? kAxisBlocksSmall
+                               : DIR >= 1 ? kAxisBlocks
+                               : (NBT <= 1 ? 6 : (NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? 3 : 2))));
+};
+
+constexpr int kMarchBlock = 128;
+
+// Node k's ray: trace it and store its column density, step count and band
+// intensities (and their sum when one chunk holds every band).
+template <int NBT, bool AMR, int FMT, int DIR>
+__device__ __forceinline__ void march_one(const GridView &g, const RayGeom &rg, const RaySource &src,
+                                          const RayOut &out, int fp64_level, const BandCtx &bc,
+                                          const BandRegs<NBT> &br, int chunk, int b0, int nbh,
+                                          int64_t k) {
+  if (src.use_prop) {
+    // the pixel's values from the proposal wave when it traced the pixel
+    // (the same trace, so the same bits); else trace it here
+    const Proposal &pr = src.prop;
+    const int L = src.lvl[k], i = src.pi[k], j = src.pj[k];
+    const int64_t b = (int64_t)(j >> L) * src.n0 + (i >> L);
+    const int64_t q = prop_index(pr.depth + 4 * b, pr.off[b], L, i, j);
+    if (q >= 0) {
+      if (chunk == 0) {
+        out.N[k] = pr.N[q];
+        out.steps[k] = pr.steps[q];
+      }
+      for (int c = 0; c < nbh; ++c)
+        out.I[(int64_t)(b0 + c) * out.stride + k] = pr.I[(int64_t)(b0 + c) * pr.stride + q];
+      if (out.p && gridDim.y == 1) out.p[k] = pr.p[q];
+      return;
+    }
+    if (chunk == 0) atomicAdd(&src.sweep->fb_sweep, 1ull);
+  }
+  RTState<NBT> st;
+  trace_ray<NBT, AMR, FMT, DIR>(st, g, rg, src.lvl[k], src.pi[k], src.pj[k], fp64_level, bc, br);
+  if (chunk == 0) {
+    out.N[k] = st.N;
+    out.steps[k] = st.steps;
+    if (out.tau0) out.tau0[k] = br.kap[0] * st.N;
+    if (out.maxlev) out.maxlev[k] = (uint8_t)st.maxlev;
+  }
+#pragma unroll
+  for (int b = 0; b < NBT; ++b)
+    if (b < nbh) out.I[(int64_t)(b0 + b) * out.stride + (k - out.ioff)] = st.I[b];
+  if (out.p && gridDim.y == 1) {
+    float p = 0.f;
+#pragma unroll
+    for (int b = 0; b < NBT; ++b)
+      if (b < nbh) p += st.I[b];
+    out.p[k] = p;
+  }
+}
+
+template <int NBT, bool AMR, int FMT, int DIR>
+__global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
+    k_march(GridView g, RayGeom rg, RaySource src, RayOut out, int fp64_level) {
+  extern __shared__ __align__(16) float smem[];
+  wait_prior_grid();
+  const int chunk = blockIdx.y;
+  const int b0 = chunk * NBT;
+  const int nbh = min(NBT, g.n_bands - b0);
+  BandCtx bc;
+  bc.tab = smem;
+  bc.nbh = nbh;
+  if (FMT == kCellXq) tab_fill<NBT>(smem, g, b0);
+  BandRegs<NBT> br;
+  band_regs<NBT>(br, g.bands, b0, nbh);
+  __syncthreads();
+
+  if (src.mode == 2) {
+    // new nodes of a sweep counted on the device: blocks take chunks of
+    // blockDim.x rays from a work counter until the rays run out
+    // (with src.advance, the last block to finish moves the state on to the
+    // next sweep)
+    SweepState *S = src.sweep;
+    if (S->done) return;
+    const int64_t count = 4 * S->tot[0], first = S->n;
+    __shared__ long long s_chunk;
+    for (;;) {
+      if (threadIdx.x == 0) s_chunk = (long long)atomicAdd(S->ray_ctr + chunk, 1ull);
+      __syncthreads();
+      const int64_t r0 = (int64_t)s_chunk * blockDim.x;
+      __syncthreads();
+      if (r0 >= count) break;
+      const int64_t r = r0 + threadIdx.x;
+      if (r < count) march_one<NBT, AMR, FMT, DIR>(g, rg, src, out, fp64_level, bc, br, chunk, b0,
+                                                   nbh, first + r);
+    }
+    if (src.advance && threadIdx.x == 0) sweep_block_finished(S, gridDim.x * gridDim.y);
+    return;
+  }
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int L, i, j;
+  int64_t k;
+  if (src.mode == 0) {
+    if (r >= src.count) return;
+    k = src.list ? (int64_t)src.list[r] : src.first + r;
+    L = src.lvl[k];
+    i = src.pi[k];
+    j = src.pj[k];
+  } else {
+    const int res = src.n0;
+    const int tw = src.tile_w, th = 32 / tw;
+    // res <= 2^16: the tiles of 32 pixels number at most 2^27 (+ a row), so
+    // 32-bit division does (64-bit division is long and uses FP64 units)
+    const uint32_t tiles_x = (uint32_t)(res + tw - 1) / (uint32_t)tw;
+    const uint32_t warp = (uint32_t)(r >> 5);
+    const uint32_t lane = (uint32_t)(r & 31);
+    const uint32_t ty = warp / tiles_x;
+    i = (int)((warp - ty * tiles_x) * tw + lane % (uint32_t)tw);
+    j = (int)(ty * th + lane / (uint32_t)tw);
+    if (i >= res || j >= res) return;
+    k = (int64_t)j * res + i;
+    L = 0;
+  }
+  RTState<NBT> st;
+  trace_ray<NBT, AMR, FMT, DIR>(st, g, rg, L, i, j, fp64_level, bc, br);
+  if (chunk == 0) {
+    out.N[k] = st.N;
+    out.steps[k] = st.steps;
+    if (out.tau0) out.tau0[k] = br.kap[0] * st.N;
+    if (out.maxlev) out.maxlev[k] = (uint8_t)st.maxlev;
+  }
+#pragma unroll
+  for (int b = 0; b < NBT; ++b)
+    if (b < nbh) out.I[(int64_t)(b0 + b) * out.stride + (k - out.ioff)] = st.I[b];
+  if (out.p && gridDim.y == 1) {
+    float p = 0.f;
+#pragma unroll
+    for (int b = 0; b < NBT; ++b)
+      if (b < nbh) p += st.I[b];
+    out.p[k] = p;
+  }
+}
+
+// The launch grid of form DIR: blocks over the rays, or, with the count on
+// the device, one wave of the form's resident blocks taking work from the
+// counter.
+template <int NBT, int DIR>
+static dim3 march_grid(const MarchLaunch &m) {
+  return dim3((unsigned)(m.src.mode == 2 ? sm_count() * MinBlocks<NBT, DIR>::value : m.blocks), m.chunks);
+}
+
+template <int NBT, bool AMR, int FMT, int DIR>
+static cudaError_t march_form(const MarchLaunch &m) {
+  const size_t smem = FMT == kCellXq ? tab_bytes<NBT>(m.g.n_tbins) : 0;
+  return launch_pdl(k_march<NBT, AMR, FMT, DIR>, march_grid<NBT, DIR>(m), dim3(kMarchBlock), smem, m.st,
+                    m.g, m.rg, m.src, m.out, m.fp64_level);
+}
+
+// Rays in any direction, NBT bands per thread.
+template <int NBT>
+cudaError_t march_general(const MarchLaunch &m) {
+  const bool amr = m.g.kind == AIR_GRID_AMR;
+  if (m.g.cell_fmt == kCellRho) return amr ? march_form<NBT, true, kCellRho, 0>(m) : march_form<NBT, false, kCellRho, 0>(m);
+  if (m.g.cell_fmt == kCellXq) return amr ? march_form<NBT, true, kCellXq, 0>(m) : march_form<NBT, false, kCellXq, 0>(m);
+  // per-cell Lambda exists for one-band grids only
+  if constexpr (NBT == 1) return amr ? march_form<1, true, kCellLam, 0>(m) : march_form<1, false, kCellLam, 0>(m);
+  return cudaErrorInvalidValue;
+}
+
+// One-band grids, every ray parallel to grid axis A: the form DIR = 1 + A, or
+// 4 + A for bricks of at most 8 cells, 7 + A or 10 + A for grids of 16^3 bricks
+// with per-cell Lambda (the ordinary one-band grid).
+template <int A, int FMT>
+static cudaError_t march_axis_fmt(const MarchLaunch &m) {
+  if (m.g.kind != AIR_GRID_AMR) return march_form<1, false, FMT, 1 + A>(m);
+  if (m.g.B <= 8) return march_form<1, true, FMT, 4 + A>(m);
+  if constexpr (FMT == kCellLam)
+    if (m.g.B == 16) return m.rg.Dhi[A] > 0.f ? march_form<1, true, FMT, 7 + A>(m) : march_form<1, true, FMT, 10 + A>(m);
+  return march_form<1, true, FMT, 1 + A>(m);
+}
+template <int A>
+cudaError_t march_axis_one(const MarchLaunch &m) {
+  if (m.g.cell_fmt == kCellRho) return march_axis_fmt<A, kCellRho>(m);
+  if (m.g.cell_fmt == kCellXq) return march_axis_fmt<A, kCellXq>(m);
+  return march_axis_fmt<A, kCellLam>(m);
+}
+
+}  // namespace air
