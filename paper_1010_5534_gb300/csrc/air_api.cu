@@ -183,19 +183,15 @@ MarchTune march_tune(const air_grid *g, int fp64_level) {
   return t;
 }
 
-// Fixed image -> output arrays: level 0, (i, j) from the row-major index.
-__global__ void k_fixed_out(int64_t n, int res, const float *N, const float *p, const float *I,
-                            int n_bands, OutView o) {
+// The pixel list of a fixed image: level 0, (i, j) from the row-major index.
+__global__ void k_fixed_out(int64_t n, uint32_t res, OutView o) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
+  const uint32_t j = (uint32_t)k / res;  // n <= 2^32
   if (o.level) o.level[k] = 0;
-  if (o.i) o.i[k] = (int32_t)(k % res);
-  if (o.j) o.j[k] = (int32_t)(k / res);
+  if (o.i) o.i[k] = (int32_t)((uint32_t)k - j * res);
+  if (o.j) o.j[k] = (int32_t)j;
   if (o.is_leaf) o.is_leaf[k] = 1;
-  if (o.N) o.N[k] = N[k];
-  if (o.p) o.p[k] = p[k];
-  if (o.I)
-    for (int b = 0; b < n_bands; ++b) o.I[(int64_t)b * o.stride + k] = I[(int64_t)b * n + k];
 }
 
 // Device address of page-locked host memory (NULL if p is not page-locked):
@@ -283,9 +279,14 @@ air_status render_fixed(air_grid *g, const air_view *view, int32_t res, int32_t 
   if ((s = init_scalars(g->ws))) return s;
   Workspace &w = g->ws;
   const int nb = g->gv.n_bands;
-  CU_TRY(ensure((void **)&w.fN, &w.fN_b, 4 * n));
-  CU_TRY(ensure((void **)&w.fI, &w.fI_b, 4 * n * nb));
-  CU_TRY(ensure((void **)&w.fp, &w.fp_b, 4 * n));
+  // the march writes the values where the output wants them (the caller's
+  // arrays, or the staging arrays of host outputs), and to scratch what the
+  // caller left out: copying them over afterwards cost 8 bytes per value
+  OutView o;
+  if ((s = out_view(g, im, n, o))) return s;
+  if (!o.N) CU_TRY(ensure((void **)&w.fN, &w.fN_b, 4 * n));
+  if (!o.I) CU_TRY(ensure((void **)&w.fI, &w.fI_b, 4 * n * nb));
+  if (!o.p) CU_TRY(ensure((void **)&w.fp, &w.fp_b, 4 * n));
   CU_TRY(ensure((void **)&w.fsteps, &w.fsteps_b, 4 * n));
   CU_TRY(ensure((void **)&w.partial, &w.partial_b, sizeof(double) * (nb + 1) * flux_blocks(n)));
   cudaStream_t st = g->stream;
@@ -296,19 +297,18 @@ air_status render_fixed(air_grid *g, const air_view *view, int32_t res, int32_t 
     const air_status sa = axis_table(g, cam, res, 0, src);
     if (sa) return sa;
   }
-  RayOut ro{w.fN, w.fI, n, w.fsteps, w.fp};
+  RayOut ro{o.N ? o.N : w.fN, o.I ? o.I : w.fI, o.I ? o.stride : n, w.fsteps, o.p ? o.p : w.fp};
   g->prof.used = 0;
   CU_TRY(prof_open(g, AIR_PHASE_MARCH, nb > (g->tune.bands_per_thread > 0 ? g->tune.bands_per_thread : default_bands_per_thread(nb)) ? 2 : 1));
   CU_TRY(launch_march(g->gv, cam, src, ro, march_tune(g, fp64_level), st));
   CU_TRY(prof_close(g));
   FluxArgs fa{};
-  fa.n = n; fa.child = nullptr; fa.lvl = nullptr; fa.I = w.fI; fa.stride = n; fa.steps = w.fsteps;
+  fa.n = n; fa.child = nullptr; fa.lvl = nullptr; fa.I = ro.I; fa.stride = ro.stride; fa.steps = w.fsteps;
   fa.n_bands = nb; fa.area0 = (2.0 * cam.H / res) * (2.0 * cam.H / res); fa.partial = w.partial;
-  OutView o;
-  if ((s = out_view(g, im, n, o))) return s;
-  CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, 3));
+  const bool list = o.level || o.i || o.j || o.is_leaf;
+  CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, list ? 3 : 2));
   CU_TRY(launch_flux(fa, w.d_flux, w.d_flux + nb, st));
-  k_fixed_out<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, res, w.fN, w.fp, w.fI, nb, o);
+  if (list) k_fixed_out<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, (uint32_t)res, o);
   CU_TRY(cudaGetLastError());
   CU_TRY(prof_close(g));
   s = finish_out(g, im, o, n);

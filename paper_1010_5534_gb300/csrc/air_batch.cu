@@ -45,10 +45,27 @@ __global__ void __launch_bounds__(256) k_vcount(TreeView t, const int16_t *view,
   }
   __syncthreads();
   const int64_t s0 = (int64_t)blockIdx.x * kScanItems, s1 = min(n, s0 + kScanItems);
-  for (int64_t k = s0 + threadIdx.x; k < s1; k += blockDim.x) {
-    const int v = view[k];
-    if (all || t.child[k] < 0) atomicAdd(&sm_cnt[v], 1);
-    atomicAdd(&sm_steps[v], (unsigned long long)t.steps[k]);
+  for (int64_t r0 = s0; r0 < s1; r0 += blockDim.x) {
+    // one addition per warp where its nodes are of one view (nodes of a view
+    // lie together), else one per node
+    const int64_t k = r0 + threadIdx.x;
+    const bool in = k < s1;
+    const int v = in ? (int)view[k] : -1;
+    const bool sel = in && (all || t.child[k] < 0);
+    const uint32_t st = in ? t.steps[k] : 0u;
+    const int v0 = __shfl_sync(0xffffffffu, v, 0);
+    const unsigned nsel = __popc(__ballot_sync(0xffffffffu, sel));
+    if (__all_sync(0xffffffffu, v == v0 || !in)) {
+      const unsigned lo = __reduce_add_sync(0xffffffffu, st & 0xffffu);
+      const unsigned hi = __reduce_add_sync(0xffffffffu, st >> 16);
+      if ((threadIdx.x & 31) == 0 && in) {
+        if (nsel) atomicAdd(&sm_cnt[v0], (int)nsel);
+        atomicAdd(&sm_steps[v0], ((unsigned long long)hi << 16) + lo);
+      }
+    } else if (in) {
+      if (sel) atomicAdd(&sm_cnt[v], 1);
+      atomicAdd(&sm_steps[v], (unsigned long long)st);
+    }
   }
   __syncthreads();
   for (int v = threadIdx.x; v < V; v += blockDim.x) {
@@ -84,44 +101,105 @@ __global__ void __launch_bounds__(256) k_vscan(const int32_t *bcnt, int64_t nblo
 struct EmitOutV {
   TreeView t;
   const OutView *outs;    // [V] (global)
-  double *sm_flux;        // shared [V][n_bands]
-  const RayGeom *geoms;   // [V]: level-0 pixel size of each view
   __device__ void operator()(int64_t k, int v, int64_t r) {
     const OutView &o = outs[v];
-    const bool leaf = t.child[k] < 0;
     if (o.level) o.level[r] = t.lvl[k];
     if (o.i) o.i[r] = t.pi[k];
     if (o.j) o.j[r] = t.pj[k];
-    if (o.is_leaf) o.is_leaf[r] = leaf;
+    if (o.is_leaf) o.is_leaf[r] = t.child[k] < 0;
     if (o.N) o.N[r] = t.N[k];
     if (o.p) o.p[r] = t.p[k];
-    const double pix = geoms[v].pix0;
-    const double area = pix * pix * __longlong_as_double((long long)(1023 - 2 * t.lvl[k]) << 52);
-    for (int b = 0; b < o.n_bands; ++b) {
-      const float I = t.I[(int64_t)b * t.cap + k];
-      if (o.I) o.I[(int64_t)b * o.stride + r] = I;
-      if (leaf) atomicAdd(&sm_flux[v * o.n_bands + b], (double)I * area);
+    if (o.I) {
+#pragma unroll 4
+      for (int b = 0; b < o.n_bands; ++b) o.I[(int64_t)b * o.stride + r] = t.I[(int64_t)b * t.cap + k];
     }
   }
 };
 
 __global__ void __launch_bounds__(256) k_vemit(TreeView t, const int16_t *view, int all, int64_t n,
-                                               int V, int n_bands, const int64_t *boff,
-                                               const OutView *outs, const RayGeom *geoms,
-                                               double *vflux) {
+                                               int V, const int64_t *boff, const OutView *outs) {
   extern __shared__ __align__(16) unsigned char sm[];
   int64_t *run = (int64_t *)sm;
-  double *flux = (double *)(run + V);
-  int32_t *wcnt = (int32_t *)(flux + (size_t)V * n_bands);
+  int32_t *wcnt = (int32_t *)(run + V);
   for (int v = threadIdx.x; v < V; v += blockDim.x) run[v] = boff[(int64_t)blockIdx.x * V + v];
-  for (int x = threadIdx.x; x < V * n_bands; x += blockDim.x) flux[x] = 0.0;
   __syncthreads();
   const int64_t s0 = (int64_t)blockIdx.x * kScanItems, s1 = min(n, s0 + kScanItems);
-  EmitOutV e{t, outs, flux, geoms};
+  EmitOutV e{t, outs};
   block_emit_by_view(LeafPred{t.child, all}, view, e, s0, s1, V, run, wcnt);
+}
+
+// Band flux of every view. A block takes 2048 nodes and kFluxBands bands
+// (blockIdx.y). Nodes of a view lie together, so a warp's strip of 32 nodes
+// mostly belongs to one view: its lanes sum on (flux_add) until the view
+// changes, and the block adds its warps' sums to the view's flux at the end.
+// (An FP64 atomic in shared memory per leaf and band, in the kernel above,
+// took most of the 2 ms that the output of 8 views x 16 bands cost.)
+constexpr int kVfluxRounds = 8;
+__global__ void __launch_bounds__(256) k_vflux(TreeView t, const int16_t *view, int64_t n,
+                                               int n_bands, const RayGeom *geoms, double *vflux) {
+  __shared__ double sums[kFluxBands][8];
+  __shared__ int views[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b0 = blockIdx.y * kFluxBands, nb = min(kFluxBands, n_bands - b0);
+  const int64_t start = (int64_t)blockIdx.x * (256 * kVfluxRounds) + threadIdx.x;
+  float hi[kFluxBands], lo[kFluxBands];
+  double tiny[kFluxBands];
+  int cur = -1;
+#pragma unroll
+  for (int q = 0; q < kFluxBands; ++q) {
+    hi[q] = lo[q] = 0.f;
+    tiny[q] = 0.0;
+  }
+  // the warp's sum of band q (to every lane), its accumulators emptied
+  auto take = [&](int q) {
+    double s = ((double)hi[q] + (double)lo[q]) + tiny[q];
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    hi[q] = lo[q] = 0.f;
+    tiny[q] = 0.0;
+    return s;
+  };
+  auto area = [&](int v) { return geoms[v].pix0 * geoms[v].pix0; };
+  for (int r = 0; r < kVfluxRounds; ++r) {
+    const int64_t k = start + (int64_t)r * 256;
+    const bool in = k < n;
+    const int v = in ? (int)view[k] : -1;
+    const bool leaf = in && t.child[k] < 0;
+    const int L = leaf ? t.lvl[k] : 0;
+    const int v0 = __shfl_sync(0xffffffffu, v, 0);
+    if (v0 < 0) break;  // past the end
+    if (__all_sync(0xffffffffu, v == v0 || !in)) {
+      if (v0 != cur) {
+        if (cur >= 0)
+          for (int q = 0; q < kFluxBands; ++q) {
+            const double s = take(q);
+            if (lane == 0 && q < nb) atomicAdd(&vflux[(int64_t)cur * n_bands + b0 + q], s * area(cur));
+          }
+        cur = v0;
+      }
+#pragma unroll
+      for (int q = 0; q < kFluxBands; ++q)
+        if (leaf && q < nb) flux_add(t.I[(int64_t)(b0 + q) * t.cap + k], L, hi[q], lo[q], tiny[q]);
+    } else if (leaf) {
+      for (int q = 0; q < nb; ++q)
+        atomicAdd(&vflux[(int64_t)v * n_bands + b0 + q],
+                  (double)t.I[(int64_t)(b0 + q) * t.cap + k] * pow4_neg(L) * area(v));
+    }
+  }
+  for (int q = 0; q < kFluxBands; ++q) {
+    const double s = take(q);
+    if (lane == 0) sums[q][warp] = s;
+  }
+  if (lane == 0) views[warp] = cur;
   __syncthreads();
-  for (int x = threadIdx.x; x < V * n_bands; x += blockDim.x)
-    if (flux[x] != 0.0) atomicAdd(&vflux[x], flux[x]);
+  if (threadIdx.x < nb) {
+    const int q = threadIdx.x;
+    for (int w = 0; w < 8;) {  // runs of warps that ended on the same view
+      const int v = views[w];
+      double s = 0.0;
+      for (; w < 8 && views[w] == v; ++w) s += sums[q][w];
+      if (v >= 0) atomicAdd(&vflux[(int64_t)v * n_bands + b0 + q], s * area(v));
+    }
+  }
 }
 
 // ---- host ---------------------------------------------------------------------
@@ -461,7 +539,7 @@ air_status render_batch(air_grid *g, const air_view *views, int32_t V, const air
   CU_TRY(cudaMemsetAsync(bw.vflux, 0, sizeof(double) * V * nb, st));
   TreeView t = w.tree(n0, Lm);
   const int64_t nblocks = scan_blocks(n);
-  CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, 3));
+  CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, 4));
   if (nblocks > 0) {
     const size_t sm1 = sizeof(int32_t) * ((V + 1) & ~1) + sizeof(unsigned long long) * V;
     k_vcount<<<(unsigned)nblocks, 256, sm1, st>>>(t, w.view, all, n, V, bw.bcnt, bw.vsteps);
@@ -469,9 +547,12 @@ air_status render_batch(air_grid *g, const air_view *views, int32_t V, const air
     CU_TRY(ensure((void **)&bw.boff, &bw.boff_b, sizeof(int64_t) * nblocks * V));
     k_vscan<<<V, 256, 0, st>>>(bw.bcnt, nblocks, V, bw.boff);
     CU_TRY(cudaGetLastError());
-    const size_t sm3 = sizeof(int64_t) * V + sizeof(double) * V * nb + sizeof(int32_t) * 8 * V;
-    CU_TRY(cudaFuncSetAttribute(k_vemit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
-    k_vemit<<<(unsigned)nblocks, 256, sm3, st>>>(t, w.view, all, n, V, nb, bw.boff, bw.outs, bw.geoms, bw.vflux);
+    const size_t sm3 = sizeof(int64_t) * V + sizeof(int32_t) * 8 * V;
+    k_vemit<<<(unsigned)nblocks, 256, sm3, st>>>(t, w.view, all, n, V, bw.boff, bw.outs);
+    CU_TRY(cudaGetLastError());
+    k_vflux<<<dim3((unsigned)((n + 256 * kVfluxRounds - 1) / (256 * kVfluxRounds)),
+                   (unsigned)((nb + kFluxBands - 1) / kFluxBands)),
+              256, 0, st>>>(t, w.view, n, nb, bw.geoms, bw.vflux);
     CU_TRY(cudaGetLastError());
   }
   CU_TRY(prof_close(g));

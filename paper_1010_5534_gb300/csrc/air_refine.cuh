@@ -106,7 +106,14 @@ __device__ __forceinline__ void sweep_block_finished(SweepState *S, unsigned nbl
 // the kernel before it (launched with cudaLaunchAttributeProgrammaticStream-
 // Serialization, the wait returns once that kernel has completed and its
 // memory is visible; launched without it, the wait returns at once).
-__device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// From then on the kernel after it may be scheduled too: its blocks come up
+// beside this kernel's last ones and wait here in their turn, so a launch
+// costs no gap. (Without the second instruction the next kernel was scheduled
+// only when this one had ended.)
+__device__ __forceinline__ void wait_prior_grid() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // Launch with programmatic stream serialization: the kernel may be scheduled
 // while the one before it in the stream is finishing, and waits for it in
@@ -126,6 +133,30 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// ---- band flux (shared by the single-view and the batched output) ----------
+constexpr int kFluxBands = 4;  // bands a block sums side by side
+
+__device__ __forceinline__ double pow4_neg(int L) {
+  return __longlong_as_double((long long)(1023 - 2 * L) << 52);
+}
+
+// A thread's leaves are summed as an unevaluated pair of FP32 numbers
+// (Knuth's two-sum: hi + lo carries the sum to ~2^-44 relative) of I 4^-L, an
+// exact scaling while the product stays a normal number; the rare smaller
+// terms go to an FP64 sum. FP64 work per thread, not per leaf (FP64 issues at
+// 1/64 of the FP32 rate here).
+__device__ __forceinline__ void flux_add(float I, int L, float &hi, float &lo, double &tiny) {
+  const float x = __fmul_rn(I, __int_as_float((127 - 2 * L) << 23));
+  if (fabsf(x) >= 0x1p-126f || x == 0.f) {
+    const float t = __fadd_rn(hi, x);
+    const float bv = __fsub_rn(t, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bv)), __fsub_rn(x, bv)));
+    hi = t;
+  } else {
+    tiny = fma((double)I, pow4_neg(L), tiny);
+  }
 }
 
 cudaError_t launch_init_base(const TreeView &t, cudaStream_t st);
