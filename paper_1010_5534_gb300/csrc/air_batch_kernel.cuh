@@ -116,11 +116,15 @@ static size_t batch_smem(const GridView &g, int V) {
   return tab + 3 * sizeof(int64_t) * V + sizeof(int32_t) * V + sizeof(int32_t) * (kBatchBlock / 32) * V;
 }
 
-// No minimum-blocks bound: with one, the compiler takes more registers (198
-// instead of 152 at 8 bands per thread) and the batch runs slower; bounds of 4
-// and more blocks per SM spill in the refinement phases and run 2.5x slower.
+// Resident blocks per SM. Left open, the compiler took 234 registers at 8 bands
+// per thread (two blocks).
+template <int NBT>
+struct BatchBlocks {
+  static constexpr int value = NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? 3 : 2));
+};
+
 template <int NBT, bool AMR, int FMT>
-__global__ void __launch_bounds__(kBatchBlock) k_air_batch(BatchArgs a) {
+__global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT>::value) k_air_batch(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const GridView &g = a.g;
   const int V = a.V, nb = g.n_bands;

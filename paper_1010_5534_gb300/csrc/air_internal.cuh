@@ -155,6 +155,8 @@ struct RaySource {
   SweepState *sweep;    // mode 2: rays [S->n, S->n + 4 S->tot[0]), none once S->done;
                         // blocks take 128-ray chunks from S->ray_ctr[band chunk]
   int advance;          // mode 2: the launch's last block moves S on to the next sweep
+  int part;             // mode 2, a sweep launched in two forms: 1 traces only counts up to
+  int64_t few;          // `few` rays, 2 only larger ones (and advances either way); 0: any
   int use_prop;         // mode 2: copy a new pixel's values from `prop` when the
   Proposal prop;        // proposal traced it; trace only the pixels it missed
   // column table of an axis view (RayGeom::tab, levels of the n0 image), or NULL

@@ -202,21 +202,11 @@ __device__ __forceinline__ void tab_pair(const float *row, int q, float w, float
 // product) are rounded explicitly (__fmul_rn), so the compiler cannot fuse
 // them into the sums' subtractions: every instantiation (band chunking, form)
 // rounds alike and gives the same bits.
-// DARK = false: without the test (for one-band callers that have made it).
-template <int NBT, int FMT, bool DARK = true>
-__device__ __forceinline__ void rt_term(RTState<NBT> &r, float rho, uint32_t aux, float ds,
-                                        const BandCtx &bc, const BandRegs<NBT> &br) {
-  const float rds = __fmul_rn(rho, ds);
-  kahan_add(r.N, r.cN, rds);
-  if (DARK && FMT != kCellRho && cell_dark<FMT>(aux, br.xz) && r.N <= FLT_MAX) {
-    if (NBT == 1) {
-      kahan_add(r.I[0], r.cI[0], 0.f);
-      r.T[0] = ex2_approx(br.nk[0] * r.N);
-    } else {
-      rt_dark<NBT>(r, r.N, 0.f);
-    }
-    return;
-  }
+
+// The band terms of a cell that brought the column density to N.
+template <int NBT, int FMT>
+__device__ __forceinline__ void rt_bands(RTState<NBT> &r, float rho, uint32_t aux, float rds, float N,
+                                         const BandCtx &bc, const BandRegs<NBT> &br) {
   if (FMT != kCellRho && NBT > 1 && r.stale) rt_refresh<NBT>(r, br);
   float w = 0.f;
   const float *row = bc.tab;
@@ -233,7 +223,7 @@ __device__ __forceinline__ void rt_term(RTState<NBT> &r, float rho, uint32_t aux
       for (int e = 0; e < (NBT == 1 ? 1 : 2); ++e) {
         const int b = 2 * q + e;
         const float dtau = br.kap[b] * rds;
-        const float Tn = ex2_approx(br.nk[b] * r.N);
+        const float Tn = ex2_approx(br.nk[b] * N);
         // rho Lambda_b
         const float rl = FMT == kCellLam ? __uint_as_float(aux) : (FMT == kCellXq ? rho * lam[e] : rho);
         const float t_small = __fmul_rn(rl * rds, r.T[b] * one_minus_exp_over_x(dtau));
@@ -246,23 +236,34 @@ __device__ __forceinline__ void rt_term(RTState<NBT> &r, float rho, uint32_t aux
   }
 }
 
-// One cell chord of length ds >= 0 on the DDA path. A zero-length chord (a
-// ray grazing an edge or corner) adds nothing and is not counted as a step.
-// Both transfer forms are evaluated and one selected per band: a per-cell
-// branch to the series form alone (same bits when kmax (rho ds) < 1/4) was
-// timed and made the batched 16-band renders 15% slower.
-template <int NBT, int FMT>
-__device__ __forceinline__ void rt_cell(RTState<NBT> &r, float rho, uint32_t aux, float ds,
+// The band terms of dark cells up to column density N.
+template <int NBT>
+__device__ __forceinline__ void rt_dark_to(RTState<NBT> &r, float N, const BandRegs<NBT> &br) {
+  if (NBT == 1) {
+    kahan_add(r.I[0], r.cI[0], 0.f);
+    r.T[0] = ex2_approx(br.nk[0] * N);
+  } else {
+    rt_dark<NBT>(r, N, 0.f);
+  }
+}
+
+// DARK = false: without the test (for callers that have made it).
+template <int NBT, int FMT, bool DARK = true>
+__device__ __forceinline__ void rt_term(RTState<NBT> &r, float rho, uint32_t aux, float ds,
                                         const BandCtx &bc, const BandRegs<NBT> &br) {
-  r.steps += ds > 0.f ? 1u : 0u;
-  rt_term<NBT, FMT>(r, rho, aux, ds, bc, br);
+  const float rds = __fmul_rn(rho, ds);
+  kahan_add(r.N, r.cN, rds);
+  if (DARK && cell_dark<FMT>(aux, br.xz) && r.N <= FLT_MAX) rt_dark_to<NBT>(r, r.N, br);
+  else rt_bands<NBT, FMT>(r, rho, aux, rds, r.N, bc, br);
 }
 
 // Cells that the DDA steps through, and requests, before it sums the first of
-// them (march_block).
-template <int NBT>
+// them (march_block). DIR = -1, the form for launches that leave most of the
+// GPU's threads idle, goes further ahead: there a ray's time is its number of
+// chunks times the L2's latency (800 cycles), and registers are free.
+template <int NBT, int DIR>
 struct DdaChunk {
-  static constexpr int value = 4;
+  static constexpr int value = DIR >= 0 ? 4 : (NBT <= 2 ? 16 : 8);
 };
 
 // Fields of cell idx: rho and the auxiliary word of the format.
@@ -527,17 +528,16 @@ struct ColumnUnroll {
 // origin.
 //
 // Which cells a ray crosses does not depend on their fields, so the walk runs
-// DdaChunk cells ahead of the sums: it steps through a chunk of cells, asking
+// K cells ahead of the sums: it steps through a chunk of cells, asking
 // for each record as its index is known, and only then sums the chunk. One
 // load latency is paid per chunk instead of one per cell, and the step's own
 // dependent operations overlap the loads.
-template <int NBT, int FMT, typename Idx>
+template <int NBT, int FMT, int K, typename Idx>
 __device__ __forceinline__ void march_block(RTState<NBT> &r, const float Q[3], const float Dl[3],
                                             const float inv[3], float tend, int lx, int ly, int lz,
                                             int nx, int ny, int nz, Idx sy, Idx sz,
                                             const void *__restrict__ cells, const BandCtx &bc,
                                             const BandRegs<NBT> &br) {
-  constexpr int K = DdaChunk<NBT>::value;
   const float INF = FLT_MAX;
   const bool p0 = Dl[0] > 0.f, p1 = Dl[1] > 0.f, p2 = Dl[2] > 0.f;
   const float a0 = fabsf(inv[0]), a1 = fabsf(inv[1]), a2 = fabsf(inv[2]);
@@ -562,18 +562,17 @@ __device__ __forceinline__ void march_block(RTState<NBT> &r, const float Q[3], c
     for (int u = 0; u < K; ++u) {
       in[u] = more;
       if (more) load_cell<FMT>(cells, idx, rh[u], xv[u]);
-      const float tn = fminf(fminf(tm0, tm1), fminf(tm2, tend));
+      const float tmin = fminf(fminf(tm0, tm1), tm2);
+      const float tn = fminf(tmin, tend);
       ds[u] = fmaxf(tn - tl, 0.f);
       tl = tn;
       // step the axis whose face comes first; an axis that is not stepped
       // keeps its count and so its boundary parameter
-      const bool x0 = tm0 <= tm1 && tm0 <= tm2;
-      const bool x1 = !x0 && tm1 <= tm2;
-      if (x0) {
+      if (tm0 == tmin) {
         k0 += 1.f;
         tm0 = fmaf(k0, a0, q0);
         idx += d0;
-      } else if (x1) {
+      } else if (tm1 == tmin) {
         k1 += 1.f;
         tm1 = fmaf(k1, a1, q1);
         idx += d1;
@@ -582,11 +581,32 @@ __device__ __forceinline__ void march_block(RTState<NBT> &r, const float Q[3], c
         tm2 = fmaf(k2, a2, q2);
         idx += d2;
       }
-      more = more && tn < tend && k0 <= km0 && k1 <= km1 && k2 <= km2;
+      more = more && tmin < tend && k0 <= km0 && k1 <= km1 && k2 <= km2;
     }
+    // the chunk's column density, and whether any of its cells emits. A
+    // zero-length chord (a ray grazing an edge or corner) adds nothing and is
+    // not counted as a step.
+    float N[K];
+    uint32_t x = 0u;
 #pragma unroll
     for (int u = 0; u < K; ++u)
-      if (in[u]) rt_cell<NBT, FMT>(r, rh[u], xv[u], ds[u], bc, br);
+      if (in[u]) {
+        r.steps += ds[u] > 0.f ? 1u : 0u;
+        ds[u] = __fmul_rn(rh[u], ds[u]);  // rho ds from here on
+        kahan_add(r.N, r.cN, ds[u]);
+        N[u] = r.N;
+        x = FMT == kCellLam ? x | xv[u] : max(x, xv[u]);
+      }
+    if (cell_dark<FMT>(x, br.xz) && r.N <= FLT_MAX) {
+      rt_dark_to<NBT>(r, r.N, br);
+    } else {
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (in[u]) {
+          if (NBT > 1 && cell_dark<FMT>(xv[u], br.xz) && N[u] <= FLT_MAX) rt_dark_to<NBT>(r, N[u], br);
+          else rt_bands<NBT, FMT>(r, rh[u], xv[u], ds[u], N[u], bc, br);
+        }
+    }
   } while (more);  // until the block is left (through its far face, or by rounding)
 }
 
@@ -838,7 +858,7 @@ __device__ __forceinline__ int axis_table_entry(const GridView &g, const RayGeom
   return (o >= 0.0 && o < (double)g.nf[a]) ? (int)o : -1;
 }
 
-template <int NBT, int FMT>
+template <int NBT, int FMT, int K>
 __device__ void march_uniform(RTState<NBT> &r, const GridView &g, const double O[3],
                               const RayGeom &rg, double t0, const BandCtx &bc,
                               const BandRegs<NBT> &br) {
@@ -856,10 +876,10 @@ __device__ void march_uniform(RTState<NBT> &r, const GridView &g, const double O
   // (indices are 32-bit where every cell has one; a step past the block may
   // lie one row beyond)
   if ((int64_t)g.nf[0] * g.nf[1] * ((int64_t)g.nf[2] + 2) <= 0x7fffffff)
-    march_block<NBT, FMT, int>(r, Q, Dl, inv, FLT_MAX, lc[0], lc[1], lc[2], g.nf[0], g.nf[1], g.nf[2],
+    march_block<NBT, FMT, K, int>(r, Q, Dl, inv, FLT_MAX, lc[0], lc[1], lc[2], g.nf[0], g.nf[1], g.nf[2],
                                g.nf[0], g.nf[0] * g.nf[1], g.cells, bc, br);
   else
-    march_block<NBT, FMT, int64_t>(r, Q, Dl, inv, FLT_MAX, lc[0], lc[1], lc[2], g.nf[0], g.nf[1],
+    march_block<NBT, FMT, K, int64_t>(r, Q, Dl, inv, FLT_MAX, lc[0], lc[1], lc[2], g.nf[0], g.nf[1],
                                    g.nf[2], (int64_t)g.nf[0], (int64_t)g.nf[0] * g.nf[1], g.cells,
                                    bc, br);
 }
@@ -923,7 +943,7 @@ __device__ __forceinline__ int brick_of(const GridView &g, int e, const int c[3]
 // is marched, so its latency overlaps the march. Per-launch constants
 // (direction, its inverse and its double-float split) are read from the
 // kernel-parameter bank, not held per thread.
-template <int NBT, int FMT>
+template <int NBT, int FMT, int K>
 __device__ void march_amr(RTState<NBT> &r, const GridView &g, const double O[3], const F2 Of[3],
                           const RayGeom &rg, double t0, int eax, int fp64_level,
                           const BandCtx &bc, const BandRegs<NBT> &br) {
@@ -1064,7 +1084,7 @@ __device__ void march_amr(RTState<NBT> &r, const GridView &g, const double O[3],
     const int64_t boff = (int64_t)code << (3 * lb);
     const void *cb = FMT == kCellRho ? (const void *)((const float *)g.cells + boff)
                                      : (const void *)((const uint2 *)g.cells + boff);
-    march_block<NBT, FMT, int>(r, Q, Dl, inv, tend, lc[0], lc[1], lc[2], B, B, B, B, B * B, cb,
+    march_block<NBT, FMT, K, int>(r, Q, Dl, inv, tend, lc[0], lc[1], lc[2], B, B, B, B, B * B, cb,
                                bc, br);
     if (out) break;
     // advance to the exit point
@@ -1272,14 +1292,14 @@ __device__ __forceinline__ void march_axis(RTState<NBT> &st, const GridView &g, 
   if constexpr (!AMR) march_uniform_axis<NBT, FMT, U>(st, g, A, c1, c2, rg, bc, br);
   else if constexpr (DIR >= 7) march_amr_axis<NBT, FMT, U, false, (DIR < 10 ? 1 : -1), (DIR - 1) % 3>(st, g, A, c1, c2, rg, bc, br);
   else if constexpr (DIR >= 4) march_amr_axis_small<NBT, FMT>(st, g, A, c1, c2, rg, bc, br);
-  else march_amr_axis<NBT, FMT, U, DIR == 0>(st, g, A, c1, c2, rg, bc, br);
+  else march_amr_axis<NBT, FMT, U, (DIR <= 0)>(st, g, A, c1, c2, rg, bc, br);
 }
 
 // One ray (pixel (L, i, j)) through the grid, bands [b0, b0 + NBT) of bc/br.
 // DIR = 1 + A: every ray of the launch is parallel to grid axis A (bricks of 16
 // cells and more, or a uniform grid); 4 + A: the same with bricks of at most 8
 // cells; 7 + A and 10 + A: with 16^3 bricks, towards higher and lower cells;
-// 0: any direction.
+// 0: any direction; -1: inclined rays in launches of few rays (DdaChunk).
 template <int NBT, bool AMR, int FMT, int DIR = 0>
 __device__ __forceinline__ void trace_ray(RTState<NBT> &st, const GridView &g, const RayGeom &rg,
                                           int L, int i, int j, int fp64_level, const BandCtx &bc,
@@ -1290,7 +1310,7 @@ __device__ __forceinline__ void trace_ray(RTState<NBT> &st, const GridView &g, c
     march_axis<NBT, AMR, FMT, DIR, U>(st, g, rg, (DIR - 1) % 3, L, i, j, bc, br);
   } else {
     const bool m0 = rg.Dhi[0] != 0.f, m1 = rg.Dhi[1] != 0.f, m2 = rg.Dhi[2] != 0.f;
-    if (m0 + m1 + m2 == 1) {
+    if (DIR == 0 && m0 + m1 + m2 == 1) {
       march_axis<NBT, AMR, FMT, DIR, U>(st, g, rg, m0 ? 0 : (m1 ? 1 : 2), L, i, j, bc, br);
       return;
     }
@@ -1298,8 +1318,9 @@ __device__ __forceinline__ void trace_ray(RTState<NBT> &st, const GridView &g, c
     F2 Of[3];
     int eax;
     if (!ray_setup(g, rg, L, i, j, O, Of, t0, eax)) return;
-    if (AMR) march_amr<NBT, FMT>(st, g, O, Of, rg, t0, eax, fp64_level, bc, br);
-    else march_uniform<NBT, FMT>(st, g, O, rg, t0, bc, br);
+    constexpr int K = DdaChunk<NBT, DIR>::value;
+    if (AMR) march_amr<NBT, FMT, K>(st, g, O, Of, rg, t0, eax, fp64_level, bc, br);
+    else march_uniform<NBT, FMT, K>(st, g, O, rg, t0, bc, br);
   }
 }
 

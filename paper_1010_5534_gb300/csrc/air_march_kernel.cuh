@@ -30,9 +30,11 @@ struct MarchLaunch {
 constexpr int kAxisBlocks = 8;
 constexpr int kAxisBlocksSmall = 6;  // bricks of at most 8 cells: two bricks' records in registers
 
+// DIR = -1 has the registers of two or three blocks (see DdaChunk).
 template <int NBT, int DIR>
 struct MinBlocks {
-  static constexpr int value = DIR >= 4 && DIR <= 6 ? kAxisBlocksSmall
+  static constexpr int value = DIR < 0 ? (NBT <= 4 ? 3 : 2)
+                               : DIR >= 4 && DIR <= 6 ? kAxisBlocksSmall
                                : DIR >= 1 ? kAxisBlocks
                                : (NBT <= 1 ? 6 : (NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? 3 : 2))));
 };
@@ -109,8 +111,9 @@ __global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
     SweepState *S = src.sweep;
     if (S->done) return;
     const int64_t count = 4 * S->tot[0], first = S->n;
+    const bool skip = (src.part == 1 && count > src.few) || (src.part == 2 && count <= src.few);
     __shared__ long long s_chunk;
-    for (;;) {
+    while (!skip) {
       if (threadIdx.x == 0) s_chunk = (long long)atomicAdd(S->ray_ctr + chunk, 1ull);
       __syncthreads();
       const int64_t r0 = (int64_t)s_chunk * blockDim.x;
@@ -182,14 +185,46 @@ static cudaError_t march_form(const MarchLaunch &m) {
                     m.g, m.rg, m.src, m.out, m.fp64_level);
 }
 
+// Rays that fill the GPU's threads once in the form for few rays.
+template <int NBT>
+static int64_t few_rays(const MarchLaunch &m) {
+  return (int64_t)sm_count() * MinBlocks<NBT, -1>::value * kMarchBlock / m.chunks;
+}
+
+// Inclined rays. A launch of few rays takes the form for them; where the count
+// is on the device both forms are launched, and the one it is not for returns.
+template <int NBT, bool AMR, int FMT>
+static cudaError_t march_inclined(const MarchLaunch &m) {
+  const int64_t few = few_rays<NBT>(m);
+  if (m.src.mode != 2)
+    return m.blocks * kMarchBlock <= few ? march_form<NBT, AMR, FMT, -1>(m) : march_form<NBT, AMR, FMT, 0>(m);
+  RaySource s1 = m.src, s2 = m.src;
+  s1.part = 1;
+  s1.advance = 0;
+  s2.part = 2;
+  s1.few = s2.few = few;
+  const cudaError_t e = march_form<NBT, AMR, FMT, -1>(MarchLaunch{m.g, m.rg, s1, m.out, m.blocks, m.chunks, m.fp64_level, m.st});
+  if (e != cudaSuccess) return e;
+  return march_form<NBT, AMR, FMT, 0>(MarchLaunch{m.g, m.rg, s2, m.out, m.blocks, m.chunks, m.fp64_level, m.st});
+}
+
+template <int NBT, bool AMR, int FMT>
+static cudaError_t march_any(const MarchLaunch &m) {
+  // 16 bands per thread leave no registers for the form for few rays
+  const int moving = (m.rg.Dhi[0] != 0.f) + (m.rg.Dhi[1] != 0.f) + (m.rg.Dhi[2] != 0.f);
+  if constexpr (NBT <= 8)
+    if (moving > 1) return march_inclined<NBT, AMR, FMT>(m);
+  return march_form<NBT, AMR, FMT, 0>(m);
+}
+
 // Rays in any direction, NBT bands per thread.
 template <int NBT>
 cudaError_t march_general(const MarchLaunch &m) {
   const bool amr = m.g.kind == AIR_GRID_AMR;
-  if (m.g.cell_fmt == kCellRho) return amr ? march_form<NBT, true, kCellRho, 0>(m) : march_form<NBT, false, kCellRho, 0>(m);
-  if (m.g.cell_fmt == kCellXq) return amr ? march_form<NBT, true, kCellXq, 0>(m) : march_form<NBT, false, kCellXq, 0>(m);
+  if (m.g.cell_fmt == kCellRho) return amr ? march_any<NBT, true, kCellRho>(m) : march_any<NBT, false, kCellRho>(m);
+  if (m.g.cell_fmt == kCellXq) return amr ? march_any<NBT, true, kCellXq>(m) : march_any<NBT, false, kCellXq>(m);
   // per-cell Lambda exists for one-band grids only
-  if constexpr (NBT == 1) return amr ? march_form<1, true, kCellLam, 0>(m) : march_form<1, false, kCellLam, 0>(m);
+  if constexpr (NBT == 1) return amr ? march_any<1, true, kCellLam>(m) : march_any<1, false, kCellLam>(m);
   return cudaErrorInvalidValue;
 }
 
