@@ -397,10 +397,10 @@ air_status sweep_loop_device(air_grid *g, const Camera &cam, const air_params *p
   s0.m = m;
   s0.done = m == 0;
   CU_TRY(cudaMemcpyAsync(w.d_sweep, &s0, sizeof(SweepState), cudaMemcpyHostToDevice, st));
-  // the fused scan and balance only set flags: the base pixels' start at zero
-  CU_TRY(cudaMemsetAsync(w.flag, 0, sizeof(uint32_t) * (size_t)nbase, st));
   int32_t *const open2[2] = {w.open[0], w.open[1]};
   const int64_t nb_cap = scan_blocks(open_max);
+  uint32_t *counts = (uint32_t *)w.boff;  // 3 x int64 per block of the whole pyramid
+  CU_TRY(launch_open_init(w.open[0], w.flag, m, counts, nb_cap, st));
   RaySource ds{};
   ds.mode = 2; ds.n0 = pr->base_res; ds.lvl = t.lvl; ds.pi = t.pi; ds.pj = t.pj; ds.sweep = w.d_sweep;
   {
@@ -425,11 +425,10 @@ air_status sweep_loop_device(air_grid *g, const Camera &cam, const air_params *p
     // step iii: scan and balance in one pass (counted as the scan phase)
     CU_TRY(prof_open(g, AIR_PHASE_SCAN, 1));
     CU_TRY(launch_sweep_scan_balance(t, open2, w.d_sweep, pr->xi_crit, pr->xi_norm, pr->refine_on,
-                                     w.flag, w.d_err, st, lmap));
+                                     w.flag, counts, nb_cap, w.d_err, st, lmap));
     CU_TRY(prof_close(g));
-    CU_TRY(prof_open(g, AIR_PHASE_REFINE, 3));
-    CU_TRY(launch_sweep_count(t, open2, w.d_sweep, w.flag, w.bcount, w.boff, nb_cap, st));
-    CU_TRY(launch_sweep_emit(t, open2, w.d_sweep, w.flag, w.boff, nb_cap, st, lmap));
+    CU_TRY(prof_open(g, AIR_PHASE_REFINE, 1));
+    CU_TRY(launch_sweep_emit(t, open2, w.d_sweep, w.flag, counts, nb_cap, st, lmap));
     CU_TRY(prof_close(g));
     // step ii on the new pixels (or their values from the proposal); the
     // march's last block (or the band sum after it) moves the state on
@@ -593,9 +592,10 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
     // open-leaf list: the base pixels, unless the base is the top level
     int cur = 0;
     int64_t m = Lm > 0 ? nbase : 0;
-    CU_TRY(launch_list_init(w.open[0], m, st));
+    if (!dev_loop) CU_TRY(launch_list_init(w.open[0], m, st));
     int32_t *lmap = nullptr;
     if ((s = level_maps(g, n0, Lm, &lmap))) return s;
+    g->last.lmap = lmap;
     if (dev_loop) {
       SweepState fin;
       if ((s = sweep_loop_device(g, cam, pr, nbase, m, bound, open_max, tune, march_launches, lmap,
@@ -687,6 +687,7 @@ air_status output_tree(air_grid *g, const Camera &cam, const air_params *pr, air
   g->raster.ok = true;
   g->raster.n0 = n0;
   g->raster.Lm = pr->max_level;
+  g->raster.lmap = g->last.lmap;
   CU_TRY(ensure((void **)&w.partial, &w.partial_b, sizeof(double) * (nb + 1) * flux_blocks(n)));
   FluxArgs fa{};
   fa.n = n; fa.child = t.child; fa.lvl = t.lvl; fa.steps = t.steps;

@@ -152,8 +152,7 @@ __global__ void __launch_bounds__(256) k_vflux(TreeView t, const int16_t *view, 
   }
   // the warp's sum of band q (to every lane), its accumulators emptied
   auto take = [&](int q) {
-    double s = ((double)hi[q] + (double)lo[q]) + tiny[q];
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    const double s = flux_warp_sum(hi[q], lo[q], tiny[q]);
     hi[q] = lo[q] = 0.f;
     tiny[q] = 0.0;
     return s;

@@ -181,6 +181,7 @@ struct SpectraWork {
 struct RasterSrc {
   bool ok = false;
   int n0 = 0, Lm = 0;
+  const int32_t *lmap = nullptr;  // the tree's level maps (NULL: it has none)
   float *scratch = nullptr;  // device staging for host outputs
   size_t scratch_b = 0;
 };
@@ -191,6 +192,7 @@ struct LastRender {
   air_params params;
   int64_t n_nodes = 0, n_refined = 0;
   int32_t n_sweeps = 0;
+  const int32_t *lmap = nullptr;  // the tree's level maps (NULL: it has none)
 };
 
 }  // namespace air

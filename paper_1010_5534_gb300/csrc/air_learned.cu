@@ -462,6 +462,7 @@ air_status render_learned(air_grid *g, const air_view *view, const air_params *p
   // the replay runs with its counts on the device when the node arrays can
   // hold the whole pyramid (as the plain render's loop)
   const bool dev_loop = pyramid_fits(g, bound);
+  g->last.lmap = nullptr;  // the host-count loop below keeps no level maps
   if ((s = ensure_nodes(g, dev_loop ? bound : std::min<int64_t>(bound, std::max<int64_t>(4 * nbase, w.cap)),
                         0, bound))) return s;
   CU_TRY(ensure((void **)&lw.x, &lw.x_b, sizeof(uint16_t) * 4 * nbase * kFeat));
@@ -526,12 +527,13 @@ air_status render_learned(air_grid *g, const air_view *view, const air_params *p
   CU_TRY(ensure((void **)&w.boff, &w.boff_b, 3 * sizeof(int64_t) * scan_blocks(bound)));
   int cur = 0;
   int64_t mo = Lm > 0 ? nbase : 0;
-  CU_TRY(launch_list_init(w.open[0], mo, st));
+  if (!dev_loop) CU_TRY(launch_list_init(w.open[0], mo, st));
   if (dev_loop) {
     // the device-count sweep loop; new pixels copy their values from the
     // proposal wave where it traced them, the march traces the rest
     int32_t *lmap = nullptr;
     if ((s = level_maps(g, n0, Lm, &lmap))) return s;
+    g->last.lmap = lmap;
     const Proposal prop{lw.depth, lw.off, lw.pN, lw.pI, lw.pp, lw.psteps, std::max<int64_t>(P, 1)};
     SweepState fin;
     if ((s = sweep_loop_device(g, cam, pr, nbase, mo, bound, open_max, tune, march_launches, lmap, &prop,

@@ -8,7 +8,8 @@
 
 namespace air {
 
-// One thread per finest pixel (x, y) of an (n0 2^Lm)^2 raster. The covering
+// One thread per finest pixel (x, y) of an (n0 2^Lm)^2 raster (for base images
+// and trees without level maps; else k_raster_maps). The covering
 // leaf is the deepest node containing the pixel. For the bilinear form, with
 // s = Lm - L, the pixel centre on the level-L grid is
 // u = (x + 1/2) 2^-s - 1/2 = (2x + 1 - 2^s) / 2^(s+1): its floor is an
@@ -39,6 +40,98 @@ __global__ void k_raster(TreeView t, int Lm, int mode, const float *__restrict__
   const float v01 = val[descend(t, 0, L, ia, jb)], v11 = val[descend(t, 0, L, ib, jb)];
   const float gu = 1.f - fu, gv = 1.f - fv;
   out[k] = (gu * gv) * v00 + (fu * gv) * v10 + (gu * fv) * v01 + (fu * fv) * v11;
+}
+
+// The same raster through the tree's level maps (air_tree.cuh), for images with
+// at least one level: a thread takes the 2 x 2 finest pixels of one level
+// Lm - 1 pixel. One map entry then tells the case:
+//   a node with children: the four pixels are its children, finest leaves,
+//     which keep their values (their index fractions are zero);
+//   a leaf: the four pixels lie between it and its 8 neighbours at its level;
+//   none: a coarser leaf, level L <= Lm - 2; the four pixels share the four
+//     level-L pixels they lie between (the cell boundary x = 2^(s-1) mod 2^s,
+//     s = Lm - L >= 2, is even).
+// Before, every pixel descended from its base pixel through up to Lm child
+// links five times: 45 us for a 2048^2 raster of which 2.5 us are its writes.
+// VEC: out is 8-byte aligned.
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_raster_maps(TreeView t, const int32_t *__restrict__ lmap, int Lm,
+                                                     int mode, const float *__restrict__ val,
+                                                     float *__restrict__ out) {
+  const int nh = t.n0 << (Lm - 1);
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= (int64_t)nh * nh) return;
+  const int jc = (int)(q / nh), ic = (int)(q - (int64_t)jc * nh);
+  float v[4];  // pixels (2 ic + (e & 1), 2 jc + (e >> 1))
+  int k;       // the level Lm - 1 node, or -1
+  if (Lm == 1) k = jc * t.n0 + ic;
+  else k = __ldg(lmap + level_map_offset(t.n0, Lm - 1) + q);
+  const int c = k >= 0 ? t.child[k] : -1;
+  if (c >= 0) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = val[c + e];
+  } else {
+    int L = Lm - 1;
+    if (k < 0) {  // a coarser leaf
+      while (k < 0) {
+        --L;
+        const int s = Lm - 1 - L;
+        if (L == 0) k = (jc >> s) * t.n0 + (ic >> s);
+        else k = __ldg(lmap + level_map_offset(t.n0, L) + (int64_t)(jc >> s) * (t.n0 << L) + (ic >> s));
+      }
+    }
+    if (mode == AIR_RASTER_NEAREST) {
+      const float x = val[k];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = x;
+    } else {
+      const int s = Lm - L, nl = t.n0 << L;
+      const float sc = __int_as_float((127 - (s + 1)) << 23);  // 2^-(s+1)
+      // columns and rows of level-L pixels the two finest columns and rows lie
+      // between: [i0, i0 + 1], and for s = 1 one further for the second
+      int i0[2], j0[2];
+      float fu[2], fv[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int nu = 2 * (2 * ic + e) + 1 - (1 << s), nv = 2 * (2 * jc + e) + 1 - (1 << s);
+        i0[e] = nu >> (s + 1);
+        j0[e] = nv >> (s + 1);
+        fu[e] = (float)(nu - i0[e] * (2 << s)) * sc;
+        fv[e] = (float)(nv - j0[e] * (2 << s)) * sc;
+      }
+      float w[3][3];  // values of level-L pixels (i0[0] + a, j0[0] + b)
+      const int na = i0[1] - i0[0] + 2;  // 2 or 3, the same for both axes
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+          if (a < na && b < na) {
+            const int ii = min(max(i0[0] + a, 0), nl - 1), jj = min(max(j0[0] + b, 0), nl - 1);
+            w[b][a] = val[map_deepest(t, lmap, L, ii, jj)];
+          }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int x = e & 1, y = e >> 1;
+        const bool dx = x && na == 3, dy = y && na == 3;
+        const float v00 = dy ? (dx ? w[1][1] : w[1][0]) : (dx ? w[0][1] : w[0][0]);
+        const float v10 = dy ? (dx ? w[1][2] : w[1][1]) : (dx ? w[0][2] : w[0][1]);
+        const float v01 = dy ? (dx ? w[2][1] : w[2][0]) : (dx ? w[1][1] : w[1][0]);
+        const float v11 = dy ? (dx ? w[2][2] : w[2][1]) : (dx ? w[1][2] : w[1][1]);
+        const float gu = 1.f - fu[x], gv = 1.f - fv[y];
+        v[e] = (gu * gv) * v00 + (fu[x] * gv) * v10 + (gu * fv[y]) * v01 + (fu[x] * fv[y]) * v11;
+      }
+    }
+  }
+  float *o = out + (int64_t)(2 * jc) * (2 * nh) + 2 * ic;
+  if (VEC) {
+    *reinterpret_cast<float2 *>(o) = make_float2(v[0], v[1]);
+    *reinterpret_cast<float2 *>(o + 2 * nh) = make_float2(v[2], v[3]);
+  } else {
+    o[0] = v[0];
+    o[1] = v[1];
+    o[2 * nh] = v[2];
+    o[2 * nh + 1] = v[3];
+  }
 }
 
 static bool is_device_ptr(const void *p) {
@@ -81,7 +174,13 @@ air_status render_raster(air_grid *g, int32_t quantity, int32_t band, int32_t mo
   }
   const int64_t blocks = (n + 255) / 256;
   if (blocks > 0x7fffffff) return set_error(AIR_ERR_ARG, "raster too large");
-  k_raster<<<(unsigned)blocks, 256, 0, st>>>(t, Lm, mode, val, dst);
+  if (Lm == 1 || (Lm > 1 && g->raster.lmap)) {
+    const unsigned quads = (unsigned)((n / 4 + 255) / 256);
+    if (((uintptr_t)dst & 7) == 0) k_raster_maps<true><<<quads, 256, 0, st>>>(t, g->raster.lmap, Lm, mode, val, dst);
+    else k_raster_maps<false><<<quads, 256, 0, st>>>(t, g->raster.lmap, Lm, mode, val, dst);
+  } else {
+    k_raster<<<(unsigned)blocks, 256, 0, st>>>(t, Lm, mode, val, dst);
+  }
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && !dev) e = cudaMemcpyAsync(out, dst, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -256,164 +256,171 @@ __global__ void __launch_bounds__(kScanBlock) k_emit3(TreeView t, const int32_t 
 }
 
 // ---- the sweep with counts on the device ----------------------------------
-// The same steps as above over open[S->cur] with m = S->m items; grids are a
-// few blocks per SM and loop over the items (k_count3d and k_emit3d over scan
-// chunks of kScanItems, chunk c's counts at bcount[sel * nb_cap + c]).
+// The same steps over open[S->cur] with m = S->m items, in two launches; grids
+// are a few blocks per SM and loop over the items. The first flags and counts,
+// the second ranks and emits: each of its blocks adds up the chunk counts in
+// front of its chunk (and in all, to know the totals) from the two count
+// arrays, a few kilobytes that lie in L2. (With a counting and a scanning
+// launch between them a sweep took 12 us more, whatever its size.)
+//
+// counts: two sets (S->cur) of [flagged | below the top level][nb_cap] chunk
+// counts. The set of the current sweep is zero when it starts; the emit kernel
+// zeroes the other one for the next. A flag word holds its leaf's position in
+// the open list (see FlagCount).
 
-__global__ void k_xi_scan_dev(TreeView t, const int32_t *__restrict__ open0,
-                              const int32_t *__restrict__ open1, const SweepState *__restrict__ S,
-                              double xi_crit, int xi_norm, int refine_on,
-                              uint32_t *__restrict__ flag, const int32_t *lmap) {
-  wait_prior_grid();
-  if (S->done) return;
-  const int64_t m = S->m;
-  const int32_t *open = S->cur ? open1 : open0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
-    const int64_t k = open[i];
-    flag[k] = xi_flag(t, NodeLookup{0, lmap}, k, xi_crit, xi_norm, refine_on);
-  }
+__device__ __forceinline__ FlagCount sweep_counts(uint32_t *counts, int64_t nb_cap, int set) {
+  uint32_t *c = counts + 2 * nb_cap * set;
+  return FlagCount{c, c + nb_cap};
 }
 
-// Scan and balance in one pass (counts on the device). Flags of the open
-// list are all zero when a sweep starts (a refined node's flag is cleared
-// with its children's, new children start at zero), so a thread only ever
-// sets flags: a leaf whose xi reaches xi_crit is flagged, and the thread that
-// moves a flag from 0 to 1 -- the scan's or a balance expansion's -- expands
-// it. Every flag is expanded once, and the flags reach the same closure as a
-// scan of every leaf followed by the balance.
-__global__ void k_scan_balance_dev(TreeView t, const int32_t *__restrict__ open0,
+// First open list: the m base pixels, flag words with their positions, and
+// the counts of the first set zeroed.
+__global__ void k_open_init(int32_t *list, uint32_t *flag, int64_t m, uint32_t *counts,
+                            int64_t nb_cap) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < m) {
+    list[i] = (int32_t)i;
+    flag[i] = (uint32_t)i << 1;
+  }
+  if (i < scan_chunks(m)) counts[i] = counts[nb_cap + i] = 0u;
+}
+
+// Scan and balance in one pass. No flag of the open list is set when a sweep
+// starts, so a thread only ever sets flags: a leaf whose xi reaches xi_crit is
+// flagged, and the thread that sets a flag -- the scan's or a balance
+// expansion's -- expands it. Every flag is expanded once, and the flags reach
+// the same closure as a scan of every leaf followed by the balance.
+__global__ void __launch_bounds__(kScanBlock) k_scan_balance_dev(TreeView t, const int32_t *__restrict__ open0,
                                    const int32_t *__restrict__ open1,
                                    const SweepState *__restrict__ S, double xi_crit, int xi_norm,
                                    int refine_on, uint32_t *__restrict__ flag,
+                                   uint32_t *__restrict__ counts, int64_t nb_cap,
                                    uint32_t *__restrict__ err, const int32_t *lmap) {
   wait_prior_grid();
   if (S->done) return;
   const int64_t m = S->m;
   const int32_t *open = S->cur ? open1 : open0;
+  const FlagCount fc = sweep_counts(counts, nb_cap, S->cur);
   const NodeLookup look{0, lmap};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
-    const int k = open[i];
-    if (xi_flag(t, look, k, xi_crit, xi_norm, refine_on) && atomicExch(flag + k, 1u) == 0u)
-      balance_from(t, look, k, flag, err);
-  }
-}
-
-__global__ void k_balance_dev(TreeView t, const int32_t *__restrict__ open0,
-                              const int32_t *__restrict__ open1, const SweepState *__restrict__ S,
-                              uint32_t *__restrict__ flag, uint32_t *__restrict__ err,
-                              const int32_t *lmap) {
-  wait_prior_grid();
-  if (S->done) return;
-  const int64_t m = S->m;
-  const int32_t *open = S->cur ? open1 : open0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
-    const int k = open[i];
-    if (flag[k] != 0) balance_from(t, NodeLookup{0, lmap}, k, flag, err);
-  }
-}
-
-__global__ void __launch_bounds__(kScanBlock) k_count3d(TreeView t, const int32_t *open0,
-                                                        const int32_t *open1,
-                                                        const SweepState *__restrict__ S,
-                                                        const uint32_t *flag, int32_t *bcount,
-                                                        int64_t nb_cap) {
-  wait_prior_grid();
-  if (S->done) return;
-  __shared__ int32_t wsum[3][kScanBlock / 32];
-  const int64_t m = S->m;
-  const int32_t *open = S->cur ? open1 : open0;
-  const int64_t nb = scan_chunks(m);
-  for (int64_t c = blockIdx.x; c < nb; c += gridDim.x) {
-    const int64_t start = c * kScanItems;
-    int32_t c0 = 0, c1 = 0, c2 = 0;
-    for (int rr = 0; rr < kScanRounds; ++rr) {
-      int k;
-      const ListSel q = list_sel(t, open, m, flag, t.Lm, start + (int64_t)rr * kScanBlock + threadIdx.x, k);
-      c0 += __popc(__ballot_sync(0xffffffffu, q.f));
-      c1 += __popc(__ballot_sync(0xffffffffu, q.keep));
-      c2 += __popc(__ballot_sync(0xffffffffu, q.co));
+  __shared__ unsigned long long queue[kScanBlock / 32][kWarpQueue];
+  // whole warps run the loop: a warp's 32 entries lie in one chunk
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < m; i0 += stride) {
+    const int64_t i = i0 + (threadIdx.x & 31);
+    const int k = i < m ? open[i] : 0;
+    bool mine = i < m && xi_flag(t, look, k, xi_crit, xi_norm, refine_on) &&
+                (atomicOr(flag + k, 1u) & 1u) == 0u;
+    const bool below = mine && t.lvl[k] + 1 < t.Lm;
+    const unsigned nf = __popc(__ballot_sync(0xffffffffu, mine));
+    const unsigned nc = __popc(__ballot_sync(0xffffffffu, below));
+    if ((threadIdx.x & 31) == 0 && nf) {
+      atomicAdd(fc.flagged + i0 / kScanItems, nf);
+      if (nc) atomicAdd(fc.below + i0 / kScanItems, nc);
     }
-    if ((threadIdx.x & 31) == 0) {
-      wsum[0][threadIdx.x >> 5] = c0;
-      wsum[1][threadIdx.x >> 5] = c1;
-      wsum[2][threadIdx.x >> 5] = c2;
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-      int32_t sum = 0;
-      for (int w = 0; w < kScanBlock / 32; ++w) sum += wsum[threadIdx.x][w];
-      bcount[threadIdx.x * nb_cap + c] = sum;
-    }
-    __syncthreads();
-  }
-}
-
-// Block b scans selection b's chunk counts; totals to S->tot, and block 0
-// sets S->done when nothing was flagged (blocks 1 and 2 may then see it and
-// return early: their totals are not needed once the loop has ended).
-__global__ void __launch_bounds__(1024) k_scan_blocks3d(const int32_t *bcount, int64_t nb_cap,
-                                                        int64_t *boff, SweepState *S) {
-  wait_prior_grid();
-  if (S->done) return;
-  __shared__ int64_t part[1024];
-  const int64_t nb = scan_chunks(S->m);
-  const int32_t *bc = bcount + blockIdx.x * nb_cap;
-  int64_t *bo = boff + blockIdx.x * nb_cap;
-  const int64_t per = (nb + 1023) / 1024;
-  const int64_t a = threadIdx.x * per, b = min(nb, a + per);
-  int64_t s = 0;
-  for (int64_t x = a; x < b; ++x) s += bc[x];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {
-    const int64_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
-    __syncthreads();
-    part[threadIdx.x] += v;
-    __syncthreads();
-  }
-  int64_t run = part[threadIdx.x] - s;
-  for (int64_t x = a; x < b; ++x) {
-    bo[x] = run;
-    run += bc[x];
-  }
-  if (threadIdx.x == 1023) {
-    S->tot[blockIdx.x] = part[1023];
-    if (blockIdx.x == 0 && part[1023] == 0) S->done = 1;  // nothing flagged: the loop ends
-  }
-}
-
-__global__ void __launch_bounds__(kScanBlock) k_emit3d(TreeView t, int32_t *open0,
-                                                       int32_t *open1, const SweepState *__restrict__ S,
-                                                       uint32_t *flag, const int64_t *boff,
-                                                       int64_t nb_cap, int32_t *lmap) {
-  wait_prior_grid();
-  if (S->done) return;
-  __shared__ int32_t wsum[3][kScanBlock / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t m = S->m, n_old = S->n, keep_total = S->tot[1];
-  const int32_t *open = S->cur ? open1 : open0;
-  int32_t *next = S->cur ? open0 : open1;
-  const int64_t nb = scan_chunks(m);
-  const uint32_t below = (1u << lane) - 1u;
-  for (int64_t c = blockIdx.x; c < nb; c += gridDim.x) {
-    const int64_t start = c * kScanItems;
-    int64_t run0 = boff[c], run1 = boff[nb_cap + c], run2 = boff[2 * nb_cap + c];
-    for (int rr = 0; rr < kScanRounds; ++rr) {
-      int k;
-      const ListSel q = list_sel(t, open, m, flag, t.Lm, start + (int64_t)rr * kScanBlock + threadIdx.x, k);
-      // a flagged node's fields, loaded before the ranks are formed
-      int Lc = 0, pi = 0, pj = 0;
-      if (q.f) {
-        Lc = t.lvl[k] + 1;
+    if (lmap) {
+      int L = 0, pi = 0, pj = 0;
+      if (mine) {
+        L = t.lvl[k];
         pi = t.pi[k];
         pj = t.pj[k];
       }
-      const uint32_t b0 = __ballot_sync(0xffffffffu, q.f);
-      const uint32_t b1 = __ballot_sync(0xffffffffu, q.keep);
-      const uint32_t b2 = __ballot_sync(0xffffffffu, q.co);
+      balance_warp(t, lmap, mine, L, pi, pj, flag, err, fc, queue[threadIdx.x >> 5]);
+    } else if (mine) {
+      balance_from(t, look, k, flag, err, fc);
+    }
+  }
+}
+
+// Sums of a and b over the block (to every thread).
+__device__ __forceinline__ void block_sum4(uint32_t (&v)[4], uint32_t (&sh)[4][kScanBlock / 32]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = __reduce_add_sync(0xffffffffu, v[q]);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sh[q][threadIdx.x >> 5] = v[q];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint32_t s = 0;
+#pragma unroll
+    for (int w = 0; w < kScanBlock / 32; ++w) s += sh[q][w];
+    v[q] = s;
+  }
+}
+
+// Step iv over the list, and the next list: kept entries first (in order),
+// then the children below the top level (in order). Block 0 leaves the totals
+// in S->tot, and sets S->done when nothing was flagged (blocks that see it
+// return, as all do then).
+__global__ void __launch_bounds__(kScanBlock) k_emit3d(TreeView t, int32_t *open0, int32_t *open1,
+                                                       SweepState *__restrict__ S, uint32_t *flag,
+                                                       uint32_t *counts, int64_t nb_cap,
+                                                       int32_t *lmap) {
+  wait_prior_grid();
+  if (S->done) return;
+  __shared__ uint32_t sums[4][kScanBlock / 32];
+  __shared__ int32_t wsum[3][kScanBlock / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t m = S->m, n_old = S->n;
+  const int cur = S->cur;
+  const int32_t *open = cur ? open1 : open0;
+  int32_t *next = cur ? open0 : open1;
+  const FlagCount fc = sweep_counts(counts, nb_cap, cur);
+  const int64_t nb = scan_chunks(m);
+  // totals, and the counts in front of the block's first chunk
+  uint32_t v[4] = {0u, 0u, 0u, 0u};
+  for (int64_t x = threadIdx.x; x < nb; x += kScanBlock) {
+    const uint32_t a = fc.flagged[x], b = fc.below[x];
+    v[0] += a;
+    v[1] += b;
+    if (x < blockIdx.x) {
+      v[2] += a;
+      v[3] += b;
+    }
+  }
+  block_sum4(v, sums);
+  const int64_t nflag = v[0], nbelow = v[1], keep_total = m - nflag;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    S->tot[0] = nflag;
+    S->tot[1] = keep_total;
+    S->tot[2] = nbelow;
+    if (nflag == 0) S->done = 1;  // nothing flagged: the loop ends
+  }
+  if (nflag == 0) return;
+  // the other set of counts, for the next sweep's list
+  {
+    const FlagCount fo = sweep_counts(counts, nb_cap, cur ^ 1);
+    const int64_t nn = scan_chunks(keep_total + 4 * nbelow);
+    for (int64_t x = (int64_t)blockIdx.x * kScanBlock + threadIdx.x; x < nn; x += (int64_t)gridDim.x * kScanBlock)
+      fo.flagged[x] = fo.below[x] = 0u;
+  }
+  int64_t front0 = v[2], front2 = v[3];  // flagged, below: entries before chunk c
+  const uint32_t below = (1u << lane) - 1u;
+  for (int64_t c = blockIdx.x; c < nb; c += gridDim.x) {
+    const int64_t start = c * kScanItems;
+    int64_t run0 = front0, run1 = start - front0, run2 = front2;
+    for (int rr = 0; rr < kScanRounds; ++rr) {
+      const int64_t at = start + (int64_t)rr * kScanBlock + threadIdx.x;
+      int k = 0;
+      bool f = false, co = false;
+      if (at < m) {
+        k = open[at];
+        f = (flag[k] & 1u) != 0u;
+      }
+      const bool keep = at < m && !f;
+      // a flagged node's fields, loaded before the ranks are formed
+      int L = 0, i = 0, j = 0;
+      if (f) {
+        L = t.lvl[k] + 1;
+        i = t.pi[k];
+        j = t.pj[k];
+        co = L < t.Lm;
+      }
+      const uint32_t b0 = __ballot_sync(0xffffffffu, f);
+      const uint32_t b1 = __ballot_sync(0xffffffffu, keep);
+      const uint32_t b2 = __ballot_sync(0xffffffffu, co);
       if (lane == 0) {
         wsum[0][warp] = __popc(b0);
         wsum[1][warp] = __popc(b1);
@@ -431,32 +438,43 @@ __global__ void __launch_bounds__(kScanBlock) k_emit3d(TreeView t, int32_t *open
         t1 += v1;
         t2 += v2;
       }
-      if (q.f) {
+      if (f) {
         const int64_t c0 = n_old + 4 * (run0 + p0 + __popc(b0 & below));
-        const int L = Lc, i = pi, j = pj;
+        const int64_t r2 = keep_total + 4 * (run2 + p2 + __popc(b2 & below));
 #pragma unroll
         for (int ch = 0; ch < 4; ++ch) {
           t.lvl[c0 + ch] = (int8_t)L;
           t.pi[c0 + ch] = 2 * i + (ch & 1);
           t.pj[c0 + ch] = 2 * j + (ch >> 1);
           t.child[c0 + ch] = -1;
-          flag[c0 + ch] = 0u;
+          flag[c0 + ch] = co ? (uint32_t)(r2 + ch) << 1 : 0u;
         }
         t.child[k] = (int32_t)c0;
         flag[k] = 0u;
-        if (q.co) {
-          const int64_t r2 = keep_total + 4 * (run2 + p2 + __popc(b2 & below));
+        if (co) {
 #pragma unroll
           for (int ch = 0; ch < 4; ++ch) next[r2 + ch] = (int32_t)(c0 + ch);
           if (lmap) set_level_map(lmap, t.n0, L, i, j, c0);
         }
-      } else if (q.keep) {
-        next[run1 + p1 + __popc(b1 & below)] = k;
+      } else if (keep) {
+        const int64_t r1 = run1 + p1 + __popc(b1 & below);
+        next[r1] = k;
+        flag[k] = (uint32_t)r1 << 1;
       }
       run0 += t0;
       run1 += t1;
       run2 += t2;
       __syncthreads();
+    }
+    if (c + gridDim.x < nb) {  // the counts up to the block's next chunk
+      uint32_t w4[4] = {0u, 0u, 0u, 0u};
+      for (int64_t x = c + threadIdx.x; x < c + gridDim.x; x += kScanBlock) {
+        w4[0] += fc.flagged[x];
+        w4[1] += fc.below[x];
+      }
+      block_sum4(w4, sums);
+      front0 += w4[0];
+      front2 += w4[1];
     }
   }
 }
@@ -543,21 +561,10 @@ __global__ void k_init_base(TreeView t) {
 // the bands of a block, and bands run beside one another. (One block summed
 // every band of 8192 entries, band after band, before: 85 us for 0.8 M leaves
 // of four bands.)
-// Sum of v over the block (256 threads), to thread 0.
-template <typename T>
-__device__ __forceinline__ T block_sum(T v, T *sh) {
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  T s = sh[0];
-  for (int w = 1; w < 8; ++w) s += sh[w];
-  return s;
-}
-
 __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
-  __shared__ double sh[8];
+  __shared__ double sh[kFluxBands][8];
   __shared__ unsigned long long shs[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t start = (int64_t)blockIdx.x * a.per_block;
   const int64_t end = min(a.n, start + a.per_block);
   double *outp = a.partial + (int64_t)blockIdx.x * (a.n_bands + 1);
@@ -565,8 +572,13 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
   if (b0 >= a.n_bands) {
     unsigned long long st = 0;
     for (int64_t k = start + threadIdx.x; k < end; k += blockDim.x) st += a.steps[k];
-    st = block_sum(st, shs);
-    if (threadIdx.x == 0) outp[0] = (double)st;
+    for (int off = 16; off > 0; off >>= 1) st += __shfl_xor_sync(0xffffffffu, st, off);
+    if (lane == 0) shs[warp] = st;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 8; ++w) st += shs[w];
+      outp[0] = (double)st;
+    }
     return;
   }
   float hi[kFluxBands], lo[kFluxBands];
@@ -604,8 +616,14 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
 #pragma unroll
   for (int q = 0; q < kFluxBands; ++q) {
     if (b0 + q >= a.n_bands) break;
-    const double s = block_sum(((double)hi[q] + (double)lo[q]) + tiny[q], sh);
-    if (threadIdx.x == 0) outp[b0 + q + 1] = s * a.area0;
+    const double s = flux_warp_sum(hi[q], lo[q], tiny[q]);
+    if (lane == 0) sh[q][warp] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < kFluxBands && b0 + (int)threadIdx.x < a.n_bands) {
+    double s = sh[threadIdx.x][0];
+    for (int w = 1; w < 8; ++w) s += sh[threadIdx.x][w];
+    outp[b0 + threadIdx.x + 1] = s * a.area0;
   }
 }
 
@@ -739,52 +757,34 @@ cudaError_t launch_emit_out(const TreeView &t, const OutView &o, int all, int64_
 // Blocks of the device-count sweep kernels: a few per SM, looping over items.
 static unsigned sweep_blocks(int per_sm) { return (unsigned)(sm_count() * per_sm); }
 
-cudaError_t launch_sweep_scan(const TreeView &t, int32_t *const open[2], const SweepState *S,
-                              double xi_crit, int xi_norm, int refine_on, uint32_t *flag,
-                              cudaStream_t st, const int32_t *lmap) {
-  return launch_pdl(k_xi_scan_dev, dim3(sweep_blocks(8)), dim3(256), 0, st, t,
-                    (const int32_t *)open[0], (const int32_t *)open[1], S, xi_crit, xi_norm,
-                    refine_on, flag, lmap);
+cudaError_t launch_open_init(int32_t *list, uint32_t *flag, int64_t m, uint32_t *counts,
+                             int64_t nb_cap, cudaStream_t st) {
+  if (m <= 0) return cudaSuccess;
+  k_open_init<<<nblk(m, 256), 256, 0, st>>>(list, flag, m, counts, nb_cap);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_sweep_scan_balance(const TreeView &t, int32_t *const open[2],
                                       const SweepState *S, double xi_crit, int xi_norm,
-                                      int refine_on, uint32_t *flag, uint32_t *err,
-                                      cudaStream_t st, const int32_t *lmap) {
+                                      int refine_on, uint32_t *flag, uint32_t *counts,
+                                      int64_t nb_cap, uint32_t *err, cudaStream_t st,
+                                      const int32_t *lmap) {
   return launch_pdl(k_scan_balance_dev, dim3(sweep_blocks(8)), dim3(256), 0, st, t,
                     (const int32_t *)open[0], (const int32_t *)open[1], S, xi_crit, xi_norm,
-                    refine_on, flag, err, lmap);
+                    refine_on, flag, counts, nb_cap, err, lmap);
 }
 
-cudaError_t launch_sweep_balance(const TreeView &t, int32_t *const open[2], const SweepState *S,
-                                 uint32_t *flag, uint32_t *err, cudaStream_t st,
-                                 const int32_t *lmap) {
-  return launch_pdl(k_balance_dev, dim3(sweep_blocks(16)), dim3(128), 0, st, t,
-                    (const int32_t *)open[0], (const int32_t *)open[1], S, flag, err, lmap);
-}
-
-cudaError_t launch_sweep_count(const TreeView &t, int32_t *const open[2], SweepState *S,
-                               const uint32_t *flag, int32_t *bcount, int64_t *boff,
-                               int64_t nb_cap, cudaStream_t st) {
-  cudaError_t e = launch_pdl(k_count3d, dim3(sweep_blocks(8)), dim3(kScanBlock), 0, st, t,
-                             (const int32_t *)open[0], (const int32_t *)open[1],
-                             (const SweepState *)S, flag, bcount, nb_cap);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(k_scan_blocks3d, dim3(3), dim3(1024), 0, st, (const int32_t *)bcount, nb_cap,
-                    boff, S);
-}
-
-cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], const SweepState *S,
-                              uint32_t *flag, const int64_t *boff, int64_t nb_cap,
-                              cudaStream_t st, int32_t *lmap) {
+cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], SweepState *S,
+                              uint32_t *flag, uint32_t *counts, int64_t nb_cap, cudaStream_t st,
+                              int32_t *lmap) {
   return launch_pdl(k_emit3d, dim3(sweep_blocks(8)), dim3(kScanBlock), 0, st, t, open[0], open[1],
-                    S, flag, boff, nb_cap, lmap);
+                    S, flag, counts, nb_cap, lmap);
 }
 
-
-// Entries of a block: 2048, 8 per thread (512 of them already fill the GPU
-// with 10^6 entries).
-constexpr int64_t kFluxPerBlock = 2048;
+// Entries of a block: 8192, 32 per thread. (2048: the FP64 sums at each
+// block's end took longer than its loads; 70 us instead of 44 for 7.7 M
+// nodes of one band.)
+constexpr int64_t kFluxPerBlock = 8192;
 
 int64_t flux_blocks(int64_t n) { return n <= 0 ? 0 : (n + kFluxPerBlock - 1) / kFluxPerBlock; }
 

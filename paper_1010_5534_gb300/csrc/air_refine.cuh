@@ -159,6 +159,25 @@ __device__ __forceinline__ void flux_add(float I, int L, float &hi, float &lo, d
   }
 }
 
+// The warp's sum of such accumulators, in every lane: pairs are added as
+// pairs (two-sum again), and one FP64 value is formed at the end.
+__device__ __forceinline__ double flux_warp_sum(float hi, float lo, double tiny) {
+  for (int off = 16; off > 0; off >>= 1) {
+    const float h2 = __shfl_xor_sync(0xffffffffu, hi, off), l2 = __shfl_xor_sync(0xffffffffu, lo, off);
+    const float t = __fadd_rn(hi, h2);
+    const float bv = __fsub_rn(t, hi);
+    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bv)), __fsub_rn(h2, bv));
+    lo = __fadd_rn(__fadd_rn(lo, l2), e);
+    hi = t;
+  }
+  double s = (double)hi + (double)lo;
+  if (__any_sync(0xffffffffu, tiny != 0.0)) {
+    for (int off = 16; off > 0; off >>= 1) tiny += __shfl_xor_sync(0xffffffffu, tiny, off);
+    s += tiny;
+  }
+  return s;
+}
+
 cudaError_t launch_init_base(const TreeView &t, cudaStream_t st);
 int64_t scan_blocks(int64_t n);
 cudaError_t launch_count_flags(const uint32_t *flag, int64_t n, int32_t *bcount, int64_t *boff,
@@ -190,27 +209,21 @@ cudaError_t launch_list_emit(const TreeView &t, const int32_t *open, int64_t m, 
                              int32_t *next, cudaStream_t st, int32_t *lmap = nullptr);
 // The same steps with every count read from the device (SweepState S; the
 // current list is open[S->cur], the next one open[S->cur ^ 1]). Grids are
-// sized for the GPU, not for the count, and loop over the items. nb_cap:
-// scan blocks the count arrays hold per selection (scan_blocks of the
-// largest list).
-cudaError_t launch_sweep_scan(const TreeView &t, int32_t *const open[2], const SweepState *S,
-                              double xi_crit, int xi_norm, int refine_on, uint32_t *flag,
-                              cudaStream_t st, const int32_t *lmap);
-// Scan and balance fused (the open list's flags must be zero on entry).
+// sized for the GPU, not for the count, and loop over the items. counts: 4 x
+// nb_cap chunk counts, nb_cap = scan_blocks of the largest list.
+// The first list (the m base pixels), its flag words, and the counts.
+cudaError_t launch_open_init(int32_t *list, uint32_t *flag, int64_t m, uint32_t *counts,
+                             int64_t nb_cap, cudaStream_t st);
+// Scan and balance fused; flagged leaves counted per chunk.
 cudaError_t launch_sweep_scan_balance(const TreeView &t, int32_t *const open[2],
                                       const SweepState *S, double xi_crit, int xi_norm,
-                                      int refine_on, uint32_t *flag, uint32_t *err,
-                                      cudaStream_t st, const int32_t *lmap);
-cudaError_t launch_sweep_balance(const TreeView &t, int32_t *const open[2], const SweepState *S,
-                                 uint32_t *flag, uint32_t *err, cudaStream_t st,
-                                 const int32_t *lmap);
-// Count the three selections and scan them; S->tot and S->done are set.
-cudaError_t launch_sweep_count(const TreeView &t, int32_t *const open[2], SweepState *S,
-                               const uint32_t *flag, int32_t *bcount, int64_t *boff,
-                               int64_t nb_cap, cudaStream_t st);
-cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], const SweepState *S,
-                              uint32_t *flag, const int64_t *boff, int64_t nb_cap,
-                              cudaStream_t st, int32_t *lmap);
+                                      int refine_on, uint32_t *flag, uint32_t *counts,
+                                      int64_t nb_cap, uint32_t *err, cudaStream_t st,
+                                      const int32_t *lmap);
+// Children, the next list and the level maps; S->tot and S->done are set.
+cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], SweepState *S,
+                              uint32_t *flag, uint32_t *counts, int64_t nb_cap, cudaStream_t st,
+                              int32_t *lmap);
 int64_t flux_blocks(int64_t n);
 cudaError_t launch_flux(FluxArgs a, double *flux, double *steps, cudaStream_t st);
 

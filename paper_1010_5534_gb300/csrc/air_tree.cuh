@@ -165,6 +165,20 @@ __device__ __forceinline__ uint32_t xi_flag(const TreeView &t, NodeLookup look, 
         const int ii = min(max(i + di, 0), nl - 1), jj = min(max(j + dj, 0), nl - 1);
         q[3 * (dj + 1) + (di + 1)] = (di == 0 && dj == 0) ? (int)k : __ldg(mL + (int64_t)jj * nl + ii);
       }
+    // (the level above in one more round of independent loads, where a
+    // balanced tree has them all)
+    const int32_t *mU = look.lmap + level_map_offset(t.n0, L - 1);
+#pragma unroll
+    for (int dj = -1; dj <= 1; ++dj)
+#pragma unroll
+      for (int di = -1; di <= 1; ++di) {
+        const int m = 3 * (dj + 1) + (di + 1);
+        const int ii = min(max(i + di, 0), nl - 1), jj = min(max(j + dj, 0), nl - 1);
+        if (q[m] < 0) {
+          if (L >= 2) q[m] = __ldg(mU + (int64_t)(jj >> 1) * (nl >> 1) + (ii >> 1));
+          else q[m] = (jj >> 1) * t.n0 + (ii >> 1);
+        }
+      }
 #pragma unroll
     for (int dj = -1; dj <= 1; ++dj)
 #pragma unroll
@@ -172,7 +186,7 @@ __device__ __forceinline__ uint32_t xi_flag(const TreeView &t, NodeLookup look, 
         const int m = 3 * (dj + 1) + (di + 1);
         if (q[m] < 0) {
           const int ii = min(max(i + di, 0), nl - 1), jj = min(max(j + dj, 0), nl - 1);
-          q[m] = map_deepest(t, look.lmap, L - 1, ii >> 1, jj >> 1);
+          q[m] = map_deepest(t, look.lmap, L - 2, ii >> 2, jj >> 2);
         }
       }
   } else {
@@ -221,51 +235,164 @@ __device__ __forceinline__ uint32_t xi_flag(const TreeView &t, NodeLookup look, 
 // is a level-L node (nothing to force) and an entry of -1 means no level-L
 // node covers that pixel, so the deepest node covering it is a leaf at a
 // level below L: it is forced without reading it. The eight entries are
-// loaded together; only the missing ones are looked up one level up.
+// loaded together, then the missing ones' covering nodes, then their flags are
+// set together. What is to be expanded is kept as (level, i, j), so nothing of
+// a forced node is read.
+
+// Counts of the leaves flagged in the open list, per scan chunk of kScanItems
+// list entries: `flagged`, and those whose children lie below the top level.
+// A flag word holds the leaf's list position (bits 1 up) beside the flag (bit
+// 0), so whoever sets a flag knows its chunk. NULL: flags are not counted (the
+// words are then the flags alone).
+struct FlagCount {
+  uint32_t *flagged, *below;
+};
+
+// A flag word set: true if it was not set before (and counted then).
+__device__ __forceinline__ bool set_flag(uint32_t *word, const FlagCount &fc) {
+  const uint32_t old = atomicOr(word, 1u);
+  if (old & 1u) return false;
+  if (fc.flagged) {
+    // a forced leaf's level is at least two below the top
+    const uint32_t c = (old >> 1) / kScanItems;
+    atomicAdd(fc.flagged + c, 1u);
+    atomicAdd(fc.below + c, 1u);
+  }
+  return true;
+}
+
+// Pixel (L, i, j), flagged: the leaves it forces through its 8 neighbours are
+// flagged. lv[d]: the level of the leaf that neighbour d made newly flagged,
+// or -1.
+__device__ __forceinline__ void force_neighbours(const TreeView &t, const int32_t *__restrict__ lmap,
+                                                 int L, int i, int j, uint32_t *__restrict__ flag,
+                                                 const FlagCount &fc, int (&lv)[8]) {
+  if (L < 1) {  // level-0 neighbours always exist
+#pragma unroll
+    for (int d = 0; d < 8; ++d) lv[d] = -1;
+    return;
+  }
+  const int nl = t.n0 << L;
+  const int32_t *mL = lmap + level_map_offset(t.n0, L);
+  const int32_t *mU = lmap + level_map_offset(t.n0, L - 1);
+  int e[8];
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    const int dd = d < 4 ? d : d + 1;  // skip the centre of the 3x3 stencil
+    const int ii = i + dd % 3 - 1, jj = j + dd / 3 - 1;
+    const bool in = ii >= 0 && jj >= 0 && ii < nl && jj < nl;
+    e[d] = in ? __ldg(mL + (int64_t)jj * nl + ii) : 0;
+  }
+  // the covering nodes of the missing ones
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    const int dd = d < 4 ? d : d + 1;
+    const int iu = (i + dd % 3 - 1) >> 1, ju = (j + dd / 3 - 1) >> 1;
+    lv[d] = e[d] < 0 ? L - 1 : -1;
+    if (e[d] < 0) e[d] = L >= 2 ? __ldg(mU + (int64_t)ju * (nl >> 1) + iu) : ju * t.n0 + iu;
+  }
+#pragma unroll
+  for (int d = 0; d < 8; ++d)
+    if (e[d] < 0) {  // not at the level above either (an unbalanced tree)
+      const int dd = d < 4 ? d : d + 1;
+      e[d] = map_deepest(t, lmap, L - 2, (i + dd % 3 - 1) >> 2, (j + dd / 3 - 1) >> 2);
+      lv[d] = t.lvl[e[d]];
+    }
+#pragma unroll
+  for (int d = 0; d < 8; ++d)
+    if (lv[d] >= 0 && !set_flag(flag + e[d], fc)) lv[d] = -1;
+}
+
+// What is to be expanded, packed: the level-lv leaf over neighbour d of (L, i, j).
+__device__ __forceinline__ unsigned long long forced_leaf(int L, int i, int j, int d, int lv) {
+  const int dd = d < 4 ? d : d + 1, s = L - lv;
+  return ((unsigned long long)lv << 40) | ((unsigned long long)((j + dd / 3 - 1) >> s) << 20) |
+         (unsigned long long)((i + dd % 3 - 1) >> s);
+}
+__device__ __forceinline__ void unpack_leaf(unsigned long long q, int &L, int &i, int &j) {
+  L = (int)(q >> 40);
+  j = (int)((q >> 20) & 0xfffffu);
+  i = (int)(q & 0xfffffu);
+}
+
+// One thread expands a flagged pixel and what it forces, depth first.
 __device__ __forceinline__ void balance_from_maps(const TreeView &t, const int32_t *__restrict__ lmap,
-                                                  int k0, uint32_t *__restrict__ flag,
-                                                  uint32_t *__restrict__ err,
-                                                  int (&stack)[kBalanceStack]) {
+                                                  int L, int i, int j, uint32_t *__restrict__ flag,
+                                                  uint32_t *__restrict__ err, const FlagCount &fc) {
+  unsigned long long stack[kBalanceStack];
   int sp = 0;
-  int q = k0;
   for (;;) {
-    const int L = t.lvl[q], i = t.pi[q], j = t.pj[q];
-    if (L >= 1) {  // level-0 neighbours always exist
-      const int nl = t.n0 << L;
-      const int32_t *mL = lmap + level_map_offset(t.n0, L);
-      int e[8];
+    int lv[8];
+    force_neighbours(t, lmap, L, i, j, flag, fc, lv);
 #pragma unroll
-      for (int d = 0; d < 8; ++d) {
-        const int dd = d < 4 ? d : d + 1;  // skip the centre of the 3x3 stencil
-        const int ii = i + dd % 3 - 1, jj = j + dd / 3 - 1;
-        const bool in = ii >= 0 && jj >= 0 && ii < nl && jj < nl;
-        e[d] = in ? __ldg(mL + (int64_t)jj * nl + ii) : 0;
+    for (int d = 0; d < 8; ++d)
+      if (lv[d] >= 0) {
+        if (sp < kBalanceStack) stack[sp++] = forced_leaf(L, i, j, d, lv[d]);
+        else atomicOr(err, 1u);
       }
+    if (sp == 0) break;
+    unpack_leaf(stack[--sp], L, i, j);
+  }
+}
+
+// A warp expands its lanes' flagged pixels (have: the lane holds one) together:
+// what they force goes to a queue in shared memory (kWarpQueue entries), from
+// which the lanes take the next 32. One thread after another's forced leaves
+// are three dependent memory accesses each, and a chain of a dozen of them was
+// most of the 16 us that a scan of a few thousand leaves took. An entry that
+// the queue has no room for is expanded by its lane.
+constexpr int kWarpQueue = 256;
+__device__ __forceinline__ void balance_warp(const TreeView &t, const int32_t *__restrict__ lmap,
+                                             bool have, int L, int i, int j,
+                                             uint32_t *__restrict__ flag, uint32_t *__restrict__ err,
+                                             const FlagCount &fc, unsigned long long *queue) {
+  const int lane = threadIdx.x & 31;
+  int n = 0;  // queued entries
+  while (__any_sync(0xffffffffu, have)) {
+    int lv[8], cnt = 0;
 #pragma unroll
-      for (int d = 0; d < 8; ++d) {
-        if (e[d] >= 0) continue;
-        const int dd = d < 4 ? d : d + 1;
-        const int ii = i + dd % 3 - 1, jj = j + dd / 3 - 1;
-        const int m = map_deepest(t, lmap, L - 1, ii >> 1, jj >> 1);
-        if (atomicExch(flag + m, 1u) == 0u) {
-          if (sp < kBalanceStack) stack[sp++] = m;
-          else atomicOr(err, 1u);
+    for (int d = 0; d < 8; ++d) lv[d] = -1;
+    if (have) force_neighbours(t, lmap, L, i, j, flag, fc, lv);
+#pragma unroll
+    for (int d = 0; d < 8; ++d) cnt += lv[d] >= 0 ? 1 : 0;
+    int before = cnt;  // inclusive prefix sum over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, before, o);
+      if (lane >= o) before += u;
+    }
+    const int total = __shfl_sync(0xffffffffu, before, 31);
+    int at = n + before - cnt;
+#pragma unroll
+    for (int d = 0; d < 8; ++d)
+      if (lv[d] >= 0) {
+        const unsigned long long q = forced_leaf(L, i, j, d, lv[d]);
+        if (at < kWarpQueue) {
+          queue[at++] = q;
+        } else {
+          int L2, i2, j2;
+          unpack_leaf(q, L2, i2, j2);
+          balance_from_maps(t, lmap, L2, i2, j2, flag, err, fc);
         }
       }
-    }
-    if (sp == 0) break;
-    q = stack[--sp];
+    n = min(n + total, kWarpQueue);
+    __syncwarp();
+    have = lane < n;
+    if (have) unpack_leaf(queue[n - 1 - lane], L, i, j);
+    n = max(n - 32, 0);
+    __syncwarp();
   }
 }
 
 __device__ __forceinline__ void balance_from(const TreeView &t, NodeLookup look, int k0,
                                              uint32_t *__restrict__ flag,
-                                             uint32_t *__restrict__ err) {
-  int stack[kBalanceStack];
+                                             uint32_t *__restrict__ err,
+                                             FlagCount fc = FlagCount{nullptr, nullptr}) {
   if (look.lmap) {
-    balance_from_maps(t, look.lmap, k0, flag, err, stack);
+    balance_from_maps(t, look.lmap, t.lvl[k0], t.pi[k0], t.pj[k0], flag, err, fc);
     return;
   }
+  int stack[kBalanceStack];
   int sp = 0;
   stack[sp++] = k0;
   while (sp > 0) {
@@ -279,7 +406,7 @@ __device__ __forceinline__ void balance_from(const TreeView &t, NodeLookup look,
         if (ii < 0 || jj < 0 || ii >= nl || jj >= nl) continue;
         const int m = look(t, L, ii, jj);
         if (t.child[m] < 0 && t.lvl[m] < L) {
-          if (atomicExch(flag + m, 1u) == 0u) {
+          if (set_flag(flag + m, fc)) {
             if (sp < kBalanceStack) stack[sp++] = m;
             else atomicOr(err, 1u);
           }
