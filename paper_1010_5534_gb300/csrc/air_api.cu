@@ -374,33 +374,46 @@ bool pyramid_fits(air_grid *g, int64_t bound) {
   return need <= 0.5 * (double)fr;
 }
 
+// Waits for the report of sweep `q` of the loop with this tag. The stream is asked now and then, so that a loop that can no longer
+// report (a CUDA error, or everything queued has run) ends the wait.
+static air_status wait_report(const SweepReport &rep, uint32_t tag, int64_t q, cudaStream_t st) {
+  const unsigned long long want = ((unsigned long long)tag << 32) | (uint32_t)(q + 1);
+  for (int64_t spin = 1;; ++spin) {
+    const bool last = spin % 4096 == 0;
+    cudaError_t e = cudaErrorNotReady;
+    if (last) e = cudaStreamQuery(st);
+    if (__atomic_load_n(&rep.progress, __ATOMIC_ACQUIRE) == want) return AIR_OK;
+    if (e == cudaSuccess) return set_error(AIR_ERR_CUDA, "the sweep loop stopped reporting");
+    if (e != cudaErrorNotReady) return cuda_fail(e, "sweep loop");
+  }
+}
+
 air_status sweep_loop_device(air_grid *g, const Camera &cam, const air_params *pr, int64_t nbase,
                              int64_t m, int64_t bound, int64_t open_max, const MarchTune &tune,
                              int march_launches, int32_t *lmap, const Proposal *prop,
-                             SweepState *fin) {
+                             SweepEnd *fin) {
   Workspace &w = g->ws;
   cudaStream_t st = g->stream;
   TreeView t = w.tree(pr->base_res, pr->max_level);
   // Steps iii-v with every count on the device: each sweep's kernels read
-  // the open-list length, the flag count and the node count from the
-  // device state, so the host queues sweep after sweep without waiting.
-  // It reads the state back two sweeps behind, only to learn that the
-  // loop has ended; the (at most two) sweeps queued past the end find
-  // `done` set and do nothing.
+  // the open-list length and the node counts from the device state, so the
+  // host queues sweep after sweep without waiting for one. It follows the
+  // loop through the report that each sweep's emit kernel writes to page-locked
+  // memory, two sweeps behind what it queues, to learn that it has ended; a
+  // sweep queued past the end finds `done` set and does nothing. (A copy of
+  // the state and an event after each sweep, instead of the report, and a last
+  // block that moved the state on, kept 12 to 16 us between the last ray of a
+  // sweep and the next scan.)
   if (!w.d_sweep) CU_TRY(cudaMalloc((void **)&w.d_sweep, sizeof(SweepState)));
-  if (!w.h_sweep) CU_TRY(cudaMallocHost((void **)&w.h_sweep, 3 * sizeof(SweepState)));
-  for (int k = 0; k < 2; ++k)
-    if (!w.ev_sweep[k]) CU_TRY(cudaEventCreateWithFlags(&w.ev_sweep[k], cudaEventDisableTiming));
-  SweepState &s0 = w.h_sweep[2];
-  std::memset(&s0, 0, sizeof(SweepState));
-  s0.n = nbase;
-  s0.m = m;
-  s0.done = m == 0;
-  CU_TRY(cudaMemcpyAsync(w.d_sweep, &s0, sizeof(SweepState), cudaMemcpyHostToDevice, st));
+  if (!w.h_report) {
+    CU_TRY(cudaMallocHost((void **)&w.h_report, 4 * sizeof(SweepReport)));
+    std::memset(w.h_report, 0, 4 * sizeof(SweepReport));
+  }
+  const uint32_t tag = ++w.sweep_tag;
   int32_t *const open2[2] = {w.open[0], w.open[1]};
   const int64_t nb_cap = scan_blocks(open_max);
   uint32_t *counts = (uint32_t *)w.boff;  // 3 x int64 per block of the whole pyramid
-  CU_TRY(launch_open_init(w.open[0], w.flag, m, counts, nb_cap, st));
+  CU_TRY(launch_open_init(w.d_sweep, nbase, w.open[0], w.flag, m, counts, nb_cap, st));
   RaySource ds{};
   ds.mode = 2; ds.n0 = pr->base_res; ds.lvl = t.lvl; ds.pi = t.pi; ds.pj = t.pj; ds.sweep = w.d_sweep;
   {
@@ -412,35 +425,45 @@ air_status sweep_loop_device(air_grid *g, const Camera &cam, const air_params *p
     ds.prop = *prop;
   }
   RayOut ro{t.N, t.I, t.cap, t.steps, t.p};
-  constexpr int kAhead = 2;
   // every sweep refines at least one pixel
-  const int64_t max_sweeps = (bound - nbase) / 4 + kAhead + 1;
-  int64_t q = 0;
-  for (;; ++q) {
-    if (q >= kAhead) {
-      CU_TRY(cudaEventSynchronize(w.ev_sweep[q % kAhead]));
-      if (w.h_sweep[q % kAhead].done) break;
+  const int64_t max_sweeps = std::min<int64_t>((bound - nbase) / 4 + 3, INT32_MAX);
+  SweepReport rep{};
+  for (int64_t q = 0;; ++q) {
+    if (q >= 2) {
+      const air_status s = wait_report(w.h_report[(q - 2) & 3], tag, q - 2, st);
+      if (s) return s;
+      rep = w.h_report[(q - 2) & 3];
+      if (rep.done) break;
     }
     if (q > max_sweeps) return set_error(AIR_ERR_NUMERIC, "sweep loop did not end");
+    ds.q = (int)q;
     // step iii: scan and balance in one pass (counted as the scan phase)
     CU_TRY(prof_open(g, AIR_PHASE_SCAN, 1));
-    CU_TRY(launch_sweep_scan_balance(t, open2, w.d_sweep, pr->xi_crit, pr->xi_norm, pr->refine_on,
+    CU_TRY(launch_sweep_scan_balance(t, open2, w.d_sweep, (int)q, pr->xi_crit, pr->xi_norm, pr->refine_on,
                                      w.flag, counts, nb_cap, w.d_err, st, lmap));
     CU_TRY(prof_close(g));
     CU_TRY(prof_open(g, AIR_PHASE_REFINE, 1));
-    CU_TRY(launch_sweep_emit(t, open2, w.d_sweep, w.flag, counts, nb_cap, st, lmap));
+    CU_TRY(launch_sweep_emit(t, open2, w.d_sweep, (int)q, w.flag, counts, nb_cap, w.d_err, w.h_report, tag,
+                             st, lmap));
     CU_TRY(prof_close(g));
-    // step ii on the new pixels (or their values from the proposal); the
-    // march's last block (or the band sum after it) moves the state on
+    // step ii on the new pixels (or their values from the proposal)
     CU_TRY(prof_open(g, AIR_PHASE_MARCH, march_launches));
     CU_TRY(launch_march(g->gv, cam, ds, ro, tune, st));
     CU_TRY(prof_close(g));
-    CU_TRY(cudaMemcpyAsync(&w.h_sweep[q % kAhead], w.d_sweep, sizeof(SweepState),
-                           cudaMemcpyDeviceToHost, st));
-    CU_TRY(cudaEventRecord(w.ev_sweep[q % kAhead], st));
   }
-  CU_TRY(cudaStreamSynchronize(st));
-  *fin = w.h_sweep[(q - 1) % kAhead];
+  if (rep.err) return set_error(AIR_ERR_NUMERIC, "balance closure overflowed its stack");
+  fin->n = rep.n;
+  fin->n_refined = rep.n_refined;
+  fin->sweeps = rep.sweeps;
+  fin->fb_total = 0;
+  fin->fb_waves = 0;
+  if (prop) {
+    SweepState s;
+    CU_TRY(cudaMemcpyAsync(&s, w.d_sweep, sizeof(s), cudaMemcpyDeviceToHost, st));
+    CU_TRY(cudaStreamSynchronize(st));
+    fin->fb_total = (int64_t)s.fb_total;
+    fin->fb_waves = s.fb_waves;
+  }
   return AIR_OK;
 }
 
@@ -597,7 +620,7 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
     if ((s = level_maps(g, n0, Lm, &lmap))) return s;
     g->last.lmap = lmap;
     if (dev_loop) {
-      SweepState fin;
+      SweepEnd fin;
       if ((s = sweep_loop_device(g, cam, pr, nbase, m, bound, open_max, tune, march_launches, lmap,
                                  nullptr, &fin)))
         return s;
@@ -642,9 +665,11 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
       m = m_next;
       cur ^= 1;
     }
-    CU_TRY(cudaMemcpyAsync(w.h_err, w.d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-    CU_TRY(cudaStreamSynchronize(st));
-    if (*w.h_err) return set_error(AIR_ERR_NUMERIC, "balance closure overflowed its stack");
+    if (!dev_loop) {  // (the device-count loop reports its own errors)
+      CU_TRY(cudaMemcpyAsync(w.h_err, w.d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+      CU_TRY(cudaStreamSynchronize(st));
+      if (*w.h_err) return set_error(AIR_ERR_NUMERIC, "balance closure overflowed its stack");
+    }
     g->last.view = *view;
     g->last.params = key;
     g->last.n_nodes = n; g->last.n_refined = n_refined; g->last.n_sweeps = sweeps;
@@ -680,6 +705,7 @@ air_status output_tree(air_grid *g, const Camera &cam, const air_params *pr, air
   im->n_out = n_out; im->n_leaves = n_leaves; im->n_rays = n; im->n_sweeps = sweeps; im->n_steps = 0;
   if (im->capacity < n_out) {
     // keep the finished tree so that a retry with larger arrays only copies it out
+    CU_TRY(cudaStreamSynchronize(st));
     g->last.valid = true;
     return set_error(AIR_ERR_CAPACITY, "capacity %lld < %lld pixels", (long long)im->capacity, (long long)n_out);
   }

@@ -201,12 +201,8 @@ void free_grid_impl(air_grid *g) {
   dfree(w.o_level); dfree(w.o_i); dfree(w.o_j); dfree(w.o_leaf); dfree(w.o_N); dfree(w.o_p);
   dfree(w.o_I);
   dfree(w.d_sweep);
-  if (w.h_sweep) cudaFreeHost(w.h_sweep);
-  w.h_sweep = nullptr;
-  for (int k = 0; k < 2; ++k) {
-    if (w.ev_sweep[k]) cudaEventDestroy(w.ev_sweep[k]);
-    w.ev_sweep[k] = nullptr;
-  }
+  if (w.h_report) cudaFreeHost(w.h_report);
+  w.h_report = nullptr;
   if (w.h_total) cudaFreeHost(w.h_total);
   if (w.h_err) cudaFreeHost(w.h_err);
   if (w.h_flux) cudaFreeHost(w.h_flux);

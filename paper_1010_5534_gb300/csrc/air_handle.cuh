@@ -52,11 +52,11 @@ struct Workspace {
   uint8_t *o_leaf = nullptr;
   float *o_N = nullptr, *o_p = nullptr, *o_I = nullptr;
   size_t o_level_b = 0, o_i_b = 0, o_j_b = 0, o_leaf_b = 0, o_N_b = 0, o_p_b = 0, o_I_b = 0;
-  // sweep loop with counts on the device: its state, pinned copies of it
-  // (two in flight, one for the initial state) and the copies' events
+  // sweep loop with counts on the device: its state, and the page-locked
+  // report of it, tagged per render
   SweepState *d_sweep = nullptr;
-  SweepState *h_sweep = nullptr;  // [3]
-  cudaEvent_t ev_sweep[2] = {nullptr, nullptr};
+  SweepReport *h_report = nullptr;
+  uint32_t sweep_tag = 0;
   // pinned host scalars
   int64_t *h_total = nullptr;  // [3]
   uint32_t *h_err = nullptr;
@@ -267,14 +267,20 @@ air_status axis_table(air_grid *g, const Camera &cam, int n0, int lmax, RaySourc
 // Whether the node arrays can be sized for a whole image pyramid of `bound`
 // nodes (at most half the free device memory beyond what is held).
 bool pyramid_fits(air_grid *g, int64_t bound);
+// How the device-count sweep loop ended.
+struct SweepEnd {
+  int64_t n, n_refined, fb_total;
+  int32_t sweeps, fb_waves;
+};
 // Steps iii-v of one view with every count on the device, over the tree in
 // the workspace (nodes [0, nbase) traced, open[0] holding the first m
 // leaves; node arrays sized for `bound`); prop: values of new pixels from a
-// learned proposal wave where it traced them, or NULL. *fin: the final state.
+// learned proposal wave where it traced them, or NULL. *fin: the final counts
+// (known before the last sweep's rays are traced: the stream is not waited for).
 air_status sweep_loop_device(air_grid *g, const Camera &cam, const air_params *pr, int64_t nbase,
                              int64_t m, int64_t bound, int64_t open_max, const MarchTune &tune,
                              int march_launches, int32_t *lmap, const Proposal *prop,
-                             SweepState *fin);
+                             SweepEnd *fin);
 // The march configuration of this handle's tuning.
 MarchTune march_tune(const air_grid *g, int fp64_level);
 air_status render_fixed(air_grid *g, const air_view *view, int32_t res, int32_t fp64_level,

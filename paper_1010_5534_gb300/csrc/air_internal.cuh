@@ -152,11 +152,11 @@ struct RaySource {
   int64_t first, count; // rays [first, first + count) of the list / image (modes 0, 1)
   int tile_w;           // grid mode: a warp covers tile_w x (32 / tile_w) pixels
   const int32_t *list;  // nodes mode: if set, ray r is node list[r] (first ignored)
-  SweepState *sweep;    // mode 2: rays [S->n, S->n + 4 S->tot[0]), none once S->done;
-                        // blocks take 128-ray chunks from S->ray_ctr[band chunk]
-  int advance;          // mode 2: the launch's last block moves S on to the next sweep
+  SweepState *sweep;    // mode 2: the new nodes of sweep q, from its slot's n to the next
+  int q;                // slot's; beyond the grid's first 128-ray chunks, blocks take more
+                        // from the slot's ray_ctr[band chunk]
   int part;             // mode 2, a sweep launched in two forms: 1 traces only counts up to
-  int64_t few;          // `few` rays, 2 only larger ones (and advances either way); 0: any
+  int64_t few;          // `few` rays, 2 only larger ones; 0: any
   int use_prop;         // mode 2: copy a new pixel's values from `prop` when the
   Proposal prop;        // proposal traced it; trace only the pixels it missed
   // column table of an axis view (RayGeom::tab, levels of the n0 image), or NULL

@@ -535,7 +535,7 @@ air_status render_learned(air_grid *g, const air_view *view, const air_params *p
     if ((s = level_maps(g, n0, Lm, &lmap))) return s;
     g->last.lmap = lmap;
     const Proposal prop{lw.depth, lw.off, lw.pN, lw.pI, lw.pp, lw.psteps, std::max<int64_t>(P, 1)};
-    SweepState fin;
+    SweepEnd fin;
     if ((s = sweep_loop_device(g, cam, pr, nbase, mo, bound, open_max, tune, march_launches, lmap, &prop,
                                &fin)))
       return s;
@@ -605,9 +605,11 @@ air_status render_learned(air_grid *g, const air_view *view, const air_params *p
     mo = mo_next;
     cur ^= 1;
   }
-  CU_TRY(cudaMemcpyAsync(w.h_err, w.d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-  CU_TRY(cudaStreamSynchronize(st));
-  if (*w.h_err) return set_error(AIR_ERR_NUMERIC, "balance closure overflowed its stack");
+  if (!dev_loop) {
+    CU_TRY(cudaMemcpyAsync(w.h_err, w.d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+    CU_TRY(cudaStreamSynchronize(st));
+    if (*w.h_err) return set_error(AIR_ERR_NUMERIC, "balance closure overflowed its stack");
+  }
   // statistics of the proposal against the final tree
   CU_TRY(cudaMemsetAsync(lw.label, 0, sizeof(int32_t) * 4 * nbase, st));
   CU_TRY(cudaMemsetAsync(lw.counters, 0, sizeof(unsigned long long) * 2, st));

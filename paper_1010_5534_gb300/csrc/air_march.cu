@@ -15,23 +15,17 @@ __global__ void k_band_sum(const float *__restrict__ I, int n_bands, int64_t str
   p[k] = s;
 }
 
-// Band sums of a sweep counted on the device (rays [S->n, S->n + 4 S->tot[0])).
-// The last block to finish moves the state on to the next sweep.
+// Band sums of the new nodes of sweep q, counted on the device.
 __global__ void k_band_sum_dev(const float *__restrict__ I, int n_bands, int64_t stride,
-                               SweepState *__restrict__ S, float *__restrict__ p) {
+                               const SweepState *__restrict__ S, int q, float *__restrict__ p) {
   wait_prior_grid();
-  if (S->done) return;
-  const int64_t first = S->n, count = 4 * S->tot[0];
+  const int64_t first = S->slot[q & 3].n, end = S->slot[(q + 1) & 3].n;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
-  if (p)
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < count; r += step) {
-      const int64_t k = first + r;
-      float s = 0.f;
-      for (int b = 0; b < n_bands; ++b) s += I[(int64_t)b * stride + k];
-      p[k] = s;
-    }
-  __syncthreads();
-  if (threadIdx.x == 0) sweep_block_finished(S, gridDim.x);
+  for (int64_t k = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < end; k += step) {
+    float s = 0.f;
+    for (int b = 0; b < n_bands; ++b) s += I[(int64_t)b * stride + k];
+    p[k] = s;
+  }
 }
 
 // Compiled in air_march_<NBT>.cu and air_march_axis.cu.
@@ -66,11 +60,7 @@ static cudaError_t launch_nbt(int NBT, const GridView &g, const Camera &cam, con
   rg.tab_slot = src.axtab_slot;
   rg.tab_byj = src.axtab_byj;
   const int moving = (rg.Dhi[0] != 0.f) + (rg.Dhi[1] != 0.f) + (rg.Dhi[2] != 0.f);
-  // with the count on the device the march ends the sweep: the last block
-  // advances the state, or the band sum after it does when bands are split
-  RaySource s2 = src;
-  s2.advance = dev && chunks == 1;
-  const MarchLaunch m{g, rg, s2, out, blocks, chunks, tune.fp64_level, st};
+  const MarchLaunch m{g, rg, src, out, blocks, chunks, tune.fp64_level, st};
   cudaError_t le;
   if (NBT == 1 && moving == 1) {
     le = rg.Dhi[0] != 0.f ? march_axis_one<0>(m) : (rg.Dhi[1] != 0.f ? march_axis_one<1>(m) : march_axis_one<2>(m));
@@ -83,9 +73,9 @@ static cudaError_t launch_nbt(int NBT, const GridView &g, const Camera &cam, con
   if (le != cudaSuccess) return le;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (dev && chunks > 1)  // band sums (if wanted), and the state moves on
+  if (dev && chunks > 1 && out.p)
     return launch_pdl(k_band_sum_dev, dim3((unsigned)(sm_count() * 8)), dim3(256), 0, st,
-                      (const float *)out.I, g.n_bands, out.stride, src.sweep, out.p);
+                      (const float *)out.I, g.n_bands, out.stride, (const SweepState *)src.sweep, src.q, out.p);
   if (chunks > 1 && out.p) {
     const int64_t first = src.mode == 0 ? src.first : 0;
     const int64_t count = src.mode == 0 ? src.count : (int64_t)src.n0 * src.n0;

@@ -65,7 +65,10 @@ __device__ __forceinline__ void march_one(const GridView &g, const RayGeom &rg, 
       if (out.p && gridDim.y == 1) out.p[k] = pr.p[q];
       return;
     }
-    if (chunk == 0) atomicAdd(&src.sweep->fb_sweep, 1ull);
+    if (chunk == 0) {
+      if (atomicAdd(&src.sweep->slot[src.q & 3].missed, 1ull) == 0ull) atomicAdd(&src.sweep->fb_waves, 1);
+      atomicAdd(&src.sweep->fb_total, 1ull);
+    }
   }
   RTState<NBT> st;
   trace_ray<NBT, AMR, FMT, DIR>(st, g, rg, src.lvl[k], src.pi[k], src.pj[k], fp64_level, bc, br);
@@ -91,7 +94,6 @@ template <int NBT, bool AMR, int FMT, int DIR>
 __global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
     k_march(GridView g, RayGeom rg, RaySource src, RayOut out, int fp64_level) {
   extern __shared__ __align__(16) float smem[];
-  wait_prior_grid();
   const int chunk = blockIdx.y;
   const int b0 = chunk * NBT;
   const int nbh = min(NBT, g.n_bands - b0);
@@ -101,29 +103,26 @@ __global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
   if (FMT == kCellXq) tab_fill<NBT>(smem, g, b0);
   BandRegs<NBT> br;
   band_regs<NBT>(br, g.bands, b0, nbh);
+  // (the tables and constants above were written when the grid was loaded)
+  wait_prior_grid();
   __syncthreads();
 
   if (src.mode == 2) {
-    // new nodes of a sweep counted on the device: blocks take chunks of
-    // blockDim.x rays from a work counter until the rays run out
-    // (with src.advance, the last block to finish moves the state on to the
-    // next sweep)
-    SweepState *S = src.sweep;
-    if (S->done) return;
-    const int64_t count = 4 * S->tot[0], first = S->n;
-    const bool skip = (src.part == 1 && count > src.few) || (src.part == 2 && count <= src.few);
+    // new nodes of a sweep counted on the device: block b takes chunk b of
+    // blockDim.x rays, and more from a work counter until the rays run out
+    SweepSlot &s0 = src.sweep->slot[src.q & 3];
+    const int64_t first = s0.n, count = src.sweep->slot[(src.q + 1) & 3].n - first;
+    if ((src.part == 1 && count > src.few) || (src.part == 2 && count <= src.few)) return;
     __shared__ long long s_chunk;
-    while (!skip) {
-      if (threadIdx.x == 0) s_chunk = (long long)atomicAdd(S->ray_ctr + chunk, 1ull);
-      __syncthreads();
-      const int64_t r0 = (int64_t)s_chunk * blockDim.x;
-      __syncthreads();
-      if (r0 >= count) break;
+    for (int64_t r0 = (int64_t)blockIdx.x * blockDim.x; r0 < count; r0 = s_chunk * blockDim.x) {
       const int64_t r = r0 + threadIdx.x;
       if (r < count) march_one<NBT, AMR, FMT, DIR>(g, rg, src, out, fp64_level, bc, br, chunk, b0,
                                                    nbh, first + r);
+      if (count <= (int64_t)gridDim.x * blockDim.x) return;
+      __syncthreads();
+      if (threadIdx.x == 0) s_chunk = gridDim.x + (long long)atomicAdd(&s0.ray_ctr[chunk], 1ull);
+      __syncthreads();
     }
-    if (src.advance && threadIdx.x == 0) sweep_block_finished(S, gridDim.x * gridDim.y);
     return;
   }
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -200,7 +199,6 @@ static cudaError_t march_inclined(const MarchLaunch &m) {
     return m.blocks * kMarchBlock <= few ? march_form<NBT, AMR, FMT, -1>(m) : march_form<NBT, AMR, FMT, 0>(m);
   RaySource s1 = m.src, s2 = m.src;
   s1.part = 1;
-  s1.advance = 0;
   s2.part = 2;
   s1.few = s2.few = few;
   const cudaError_t e = march_form<NBT, AMR, FMT, -1>(MarchLaunch{m.g, m.rg, s1, m.out, m.blocks, m.chunks, m.fp64_level, m.st});

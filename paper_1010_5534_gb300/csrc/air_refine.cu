@@ -10,6 +10,7 @@
 // found by descending from the base node through the child links; this gives
 // the deepest existing node at a level <= L, which is the value a missing
 // neighbour takes in the stencil.
+#include <algorithm>
 #include <atomic>
 #include <cfloat>
 
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(kScanBlock) k_emit3(TreeView t, const int32_t 
 // arrays, a few kilobytes that lie in L2. (With a counting and a scanning
 // launch between them a sweep took 12 us more, whatever its size.)
 //
-// counts: two sets (S->cur) of [flagged | below the top level][nb_cap] chunk
+// counts: two sets (q & 1) of [flagged | below the top level][nb_cap] chunk
 // counts. The set of the current sweep is zero when it starts; the emit kernel
 // zeroes the other one for the next. A flag word holds its leaf's position in
 // the open list (see FlagCount).
@@ -273,16 +274,30 @@ __device__ __forceinline__ FlagCount sweep_counts(uint32_t *counts, int64_t nb_c
   return FlagCount{c, c + nb_cap};
 }
 
-// First open list: the m base pixels, flag words with their positions, and
-// the counts of the first set zeroed.
-__global__ void k_open_init(int32_t *list, uint32_t *flag, int64_t m, uint32_t *counts,
-                            int64_t nb_cap) {
+// The first slot, the first open list (the m base pixels), flag words with
+// their positions, and the counts of the first set zeroed.
+__global__ void k_open_init(SweepState *S, int64_t n, int32_t *list, uint32_t *flag, int64_t m,
+                            uint32_t *counts, int64_t nb_cap) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < m) {
     list[i] = (int32_t)i;
     flag[i] = (uint32_t)i << 1;
   }
   if (i < scan_chunks(m)) counts[i] = counts[nb_cap + i] = 0u;
+  if (blockIdx.x == 0) {
+    SweepSlot &s = S->slot[0];
+    if (threadIdx.x < kMaxBands) s.ray_ctr[threadIdx.x] = 0ull;
+    if (threadIdx.x == 0) {
+      s.n = n;
+      s.m = m;
+      s.n_refined = 0;
+      s.sweeps = 0;
+      s.done = m == 0;
+      s.missed = 0ull;
+      S->fb_total = 0ull;
+      S->fb_waves = 0;
+    }
+  }
 }
 
 // Scan and balance in one pass. No flag of the open list is set when a sweep
@@ -290,17 +305,16 @@ __global__ void k_open_init(int32_t *list, uint32_t *flag, int64_t m, uint32_t *
 // flagged, and the thread that sets a flag -- the scan's or a balance
 // expansion's -- expands it. Every flag is expanded once, and the flags reach
 // the same closure as a scan of every leaf followed by the balance.
-__global__ void __launch_bounds__(kScanBlock) k_scan_balance_dev(TreeView t, const int32_t *__restrict__ open0,
-                                   const int32_t *__restrict__ open1,
-                                   const SweepState *__restrict__ S, double xi_crit, int xi_norm,
-                                   int refine_on, uint32_t *__restrict__ flag,
-                                   uint32_t *__restrict__ counts, int64_t nb_cap,
-                                   uint32_t *__restrict__ err, const int32_t *lmap) {
+__global__ void __launch_bounds__(kScanBlock)
+    k_scan_balance_dev(TreeView t, const int32_t *__restrict__ open, const SweepState *__restrict__ S,
+                       int q, double xi_crit, int xi_norm, int refine_on, uint32_t *__restrict__ flag,
+                       uint32_t *__restrict__ counts, int64_t nb_cap, uint32_t *__restrict__ err,
+                       const int32_t *lmap) {
   wait_prior_grid();
-  if (S->done) return;
-  const int64_t m = S->m;
-  const int32_t *open = S->cur ? open1 : open0;
-  const FlagCount fc = sweep_counts(counts, nb_cap, S->cur);
+  const SweepSlot &sl = S->slot[q & 3];
+  if (sl.done) return;
+  const int64_t m = sl.m;
+  const FlagCount fc = sweep_counts(counts, nb_cap, q & 1);
   const NodeLookup look{0, lmap};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   __shared__ unsigned long long queue[kScanBlock / 32][kWarpQueue];
@@ -351,24 +365,23 @@ __device__ __forceinline__ void block_sum4(uint32_t (&v)[4], uint32_t (&sh)[4][k
 }
 
 // Step iv over the list, and the next list: kept entries first (in order),
-// then the children below the top level (in order). Block 0 leaves the totals
-// in S->tot, and sets S->done when nothing was flagged (blocks that see it
-// return, as all do then).
-__global__ void __launch_bounds__(kScanBlock) k_emit3d(TreeView t, int32_t *open0, int32_t *open1,
-                                                       SweepState *__restrict__ S, uint32_t *flag,
-                                                       uint32_t *counts, int64_t nb_cap,
-                                                       int32_t *lmap) {
+// then the children below the top level (in order). Block 0 writes the next
+// slot and the host's report.
+__global__ void __launch_bounds__(kScanBlock)
+    k_emit3d(TreeView t, const int32_t *__restrict__ open, int32_t *__restrict__ next,
+             SweepState *__restrict__ S, int q, uint32_t *flag, uint32_t *counts, int64_t nb_cap,
+             const uint32_t *__restrict__ err, SweepReport *rep, uint32_t tag, int32_t *lmap) {
   wait_prior_grid();
-  if (S->done) return;
   __shared__ uint32_t sums[4][kScanBlock / 32];
   __shared__ int32_t wsum[3][kScanBlock / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t m = S->m, n_old = S->n;
-  const int cur = S->cur;
-  const int32_t *open = cur ? open1 : open0;
-  int32_t *next = cur ? open0 : open1;
+  const SweepSlot &sl = S->slot[q & 3];
+  const int done = sl.done;
+  const int64_t m = sl.m, n_old = sl.n;
+  if (done && blockIdx.x != 0) return;
+  const int cur = q & 1;
   const FlagCount fc = sweep_counts(counts, nb_cap, cur);
-  const int64_t nb = scan_chunks(m);
+  const int64_t nb = done ? 0 : scan_chunks(m);
   // totals, and the counts in front of the block's first chunk
   uint32_t v[4] = {0u, 0u, 0u, 0u};
   for (int64_t x = threadIdx.x; x < nb; x += kScanBlock) {
@@ -382,11 +395,29 @@ __global__ void __launch_bounds__(kScanBlock) k_emit3d(TreeView t, int32_t *open
   }
   block_sum4(v, sums);
   const int64_t nflag = v[0], nbelow = v[1], keep_total = m - nflag;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    S->tot[0] = nflag;
-    S->tot[1] = keep_total;
-    S->tot[2] = nbelow;
-    if (nflag == 0) S->done = 1;  // nothing flagged: the loop ends
+  if (blockIdx.x == 0) {
+    SweepSlot &sn = S->slot[(q + 1) & 3];
+    if (threadIdx.x < kMaxBands) sn.ray_ctr[threadIdx.x] = 0ull;
+    if (threadIdx.x == 0) {
+      const int64_t m1 = keep_total + 4 * nbelow;
+      const int sweeps = sl.sweeps + (nflag ? 1 : 0);
+      const int end = done || nflag == 0 || m1 == 0;  // flagged nothing, or no leaf is left to scan
+      const int64_t n1 = n_old + 4 * nflag, refined = sl.n_refined + nflag;
+      sn.n = n1;
+      sn.m = m1;
+      sn.n_refined = refined;
+      sn.sweeps = sweeps;
+      sn.done = end;
+      sn.missed = 0ull;
+      SweepReport &r = rep[q & 3];
+      r.n = n1;
+      r.n_refined = refined;
+      r.sweeps = sweeps;
+      r.done = end;
+      r.err = *err;
+      __threadfence_system();
+      *(volatile unsigned long long *)&r.progress = ((unsigned long long)tag << 32) | (unsigned)(q + 1);
+    }
   }
   if (nflag == 0) return;
   // the other set of counts, for the next sweep's list
@@ -757,28 +788,29 @@ cudaError_t launch_emit_out(const TreeView &t, const OutView &o, int all, int64_
 // Blocks of the device-count sweep kernels: a few per SM, looping over items.
 static unsigned sweep_blocks(int per_sm) { return (unsigned)(sm_count() * per_sm); }
 
-cudaError_t launch_open_init(int32_t *list, uint32_t *flag, int64_t m, uint32_t *counts,
-                             int64_t nb_cap, cudaStream_t st) {
-  if (m <= 0) return cudaSuccess;
-  k_open_init<<<nblk(m, 256), 256, 0, st>>>(list, flag, m, counts, nb_cap);
+cudaError_t launch_open_init(SweepState *S, int64_t n, int32_t *list, uint32_t *flag, int64_t m,
+                             uint32_t *counts, int64_t nb_cap, cudaStream_t st) {
+  k_open_init<<<nblk(std::max<int64_t>(m, 1), 256), 256, 0, st>>>(S, n, list, flag, m, counts, nb_cap);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sweep_scan_balance(const TreeView &t, int32_t *const open[2],
-                                      const SweepState *S, double xi_crit, int xi_norm,
+                                      const SweepState *S, int q, double xi_crit, int xi_norm,
                                       int refine_on, uint32_t *flag, uint32_t *counts,
                                       int64_t nb_cap, uint32_t *err, cudaStream_t st,
                                       const int32_t *lmap) {
-  return launch_pdl(k_scan_balance_dev, dim3(sweep_blocks(8)), dim3(256), 0, st, t,
-                    (const int32_t *)open[0], (const int32_t *)open[1], S, xi_crit, xi_norm,
-                    refine_on, flag, counts, nb_cap, err, lmap);
+  return launch_pdl(k_scan_balance_dev, dim3(sweep_blocks(8)), dim3(kScanBlock), 0, st, t,
+                    (const int32_t *)open[q & 1], S, q, xi_crit, xi_norm, refine_on, flag, counts,
+                    nb_cap, err, lmap);
 }
 
-cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], SweepState *S,
-                              uint32_t *flag, uint32_t *counts, int64_t nb_cap, cudaStream_t st,
+cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], SweepState *S, int q,
+                              uint32_t *flag, uint32_t *counts, int64_t nb_cap,
+                              const uint32_t *err, SweepReport *rep, uint32_t tag, cudaStream_t st,
                               int32_t *lmap) {
-  return launch_pdl(k_emit3d, dim3(sweep_blocks(8)), dim3(kScanBlock), 0, st, t, open[0], open[1],
-                    S, flag, counts, nb_cap, lmap);
+  return launch_pdl(k_emit3d, dim3(sweep_blocks(8)), dim3(kScanBlock), 0, st, t,
+                    (const int32_t *)open[q & 1], open[(q + 1) & 1], S, q, flag, counts, nb_cap, err,
+                    rep, tag, lmap);
 }
 
 // Entries of a block: 8192, 32 per thread. (2048: the FP64 sums at each

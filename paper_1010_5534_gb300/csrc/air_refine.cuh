@@ -56,51 +56,41 @@ struct FluxArgs {
 };
 
 // Device-resident bookkeeping of the sweep loop when the counts stay on the
-// device (render_adaptive without a read-back per sweep). Every kernel of a
-// sweep reads its item count here; once `done` is set, every later kernel
-// returns at once, so sweeps queued past the end do nothing.
-struct SweepState {
-  long long n;          // traced nodes so far
-  long long m;          // length of the current open-leaf list
+// device (render_adaptive without a read-back per sweep). Sweep q starts from
+// slot q & 3; its emit kernel knows what the sweep adds and writes the next
+// slot, which the march of the new pixels reads beside the first (so no kernel
+// waits for a last block to move the state on). Once a slot is `done`, later
+// kernels return at once and the next slots are copies of it, so sweeps queued
+// past the end do nothing. A slot is written again four sweeps later, when
+// every kernel that reads it has ended.
+struct SweepSlot {
+  long long n;          // traced nodes when the sweep starts
+  long long m;          // length of its open-leaf list
   long long n_refined;  // refined nodes so far
-  long long tot[3];     // this sweep: flagged, kept, flagged with children below the top level
-  int cur;              // which open-leaf list is current (0 or 1)
-  int sweeps;           // sweeps that refined something
-  int done;             // the last scan flagged nothing (or nothing is left to scan)
-  unsigned blocks_done; // blocks of the sweep's last kernel that have finished
+  int sweeps;           // sweeps so far that refined something
+  int done;             // nothing is left to scan, or the sweep before flagged nothing
   unsigned long long ray_ctr[kMaxBands];  // march work counters, one per band chunk
-  // with a learned proposal: pixels it missed, traced this sweep / in all
-  // sweeps, and the sweeps that traced any
-  unsigned long long fb_sweep, fb_total;
+  // with a learned proposal: pixels of this sweep that it missed
+  unsigned long long missed;
+};
+struct SweepState {
+  SweepSlot slot[4];
+  // with a learned proposal: pixels it missed, and the sweeps that had any
+  unsigned long long fb_total;
   int fb_waves;
 };
 
-// After the new pixels are traced: n, m, cur, sweeps and n_refined move on to
-// the next sweep, and the work counters are reset. Run by one thread once no
-// other thread of the sweep reads the state any more.
-__device__ __forceinline__ void sweep_advance(SweepState *S) {
-  const long long nflag = S->tot[0];
-  S->n += 4 * nflag;
-  S->n_refined += nflag;
-  S->m = S->tot[1] + 4 * S->tot[2];
-  S->cur ^= 1;
-  S->sweeps += 1;
-  if (S->m == 0) S->done = 1;  // no leaf below the top level is left
-  for (int b = 0; b < kMaxBands; ++b) S->ray_ctr[b] = 0ull;
-  S->blocks_done = 0u;
-  if (S->fb_sweep) {
-    S->fb_total += S->fb_sweep;
-    S->fb_waves += 1;
-    S->fb_sweep = 0ull;
-  }
-}
-
-// Called by thread 0 of every block of the sweep's last kernel as the block
-// finishes (after a __syncthreads): the last block to finish advances.
-__device__ __forceinline__ void sweep_block_finished(SweepState *S, unsigned nblocks) {
-  __threadfence();
-  if (atomicAdd(&S->blocks_done, 1u) == nblocks - 1u) sweep_advance(S);
-}
+// What the host sees of it: page-locked memory, of which the emit kernel of
+// sweep q writes entry q & 3 (`progress` last: the render's tag in the high
+// word, q + 1 in the low one), so the host follows the loop without a copy or
+// an event in the stream. It reads an entry before it queues the sweep that
+// will write it again.
+struct SweepReport {
+  long long n, n_refined;
+  int sweeps, done;
+  unsigned int err;  // the balance's error word
+  unsigned long long progress;
+};
 
 // Programmatic dependent launch: a kernel of the sweep chain waits here for
 // the kernel before it (launched with cudaLaunchAttributeProgrammaticStream-
@@ -207,22 +197,24 @@ cudaError_t launch_list_count(const TreeView &t, const int32_t *open, int64_t m,
 cudaError_t launch_list_emit(const TreeView &t, const int32_t *open, int64_t m, uint32_t *flag,
                              const int64_t *boff, const int64_t *totals, int64_t n_old,
                              int32_t *next, cudaStream_t st, int32_t *lmap = nullptr);
-// The same steps with every count read from the device (SweepState S; the
-// current list is open[S->cur], the next one open[S->cur ^ 1]). Grids are
-// sized for the GPU, not for the count, and loop over the items. counts: 4 x
-// nb_cap chunk counts, nb_cap = scan_blocks of the largest list.
-// The first list (the m base pixels), its flag words, and the counts.
-cudaError_t launch_open_init(int32_t *list, uint32_t *flag, int64_t m, uint32_t *counts,
-                             int64_t nb_cap, cudaStream_t st);
+// The same steps with every count read from the device: sweep q of the loop
+// (SweepState S). The current list is open[q & 1], the next one
+// open[(q + 1) & 1]. Grids are sized for the GPU, not for the count, and loop
+// over the items. counts: 4 x nb_cap chunk counts, nb_cap = scan_blocks of the
+// largest list.
+// The state, the first list (the m base pixels), its flag words and the counts.
+cudaError_t launch_open_init(SweepState *S, int64_t n, int32_t *list, uint32_t *flag, int64_t m,
+                             uint32_t *counts, int64_t nb_cap, cudaStream_t st);
 // Scan and balance fused; flagged leaves counted per chunk.
 cudaError_t launch_sweep_scan_balance(const TreeView &t, int32_t *const open[2],
-                                      const SweepState *S, double xi_crit, int xi_norm,
+                                      const SweepState *S, int q, double xi_crit, int xi_norm,
                                       int refine_on, uint32_t *flag, uint32_t *counts,
                                       int64_t nb_cap, uint32_t *err, cudaStream_t st,
                                       const int32_t *lmap);
-// Children, the next list and the level maps; S->tot and S->done are set.
-cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], SweepState *S,
-                              uint32_t *flag, uint32_t *counts, int64_t nb_cap, cudaStream_t st,
+// Children, the next list, the level maps, the next slot and the report.
+cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], SweepState *S, int q,
+                              uint32_t *flag, uint32_t *counts, int64_t nb_cap,
+                              const uint32_t *err, SweepReport *rep, uint32_t tag, cudaStream_t st,
                               int32_t *lmap);
 int64_t flux_blocks(int64_t n);
 cudaError_t launch_flux(FluxArgs a, double *flux, double *steps, cudaStream_t st);

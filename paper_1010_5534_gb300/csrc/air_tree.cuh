@@ -148,9 +148,8 @@ __device__ __forceinline__ int xi_at_least_f32(const float f[9], int xi_norm, do
 // Step iii for node k: 1 if it is a leaf below max_level with xi >= xi_crit.
 __device__ __forceinline__ uint32_t xi_flag(const TreeView &t, NodeLookup look, int64_t k,
                                             double xi_crit, int xi_norm, int refine_on) {
-  const int L = t.lvl[k];
+  const int L = t.lvl[k], i = t.pi[k], j = t.pj[k];
   if (t.child[k] >= 0 || L >= t.Lm) return 0u;
-  const int i = t.pi[k], j = t.pj[k];
   const int nl = t.n0 << L;
   int q[9];
   if (look.lmap && L >= 1) {
@@ -248,9 +247,9 @@ struct FlagCount {
   uint32_t *flagged, *below;
 };
 
-// A flag word set: true if it was not set before (and counted then).
-__device__ __forceinline__ bool set_flag(uint32_t *word, const FlagCount &fc) {
-  const uint32_t old = atomicOr(word, 1u);
+// A flag word that was `old` has been set: true if it was not set before (and
+// counted then).
+__device__ __forceinline__ bool newly_set(uint32_t old, const FlagCount &fc) {
   if (old & 1u) return false;
   if (fc.flagged) {
     // a forced leaf's level is at least two below the top
@@ -298,9 +297,16 @@ __device__ __forceinline__ void force_neighbours(const TreeView &t, const int32_
       e[d] = map_deepest(t, lmap, L - 2, (i + dd % 3 - 1) >> 2, (j + dd / 3 - 1) >> 2);
       lv[d] = t.lvl[e[d]];
     }
+  // all flags are set before the first answer is waited for
+  uint32_t old[8];
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    old[d] = 1u;
+    if (lv[d] >= 0) old[d] = atomicOr(flag + e[d], 1u);
+  }
 #pragma unroll
   for (int d = 0; d < 8; ++d)
-    if (lv[d] >= 0 && !set_flag(flag + e[d], fc)) lv[d] = -1;
+    if (lv[d] >= 0 && !newly_set(old[d], fc)) lv[d] = -1;
 }
 
 // What is to be expanded, packed: the level-lv leaf over neighbour d of (L, i, j).
@@ -406,7 +412,7 @@ __device__ __forceinline__ void balance_from(const TreeView &t, NodeLookup look,
         if (ii < 0 || jj < 0 || ii >= nl || jj >= nl) continue;
         const int m = look(t, L, ii, jj);
         if (t.child[m] < 0 && t.lvl[m] < L) {
-          if (set_flag(flag + m, fc)) {
+          if (newly_set(atomicOr(flag + m, 1u), fc)) {
             if (sp < kBalanceStack) stack[sp++] = m;
             else atomicOr(err, 1u);
           }
