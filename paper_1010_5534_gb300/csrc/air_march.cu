@@ -1,5 +1,7 @@
 // air_march.cu -- launches of the per-ray march (device code in air_march.cuh,
 // the kernel and its forms in air_march_kernel.cuh).
+#include <algorithm>
+
 #include "air_march_kernel.cuh"
 
 namespace air {
@@ -15,17 +17,28 @@ __global__ void k_band_sum(const float *__restrict__ I, int n_bands, int64_t str
   p[k] = s;
 }
 
-// Band sums of the new nodes of sweep q, counted on the device.
+// Band sums of the new nodes of sweep q, counted on the device, unless they are
+// more than `most` (their threads then held all bands and summed them).
 __global__ void k_band_sum_dev(const float *__restrict__ I, int n_bands, int64_t stride,
-                               const SweepState *__restrict__ S, int q, float *__restrict__ p) {
+                               const SweepState *__restrict__ S, int q, int64_t most,
+                               float *__restrict__ p) {
   wait_prior_grid();
   const int64_t first = S->slot[q & 3].n, end = S->slot[(q + 1) & 3].n;
+  if (end - first > most) return;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   for (int64_t k = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < end; k += step) {
     float s = 0.f;
     for (int b = 0; b < n_bands; ++b) s += I[(int64_t)b * stride + k];
     p[k] = s;
   }
+}
+
+// Rays whose threads (one per band chunk) fill the GPU twice in the form for
+// few rays, or in the ordinary one of that width.
+static int64_t few_rays(int NBT, bool lone, int chunks) {
+  const int blocks = lone ? (NBT <= 4 ? MinBlocks<4, -1>::value : MinBlocks<8, -1>::value)
+                          : (NBT <= 1 ? kAxisBlocksSmall : (NBT <= 2 ? MinBlocks<2, 0>::value : MinBlocks<4, 0>::value));
+  return (int64_t)sm_count() * blocks * kMarchBlock * 2 / chunks;
 }
 
 // Compiled in air_march_<NBT>.cu and air_march_axis.cu.
@@ -38,10 +51,11 @@ extern template cudaError_t march_axis_one<0>(const MarchLaunch &);
 extern template cudaError_t march_axis_one<1>(const MarchLaunch &);
 extern template cudaError_t march_axis_one<2>(const MarchLaunch &);
 
-static cudaError_t launch_nbt(int NBT, const GridView &g, const Camera &cam, const RaySource &src,
-                              const RayOut &out, const MarchTune &tune, cudaStream_t st) {
+// The march kernel with NBT bands per thread.
+static cudaError_t launch_nbt(int NBT, bool few, const GridView &g, const RayGeom &rg,
+                              const RaySource &src, const RayOut &out, const MarchTune &tune,
+                              cudaStream_t st) {
   const int chunks = (g.n_bands + NBT - 1) / NBT;
-  const bool dev = src.mode == 2;
   int64_t threads;
   if (src.mode == 0) {
     threads = src.count;
@@ -55,12 +69,8 @@ static cudaError_t launch_nbt(int NBT, const GridView &g, const Camera &cam, con
   if (threads <= 0) return cudaSuccess;
   const int64_t blocks = (threads + kMarchBlock - 1) / kMarchBlock;
   if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-  RayGeom rg = make_geom(g, cam, src.n0);
-  rg.tab = src.axtab;
-  rg.tab_slot = src.axtab_slot;
-  rg.tab_byj = src.axtab_byj;
   const int moving = (rg.Dhi[0] != 0.f) + (rg.Dhi[1] != 0.f) + (rg.Dhi[2] != 0.f);
-  const MarchLaunch m{g, rg, src, out, blocks, chunks, tune.fp64_level, st};
+  const MarchLaunch m{g, rg, src, out, blocks, chunks, tune.fp64_level, st, few};
   cudaError_t le;
   if (NBT == 1 && moving == 1) {
     le = rg.Dhi[0] != 0.f ? march_axis_one<0>(m) : (rg.Dhi[1] != 0.f ? march_axis_one<1>(m) : march_axis_one<2>(m));
@@ -71,37 +81,67 @@ static cudaError_t launch_nbt(int NBT, const GridView &g, const Camera &cam, con
          : NBT == 8 ? march_general<8>(m) : march_general<16>(m);
   }
   if (le != cudaSuccess) return le;
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (dev && chunks > 1 && out.p)
-    return launch_pdl(k_band_sum_dev, dim3((unsigned)(sm_count() * 8)), dim3(256), 0, st,
-                      (const float *)out.I, g.n_bands, out.stride, (const SweepState *)src.sweep, src.q, out.p);
-  if (chunks > 1 && out.p) {
-    const int64_t first = src.mode == 0 ? src.first : 0;
-    const int64_t count = src.mode == 0 ? src.count : (int64_t)src.n0 * src.n0;
-    if (src.list) {
-      k_band_sum<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(out.I, g.n_bands, out.stride, 0,
-                                                                  count, src.list, out.p, out.ioff);
-      return cudaGetLastError();
-    }
-    return launch_band_sum(out.I, g.n_bands, out.stride, first, count, out.p, st, out.ioff);
-  }
-  return cudaSuccess;
+  return cudaGetLastError();
 }
+
+// The kernel's width for a number of bands per thread.
+static int width_of(int nbt) { return nbt <= 1 ? 1 : (nbt <= 2 ? 2 : (nbt <= 4 ? 4 : (nbt <= 8 ? 8 : 16))); }
 
 cudaError_t launch_march(const GridView &g, const Camera &cam, const RaySource &src,
                          const RayOut &out, const MarchTune &tune, cudaStream_t st) {
   // default: every band in one thread up to 8 bands, chunks of 8 above
   // (32-band adaptive / fixed images of the large grid, one view: 4 bands
   // 1315 / 1365 ms, 8 bands 1251 / 1328 ms, 16 bands 1512 / 1653 ms)
-  int nbt = tune.nbt;
-  if (nbt <= 0) nbt = default_bands_per_thread(g.n_bands);
-  if (g.cell_fmt == kCellLam) nbt = 1;  // one band
-  if (nbt <= 1) return launch_nbt(1, g, cam, src, out, tune, st);
-  if (nbt <= 2) return launch_nbt(2, g, cam, src, out, tune, st);
-  if (nbt <= 4) return launch_nbt(4, g, cam, src, out, tune, st);
-  if (nbt <= 8) return launch_nbt(8, g, cam, src, out, tune, st);
-  return launch_nbt(16, g, cam, src, out, tune, st);
+  const int want = tune.nbt > 0 ? tune.nbt : default_bands_per_thread(g.n_bands);
+  const int nbt = g.cell_fmt == kCellLam ? 1 : width_of(want);  // per-cell Lambda: one band
+  RayGeom rg = make_geom(g, cam, src.n0);
+  rg.tab = src.axtab;
+  rg.tab_slot = src.axtab_slot;
+  rg.tab_byj = src.axtab_byj;
+  const int moving = (rg.Dhi[0] != 0.f) + (rg.Dhi[1] != 0.f) + (rg.Dhi[2] != 0.f);
+  const int chunks = (g.n_bands + nbt - 1) / nbt;
+  if (src.mode == 0 && src.count <= 0) return cudaSuccess;
+
+  // A launch that leaves most of the GPU idle takes as long as its longest ray,
+  // and a ray's time is that of one warp working alone, so its bands are spread
+  // over more threads (unless the caller has set the bands per thread), and
+  // inclined rays take the form DIR = -1. `few`: the rays that fill that form's
+  // threads twice. Where the count is on the device, both launches are queued
+  // and the one that it is not for returns.
+  const int narrow = tune.nbt > 0 ? nbt : std::min(nbt, g.n_bands <= 8 ? 1 : (g.n_bands <= 16 ? 2 : 4));
+  const int nchunks = (g.n_bands + narrow - 1) / narrow;
+  const bool lone = moving > 1 && narrow <= 8;  // there is a form for few rays
+  const int64_t few = lone || narrow < nbt ? few_rays(narrow, lone, nchunks) : 0;
+  const int64_t total = src.mode == 0 ? src.count : (src.mode == 1 ? (int64_t)src.n0 * src.n0 : 0);
+  cudaError_t e;
+  if (src.mode != 2) {
+    const bool is_few = total <= few;
+    e = launch_nbt(is_few ? narrow : nbt, is_few && lone, g, rg, src, out, tune, st);
+    if (e != cudaSuccess || !out.p || (is_few ? nchunks : chunks) == 1) return e;
+    const int64_t first = src.mode == 0 ? src.first : 0;
+    if (src.list) {
+      k_band_sum<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(out.I, g.n_bands, out.stride, 0, total,
+                                                                  src.list, out.p, out.ioff);
+      return cudaGetLastError();
+    }
+    return launch_band_sum(out.I, g.n_bands, out.stride, first, total, out.p, st, out.ioff);
+  }
+  RaySource s2 = src;
+  s2.few = few;
+  if (few > 0) {
+    s2.part = 1;
+    e = launch_nbt(narrow, lone, g, rg, s2, out, tune, st);
+    if (e != cudaSuccess) return e;
+    s2.part = 2;
+  }
+  e = launch_nbt(nbt, false, g, rg, s2, out, tune, st);
+  if (e != cudaSuccess || !out.p) return e;
+  const int64_t most = chunks > 1 ? INT64_MAX : (few > 0 && nchunks > 1 ? few : 0);
+  if (most > 0)
+    return launch_pdl(k_band_sum_dev, dim3((unsigned)(sm_count() * 8)), dim3(256), 0, st,
+                      (const float *)out.I, g.n_bands, out.stride, (const SweepState *)src.sweep, src.q, most,
+                      out.p);
+  return cudaSuccess;
 }
 
 // Column-table entries (axis_table_entry), one per thread.

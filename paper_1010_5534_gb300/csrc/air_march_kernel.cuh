@@ -18,6 +18,7 @@ struct MarchLaunch {
   int chunks;      // band chunks
   int fp64_level;
   cudaStream_t st;
+  bool few;        // inclined rays that leave most threads idle: the form DIR = -1
 };
 
 // Resident blocks per SM of the one-band kernels of rays parallel to an axis
@@ -184,34 +185,11 @@ static cudaError_t march_form(const MarchLaunch &m) {
                     m.g, m.rg, m.src, m.out, m.fp64_level);
 }
 
-// Rays that fill the GPU's threads once in the form for few rays.
-template <int NBT>
-static int64_t few_rays(const MarchLaunch &m) {
-  return (int64_t)sm_count() * MinBlocks<NBT, -1>::value * kMarchBlock / m.chunks;
-}
-
-// Inclined rays. A launch of few rays takes the form for them; where the count
-// is on the device both forms are launched, and the one it is not for returns.
-template <int NBT, bool AMR, int FMT>
-static cudaError_t march_inclined(const MarchLaunch &m) {
-  const int64_t few = few_rays<NBT>(m);
-  if (m.src.mode != 2)
-    return m.blocks * kMarchBlock <= few ? march_form<NBT, AMR, FMT, -1>(m) : march_form<NBT, AMR, FMT, 0>(m);
-  RaySource s1 = m.src, s2 = m.src;
-  s1.part = 1;
-  s2.part = 2;
-  s1.few = s2.few = few;
-  const cudaError_t e = march_form<NBT, AMR, FMT, -1>(MarchLaunch{m.g, m.rg, s1, m.out, m.blocks, m.chunks, m.fp64_level, m.st});
-  if (e != cudaSuccess) return e;
-  return march_form<NBT, AMR, FMT, 0>(MarchLaunch{m.g, m.rg, s2, m.out, m.blocks, m.chunks, m.fp64_level, m.st});
-}
-
 template <int NBT, bool AMR, int FMT>
 static cudaError_t march_any(const MarchLaunch &m) {
   // 16 bands per thread leave no registers for the form for few rays
-  const int moving = (m.rg.Dhi[0] != 0.f) + (m.rg.Dhi[1] != 0.f) + (m.rg.Dhi[2] != 0.f);
   if constexpr (NBT <= 8)
-    if (moving > 1) return march_inclined<NBT, AMR, FMT>(m);
+    if (m.few) return march_form<NBT, AMR, FMT, -1>(m);
   return march_form<NBT, AMR, FMT, 0>(m);
 }
 
