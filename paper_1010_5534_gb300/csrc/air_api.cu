@@ -50,7 +50,6 @@ cudaError_t ensure(void **p, size_t *have, size_t bytes) {
 air_status init_scalars(Workspace &w) {
   if (!w.d_total) CU_TRY(cudaMalloc((void **)&w.d_total, 3 * sizeof(int64_t)));
   if (!w.d_err) CU_TRY(cudaMalloc((void **)&w.d_err, sizeof(uint32_t)));
-  if (!w.d_flux) CU_TRY(cudaMalloc((void **)&w.d_flux, sizeof(double) * (kMaxBands + 1)));
   if (!w.h_total) CU_TRY(cudaMallocHost((void **)&w.h_total, 3 * sizeof(int64_t)));
   if (!w.h_err) CU_TRY(cudaMallocHost((void **)&w.h_err, sizeof(uint32_t)));
   if (!w.h_flux) CU_TRY(cudaMallocHost((void **)&w.h_flux, sizeof(double) * (kMaxBands + 1)));
@@ -233,7 +232,8 @@ static air_status out_view(air_grid *g, const air_image *im, int64_t n, OutView 
   return AIR_OK;
 }
 
-// Staging -> host arrays (host-memory outputs), then band flux and step count.
+// Staging -> host arrays (host-memory outputs); band flux and step count from
+// the page-locked copy that k_flux_final left.
 static air_status finish_out(air_grid *g, air_image *im, const OutView &o, int64_t n) {
   cudaStream_t st = g->stream;
   const int nb = g->gv.n_bands;
@@ -250,9 +250,6 @@ static air_status finish_out(air_grid *g, air_image *im, const OutView &o, int64
         CU_TRY(cudaMemcpyAsync(im->intensity + (size_t)b * im->capacity, o.I + (size_t)b * o.stride,
                                4 * n, cudaMemcpyDeviceToHost, st));
   }
-  CU_TRY(cudaMemcpyAsync(w.h_flux, w.d_flux, sizeof(double) * (nb + 1), cudaMemcpyDeviceToHost, st));
-  if (im->band_flux && im->mem == AIR_DEVICE)
-    CU_TRY(cudaMemcpyAsync(im->band_flux, w.d_flux, sizeof(double) * nb, cudaMemcpyDeviceToDevice, st));
   CU_TRY(cudaStreamSynchronize(st));
   if (im->band_flux && im->mem == AIR_HOST) std::memcpy(im->band_flux, w.h_flux, sizeof(double) * nb);
   im->n_steps = (int64_t)w.h_flux[nb];
@@ -305,9 +302,12 @@ air_status render_fixed(air_grid *g, const air_view *view, int32_t res, int32_t 
   FluxArgs fa{};
   fa.n = n; fa.child = nullptr; fa.lvl = nullptr; fa.I = ro.I; fa.stride = ro.stride; fa.steps = w.fsteps;
   fa.n_bands = nb; fa.area0 = (2.0 * cam.H / res) * (2.0 * cam.H / res); fa.partial = w.partial;
+  fa.flux = im->mem == AIR_DEVICE ? im->band_flux : nullptr;
+  fa.host = w.h_flux;
   const bool list = o.level || o.i || o.j || o.is_leaf;
   CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, list ? 3 : 2));
-  CU_TRY(launch_flux(fa, w.d_flux, w.d_flux + nb, st));
+  CU_TRY(launch_flux_partial(fa, st));
+  CU_TRY(launch_flux_final(fa, st));
   if (list) k_fixed_out<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, (uint32_t)res, o);
   CU_TRY(cudaGetLastError());
   CU_TRY(prof_close(g));
@@ -720,12 +720,18 @@ air_status output_tree(air_grid *g, const Camera &cam, const air_params *pr, air
   fa.I = spectra_dev ? spectra_dev : t.I;
   fa.stride = spectra_dev ? spectra_cap : t.cap;
   fa.n_bands = nb; fa.area0 = (2.0 * cam.H / n0) * (2.0 * cam.H / n0); fa.partial = w.partial;
+  fa.flux = im->mem == AIR_DEVICE ? im->band_flux : nullptr;
+  fa.host = w.h_flux;
+  if (!all) {  // (both arrays hold 3 entries per scan chunk of the whole pyramid)
+    fa.chunk_leaves = w.bcount;
+    fa.block_leaves = (int32_t *)w.boff;
+  }
   OutView o;
   if ((s = out_view(g, im, n_out, o))) return s;
-  CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, 5));
-  CU_TRY(launch_flux(fa, w.d_flux, w.d_flux + nb, st));
-  CU_TRY(launch_count_leaves(t, all, n, w.bcount, w.boff, w.d_total, st));
-  CU_TRY(launch_emit_out(t, o, all, n, w.boff, st));
+  CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, 3));
+  CU_TRY(launch_flux_partial(fa, st));
+  CU_TRY(launch_emit_out(t, o, all, n, fa.chunk_leaves, fa.block_leaves, st));
+  CU_TRY(launch_flux_final(fa, st));
   CU_TRY(prof_close(g));
   s = finish_out(g, im, o, n_out);
   if (s) return s;

@@ -42,7 +42,6 @@ struct Workspace {
   uint32_t *d_err = nullptr;
   double *partial = nullptr;
   size_t partial_b = 0;
-  double *d_flux = nullptr;  // [kMaxBands + 1]: flux then steps
   // fixed image
   float *fN = nullptr, *fI = nullptr, *fp = nullptr;
   uint32_t *fsteps = nullptr;

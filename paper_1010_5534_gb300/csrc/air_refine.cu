@@ -29,11 +29,6 @@ struct PredFlag {
   const uint32_t *flag;
   __device__ bool operator()(int64_t k) const { return flag[k] != 0; }
 };
-struct PredLeaf {
-  const int32_t *child;
-  int all;
-  __device__ bool operator()(int64_t k) const { return all || child[k] < 0; }
-};
 
 template <class Pred>
 __global__ void __launch_bounds__(kScanBlock) k_count(Pred pred, int64_t n, int32_t *bcount) {
@@ -513,12 +508,26 @@ __global__ void __launch_bounds__(kScanBlock)
 // Step vi: copy the selected nodes (leaves, or all) to the output arrays.
 
 // The fields of every round's node are loaded before the ranks are formed,
-// so their latency overlaps the block's ballots and barriers.
+// so their latency overlaps the block's ballots and barriers. The leaves in
+// front of the block are added up from the counts of k_flux_partial: those of
+// the flux blocks before, and of the chunks before within its flux block. (A
+// counting and a scanning launch of their own took 25 us for 7.7 M nodes.)
 __global__ void __launch_bounds__(kScanBlock) k_emit_out(TreeView t, OutView o, int all, int64_t n,
-                                                         const int64_t *boff) {
+                                                         const int32_t *__restrict__ chunk_leaves,
+                                                         const int32_t *__restrict__ block_leaves) {
+  wait_prior_grid();
   __shared__ int32_t wsum[kScanBlock / 32];
+  __shared__ uint32_t fsum[kScanBlock / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t start = (int64_t)blockIdx.x * kScanItems;
+  uint32_t front = 0;
+  if (!all) {
+    const int fb = blockIdx.x / kFluxChunks, c0 = fb * kFluxChunks;
+    for (int x = threadIdx.x; x < fb; x += kScanBlock) front += (uint32_t)block_leaves[x];
+    if (c0 + (int)threadIdx.x < (int)blockIdx.x) front += (uint32_t)chunk_leaves[c0 + threadIdx.x];
+    front = __reduce_add_sync(0xffffffffu, front);
+    if (lane == 0) fsum[warp] = front;
+  }
   bool sel[kScanRounds];
   int lv[kScanRounds], pi[kScanRounds], pj[kScanRounds], cl[kScanRounds];
   float N[kScanRounds], P[kScanRounds], I0[kScanRounds];
@@ -537,7 +546,14 @@ __global__ void __launch_bounds__(kScanBlock) k_emit_out(TreeView t, OutView o, 
       I0[rr] = o.I ? t.I[k] : 0.f;  // no tree intensities are read without o.I
     }
   }
-  int64_t run = boff[blockIdx.x];
+  int64_t run = start;
+  if (!all) {
+    __syncthreads();
+    uint32_t f = 0;
+#pragma unroll
+    for (int w = 0; w < kScanBlock / 32; ++w) f += fsum[w];
+    run = f;
+  }
 #pragma unroll
   for (int rr = 0; rr < kScanRounds; ++rr) {
     const int64_t k = start + (int64_t)rr * kScanBlock + threadIdx.x;
@@ -593,11 +609,13 @@ __global__ void k_init_base(TreeView t) {
 // every band of 8192 entries, band after band, before: 85 us for 0.8 M leaves
 // of four bands.)
 __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
+  wait_prior_grid();
+  __shared__ int32_t chunk_sum[kFluxChunks];
   __shared__ double sh[kFluxBands][8];
   __shared__ unsigned long long shs[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t start = (int64_t)blockIdx.x * a.per_block;
-  const int64_t end = min(a.n, start + a.per_block);
+  const int64_t start = (int64_t)blockIdx.x * kFluxPerBlock;
+  const int64_t end = min(a.n, start + kFluxPerBlock);
   double *outp = a.partial + (int64_t)blockIdx.x * (a.n_bands + 1);
   const int b0 = blockIdx.y * kFluxBands;
   if (b0 >= a.n_bands) {
@@ -622,7 +640,12 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
   // four entries per thread at a time, their loads issued together (a leaf's
   // intensity is not made to wait for its flag)
   constexpr int R = 4;
-  for (int64_t k0 = start + threadIdx.x; k0 < end; k0 += R * blockDim.x) {
+  const bool count = a.chunk_leaves && b0 == 0;
+  if (count) {
+    if (threadIdx.x < kFluxChunks) chunk_sum[threadIdx.x] = 0;
+    __syncthreads();
+  }
+  for (int64_t k0 = start + threadIdx.x; k0 - threadIdx.x < end; k0 += R * blockDim.x) {
     bool leaf[R];
     int L[R];
     float I[R][kFluxBands];
@@ -635,6 +658,13 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
 #pragma unroll
       for (int q = 0; q < kFluxBands; ++q)
         I[r][q] = in && b0 + q < a.n_bands ? a.I[(int64_t)(b0 + q) * a.stride + k] : 0.f;
+    }
+    if (count) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {  // 256 nodes of a round lie in one chunk
+        const int c = __popc(__ballot_sync(0xffffffffu, leaf[r]));
+        if (lane == 0 && c) atomicAdd(&chunk_sum[(int)(k0 + r * blockDim.x - start) / kScanItems], c);
+      }
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
@@ -651,6 +681,15 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
     if (lane == 0) sh[q][warp] = s;
   }
   __syncthreads();
+  if (count) {
+    const int nc = (int)((end - start + kScanItems - 1) / kScanItems);
+    if (threadIdx.x < nc) a.chunk_leaves[(int64_t)blockIdx.x * kFluxChunks + threadIdx.x] = chunk_sum[threadIdx.x];
+    if (threadIdx.x == 32) {
+      int s = 0;
+      for (int c = 0; c < nc; ++c) s += chunk_sum[c];
+      a.block_leaves[blockIdx.x] = s;
+    }
+  }
   if (threadIdx.x < kFluxBands && b0 + (int)threadIdx.x < a.n_bands) {
     double s = sh[threadIdx.x][0];
     for (int w = 1; w < 8; ++w) s += sh[threadIdx.x][w];
@@ -658,22 +697,22 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
   }
 }
 
-// One block per output: block 0 the step count, block b + 1 band b.
-__global__ void __launch_bounds__(256) k_flux_final(const double *partial, int64_t nblocks,
-                                                    int n_bands, double *flux, double *steps) {
-  __shared__ double sh[256];
+// One block per output: block 0 the step count, block b + 1 band b. The host
+// reads its copy in page-locked memory once the stream has been waited for (a
+// copy of its own behind the kernel cost 4 us per image).
+__global__ void __launch_bounds__(256) k_flux_final(FluxArgs a, int64_t nblocks) {
+  wait_prior_grid();
+  __shared__ double sh[8];
   const int b = (int)blockIdx.x - 1;
   double s = 0.0;
-  for (int64_t x = threadIdx.x; x < nblocks; x += blockDim.x) s += partial[x * (n_bands + 1) + b + 1];
-  sh[threadIdx.x] = s;
+  for (int64_t x = threadIdx.x; x < nblocks; x += blockDim.x) s += a.partial[x * (a.n_bands + 1) + b + 1];
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int off = 128; off > 0; off >>= 1) {
-    if (threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
-    __syncthreads();
-  }
   if (threadIdx.x == 0) {
-    if (b < 0) *steps = sh[0];
-    else flux[b] = sh[0];
+    for (int w = 1; w < 8; ++w) s += sh[w];
+    a.host[b < 0 ? a.n_bands : b] = s;
+    if (b >= 0 && a.flux) a.flux[b] = s;
   }
 }
 
@@ -768,21 +807,12 @@ cudaError_t launch_scan_offsets(const int32_t *bcount, int64_t nb, int64_t *boff
 }
 
 
-cudaError_t launch_count_leaves(const TreeView &t, int all, int64_t n, int32_t *bcount,
-                                int64_t *boff, int64_t *total, cudaStream_t st) {
-  const int64_t nb = scan_blocks(n);
-  if (nb == 0) return cudaMemsetAsync(total, 0, sizeof(int64_t), st);
-  k_count<<<(unsigned)nb, kScanBlock, 0, st>>>(PredLeaf{t.child, all}, n, bcount);
-  k_scan_blocks<<<1, 1024, 0, st>>>(bcount, nb, boff, total);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_emit_out(const TreeView &t, const OutView &o, int all, int64_t n,
-                            const int64_t *boff, cudaStream_t st) {
+                            const int32_t *chunk_leaves, const int32_t *block_leaves, cudaStream_t st) {
   const int64_t nb = scan_blocks(n);
   if (nb == 0) return cudaSuccess;
-  k_emit_out<<<(unsigned)nb, kScanBlock, 0, st>>>(t, o, all, n, boff);
-  return cudaGetLastError();
+  return launch_pdl(k_emit_out, dim3((unsigned)nb), dim3(kScanBlock), 0, st, t, o, all, n, chunk_leaves,
+                    block_leaves);
 }
 
 // Blocks of the device-count sweep kernels: a few per SM, looping over items.
@@ -813,25 +843,17 @@ cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], SweepSt
                     rep, tag, lmap);
 }
 
-// Entries of a block: 8192, 32 per thread. (2048: the FP64 sums at each
-// block's end took longer than its loads; 70 us instead of 44 for 7.7 M
-// nodes of one band.)
-constexpr int64_t kFluxPerBlock = 8192;
-
 int64_t flux_blocks(int64_t n) { return n <= 0 ? 0 : (n + kFluxPerBlock - 1) / kFluxPerBlock; }
 
-cudaError_t launch_flux(FluxArgs a, double *flux, double *steps, cudaStream_t st) {
-  a.per_block = kFluxPerBlock;
+cudaError_t launch_flux_partial(const FluxArgs &a, cudaStream_t st) {
   const int64_t nb = flux_blocks(a.n);
-  if (nb == 0) {
-    cudaError_t e = cudaMemsetAsync(flux, 0, sizeof(double) * a.n_bands, st);
-    if (e != cudaSuccess) return e;
-    return cudaMemsetAsync(steps, 0, sizeof(double), st);
-  }
+  if (nb == 0) return cudaSuccess;
   const unsigned rows = (unsigned)((a.n_bands + kFluxBands - 1) / kFluxBands) + 1;
-  k_flux_partial<<<dim3((unsigned)nb, rows), 256, 0, st>>>(a);
-  k_flux_final<<<(unsigned)(a.n_bands + 1), 256, 0, st>>>(a.partial, nb, a.n_bands, flux, steps);
-  return cudaGetLastError();
+  return launch_pdl(k_flux_partial, dim3((unsigned)nb, rows), dim3(256), 0, st, a);
+}
+
+cudaError_t launch_flux_final(const FluxArgs &a, cudaStream_t st) {
+  return launch_pdl(k_flux_final, dim3((unsigned)(a.n_bands + 1)), dim3(256), 0, st, a, flux_blocks(a.n));
 }
 
 }  // namespace air

@@ -52,8 +52,18 @@ struct FluxArgs {
   int n_bands;
   double area0;          // pixel area at level 0
   double *partial;       // [blocks][n_bands + 1]
-  int64_t per_block;
+  // leaves counted on the way (NULL: not): per scan chunk of kScanItems nodes,
+  // and per block of kFluxPerBlock nodes
+  int32_t *chunk_leaves, *block_leaves;
+  // where the sums go: the flux to device memory (may be NULL), and to
+  // page-locked memory, [n_bands], with the step count behind it
+  double *flux, *host;
 };
+// Nodes of a flux block: 8192, 32 per thread. (2048: the FP64 sums at each
+// block's end took longer than its loads; 70 us instead of 44 for 7.7 M nodes
+// of one band.)
+constexpr int64_t kFluxPerBlock = 8192;
+constexpr int kFluxChunks = kFluxPerBlock / kScanItems;
 
 // Device-resident bookkeeping of the sweep loop when the counts stay on the
 // device (render_adaptive without a read-back per sweep). Sweep q starts from
@@ -172,10 +182,9 @@ cudaError_t launch_init_base(const TreeView &t, cudaStream_t st);
 int64_t scan_blocks(int64_t n);
 cudaError_t launch_count_flags(const uint32_t *flag, int64_t n, int32_t *bcount, int64_t *boff,
                                int64_t *total, cudaStream_t st);
-cudaError_t launch_count_leaves(const TreeView &t, int all, int64_t n, int32_t *bcount,
-                                int64_t *boff, int64_t *total, cudaStream_t st);
+// chunk_leaves, block_leaves: from launch_flux_partial (unused with `all`).
 cudaError_t launch_emit_out(const TreeView &t, const OutView &o, int all, int64_t n,
-                            const int64_t *boff, cudaStream_t st);
+                            const int32_t *chunk_leaves, const int32_t *block_leaves, cudaStream_t st);
 // Exclusive scan of nb per-block counts (one block) -> boff, total.
 cudaError_t launch_scan_offsets(const int32_t *bcount, int64_t nb, int64_t *boff, int64_t *total,
                                 cudaStream_t st);
@@ -217,6 +226,7 @@ cudaError_t launch_sweep_emit(const TreeView &t, int32_t *const open[2], SweepSt
                               const uint32_t *err, SweepReport *rep, uint32_t tag, cudaStream_t st,
                               int32_t *lmap);
 int64_t flux_blocks(int64_t n);
-cudaError_t launch_flux(FluxArgs a, double *flux, double *steps, cudaStream_t st);
+cudaError_t launch_flux_partial(const FluxArgs &a, cudaStream_t st);
+cudaError_t launch_flux_final(const FluxArgs &a, cudaStream_t st);
 
 }  // namespace air
