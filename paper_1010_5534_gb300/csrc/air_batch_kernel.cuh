@@ -112,32 +112,32 @@ struct EmitChildrenV {
 // per-view counters.
 template <int NBT>
 static size_t batch_smem(const GridView &g, int V) {
-  const size_t tab = g.cell_fmt == kCellXq ? ((g.n_bands + NBT - 1) / NBT) * tab_bytes<NBT>(g.n_tbins) : 0;
+  const size_t tab = ((g.n_bands + NBT - 1) / NBT) * chunk_bytes<NBT>(g.cell_fmt == kCellXq, g.n_tbins);
   return tab + 3 * sizeof(int64_t) * V + sizeof(int32_t) * V + sizeof(int32_t) * (kBatchBlock / 32) * V;
 }
 
-// Resident blocks per SM. Left open, the compiler took 234 registers at 8 bands
-// per thread (two blocks).
-template <int NBT>
+// DIR: 0 for any views, -2 when every view is inclined (trace_ray): without the
+// column march of axis rays, which holds a chunk's band constants and partial
+// sums in registers, a block needs 124 registers instead of 168 at 8 bands per
+// thread and 160 instead of 250 at 16.
+template <int NBT, int DIR>
 struct BatchBlocks {
-  static constexpr int value = NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? 3 : 2));
+  static constexpr int value = NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? (DIR == 0 ? 3 : 4) : (DIR == 0 ? 2 : 3)));
 };
 
-template <int NBT, bool AMR, int FMT>
-__global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT>::value) k_air_batch(BatchArgs a) {
+template <int NBT, bool AMR, int FMT, int DIR>
+__global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_air_batch(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const GridView &g = a.g;
   const int V = a.V, nb = g.n_bands;
-  float *tab = (float *)smem_raw;
-  int64_t *run = (int64_t *)(smem_raw + (FMT == kCellXq ? a.chunks * tab_bytes<NBT>(g.n_tbins) : 0));
+  int64_t *run = (int64_t *)(smem_raw + a.chunks * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins));
   int64_t *tot = run + V;
   int64_t *vbase = tot + V;
   int32_t *cnt = (int32_t *)(vbase + V);
   int32_t *wcnt = cnt + V;
   __shared__ int64_t s_total;
-  if (FMT == kCellXq)
-    for (int c = 0; c < a.chunks; ++c)
-      tab_fill<NBT>(tab + c * (tab_bytes<NBT>(g.n_tbins) / sizeof(float)), g, c * NBT);
+  for (int c = 0; c < a.chunks; ++c)
+    chunk_fill<NBT, FMT>(smem_raw + c * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g, c * NBT);
   __syncthreads();
 
   const TreeView t = a.t;
@@ -178,14 +178,13 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT>::value) k_air_ba
         const int chunk = (int)(it / (unsigned long long)a.P);
         const int64_t q = (int64_t)(it - (unsigned long long)chunk * a.P);
         const int b0 = chunk * NBT;
-        BandCtx bc;
-        bc.tab = tab + chunk * (tab_bytes<NBT>(g.n_tbins) / sizeof(float));
-        bc.nbh = min(NBT, nb - b0);
+        const BandCtx bc = chunk_ctx<NBT, FMT>(smem_raw + chunk * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g,
+                                               min(NBT, nb - b0));
         BandRegs<NBT> br;
-        band_regs<NBT>(br, g.bands, b0, bc.nbh);
+        band_regs<NBT>(br, bc);
         const RayGeom &rg = a.geoms[a.pview[q]];
         RTState<NBT> st;
-        trace_ray<NBT, AMR, FMT>(st, g, rg, a.plvl[q], a.ppi[q], a.ppj[q], a.fp64_level, bc, br);
+        trace_ray<NBT, AMR, FMT, DIR>(st, g, rg, a.plvl[q], a.ppi[q], a.ppj[q], a.fp64_level, bc, br);
         if (chunk == 0) {
           a.pN[q] = st.N;
           a.psteps[q] = st.steps;
@@ -245,14 +244,13 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT>::value) k_air_ba
         }
       }
       if (todo) {
-        BandCtx bc;
-        bc.tab = tab + chunk * (tab_bytes<NBT>(g.n_tbins) / sizeof(float));
-        bc.nbh = min(NBT, nb - b0);
+        const BandCtx bc = chunk_ctx<NBT, FMT>(smem_raw + chunk * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g,
+                                               min(NBT, nb - b0));
         BandRegs<NBT> br;
-        band_regs<NBT>(br, g.bands, b0, bc.nbh);
+        band_regs<NBT>(br, bc);
         const RayGeom &rg = a.geoms[v];
         RTState<NBT> st;
-        trace_ray<NBT, AMR, FMT>(st, g, rg, t.lvl[k], t.pi[k], t.pj[k], a.fp64_level, bc, br);
+        trace_ray<NBT, AMR, FMT, DIR>(st, g, rg, t.lvl[k], t.pi[k], t.pj[k], a.fp64_level, bc, br);
         if (chunk == 0) {
           t.N[k] = st.N;
           t.steps[k] = st.steps;
@@ -353,14 +351,14 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT>::value) k_air_ba
   }
 }
 
-template <int NBT, bool AMR, int FMT>
+template <int NBT, bool AMR, int FMT, int DIR>
 static cudaError_t batch_occupancy(int *blocks_per_sm, size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(k_air_batch<NBT, AMR, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_air_batch<NBT, AMR, FMT, DIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_air_batch<NBT, AMR, FMT>, kBatchBlock, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_air_batch<NBT, AMR, FMT, DIR>, kBatchBlock, smem);
 }
 
-template <int NBT, bool AMR, int FMT>
+template <int NBT, bool AMR, int FMT, int DIR>
 static cudaError_t batch_launch(const BatchArgs &a, int grid, size_t smem, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
@@ -372,31 +370,37 @@ static cudaError_t batch_launch(const BatchArgs &a, int grid, size_t smem, cudaS
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_air_batch<NBT, AMR, FMT>, a);
+  return cudaLaunchKernelEx(&cfg, k_air_batch<NBT, AMR, FMT, DIR>, a);
+}
+
+template <int NBT, int FMT, int DIR>
+static void batch_pick(bool amr, BatchOccFn *occ, BatchLaunchFn *launch) {
+  *occ = amr ? batch_occupancy<NBT, true, FMT, DIR> : batch_occupancy<NBT, false, FMT, DIR>;
+  *launch = amr ? batch_launch<NBT, true, FMT, DIR> : batch_launch<NBT, false, FMT, DIR>;
 }
 
 // Occupancy and launch functions and shared memory of the kernel for a grid
-// and V views with NBT bands per thread; false where there is no such form.
+// and V views (inclined: all of them are) with NBT bands per thread; false
+// where there is no such form.
 template <int NBT>
-bool batch_fns(const GridView &g, int V, BatchOccFn *occ, BatchLaunchFn *launch, size_t *smem) {
+bool batch_fns(const GridView &g, int V, bool inclined, BatchOccFn *occ, BatchLaunchFn *launch, size_t *smem) {
   const bool amr = g.kind == AIR_GRID_AMR;
-  const int fmt = g.cell_fmt;
   *smem = batch_smem<NBT>(g, V);
-  if (fmt == kCellLam) {
+  if (g.cell_fmt == kCellLam) {
     // per-cell Lambda exists for one-band grids only
     if constexpr (NBT == 1) {
-      *occ = amr ? batch_occupancy<1, true, kCellLam> : batch_occupancy<1, false, kCellLam>;
-      *launch = amr ? batch_launch<1, true, kCellLam> : batch_launch<1, false, kCellLam>;
+      if (inclined) batch_pick<1, kCellLam, -2>(amr, occ, launch);
+      else batch_pick<1, kCellLam, 0>(amr, occ, launch);
       return true;
     }
     return false;
   }
-  if (fmt == kCellXq) {
-    *occ = amr ? batch_occupancy<NBT, true, kCellXq> : batch_occupancy<NBT, false, kCellXq>;
-    *launch = amr ? batch_launch<NBT, true, kCellXq> : batch_launch<NBT, false, kCellXq>;
+  if (g.cell_fmt == kCellXq) {
+    if (inclined) batch_pick<NBT, kCellXq, -2>(amr, occ, launch);
+    else batch_pick<NBT, kCellXq, 0>(amr, occ, launch);
   } else {
-    *occ = amr ? batch_occupancy<NBT, true, kCellRho> : batch_occupancy<NBT, false, kCellRho>;
-    *launch = amr ? batch_launch<NBT, true, kCellRho> : batch_launch<NBT, false, kCellRho>;
+    if (inclined) batch_pick<NBT, kCellRho, -2>(amr, occ, launch);
+    else batch_pick<NBT, kCellRho, 0>(amr, occ, launch);
   }
   return true;
 }

@@ -37,7 +37,7 @@ __global__ void k_band_sum_dev(const float *__restrict__ I, int n_bands, int64_t
 // few rays, or in the ordinary one of that width.
 static int64_t few_rays(int NBT, bool lone, int chunks) {
   const int blocks = lone ? (NBT <= 4 ? MinBlocks<4, -1>::value : MinBlocks<8, -1>::value)
-                          : (NBT <= 1 ? kAxisBlocksSmall : (NBT <= 2 ? MinBlocks<2, 0>::value : MinBlocks<4, 0>::value));
+                          : (NBT <= 1 ? kAxisBlocksSmall : (NBT <= 2 ? MinBlocks<2, -3>::value : MinBlocks<4, -3>::value));
   return (int64_t)sm_count() * blocks * kMarchBlock * 2 / chunks;
 }
 

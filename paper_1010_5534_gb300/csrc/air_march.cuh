@@ -80,12 +80,39 @@ __device__ __forceinline__ void tab_fill(float *tab, const GridView &g, int b0) 
   }
 }
 
+// Shared memory of a band chunk: its table (kCellXq) and its bands' constants.
+template <int NBT>
+__host__ __device__ constexpr size_t chunk_bytes(bool table, int n_tbins) {
+  return (table ? tab_bytes<NBT>(n_tbins) : 0) + sizeof(BandConst) * NBT;
+}
+
 struct BandCtx {
-  const float *tab;  // shared: the chunk's table (tab_fill)
+  const float *tab;      // shared: the chunk's table (tab_fill)
+  const BandConst *band; // shared: the chunk's bands (zero opacity beyond the last)
   int nbh;
 };
 
-// Per-band constants held in registers for the whole ray.
+// Fill a chunk's shared memory at `sm` by one block.
+template <int NBT, int FMT>
+__device__ __forceinline__ void chunk_fill(unsigned char *sm, const GridView &g, int b0) {
+  if (FMT == kCellXq) tab_fill<NBT>(reinterpret_cast<float *>(sm), g, b0);
+  BandConst *band = reinterpret_cast<BandConst *>(sm + (FMT == kCellXq ? tab_bytes<NBT>(g.n_tbins) : 0));
+  for (int b = threadIdx.x; b < NBT; b += blockDim.x)
+    band[b] = b0 + b < g.n_bands ? g.bands[b0 + b] : BandConst{0.f, 0.f, -0.f, 0xffffffffu};
+}
+template <int NBT, int FMT>
+__device__ __forceinline__ BandCtx chunk_ctx(const unsigned char *sm, const GridView &g, int nbh) {
+  BandCtx bc;
+  bc.tab = reinterpret_cast<const float *>(sm);
+  bc.band = reinterpret_cast<const BandConst *>(sm + (FMT == kCellXq ? tab_bytes<NBT>(g.n_tbins) : 0));
+  bc.nbh = nbh;
+  return bc;
+}
+
+// Per-band constants in registers. One band keeps them for the whole ray; with
+// more, only the column march of axis rays does (band_load), and the cells of
+// inclined rays read their band's constants from shared memory (one 16-byte
+// load that every lane shares, against 24 registers at 8 bands).
 template <int NBT>
 struct BandRegs {
   float kap[NBT];  // kappa_b
@@ -95,22 +122,30 @@ struct BandRegs {
   uint32_t xz;     // table coordinates below xz emit nothing in any band (kCellXq)
 };
 
-// Per-band registers of bands [b0, b0 + nbh) (zero beyond).
 template <int NBT>
-__device__ __forceinline__ void band_regs(BandRegs<NBT> &br, const BandConst *bands, int b0,
-                                          int nbh) {
+__device__ __forceinline__ BandConst band_const(const BandCtx &bc, int b) {
+  const float4 c = *reinterpret_cast<const float4 *>(bc.band + b);
+  return BandConst{c.x, c.y, c.z, __float_as_uint(c.w)};
+}
+template <int NBT>
+__device__ __forceinline__ void band_load(BandRegs<NBT> &br, const BandCtx &bc) {
   br.kmax = 0.f;
-  br.xz = 0xffffffffu;
 #pragma unroll
   for (int b = 0; b < NBT; ++b) {
-    float4 c = make_float4(0.f, 0.f, -0.f, __uint_as_float(0xffffffffu));
-    if (b < nbh) c = __ldg(reinterpret_cast<const float4 *>(bands + b0 + b));
-    br.kap[b] = c.x;
-    br.ik[b] = c.y;
-    br.nk[b] = c.z;
-    br.xz = min(br.xz, __float_as_uint(c.w));
-    br.kmax = fmaxf(br.kmax, br.kap[b]);
+    const BandConst c = band_const<NBT>(bc, b);
+    br.kap[b] = c.kap;
+    br.ik[b] = c.ik;
+    br.nk[b] = c.nk;
+    br.kmax = fmaxf(br.kmax, c.kap);
   }
+}
+// What a ray starts with: xz, and one band's constants.
+template <int NBT>
+__device__ __forceinline__ void band_regs(BandRegs<NBT> &br, const BandCtx &bc) {
+  br.xz = 0xffffffffu;
+#pragma unroll
+  for (int b = 0; b < NBT; ++b) br.xz = min(br.xz, bc.band[b].xz);
+  if (NBT == 1) band_load<NBT>(br, bc);
 }
 
 // Whether a cell emits nothing in any band of the chunk, from its auxiliary
@@ -150,10 +185,12 @@ __device__ __forceinline__ void rt_init(RTState<NBT> &r) {
 
 // T[] brought up to the current N after cells that emit nothing.
 template <int NBT>
-__device__ __forceinline__ void rt_refresh(RTState<NBT> &r, const BandRegs<NBT> &br) {
+__device__ __forceinline__ void rt_refresh(RTState<NBT> &r, const BandCtx &bc) {
 #pragma unroll
-  for (int b = 0; b < NBT; ++b)
-    r.T[b] = ex2_approx(fmaf(br.nk[b], r.tp, __fmul_rn(br.nk[b], r.tN)));
+  for (int b = 0; b < NBT; ++b) {
+    const float nk = bc.band[b].nk;
+    r.T[b] = ex2_approx(fmaf(nk, r.tp, __fmul_rn(nk, r.tN)));
+  }
   r.stale = false;
 }
 
@@ -207,7 +244,7 @@ __device__ __forceinline__ void tab_pair(const float *row, int q, float w, float
 template <int NBT, int FMT>
 __device__ __forceinline__ void rt_bands(RTState<NBT> &r, float rho, uint32_t aux, float rds, float N,
                                          const BandCtx &bc, const BandRegs<NBT> &br) {
-  if (FMT != kCellRho && NBT > 1 && r.stale) rt_refresh<NBT>(r, br);
+  if (FMT != kCellRho && NBT > 1 && r.stale) rt_refresh<NBT>(r, bc);
   float w = 0.f;
   const float *row = bc.tab;
   if (FMT == kCellXq) {
@@ -222,12 +259,13 @@ __device__ __forceinline__ void rt_bands(RTState<NBT> &r, float rho, uint32_t au
 #pragma unroll
       for (int e = 0; e < (NBT == 1 ? 1 : 2); ++e) {
         const int b = 2 * q + e;
-        const float dtau = br.kap[b] * rds;
-        const float Tn = ex2_approx(br.nk[b] * N);
+        const BandConst c = NBT == 1 ? BandConst{br.kap[0], br.ik[0], br.nk[0], 0u} : band_const<NBT>(bc, b);
+        const float dtau = c.kap * rds;
+        const float Tn = ex2_approx(c.nk * N);
         // rho Lambda_b
         const float rl = FMT == kCellLam ? __uint_as_float(aux) : (FMT == kCellXq ? rho * lam[e] : rho);
         const float t_small = __fmul_rn(rl * rds, r.T[b] * one_minus_exp_over_x(dtau));
-        const float t_large = __fmul_rn(rl * br.ik[b], r.T[b] - Tn);
+        const float t_large = __fmul_rn(rl * c.ik, r.T[b] - Tn);
         const float term = dtau < 0.25f ? t_small : t_large;
         r.T[b] = Tn;
         kahan_add(r.I[b], r.cI[b], term);
@@ -263,7 +301,7 @@ __device__ __forceinline__ void rt_term(RTState<NBT> &r, float rho, uint32_t aux
 // chunks times the L2's latency (800 cycles), and registers are free.
 template <int NBT, int DIR>
 struct DdaChunk {
-  static constexpr int value = DIR >= 0 ? 4 : (NBT <= 2 ? 16 : 8);
+  static constexpr int value = DIR != -1 ? 4 : (NBT <= 2 ? 16 : 8);
 };
 
 // Fields of cell idx: rho and the auxiliary word of the format.
@@ -429,7 +467,7 @@ __device__ __forceinline__ void column_cells(RTState<NBT> &r, float (&rh)[U],
 #pragma unroll
     for (int u = 1; u < U; ++u) x = FMT == kCellLam ? x | xv[u] : max(x, xv[u]);
     if (cell_dark<FMT>(x, br.xz) && column_group_dark<NBT, FMT, U>(r, rh, ds, br)) return;
-    if (NBT > 1 && r.stale) rt_refresh<NBT>(r, br);
+    if (NBT > 1 && r.stale) rt_refresh<NBT>(r, bc);
   }
   const float m = max_of<U>(rh);
   const float dmax = br.kmax * (FMT == kCellLam ? m : __fmul_rn(m, ds));
@@ -1286,9 +1324,10 @@ __device__ __forceinline__ void march_uniform_axis(RTState<NBT> &r, const GridVi
 template <int NBT, bool AMR, int FMT, int DIR, int U>
 __device__ __forceinline__ void march_axis(RTState<NBT> &st, const GridView &g, const RayGeom &rg,
                                            int A, int L, int i, int j, const BandCtx &bc,
-                                           const BandRegs<NBT> &br) {
+                                           BandRegs<NBT> &br) {
   int c1, c2;
   if (!axis_ray_setup(g, rg, A, L, i, j, c1, c2)) return;
+  if (NBT > 1) band_load<NBT>(br, bc);
   if constexpr (!AMR) march_uniform_axis<NBT, FMT, U>(st, g, A, c1, c2, rg, bc, br);
   else if constexpr (DIR >= 7) march_amr_axis<NBT, FMT, U, false, (DIR < 10 ? 1 : -1), (DIR - 1) % 3>(st, g, A, c1, c2, rg, bc, br);
   else if constexpr (DIR >= 4) march_amr_axis_small<NBT, FMT>(st, g, A, c1, c2, rg, bc, br);
@@ -1296,24 +1335,32 @@ __device__ __forceinline__ void march_axis(RTState<NBT> &st, const GridView &g, 
 }
 
 // One ray (pixel (L, i, j)) through the grid, bands [b0, b0 + NBT) of bc/br.
-// DIR = 1 + A: every ray of the launch is parallel to grid axis A (bricks of 16
-// cells and more, or a uniform grid); 4 + A: the same with bricks of at most 8
-// cells; 7 + A and 10 + A: with 16^3 bricks, towards higher and lower cells;
-// 0: any direction; -1: inclined rays in launches of few rays (DdaChunk).
+// DIR, the kernel's form:
+//   0: any direction (the batched kernel);
+//   1 + A: every ray of the launch is parallel to grid axis A, one band (bricks
+//     of 16 cells and more, or a uniform grid); 4 + A: the same with bricks of
+//     at most 8 cells; 7 + A and 10 + A: with 16^3 bricks, towards higher and
+//     lower cells;
+//   -1: inclined rays in launches of few rays (DdaChunk); -2: inclined rays;
+//   -3: rays parallel to some axis, any number of bands.
 template <int NBT, bool AMR, int FMT, int DIR = 0>
 __device__ __forceinline__ void trace_ray(RTState<NBT> &st, const GridView &g, const RayGeom &rg,
                                           int L, int i, int j, int fp64_level, const BandCtx &bc,
-                                          const BandRegs<NBT> &br) {
+                                          BandRegs<NBT> &br) {
   rt_init<NBT>(st);
   constexpr int U = ColumnUnroll<DIR>::value;
   if constexpr (DIR >= 1) {
     march_axis<NBT, AMR, FMT, DIR, U>(st, g, rg, (DIR - 1) % 3, L, i, j, bc, br);
-  } else {
+    return;
+  }
+  if constexpr (DIR == 0 || DIR == -3) {
     const bool m0 = rg.Dhi[0] != 0.f, m1 = rg.Dhi[1] != 0.f, m2 = rg.Dhi[2] != 0.f;
-    if (DIR == 0 && m0 + m1 + m2 == 1) {
+    if (DIR == -3 || m0 + m1 + m2 == 1) {
       march_axis<NBT, AMR, FMT, DIR, U>(st, g, rg, m0 ? 0 : (m1 ? 1 : 2), L, i, j, bc, br);
       return;
     }
+  }
+  if constexpr (DIR <= 0 && DIR != -3) {
     double O[3], t0;
     F2 Of[3];
     int eax;

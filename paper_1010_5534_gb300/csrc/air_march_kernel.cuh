@@ -34,7 +34,8 @@ constexpr int kAxisBlocksSmall = 6;  // bricks of at most 8 cells: two bricks' r
 // DIR = -1 has the registers of two or three blocks (see DdaChunk).
 template <int NBT, int DIR>
 struct MinBlocks {
-  static constexpr int value = DIR < 0 ? (NBT <= 4 ? 3 : 2)
+  static constexpr int value = DIR == -1 ? (NBT <= 4 ? 3 : 2)
+                               : DIR == -2 ? (NBT <= 1 ? 6 : (NBT <= 2 ? 5 : (NBT <= 8 ? 4 : 3)))
                                : DIR >= 4 && DIR <= 6 ? kAxisBlocksSmall
                                : DIR >= 1 ? kAxisBlocks
                                : (NBT <= 1 ? 6 : (NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? 3 : 2))));
@@ -47,7 +48,7 @@ constexpr int kMarchBlock = 128;
 template <int NBT, bool AMR, int FMT, int DIR>
 __device__ __forceinline__ void march_one(const GridView &g, const RayGeom &rg, const RaySource &src,
                                           const RayOut &out, int fp64_level, const BandCtx &bc,
-                                          const BandRegs<NBT> &br, int chunk, int b0, int nbh,
+                                          BandRegs<NBT> &br, int chunk, int b0, int nbh,
                                           int64_t k) {
   if (src.use_prop) {
     // the pixel's values from the proposal wave when it traced the pixel
@@ -76,7 +77,7 @@ __device__ __forceinline__ void march_one(const GridView &g, const RayGeom &rg, 
   if (chunk == 0) {
     out.N[k] = st.N;
     out.steps[k] = st.steps;
-    if (out.tau0) out.tau0[k] = br.kap[0] * st.N;
+    if (out.tau0) out.tau0[k] = bc.band[0].kap * st.N;
     if (out.maxlev) out.maxlev[k] = (uint8_t)st.maxlev;
   }
 #pragma unroll
@@ -94,19 +95,17 @@ __device__ __forceinline__ void march_one(const GridView &g, const RayGeom &rg, 
 template <int NBT, bool AMR, int FMT, int DIR>
 __global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
     k_march(GridView g, RayGeom rg, RaySource src, RayOut out, int fp64_level) {
-  extern __shared__ __align__(16) float smem[];
+  extern __shared__ __align__(16) unsigned char smem[];
   const int chunk = blockIdx.y;
   const int b0 = chunk * NBT;
   const int nbh = min(NBT, g.n_bands - b0);
-  BandCtx bc;
-  bc.tab = smem;
-  bc.nbh = nbh;
-  if (FMT == kCellXq) tab_fill<NBT>(smem, g, b0);
-  BandRegs<NBT> br;
-  band_regs<NBT>(br, g.bands, b0, nbh);
-  // (the tables and constants above were written when the grid was loaded)
+  chunk_fill<NBT, FMT>(smem, g, b0);
+  const BandCtx bc = chunk_ctx<NBT, FMT>(smem, g, nbh);
+  // (what fills the shared memory was written when the grid was loaded)
   wait_prior_grid();
   __syncthreads();
+  BandRegs<NBT> br;
+  band_regs<NBT>(br, bc);
 
   if (src.mode == 2) {
     // new nodes of a sweep counted on the device: block b takes chunk b of
@@ -155,7 +154,7 @@ __global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
   if (chunk == 0) {
     out.N[k] = st.N;
     out.steps[k] = st.steps;
-    if (out.tau0) out.tau0[k] = br.kap[0] * st.N;
+    if (out.tau0) out.tau0[k] = bc.band[0].kap * st.N;
     if (out.maxlev) out.maxlev[k] = (uint8_t)st.maxlev;
   }
 #pragma unroll
@@ -180,17 +179,20 @@ static dim3 march_grid(const MarchLaunch &m) {
 
 template <int NBT, bool AMR, int FMT, int DIR>
 static cudaError_t march_form(const MarchLaunch &m) {
-  const size_t smem = FMT == kCellXq ? tab_bytes<NBT>(m.g.n_tbins) : 0;
+  const size_t smem = chunk_bytes<NBT>(FMT == kCellXq, m.g.n_tbins);
   return launch_pdl(k_march<NBT, AMR, FMT, DIR>, march_grid<NBT, DIR>(m), dim3(kMarchBlock), smem, m.st,
                     m.g, m.rg, m.src, m.out, m.fp64_level);
 }
 
 template <int NBT, bool AMR, int FMT>
 static cudaError_t march_any(const MarchLaunch &m) {
+  const int moving = (m.rg.Dhi[0] != 0.f) + (m.rg.Dhi[1] != 0.f) + (m.rg.Dhi[2] != 0.f);
+  if constexpr (NBT > 1)  // (one band: march_axis_one)
+    if (moving == 1) return march_form<NBT, AMR, FMT, -3>(m);
   // 16 bands per thread leave no registers for the form for few rays
   if constexpr (NBT <= 8)
     if (m.few) return march_form<NBT, AMR, FMT, -1>(m);
-  return march_form<NBT, AMR, FMT, 0>(m);
+  return march_form<NBT, AMR, FMT, -2>(m);
 }
 
 // Rays in any direction, NBT bands per thread.
