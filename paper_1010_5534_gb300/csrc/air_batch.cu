@@ -416,7 +416,7 @@ air_status render_batch(air_grid *g, const air_view *views, int32_t V, const air
     }
     // the graph holds: reset of the control words, the cooperative launch
     const bool same = bw.exec && !std::memcmp(&bw.key, &a, sizeof(BatchArgs)) && bw.key_grid == grid &&
-                      bw.key_smem == smem && bw.key_nbt == nbt;
+                      bw.key_smem == smem && bw.key_launch == launch;
     CU_TRY(prof_open(g, AIR_PHASE_BATCH, 1));
     if (op.use_graph) {
       if (!same) {
@@ -446,7 +446,7 @@ air_status render_batch(air_grid *g, const air_view *views, int32_t V, const air
         bw.key = a;
         bw.key_grid = grid;
         bw.key_smem = smem;
-        bw.key_nbt = nbt;
+        bw.key_launch = launch;
       }
       CU_TRY(cudaGraphLaunch(bw.exec, st));
     } else {

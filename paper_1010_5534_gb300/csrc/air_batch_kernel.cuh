@@ -9,7 +9,6 @@
 namespace air {
 
 typedef cudaError_t (*BatchOccFn)(int *, size_t);
-typedef cudaError_t (*BatchLaunchFn)(const BatchArgs &, int, size_t, cudaStream_t);
 
 constexpr int kBatchBlock = 128;
 constexpr int kBatchMaxViews = 256;

@@ -125,6 +125,8 @@ struct BatchArgs {
   uint32_t *psteps;      // [P]
 };
 
+typedef cudaError_t (*BatchLaunchFn)(const BatchArgs &, int, size_t, cudaStream_t);
+
 // Buffers and the captured graph of batched renders.
 struct BatchWork {
   RayGeom *geoms = nullptr;
@@ -143,7 +145,8 @@ struct BatchWork {
   cudaGraphExec_t exec = nullptr;
   cudaStream_t cap_stream = nullptr;  // private stream the graph is captured on
   BatchArgs key{};
-  int key_grid = 0, key_nbt = 0;
+  int key_grid = 0;
+  BatchLaunchFn key_launch = nullptr;
   size_t key_smem = 0;
 };
 
