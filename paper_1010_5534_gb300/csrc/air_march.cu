@@ -108,7 +108,10 @@ cudaError_t launch_march(const GridView &g, const Camera &cam, const RaySource &
   // inclined rays take the form DIR = -1. `few`: the rays that fill that form's
   // threads twice. Where the count is on the device, both launches are queued
   // and the one that it is not for returns.
-  const int narrow = tune.nbt > 0 ? nbt : std::min(nbt, g.n_bands <= 8 ? 1 : (g.n_bands <= 16 ? 2 : 4));
+  // Rays along an axis keep the chunks of large launches: their series
+  // (column_group) is chosen by the largest opacity of the chunk, so another
+  // width gives other last bits.
+  const int narrow = tune.nbt > 0 || moving == 1 ? nbt : std::min(nbt, g.n_bands <= 8 ? 1 : (g.n_bands <= 16 ? 2 : 4));
   const int nchunks = (g.n_bands + narrow - 1) / narrow;
   const bool lone = moving > 1 && narrow <= 8;  // there is a form for few rays
   const int64_t few = lone || narrow < nbt ? few_rays(narrow, lone, nchunks) : 0;
