@@ -738,7 +738,7 @@ def large_view_record(air, torch, st, reps=2):
 
 def batch_record(air, torch, st):
     """The batched configuration in brief: the cone grid with 16 bands
-    (0.5-10 keV) at 64 random views, one persistent launch (8 bands per
+    (0.5-10 keV) at 64 random views, one persistent launch (16 bands per
     thread), against fixed 4096^2 images of two of the views (extrapolated to
     64) with the band-summed flux error on those two, and the batched march's
     FP32-issue fraction. Scene generation, upload and one warm-up render are
@@ -766,7 +766,7 @@ def batch_record(air, torch, st):
     band_steps_s = 16 * steps / (prof["batch"][0] * 1e-3)
     peak_ops = 152 * 128 * 2.07e9
     rec = dict(workload="cone grid, 64 random views x 16 bands (0.5-10 keV), base 256^2, max level 4, "
-                        "xi_crit 0.5, one persistent launch, 8 bands per thread",
+                        "xi_crit 0.5, one persistent launch, 16 bands per thread",
                setup_s=setup_s, batched_ms=ms, rays=int(sum(r["n_rays"] for r in b)), steps=int(steps),
                band_steps_per_s=16 * steps / ms * 1e3, kernel_ms=prof["batch"][0],
                fixed_per_view_ms=fixed_view_ms, fixed_64_views_ms_extrapolated=fixed_view_ms * len(vs),

@@ -25,7 +25,7 @@ LIB_PATH = os.path.join(_HERE, "libair_gb300.so")
 SOURCES = ["air_api.cu", "air_grid.cu", "air_march.cu", "air_refine.cu", "air_static.cu",
            "air_batch.cu", "air_mlp.cu", "air_learned.cu", "air_tune.cu", "air_raster.cu",
            "air_march_axis.cu"] + \
-    [f"air_{k}_{n}.cu" for k in ("march", "batch") for n in (1, 2, 4, 8, 16)]
+    [f"air_{k}_{n}.cu" for k in ("march", "batch") for n in (1, 2, 4, 8, 16)] + ["air_batch_wide.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
 

@@ -74,9 +74,10 @@ cudaError_t prof_open(air_grid *g, int phase, int nlaunch) {
   return cudaEventRecord(P.ev[2 * P.used], g->stream);
 }
 
-cudaError_t prof_close(air_grid *g) {
+cudaError_t prof_close(air_grid *g, int nlaunch) {
   Profiler &P = g->prof;
   if (!P.on) return cudaSuccess;
+  P.nlaunch[P.used] += nlaunch;
   cudaError_t r = cudaEventRecord(P.ev[2 * P.used + 1], g->stream);
   ++P.used;
   return r;
@@ -296,9 +297,10 @@ air_status render_fixed(air_grid *g, const air_view *view, int32_t res, int32_t 
   }
   RayOut ro{o.N ? o.N : w.fN, o.I ? o.I : w.fI, o.I ? o.stride : n, w.fsteps, o.p ? o.p : w.fp};
   g->prof.used = 0;
-  CU_TRY(prof_open(g, AIR_PHASE_MARCH, nb > (g->tune.bands_per_thread > 0 ? g->tune.bands_per_thread : default_bands_per_thread(nb)) ? 2 : 1));
-  CU_TRY(launch_march(g->gv, cam, src, ro, march_tune(g, fp64_level), st));
-  CU_TRY(prof_close(g));
+  int nl = 0;
+  CU_TRY(prof_open(g, AIR_PHASE_MARCH, 0));
+  CU_TRY(launch_march(g->gv, cam, src, ro, march_tune(g, fp64_level), st, &nl));
+  CU_TRY(prof_close(g, nl));
   FluxArgs fa{};
   fa.n = n; fa.child = nullptr; fa.lvl = nullptr; fa.I = ro.I; fa.stride = ro.stride; fa.steps = w.fsteps;
   fa.n_bands = nb; fa.area0 = (2.0 * cam.H / res) * (2.0 * cam.H / res); fa.partial = w.partial;
@@ -390,7 +392,7 @@ static air_status wait_report(const SweepReport &rep, uint32_t tag, int64_t q, c
 
 air_status sweep_loop_device(air_grid *g, const Camera &cam, const air_params *pr, int64_t nbase,
                              int64_t m, int64_t bound, int64_t open_max, const MarchTune &tune,
-                             int march_launches, int32_t *lmap, const Proposal *prop,
+                             int32_t *lmap, const Proposal *prop,
                              SweepEnd *fin) {
   Workspace &w = g->ws;
   cudaStream_t st = g->stream;
@@ -447,9 +449,10 @@ air_status sweep_loop_device(air_grid *g, const Camera &cam, const air_params *p
                              st, lmap));
     CU_TRY(prof_close(g));
     // step ii on the new pixels (or their values from the proposal)
-    CU_TRY(prof_open(g, AIR_PHASE_MARCH, march_launches));
-    CU_TRY(launch_march(g->gv, cam, ds, ro, tune, st));
-    CU_TRY(prof_close(g));
+    int nl = 0;
+    CU_TRY(prof_open(g, AIR_PHASE_MARCH, 0));
+    CU_TRY(launch_march(g->gv, cam, ds, ro, tune, st, &nl));
+    CU_TRY(prof_close(g, nl));
   }
   if (rep.err) return set_error(AIR_ERR_NUMERIC, "balance closure overflowed its stack");
   fin->n = rep.n;
@@ -533,7 +536,7 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
   // writes them to staging buffer k, which the copy stream then moves to the
   // host array while the next sweep proceeds; buffer k is reused only after
   // its copy has finished.
-  auto march_nodes = [&](const TreeView &tv, RaySource src, const MarchTune &tune, int launches) -> air_status {
+  auto march_nodes = [&](const TreeView &tv, RaySource src, const MarchTune &tune) -> air_status {
     RayOut ro{tv.N, tv.I, tv.cap, tv.steps, tv.p};
     const int k = stage_k;
     if (streamed) {
@@ -543,6 +546,7 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
       ro.stride = src.count;
       ro.ioff = src.first;
     }
+    int nl = 0;
     if (sharded) {
       // this rank's slice of the sweep's rays, then the other slices from
       // the other ranks (Section 2: trace distributed, gather for the scan)
@@ -552,9 +556,9 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
       src.first = first + lo;
       src.count = hi - lo;
       if (src.count > 0) {
-        CU_TRY(prof_open(g, AIR_PHASE_MARCH, launches));
-        CU_TRY(launch_march(g->gv, cam, src, ro, tune, g->stream));
-        CU_TRY(prof_close(g));
+        CU_TRY(prof_open(g, AIR_PHASE_MARCH, 0));
+        CU_TRY(launch_march(g->gv, cam, src, ro, tune, g->stream, &nl));
+        CU_TRY(prof_close(g, nl));
       }
       CU_TRY(cudaStreamSynchronize(g->stream));
       if (shard->exchange(shard->user, first, count, nb, tv.N, tv.I, tv.cap, tv.p, tv.steps) != 0)
@@ -562,9 +566,9 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
                          (long long)(first + count));
       return AIR_OK;
     }
-    CU_TRY(prof_open(g, AIR_PHASE_MARCH, launches));
-    CU_TRY(launch_march(g->gv, cam, src, ro, tune, g->stream));
-    CU_TRY(prof_close(g));
+    CU_TRY(prof_open(g, AIR_PHASE_MARCH, 0));
+    CU_TRY(launch_march(g->gv, cam, src, ro, tune, g->stream, &nl));
+    CU_TRY(prof_close(g, nl));
     if (streamed) {
       if (src.first + src.count <= spectra_cap) {
         CU_TRY(cudaEventRecord(sp.marched[k], g->stream));
@@ -600,17 +604,15 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
     t = w.tree(n0, Lm);
     const MarchTune tune = march_tune(g, pr->fp64_level);
     g->prof.used = 0;
-    const int nbt_eff = tune.nbt > 0 ? tune.nbt : default_bands_per_thread(nb);
-    const int march_launches = nb > nbt_eff ? 2 : 1;  // march (+ band sum when bands are chunked)
     // step i + ii: base image
     CU_TRY(prof_open(g, AIR_PHASE_REFINE, 1));
     CU_TRY(launch_init_base(t, st));
     CU_TRY(prof_close(g));
     CU_TRY(cudaMemsetAsync(w.d_err, 0, sizeof(uint32_t), st));
     RaySource src{};
-    src.mode = 0; src.n0 = n0; src.lvl = t.lvl; src.pi = t.pi; src.pj = t.pj; src.first = 0; src.count = nbase;
+    src.mode = 0; src.base = 1; src.n0 = n0; src.lvl = t.lvl; src.pi = t.pi; src.pj = t.pj; src.first = 0; src.count = nbase;
     if ((s = axis_table(g, cam, n0, Lm, src))) return s;
-    if ((s = march_nodes(t, src, tune, march_launches))) return s;
+    if ((s = march_nodes(t, src, tune))) return s;
     n = nbase;
     // open-leaf list: the base pixels, unless the base is the top level
     int cur = 0;
@@ -621,7 +623,7 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
     g->last.lmap = lmap;
     if (dev_loop) {
       SweepEnd fin;
-      if ((s = sweep_loop_device(g, cam, pr, nbase, m, bound, open_max, tune, march_launches, lmap,
+      if ((s = sweep_loop_device(g, cam, pr, nbase, m, bound, open_max, tune, lmap,
                                  nullptr, &fin)))
         return s;
       n = fin.n;
@@ -658,7 +660,7 @@ air_status render_adaptive(air_grid *g, const air_view *view, const air_params *
       CU_TRY(launch_list_emit(t, w.open[cur], m, w.flag, w.boff, w.d_total, n, w.open[cur ^ 1], st, lmap));
       CU_TRY(prof_close(g));
       src.lvl = t.lvl; src.pi = t.pi; src.pj = t.pj; src.first = n; src.count = 4 * nflag;
-      if ((s = march_nodes(t, src, tune, march_launches))) return s;
+      if ((s = march_nodes(t, src, tune))) return s;
       n = n_new;
       n_refined += nflag;
       ++sweeps;

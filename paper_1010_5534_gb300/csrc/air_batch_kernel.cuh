@@ -12,6 +12,7 @@ typedef cudaError_t (*BatchOccFn)(int *, size_t);
 
 constexpr int kBatchBlock = 128;
 constexpr int kBatchMaxViews = 256;
+constexpr size_t kBatchMaxSmem = 227 * 1024;  // shared memory that a block can have
 constexpr uint32_t kErrBalance = 1u, kErrTimeout = 2u, kErrCapacity = 4u;
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -109,9 +110,13 @@ struct EmitChildrenV {
 
 // Shared memory of a block: the emission tables of every band chunk, and the
 // per-view counters.
+// (NBT = 0, the wide form: of every chunk of `width` bands, and the sums.)
 template <int NBT>
-static size_t batch_smem(const GridView &g, int V) {
-  const size_t tab = ((g.n_bands + NBT - 1) / NBT) * chunk_bytes<NBT>(g.cell_fmt == kCellXq, g.n_tbins);
+static size_t batch_smem(const GridView &g, int V, int width) {
+  const bool table = g.cell_fmt == kCellXq;
+  const size_t tab = NBT == 0 ? ((g.n_bands + width - 1) / width) * wide_tab_bytes(table, g.n_tbins, width) +
+                                    wide_sum_bytes(width, kBatchBlock)
+                              : ((g.n_bands + NBT - 1) / NBT) * chunk_bytes<NBT>(table, g.n_tbins);
   return tab + 3 * sizeof(int64_t) * V + sizeof(int32_t) * V + sizeof(int32_t) * (kBatchBlock / 32) * V;
 }
 
@@ -119,24 +124,101 @@ static size_t batch_smem(const GridView &g, int V) {
 // column march of axis rays, which holds a chunk's band constants and partial
 // sums in registers, a block needs 124 registers instead of 168 at 8 bands per
 // thread and 160 instead of 250 at 16.
+constexpr int kBatchWideBlocks = 4;
 template <int NBT, int DIR>
 struct BatchBlocks {
-  static constexpr int value = NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? (DIR == 0 ? 3 : 4) : (DIR == 0 ? 2 : 3)));
+  static constexpr int value = NBT == 0 ? kBatchWideBlocks : NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? (DIR == 0 ? 3 : 4) : (DIR == 0 ? 2 : 3)));
 };
+
+// Where a traced ray's values go.
+struct BatchOut {
+  float *N, *I, *p;
+  uint32_t *steps;
+  uint8_t *maxlev;  // or NULL
+  int64_t stride;
+};
+
+// Part `part` of band chunk `chunk` of the ray of pixel (L, i, j), to entry k.
+// `all`: the part is the only one.
+template <int NBT, bool AMR, int FMT, int DIR>
+__device__ __forceinline__ void batch_trace(const BatchArgs &a, unsigned char *sm, const RayGeom &rg, int L,
+                                            int i, int j, int chunk, int part, int parts, bool all,
+                                            const BatchOut &o, int64_t k) {
+  const GridView &g = a.g;
+  if constexpr (NBT == 0) {
+    const size_t tab = wide_tab_bytes(FMT == kCellXq, g.n_tbins, a.width);
+    int b0;
+    const int c0 = chunk * a.width;
+    const WideCtx wc = wide_ctx<FMT>(sm + chunk * tab, reinterpret_cast<float4 *>(sm + a.chunks * tab), a.width,
+                                     min(a.width, g.n_bands - c0), part, parts, &b0);
+    b0 += c0;
+    if (wc.pairs <= 0) return;
+    RTState<0> st;
+    trace_wide<AMR, FMT>(st, g, rg, L, i, j, a.fp64_level, wc);
+    if (b0 == 0) {
+      o.N[k] = st.N;
+      o.steps[k] = st.steps;
+      if (o.maxlev) o.maxlev[k] = (uint8_t)st.maxlev;
+    }
+    float p = 0.f;
+    for (int q = 0; q < wc.pairs; ++q) {
+      const float4 s = wc.sums[q * blockDim.x];
+      float *I = o.I + (int64_t)(b0 + 2 * q) * o.stride + k;
+      I[0] = s.x;
+      p += s.x;
+      if (2 * q + 1 < wc.nbh) {
+        I[o.stride] = s.z;
+        p += s.z;
+      }
+    }
+    if (all) o.p[k] = p;
+  } else {
+    const int b0 = chunk * NBT;
+    const BandCtx bc = chunk_ctx<NBT, FMT>(sm + chunk * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g,
+                                           min(NBT, g.n_bands - b0));
+    BandRegs<NBT> br;
+    band_regs<NBT>(br, bc);
+    RTState<NBT> st;
+    trace_ray<NBT, AMR, FMT, DIR>(st, g, rg, L, i, j, a.fp64_level, bc, br);
+    if (chunk == 0) {
+      o.N[k] = st.N;
+      o.steps[k] = st.steps;
+      if (o.maxlev) o.maxlev[k] = (uint8_t)st.maxlev;
+    }
+#pragma unroll
+    for (int c = 0; c < NBT; ++c)
+      if (c < bc.nbh) o.I[(int64_t)(b0 + c) * o.stride + k] = st.I[c];
+    if (all) {
+      float p = 0.f;
+#pragma unroll
+      for (int c = 0; c < NBT; ++c)
+        if (c < bc.nbh) p += st.I[c];
+      o.p[k] = p;
+    }
+  }
+}
 
 template <int NBT, bool AMR, int FMT, int DIR>
 __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_air_batch(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const GridView &g = a.g;
   const int V = a.V, nb = g.n_bands;
-  int64_t *run = (int64_t *)(smem_raw + a.chunks * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins));
+  size_t tab_end;
+  if constexpr (NBT == 0) {
+    const size_t tab = wide_tab_bytes(FMT == kCellXq, g.n_tbins, a.width);
+    for (int c = 0; c < a.chunks; ++c) wide_fill<FMT>(smem_raw + c * tab, g, c * a.width, a.width);
+    tab_end = a.chunks * tab + wide_sum_bytes(a.width, kBatchBlock);
+  } else {
+    for (int c = 0; c < a.chunks; ++c)
+      chunk_fill<NBT, FMT>(smem_raw + c * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g, c * NBT);
+    tab_end = a.chunks * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins);
+  }
+  int64_t *run = (int64_t *)(smem_raw + tab_end);
   int64_t *tot = run + V;
   int64_t *vbase = tot + V;
   int32_t *cnt = (int32_t *)(vbase + V);
   int32_t *wcnt = cnt + V;
   __shared__ int64_t s_total;
-  for (int c = 0; c < a.chunks; ++c)
-    chunk_fill<NBT, FMT>(smem_raw + c * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g, c * NBT);
   __syncthreads();
 
   const TreeView t = a.t;
@@ -166,38 +248,31 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
   int64_t first = a.mode == 2 ? nbase : 0, n = nbase;
   if (a.mode == 2 && a.P > 0) {
     // the proposal wave of every view: (ray, band chunk) items from the queue
-    const unsigned long long items = (unsigned long long)a.P * (unsigned long long)a.chunks;
+    const int parts = NBT == 0 ? wide_parts(a.P * a.chunks, min(a.width, nb), a.fill) : 1;
+    const unsigned long long items = (unsigned long long)a.P * (unsigned long long)(a.chunks * parts);
+    const BatchOut o{a.pN, a.pI, a.pp, a.psteps, nullptr, a.P};
+    const int rpw = rays_per_warp(a.P, a.chunks * parts, (int64_t)nblk * (kBatchBlock / 32));
     for (;;) {
       unsigned long long b = 0;
-      if (lane == 0) b = atomicAdd(&a.ctl->q_head, 32ull);
+      if (lane == 0) b = atomicAdd(&a.ctl->q_head, (unsigned long long)rpw);
       b = __shfl_sync(0xffffffffu, b, 0);
       if (b >= items) break;
-      const unsigned long long it = b + lane;
+      const unsigned long long it = lane < rpw ? b + lane : items;
       if (it < items) {
-        const int chunk = (int)(it / (unsigned long long)a.P);
-        const int64_t q = (int64_t)(it - (unsigned long long)chunk * a.P);
-        const int b0 = chunk * NBT;
-        const BandCtx bc = chunk_ctx<NBT, FMT>(smem_raw + chunk * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g,
-                                               min(NBT, nb - b0));
-        BandRegs<NBT> br;
-        band_regs<NBT>(br, bc);
-        const RayGeom &rg = a.geoms[a.pview[q]];
-        RTState<NBT> st;
-        trace_ray<NBT, AMR, FMT, DIR>(st, g, rg, a.plvl[q], a.ppi[q], a.ppj[q], a.fp64_level, bc, br);
-        if (chunk == 0) {
-          a.pN[q] = st.N;
-          a.psteps[q] = st.steps;
-        }
-#pragma unroll
-        for (int c = 0; c < NBT; ++c)
-          if (c < bc.nbh) a.pI[(int64_t)(b0 + c) * a.P + q] = st.I[c];
-        if (a.chunks == 1) {
-          float p = 0.f;
-#pragma unroll
-          for (int c = 0; c < NBT; ++c)
-            if (c < bc.nbh) p += st.I[c];
-          a.pp[q] = p;
-        }
+        const int cp = (int)(it / (unsigned long long)a.P), chunk = cp / parts;
+        const int64_t q = (int64_t)(it - (unsigned long long)cp * a.P);
+        batch_trace<NBT, AMR, FMT, DIR>(a, smem_raw, a.geoms[a.pview[q]], a.plvl[q], a.ppi[q], a.ppj[q], chunk,
+                                        cp - chunk * parts, parts, a.chunks * parts == 1, o, q);
+      }
+    }
+    // (the band sums of rays dealt to parts of one chunk: those of several
+    // chunks are formed where the pixels take their values)
+    if (a.chunks == 1 && parts > 1) {
+      if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
+      for (int64_t k = gtid; k < a.P; k += gstride) {
+        float s = 0.f;
+        for (int q = 0; q < nb; ++q) s += a.pI[(int64_t)q * a.P + k];
+        a.pp[k] = s;
       }
     }
     if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
@@ -207,21 +282,24 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
   for (;; ++sweep) {
     // step ii: trace the rays added last sweep, all views and band chunks
     const int64_t cnt_r = n - first;
-    const unsigned long long items = (unsigned long long)cnt_r * (unsigned long long)a.chunks;
+    const int parts = NBT == 0 ? wide_parts(cnt_r * a.chunks, min(a.width, nb), a.fill) : 1;
+    const int shares = a.chunks * parts;
+    const unsigned long long items = (unsigned long long)cnt_r * (unsigned long long)shares;
+    const BatchOut o{t.N, t.I, t.p, t.steps, a.mode == 1 ? a.maxlev : nullptr, t.cap};
+    const int rpw = rays_per_warp(cnt_r, shares, (int64_t)nblk * (kBatchBlock / 32));
     for (;;) {
       unsigned long long b = 0;
-      if (lane == 0) b = atomicAdd(&a.ctl->q_head, 32ull);
+      if (lane == 0) b = atomicAdd(&a.ctl->q_head, (unsigned long long)rpw);
       b = __shfl_sync(0xffffffffu, b, 0);
       if (b >= items) break;
-      const unsigned long long it = b + lane;
+      const unsigned long long it = lane < rpw ? b + lane : items;
       bool todo = it < items;
-      int chunk = 0, v = 0, b0 = 0;
+      int cp = 0, v = 0;
       int64_t k = 0;
       if (todo) {
-        chunk = (int)(it / (unsigned long long)cnt_r);
-        k = first + (int64_t)(it - (unsigned long long)chunk * cnt_r);
+        cp = (int)(it / (unsigned long long)cnt_r);
+        k = first + (int64_t)(it - (unsigned long long)cp * cnt_r);
         v = a.view[k];
-        b0 = chunk * NBT;
       }
       if (todo && a.mode == 2) {
         // the pixel's values from its view's proposal wave when the wave
@@ -230,46 +308,27 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
         const int64_t pb = (int64_t)v * nn0 + (int64_t)(j >> L) * n0 + (i >> L);
         const int64_t q = prop_index(a.pdepth + 4 * pb, a.poff[pb], L, i, j);
         if (q >= 0) {
-          if (chunk == 0) {
+          if (cp == 0) {
             t.N[k] = a.pN[q];
             t.steps[k] = a.psteps[q];
           }
-          const int nbh = min(NBT, nb - b0);
-          for (int c = 0; c < nbh; ++c) t.I[(int64_t)(b0 + c) * t.cap + k] = a.pI[(int64_t)(b0 + c) * a.P + q];
-          if (a.chunks == 1) t.p[k] = a.pp[q];
+          const int b0 = (int)((int64_t)nb * cp / shares), b1 = (int)((int64_t)nb * (cp + 1) / shares);
+          for (int c = b0; c < b1; ++c) t.I[(int64_t)c * t.cap + k] = a.pI[(int64_t)c * a.P + q];
+          if (a.chunks == 1 && cp == 0) t.p[k] = a.pp[q];
           todo = false;
-        } else if (chunk == 0) {
+        } else if (cp == 0) {
           atomicAdd(&a.ctl->fb_rays, 1ull);
         }
       }
       if (todo) {
-        const BandCtx bc = chunk_ctx<NBT, FMT>(smem_raw + chunk * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g,
-                                               min(NBT, nb - b0));
-        BandRegs<NBT> br;
-        band_regs<NBT>(br, bc);
-        const RayGeom &rg = a.geoms[v];
-        RTState<NBT> st;
-        trace_ray<NBT, AMR, FMT, DIR>(st, g, rg, t.lvl[k], t.pi[k], t.pj[k], a.fp64_level, bc, br);
-        if (chunk == 0) {
-          t.N[k] = st.N;
-          t.steps[k] = st.steps;
-          if (a.mode == 1) a.maxlev[k] = (uint8_t)st.maxlev;
-        }
-#pragma unroll
-        for (int q = 0; q < NBT; ++q)
-          if (q < bc.nbh) t.I[(int64_t)(b0 + q) * t.cap + k] = st.I[q];
-        if (a.chunks == 1) {
-          float p = 0.f;
-#pragma unroll
-          for (int q = 0; q < NBT; ++q)
-            if (q < bc.nbh) p += st.I[q];
-          t.p[k] = p;
-        }
+        const int chunk = cp / parts;
+        batch_trace<NBT, AMR, FMT, DIR>(a, smem_raw, a.geoms[v], t.lvl[k], t.pi[k], t.pj[k], chunk,
+                                        cp - chunk * parts, parts, shares == 1, o, k);
       }
     }
     if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->q_head = 0ull;  // next sweep's queue
-    if (a.chunks > 1) {
+    if (shares > 1) {
       for (int64_t k = first + gtid; k < n; k += gstride) {
         float s = 0.f;
         for (int q = 0; q < nb; ++q) s += t.I[(int64_t)q * t.cap + k];
@@ -379,12 +438,13 @@ static void batch_pick(bool amr, BatchOccFn *occ, BatchLaunchFn *launch) {
 }
 
 // Occupancy and launch functions and shared memory of the kernel for a grid
-// and V views (inclined: all of them are) with NBT bands per thread; false
-// where there is no such form.
+// and V views (inclined: all of them are) with NBT bands per thread (0: the
+// wide form, `width` bands per chunk); false where there is no such form.
 template <int NBT>
-bool batch_fns(const GridView &g, int V, bool inclined, BatchOccFn *occ, BatchLaunchFn *launch, size_t *smem) {
+bool batch_fns(const GridView &g, int V, bool inclined, int width, BatchOccFn *occ, BatchLaunchFn *launch,
+               size_t *smem) {
   const bool amr = g.kind == AIR_GRID_AMR;
-  *smem = batch_smem<NBT>(g, V);
+  *smem = batch_smem<NBT>(g, V, width);
   if (g.cell_fmt == kCellLam) {
     // per-cell Lambda exists for one-band grids only
     if constexpr (NBT == 1) {
@@ -394,13 +454,16 @@ bool batch_fns(const GridView &g, int V, bool inclined, BatchOccFn *occ, BatchLa
     }
     return false;
   }
-  if (g.cell_fmt == kCellXq) {
-    if (inclined) batch_pick<NBT, kCellXq, -2>(amr, occ, launch);
-    else batch_pick<NBT, kCellXq, 0>(amr, occ, launch);
-  } else {
-    if (inclined) batch_pick<NBT, kCellRho, -2>(amr, occ, launch);
-    else batch_pick<NBT, kCellRho, 0>(amr, occ, launch);
-  }
+  // inclined views with more than 8 bands per thread take the wide form
+  constexpr int DIR = NBT == 0 ? -2 : 0;
+  if constexpr (NBT >= 1 && NBT <= 8)
+    if (inclined) {
+      if (g.cell_fmt == kCellXq) batch_pick<NBT, kCellXq, -2>(amr, occ, launch);
+      else batch_pick<NBT, kCellRho, -2>(amr, occ, launch);
+      return true;
+    }
+  if (g.cell_fmt == kCellXq) batch_pick<NBT, kCellXq, DIR>(amr, occ, launch);
+  else batch_pick<NBT, kCellRho, DIR>(amr, occ, launch);
   return true;
 }
 

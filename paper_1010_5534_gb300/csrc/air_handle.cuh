@@ -99,6 +99,8 @@ struct BatchArgs {
   GridView g;
   const RayGeom *geoms;  // [V]
   int V, chunks, fp64_level, xi_norm, refine_on, stall;
+  int width;             // the wide march: bands of a chunk, and the threads that a
+  int64_t fill;          // chunk's parts should fill (wide_parts)
   double xi_crit;
   TreeView t;
   int16_t *view;
@@ -224,7 +226,7 @@ air_status load_grid_impl(const air_grid_desc *d, air_grid *g);
 // Profiling: open a launch group of `phase` containing `nlaunch` kernels; close
 // it after the launches; resolve all groups after the render's final sync.
 cudaError_t prof_open(air_grid *g, int phase, int nlaunch);
-cudaError_t prof_close(air_grid *g);
+cudaError_t prof_close(air_grid *g, int nlaunch = 0);  // nlaunch more than prof_open counted
 cudaError_t prof_resolve(air_grid *g);
 void free_grid_impl(air_grid *g);
 void free_batch(air_grid *g);
@@ -281,7 +283,7 @@ struct SweepEnd {
 // (known before the last sweep's rays are traced: the stream is not waited for).
 air_status sweep_loop_device(air_grid *g, const Camera &cam, const air_params *pr, int64_t nbase,
                              int64_t m, int64_t bound, int64_t open_max, const MarchTune &tune,
-                             int march_launches, int32_t *lmap, const Proposal *prop,
+                             int32_t *lmap, const Proposal *prop,
                              SweepEnd *fin);
 // The march configuration of this handle's tuning.
 MarchTune march_tune(const air_grid *g, int fp64_level);

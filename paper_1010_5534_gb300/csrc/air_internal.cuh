@@ -150,6 +150,7 @@ struct RaySource {
   const int8_t *lvl;
   const int32_t *pi, *pj;
   int64_t first, count; // rays [first, first + count) of the list / image (modes 0, 1)
+  int base;             // mode 0: lvl, pi, pj begin with the n0 x n0 base image, row by row
   int tile_w;           // grid mode: a warp covers tile_w x (32 / tile_w) pixels
   const int32_t *list;  // nodes mode: if set, ray r is node list[r] (first ignored)
   SweepState *sweep;    // mode 2: the new nodes of sweep q, from its slot's n to the next
@@ -157,6 +158,9 @@ struct RaySource {
                         // from the slot's ray_ctr[band chunk]
   int part;             // mode 2, a sweep launched in two forms: 1 traces only counts up to
   int64_t few;          // `few` rays, 2 only larger ones; 0: any
+  int rpw;              // modes 0, 1: rays per warp (rays_per_warp)
+  int width;            // the wide march: bands of a chunk (even), and the threads that its
+  int64_t fill;         // parts should fill (wide_parts)
   int use_prop;         // mode 2: copy a new pixel's values from `prop` when the
   Proposal prop;        // proposal traced it; trace only the pixels it missed
   // column table of an axis view (RayGeom::tab, levels of the n0 image), or NULL
@@ -223,8 +227,9 @@ inline int64_t axis_table_slot(int n0, int lmax) {
 // nothing launched) when the view does not qualify.
 cudaError_t launch_axis_table(const GridView &g, const Camera &cam, int n0, int lmax,
                               int32_t *tab, int *byj, int64_t *slot, bool *ok, cudaStream_t st);
+// *launches: kernels launched (forms, and the band sums).
 cudaError_t launch_march(const GridView &g, const Camera &cam, const RaySource &src,
-                         const RayOut &out, const MarchTune &tune, cudaStream_t st);
+                         const RayOut &out, const MarchTune &tune, cudaStream_t st, int *launches);
 // Bands one thread carries when the tuning leaves it open (launch_march).
 inline int default_bands_per_thread(int n_bands) { return n_bands <= 8 ? n_bands : 8; }
 cudaError_t launch_band_sum(const float *I, int n_bands, int64_t stride, int64_t first,

@@ -324,16 +324,17 @@ static air_status base_and_features(air_grid *g, const Camera &cam, const air_pa
   CU_TRY(ensure((void **)&lw.xi_n, &lw.xi_n_b, sizeof(float) * nbase));
   CU_TRY(launch_init_base(t, st));
   RaySource src{};
-  src.mode = 0; src.n0 = n0; src.lvl = t.lvl; src.pi = t.pi; src.pj = t.pj; src.first = 0; src.count = nbase;
+  src.mode = 0; src.base = 1; src.n0 = n0; src.lvl = t.lvl; src.pi = t.pi; src.pj = t.pj; src.first = 0; src.count = nbase;
   {
     const air_status sa = axis_table(g, cam, n0, pr->max_level, src);
     if (sa) return sa;
   }
   RayOut ro{t.N, t.I, t.cap, t.steps, t.p, lw.tau0, lw.maxlev};
   const MarchTune tune = march_tune(g, pr->fp64_level);
-  CU_TRY(prof_open(g, AIR_PHASE_MARCH, g->gv.n_bands > (tune.nbt > 0 ? tune.nbt : default_bands_per_thread(g->gv.n_bands)) ? 2 : 1));
-  CU_TRY(launch_march(g->gv, cam, src, ro, tune, st));
-  CU_TRY(prof_close(g));
+  int nl = 0;
+  CU_TRY(prof_open(g, AIR_PHASE_MARCH, 0));
+  CU_TRY(launch_march(g->gv, cam, src, ro, tune, st, &nl));
+  CU_TRY(prof_close(g, nl));
   CU_TRY(prof_open(g, AIR_PHASE_LEARN, 2));
   k_base_xi<<<nblk(nbase, 256), 256, 0, st>>>(t.p, t.N, n0, lw.xi_p, lw.xi_n);
   k_features<<<nblk(4 * nbase, 256), 256, 0, st>>>(t.p, t.N, lw.tau0, lw.maxlev, lw.xi_p, lw.xi_n, n0,
@@ -502,16 +503,16 @@ air_status render_learned(air_grid *g, const air_view *view, const air_params *p
   CU_TRY(cudaGetLastError());
   CU_TRY(prof_close(g));
   const MarchTune tune = march_tune(g, pr->fp64_level);
-  const int march_launches = nb > (tune.nbt > 0 ? tune.nbt : default_bands_per_thread(nb)) ? 2 : 1;
   if (P > 0) {
     // the proposal wave: every pixel of every proposed subtree
     RaySource ps{};
     ps.mode = 0; ps.n0 = n0; ps.lvl = lw.plvl; ps.pi = lw.ppi; ps.pj = lw.ppj; ps.first = 0; ps.count = P;
     if ((s = axis_table(g, cam, n0, Lm, ps))) return s;
     RayOut po{lw.pN, lw.pI, std::max<int64_t>(P, 1), lw.psteps, lw.pp};
-    CU_TRY(prof_open(g, AIR_PHASE_MARCH, march_launches));
-    CU_TRY(launch_march(g->gv, cam, ps, po, tune, st));
-    CU_TRY(prof_close(g));
+    int nl = 0;
+    CU_TRY(prof_open(g, AIR_PHASE_MARCH, 0));
+    CU_TRY(launch_march(g->gv, cam, ps, po, tune, st, &nl));
+    CU_TRY(prof_close(g, nl));
     ++waves;
   }
   // plain AIR over the traced values (steps iii-v)
@@ -536,7 +537,7 @@ air_status render_learned(air_grid *g, const air_view *view, const air_params *p
     g->last.lmap = lmap;
     const Proposal prop{lw.depth, lw.off, lw.pN, lw.pI, lw.pp, lw.psteps, std::max<int64_t>(P, 1)};
     SweepEnd fin;
-    if ((s = sweep_loop_device(g, cam, pr, nbase, mo, bound, open_max, tune, march_launches, lmap, &prop,
+    if ((s = sweep_loop_device(g, cam, pr, nbase, mo, bound, open_max, tune, lmap, &prop,
                                &fin)))
       return s;
     n = fin.n;
@@ -593,9 +594,10 @@ air_status render_learned(air_grid *g, const air_view *view, const air_params *p
       fs.mode = 0; fs.n0 = n0; fs.lvl = t.lvl; fs.pi = t.pi; fs.pj = t.pj; fs.count = miss; fs.list = lw.list;
       if ((s = axis_table(g, cam, n0, Lm, fs))) return s;
       RayOut fo{t.N, t.I, t.cap, t.steps, t.p};
-      CU_TRY(prof_open(g, AIR_PHASE_MARCH, march_launches));
-      CU_TRY(launch_march(g->gv, cam, fs, fo, tune, st));
-      CU_TRY(prof_close(g));
+      int nl = 0;
+      CU_TRY(prof_open(g, AIR_PHASE_MARCH, 0));
+      CU_TRY(launch_march(g->gv, cam, fs, fo, tune, st, &nl));
+      CU_TRY(prof_close(g, nl));
       fallback += miss;
       ++waves;
     }

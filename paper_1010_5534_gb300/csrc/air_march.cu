@@ -34,10 +34,9 @@ __global__ void k_band_sum_dev(const float *__restrict__ I, int n_bands, int64_t
 }
 
 // Rays whose threads (one per band chunk) fill the GPU twice in the form for
-// few rays, or in the ordinary one of that width.
-static int64_t few_rays(int NBT, bool lone, int chunks) {
-  const int blocks = lone ? (NBT <= 4 ? MinBlocks<4, -1>::value : MinBlocks<8, -1>::value)
-                          : (NBT <= 1 ? kAxisBlocksSmall : (NBT <= 2 ? MinBlocks<2, -3>::value : MinBlocks<4, -3>::value));
+// few rays.
+static int64_t few_rays(int NBT, int chunks) {
+  const int blocks = NBT <= 4 ? MinBlocks<4, -1>::value : MinBlocks<8, -1>::value;
   return (int64_t)sm_count() * blocks * kMarchBlock * 2 / chunks;
 }
 
@@ -51,10 +50,23 @@ extern template cudaError_t march_axis_one<0>(const MarchLaunch &);
 extern template cudaError_t march_axis_one<1>(const MarchLaunch &);
 extern template cudaError_t march_axis_one<2>(const MarchLaunch &);
 
-// The march kernel with NBT bands per thread.
-static cudaError_t launch_nbt(int NBT, bool few, const GridView &g, const RayGeom &rg,
+// Threads that the parts of a wide launch should fill (wide_parts): twice those
+// resident at once (32-band clumps: 8.27 ms; filled once 9.15, four times 8.62).
+static int64_t wide_fill_threads() { return (int64_t)sm_count() * kWideBlocks * kMarchBlock * 2; }
+
+// Inclined rays with more than 8 bands per thread go to the wide form. (Bands in
+// registers up to 8: the 8-band cone, 1500^2 fixed, 1.09 ms, 1.17 in the wide
+// form; 5 hot bands 300 us, 318. With 32 bands the wide form's one walk wins over
+// four: clumps 11.8 -> 7.9 ms, and 8 views x 16 bands 16.4 -> 13.2.)
+static bool is_wide(int nbt, int moving) { return moving > 1 && nbt > 8; }
+
+// The march kernel with NBT bands per thread (the wide form: per chunk, any
+// even number, and `fill` threads to fill).
+static cudaError_t launch_nbt(int NBT, bool few, int64_t fill, const GridView &g, const RayGeom &rg,
                               const RaySource &src, const RayOut &out, const MarchTune &tune,
                               cudaStream_t st) {
+  const int moving = (rg.Dhi[0] != 0.f) + (rg.Dhi[1] != 0.f) + (rg.Dhi[2] != 0.f);
+  const bool wide = is_wide(NBT, moving) && !few;
   const int chunks = (g.n_bands + NBT - 1) / NBT;
   int64_t threads;
   if (src.mode == 0) {
@@ -67,10 +79,20 @@ static cudaError_t launch_nbt(int NBT, bool few, const GridView &g, const RayGeo
     threads = 1;  // the count is on the device; the grid is sized per form
   }
   if (threads <= 0) return cudaSuccess;
-  const int64_t blocks = (threads + kMarchBlock - 1) / kMarchBlock;
+  const int64_t warps = (int64_t)sm_count() * (kMarchBlock / 32) *
+                        (wide ? kWideBlocks : (few ? (NBT <= 4 ? MinBlocks<4, -1>::value : MinBlocks<8, -1>::value) : 4));
+  RaySource rs = src;
+  rs.width = NBT;
+  rs.fill = fill;
+  rs.rpw = moving == 1 ? 32 : rays_per_warp(threads, chunks * (wide ? wide_parts(threads, std::min(NBT, g.n_bands), fill) : 1), warps);
+  const int64_t per_block = kMarchBlock / 32 * rs.rpw;
+  const int64_t blocks = (threads + per_block - 1) / per_block;
   if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-  const int moving = (rg.Dhi[0] != 0.f) + (rg.Dhi[1] != 0.f) + (rg.Dhi[2] != 0.f);
-  const MarchLaunch m{g, rg, src, out, blocks, chunks, tune.fp64_level, st, few};
+  const MarchLaunch m{g, rg, rs, out, blocks, chunks, tune.fp64_level, st, few};
+  if (wide) {
+    const cudaError_t e = march_wide(m, threads);
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
   cudaError_t le;
   if (NBT == 1 && moving == 1) {
     le = rg.Dhi[0] != 0.f ? march_axis_one<0>(m) : (rg.Dhi[1] != 0.f ? march_axis_one<1>(m) : march_axis_one<2>(m));
@@ -87,41 +109,54 @@ static cudaError_t launch_nbt(int NBT, bool few, const GridView &g, const RayGeo
 // The kernel's width for a number of bands per thread.
 static int width_of(int nbt) { return nbt <= 1 ? 1 : (nbt <= 2 ? 2 : (nbt <= 4 ? 4 : (nbt <= 8 ? 8 : 16))); }
 
-cudaError_t launch_march(const GridView &g, const Camera &cam, const RaySource &src,
-                         const RayOut &out, const MarchTune &tune, cudaStream_t st) {
-  // default: every band in one thread up to 8 bands, chunks of 8 above
-  // (32-band adaptive / fixed images of the large grid, one view: 4 bands
-  // 1315 / 1365 ms, 8 bands 1251 / 1328 ms, 16 bands 1512 / 1653 ms)
-  const int want = tune.nbt > 0 ? tune.nbt : default_bands_per_thread(g.n_bands);
-  const int nbt = g.cell_fmt == kCellLam ? 1 : width_of(want);  // per-cell Lambda: one band
-  RayGeom rg = make_geom(g, cam, src.n0);
-  rg.tab = src.axtab;
-  rg.tab_slot = src.axtab_slot;
-  rg.tab_byj = src.axtab_byj;
+cudaError_t launch_march(const GridView &g, const Camera &cam, const RaySource &rays,
+                         const RayOut &out, const MarchTune &tune, cudaStream_t st, int *launches) {
+  *launches = 0;
+  // default: every band in one thread up to 8 bands; above, chunks of 8 for rays
+  // along an axis, and the wide form for inclined ones
+  int nbt = g.cell_fmt == kCellLam ? 1 : width_of(tune.nbt > 0 ? tune.nbt : default_bands_per_thread(g.n_bands));
+  RayGeom rg = make_geom(g, cam, rays.n0);
+  rg.tab = rays.axtab;
+  rg.tab_slot = rays.axtab_slot;
+  rg.tab_byj = rays.axtab_byj;
   const int moving = (rg.Dhi[0] != 0.f) + (rg.Dhi[1] != 0.f) + (rg.Dhi[2] != 0.f);
-  const int chunks = (g.n_bands + nbt - 1) / nbt;
-  if (src.mode == 0 && src.count <= 0) return cudaSuccess;
+  if (rays.mode == 0 && rays.count <= 0) return cudaSuccess;
+  RaySource src = rays;
+  if (moving > 1 && src.mode == 0 && src.base && src.first == 0 && src.count == (int64_t)src.n0 * src.n0) {
+    // a base image in node order is the fixed image of its resolution: a warp
+    // takes 8 x 4 pixels, whose rays stay closer than those of 32 in a row
+    src.mode = 1;
+    src.tile_w = 8;
+  }
 
-  // A launch that leaves most of the GPU idle takes as long as its longest ray,
-  // and a ray's time is that of one warp working alone, so its bands are spread
-  // over more threads (unless the caller has set the bands per thread), and
-  // inclined rays take the form DIR = -1. `few`: the rays that fill that form's
-  // threads twice. Where the count is on the device, both launches are queued
-  // and the one that it is not for returns.
-  // Rays along an axis keep the chunks of large launches: their series
-  // (column_group) is chosen by the largest opacity of the chunk, so another
-  // width gives other last bits.
-  const int narrow = tune.nbt > 0 || moving == 1 ? nbt : std::min(nbt, g.n_bands <= 8 ? 1 : (g.n_bands <= 16 ? 2 : 4));
+  // A launch of few inclined rays takes as long as its longest ray, and a ray's
+  // time is that of one warp working alone, so its bands are spread over more
+  // threads, at most four each (unless the caller has set the bands per thread),
+  // and it takes the form DIR = -1. `few`: the rays that fill that form's threads
+  // twice. Where the count is on the device, both launches are queued and the one
+  // that it is not for returns. (Inclined cone, 101^2 base, 4 bands, 30 sweeps,
+  // the march: 3.40 ms; with one band per thread 3.75, two 3.71.) Rays along an
+  // axis keep the chunks of large launches: their series (column_group) is chosen
+  // by the largest opacity of the chunk, so another width gives other last bits.
+  const int narrow = tune.nbt > 0 || moving == 1 ? nbt : std::min(nbt, 4);
   const int nchunks = (g.n_bands + narrow - 1) / narrow;
+  if (tune.nbt <= 0 && g.n_bands > 8 && moving > 1) nbt = 16;  // inclined: the wide form
+  const bool wide = is_wide(nbt, moving);
   const bool lone = moving > 1 && narrow <= 8;  // there is a form for few rays
-  const int64_t few = lone || narrow < nbt ? few_rays(narrow, lone, nchunks) : 0;
+  const int64_t few = lone ? few_rays(narrow, nchunks) : 0;
+  if (wide && tune.nbt <= 0) nbt = wide_width(g, kMarchBlock);
+  const int64_t fill = wide && tune.nbt <= 0 ? wide_fill_threads() : 0;
+  const int chunks = (g.n_bands + nbt - 1) / nbt;
   const int64_t total = src.mode == 0 ? src.count : (src.mode == 1 ? (int64_t)src.n0 * src.n0 : 0);
   cudaError_t e;
   if (src.mode != 2) {
     const bool is_few = total <= few;
-    e = launch_nbt(is_few ? narrow : nbt, is_few && lone, g, rg, src, out, tune, st);
-    if (e != cudaSuccess || !out.p || (is_few ? nchunks : chunks) == 1) return e;
+    *launches = 1;
+    e = launch_nbt(is_few ? narrow : nbt, is_few && lone, fill, g, rg, src, out, tune, st);
+    if (e != cudaSuccess || !out.p) return e;
+    if (is_few ? nchunks == 1 : chunks == 1 && (!wide || wide_parts(total, g.n_bands, fill) == 1)) return e;
     const int64_t first = src.mode == 0 ? src.first : 0;
+    *launches = 2;
     if (src.list) {
       k_band_sum<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(out.I, g.n_bands, out.stride, 0, total,
                                                                   src.list, out.p, out.ioff);
@@ -133,17 +168,22 @@ cudaError_t launch_march(const GridView &g, const Camera &cam, const RaySource &
   s2.few = few;
   if (few > 0) {
     s2.part = 1;
-    e = launch_nbt(narrow, lone, g, rg, s2, out, tune, st);
+    e = launch_nbt(narrow, lone, fill, g, rg, s2, out, tune, st);
     if (e != cudaSuccess) return e;
+    *launches = 1;
     s2.part = 2;
   }
-  e = launch_nbt(nbt, false, g, rg, s2, out, tune, st);
+  e = launch_nbt(nbt, false, fill, g, rg, s2, out, tune, st);
+  ++*launches;
   if (e != cudaSuccess || !out.p) return e;
-  const int64_t most = chunks > 1 ? INT64_MAX : (few > 0 && nchunks > 1 ? few : 0);
-  if (most > 0)
+  int64_t most = chunks > 1 ? INT64_MAX : (few > 0 && nchunks > 1 ? few : 0);
+  if (wide && g.n_bands > 2) most = std::max(most, fill / 2);  // dealt to parts up to there
+  if (most > 0) {
+    ++*launches;
     return launch_pdl(k_band_sum_dev, dim3((unsigned)(sm_count() * 8)), dim3(256), 0, st,
                       (const float *)out.I, g.n_bands, out.stride, (const SweepState *)src.sweep, src.q, most,
                       out.p);
+  }
   return cudaSuccess;
 }
 

@@ -50,6 +50,16 @@ struct RTState {
   float tN, tp;
 };
 
+// NBT = 0, the wide form of inclined rays: any number of bands per thread (up
+// to kWideBands), their sums in shared memory (WideCtx).
+template <>
+struct RTState<0> {
+  float N, cN;
+  uint32_t steps;
+  int maxlev;
+  bool due;  // cells that emit nothing since the last one that emits
+};
+
 // Emission table of a band chunk in shared memory (kCellXq): per table bin
 // the pairs {Lambda_b, next bin's Lambda_b - Lambda_b} of the chunk's NBT bands
 // side by side, so a cell's look-up is one 16-byte load per two bands and one
@@ -92,6 +102,103 @@ struct BandCtx {
   int nbh;
 };
 
+// The wide form (RTState<0>). A band's T is 2^(nk N) at every point of the ray,
+// so its only state is its compensated sum, two words, and only a cell that
+// emits needs them. They lie in shared memory, one float4 {I, c, I, c} per pair
+// of bands and thread: a thread's registers do not grow with its bands, so one
+// walk through the cells serves up to 32 bands, where 8 bands in registers took
+// 124 of them and a walk for every 8 bands. A chunk of cells with an emitting
+// one (wide_chunk) goes through the bands pair by pair: constants and sums are
+// read once, and every cell of the chunk is added to them.
+constexpr int kWideBands = 32;
+struct WideCtx {
+  const float *tab;       // the first pair's table entries (kCellXq), rows of `row` floats
+  const BandConst *band;  // the first band's constants
+  float4 *sums;           // [pairs][blockDim.x], this thread's column
+  int row, pairs;
+  int nbh;                // bands; an odd one's partner has zero opacity and table
+};
+// Floats per table bin: 4 modulo 8, so that rows of neighbouring bins start in
+// different banks.
+__host__ __device__ constexpr int wide_row(int width) { return (2 * width + 7) / 8 * 8 + 4; }
+// Table and constants of `width` (even) bands, and the sums of a block.
+__host__ __device__ constexpr size_t wide_tab_bytes(bool table, int n_tbins, int width) {
+  return (table ? sizeof(float) * (size_t)wide_row(width) * n_tbins : 0) + sizeof(BandConst) * width;
+}
+__host__ __device__ constexpr size_t wide_sum_bytes(int width, int threads) {
+  return sizeof(float4) * (size_t)(width / 2) * threads;
+}
+// Fill table and constants of bands [b0, b0 + width) at `sm` by one block (zero
+// beyond n_bands).
+template <int FMT>
+__device__ __forceinline__ void wide_fill(unsigned char *sm, const GridView &g, int b0, int width) {
+  BandConst *band = reinterpret_cast<BandConst *>(sm);
+  for (int b = threadIdx.x; b < width; b += blockDim.x)
+    band[b] = b0 + b < g.n_bands ? g.bands[b0 + b] : BandConst{0.f, 0.f, -0.f, 0xffffffffu};
+  if (FMT == kCellXq) {
+    float *tab = reinterpret_cast<float *>(band + width);
+    const int ts = g.n_tbins + 1, row = wide_row(width);
+    for (int k = threadIdx.x >> 5; k < g.n_tbins; k += blockDim.x >> 5)
+      for (int b = threadIdx.x & 31; b < width; b += 32) {
+        float v = 0.f, d = 0.f;
+        if (b0 + b < g.n_bands) {
+          v = g.table[(b0 + b) * ts + k];
+          d = g.table[(b0 + b) * ts + k + 1] - v;
+        }
+        *reinterpret_cast<float2 *>(tab + k * row + 2 * b) = make_float2(v, d);
+      }
+  }
+}
+// Part `part` of `parts` of the chunk at `sm` (nb of its `width` bands exist);
+// *first: its first band within the chunk. parts <= the chunk's pairs.
+template <int FMT>
+__device__ __forceinline__ WideCtx wide_ctx(unsigned char *sm, float4 *sums, int width, int nb, int part,
+                                            int parts, int *first) {
+  const int pairs = (nb + 1) / 2, per = (pairs + parts - 1) / parts;
+  const int q0 = min(part * per, pairs);
+  WideCtx c;
+  c.band = reinterpret_cast<const BandConst *>(sm) + 2 * q0;
+  c.tab = reinterpret_cast<const float *>(sm + sizeof(BandConst) * width) + 4 * q0;
+  c.sums = sums + threadIdx.x;
+  c.row = wide_row(width);
+  c.pairs = min(per, pairs - q0);
+  c.nbh = min(2 * c.pairs, nb - 2 * q0);
+  *first = 2 * q0;
+  return c;
+}
+// Parts that a chunk's bands are dealt to for `rays` rays, so that the rays'
+// parts are at least about `fill` threads: a walk of its own for each part, but
+// a launch that leaves the GPU idle takes as long as its longest ray.
+__host__ __device__ __forceinline__ int wide_parts(int64_t rays, int nb, int64_t fill) {
+  int parts = 1;
+  while (2 * parts <= (nb + 1) / 2 && 2 * parts * rays <= fill) parts *= 2;
+  return parts;
+}
+
+// Bands of a chunk of the wide form: all of them, or as equal parts as let the
+// shared memory of four blocks fit an SM (and kWideBands).
+static inline int wide_width(const GridView &g, int threads) {
+  int chunks = (g.n_bands + kWideBands - 1) / kWideBands;
+  for (;; ++chunks) {
+    const int width = ((g.n_bands + chunks - 1) / chunks + 1) & ~1;
+    const size_t b = wide_tab_bytes(g.cell_fmt == kCellXq, g.n_tbins, width) + wide_sum_bytes(width, threads);
+    if (b <= 54 * 1024 || width <= 8) return width;
+  }
+}
+
+// Rays that a warp takes at a time, of `rays` inclined rays in `chunks` chunks
+// or parts, for `warps` warps at work at once. The lanes of a warp meet brick
+// faces and emitting cells at different steps, so a warp of 32 rays issues a
+// multiple of one ray's instructions (of 32 lanes 7 to 14 are active); a launch
+// of few rays spreads them over the idle warps. (The march of the inclined cone
+// above 3.65 -> 3.40 ms, 8 views x 16 bands 12.34 -> 11.92. Rays along an axis
+// share their steps and their cache lines: 126 -> 158 us, so they stay together.)
+__host__ __device__ __forceinline__ int rays_per_warp(int64_t rays, int chunks, int64_t warps) {
+  int rpw = 32;
+  while (rpw > 1 && rays * chunks <= warps * (rpw / 2)) rpw >>= 1;
+  return rpw;
+}
+
 // Fill a chunk's shared memory at `sm` by one block.
 template <int NBT, int FMT>
 __device__ __forceinline__ void chunk_fill(unsigned char *sm, const GridView &g, int b0) {
@@ -120,6 +227,11 @@ struct BandRegs {
   float nk[NBT];   // -kappa_b log2(e): T_b = 2^(nk_b N)
   float kmax;      // largest kappa_b of the chunk
   uint32_t xz;     // table coordinates below xz emit nothing in any band (kCellXq)
+};
+
+template <>
+struct BandRegs<0> {
+  uint32_t xz;
 };
 
 template <int NBT>
@@ -164,6 +276,16 @@ __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// The wide form's start: sums of zero.
+__device__ __forceinline__ void wide_init(RTState<0> &r, const WideCtx &wc) {
+  r.N = 0.f;
+  r.cN = 0.f;
+  r.steps = 0;
+  r.maxlev = 0;
+  r.due = false;
+  for (int q = 0; q < wc.pairs; ++q) wc.sums[q * blockDim.x] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 template <int NBT>
@@ -285,6 +407,71 @@ __device__ __forceinline__ void rt_dark_to(RTState<NBT> &r, float N, const BandR
   }
 }
 
+// The band terms of a chunk of K cells in the wide form (cell u lies on the ray
+// where in[u]): the operations of rt_bands and rt_dark in their order, for one
+// pair of bands after the other. N0: the column density before the chunk.
+template <int FMT, int K>
+__device__ __forceinline__ void wide_chunk(RTState<0> &r, const bool (&in)[K], const float (&rh)[K],
+                                           const uint32_t (&xv)[K], const float (&rds)[K],
+                                           const float (&N)[K], float N0, const WideCtx &wc, uint32_t xz) {
+  uint32_t emits = 0u, zero = 0u;  // cells that emit; those with dark cells before them
+#pragma unroll
+  for (int u = 0; u < K; ++u)
+    if (in[u]) {
+      if (cell_dark<FMT>(xv[u], xz) && N[u] <= FLT_MAX) {
+        r.due = true;
+      } else {
+        emits |= 1u << u;
+        if (r.due) zero |= 1u << u;
+        r.due = false;
+      }
+    }
+  if (!emits) return;
+  const bool start = N0 == 0.f;  // T = 1, whatever the opacity
+  int row[K];
+  float w[K];
+#pragma unroll
+  for (int u = 0; u < K; ++u) {
+    row[u] = FMT == kCellXq ? (int)(xv[u] >> kXqFracBits) * wc.row : 0;
+    w[u] = FMT == kCellXq ? (float)(xv[u] & ((1u << kXqFracBits) - 1u)) * (1.0f / (float)(1u << kXqFracBits)) : 0.f;
+  }
+#pragma unroll 1
+  for (int q = 0; q < wc.pairs; ++q) {
+    const float4 ca = *reinterpret_cast<const float4 *>(wc.band + 2 * q);
+    const float4 cb = *reinterpret_cast<const float4 *>(wc.band + 2 * q + 1);
+    float4 s = wc.sums[q * blockDim.x];
+    float T0 = start ? 1.f : ex2_approx(ca.z * N0);
+    float T1 = start ? 1.f : ex2_approx(cb.z * N0);
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+      const float Tn0 = ex2_approx(ca.z * N[u]);
+      const float Tn1 = ex2_approx(cb.z * N[u]);
+      if (emits >> u & 1u) {
+        if (zero >> u & 1u) {
+          kahan_add(s.x, s.y, 0.f);
+          kahan_add(s.z, s.w, 0.f);
+        }
+        float rl0 = rh[u], rl1 = rh[u];  // rho Lambda_b
+        if (FMT == kCellXq) {
+          const float4 t = *reinterpret_cast<const float4 *>(wc.tab + row[u] + 4 * q);
+          rl0 *= fmaf(w[u], t.y, t.x);
+          rl1 *= fmaf(w[u], t.w, t.z);
+        }
+        const float d0 = ca.x * rds[u], d1 = cb.x * rds[u];  // dtau
+        const float small0 = __fmul_rn(rl0 * rds[u], T0 * one_minus_exp_over_x(d0));
+        const float small1 = __fmul_rn(rl1 * rds[u], T1 * one_minus_exp_over_x(d1));
+        const float large0 = __fmul_rn(rl0 * ca.y, T0 - Tn0);
+        const float large1 = __fmul_rn(rl1 * cb.y, T1 - Tn1);
+        kahan_add(s.x, s.y, d0 < 0.25f ? small0 : large0);
+        kahan_add(s.z, s.w, d1 < 0.25f ? small1 : large1);
+      }
+      T0 = Tn0;
+      T1 = Tn1;
+    }
+    wc.sums[q * blockDim.x] = s;
+  }
+}
+
 // DARK = false: without the test (for callers that have made it).
 template <int NBT, int FMT, bool DARK = true>
 __device__ __forceinline__ void rt_term(RTState<NBT> &r, float rho, uint32_t aux, float ds,
@@ -299,9 +486,10 @@ __device__ __forceinline__ void rt_term(RTState<NBT> &r, float rho, uint32_t aux
 // them (march_block). DIR = -1, the form for launches that leave most of the
 // GPU's threads idle, goes further ahead: there a ray's time is its number of
 // chunks times the L2's latency (800 cycles), and registers are free.
+constexpr int kWideAhead = 4;  // (8: batched 16 bands 13.5 -> 14.4 ms)
 template <int NBT, int DIR>
 struct DdaChunk {
-  static constexpr int value = DIR != -1 ? 4 : (NBT <= 2 ? 16 : 8);
+  static constexpr int value = NBT == 0 ? kWideAhead : DIR != -1 ? 4 : (NBT <= 2 ? 16 : 8);
 };
 
 // Fields of cell idx: rho and the auxiliary word of the format.
@@ -570,11 +758,11 @@ struct ColumnUnroll {
 // for each record as its index is known, and only then sums the chunk. One
 // load latency is paid per chunk instead of one per cell, and the step's own
 // dependent operations overlap the loads.
-template <int NBT, int FMT, int K, typename Idx>
+template <int NBT, int FMT, int K, typename Idx, class Ctx>
 __device__ __forceinline__ void march_block(RTState<NBT> &r, const float Q[3], const float Dl[3],
                                             const float inv[3], float tend, int lx, int ly, int lz,
                                             int nx, int ny, int nz, Idx sy, Idx sz,
-                                            const void *__restrict__ cells, const BandCtx &bc,
+                                            const void *__restrict__ cells, const Ctx &bc,
                                             const BandRegs<NBT> &br) {
   const float INF = FLT_MAX;
   const bool p0 = Dl[0] > 0.f, p1 = Dl[1] > 0.f, p2 = Dl[2] > 0.f;
@@ -625,9 +813,11 @@ __device__ __forceinline__ void march_block(RTState<NBT> &r, const float Q[3], c
     // zero-length chord (a ray grazing an edge or corner) adds nothing and is
     // not counted as a step.
     float N[K];
+    const float N0 = r.N;
     uint32_t x = 0u;
 #pragma unroll
-    for (int u = 0; u < K; ++u)
+    for (int u = 0; u < K; ++u) {
+      N[u] = r.N;
       if (in[u]) {
         r.steps += ds[u] > 0.f ? 1u : 0u;
         ds[u] = __fmul_rn(rh[u], ds[u]);  // rho ds from here on
@@ -635,7 +825,11 @@ __device__ __forceinline__ void march_block(RTState<NBT> &r, const float Q[3], c
         N[u] = r.N;
         x = FMT == kCellLam ? x | xv[u] : max(x, xv[u]);
       }
-    if (cell_dark<FMT>(x, br.xz) && r.N <= FLT_MAX) {
+    }
+    if constexpr (NBT == 0) {
+      if (cell_dark<FMT>(x, br.xz) && r.N <= FLT_MAX) r.due = true;
+      else wide_chunk<FMT, K>(r, in, rh, xv, ds, N, N0, bc, br.xz);
+    } else if (cell_dark<FMT>(x, br.xz) && r.N <= FLT_MAX) {
       rt_dark_to<NBT>(r, r.N, br);
     } else {
 #pragma unroll
@@ -896,9 +1090,9 @@ __device__ __forceinline__ int axis_table_entry(const GridView &g, const RayGeom
   return (o >= 0.0 && o < (double)g.nf[a]) ? (int)o : -1;
 }
 
-template <int NBT, int FMT, int K>
+template <int NBT, int FMT, int K, class Ctx>
 __device__ void march_uniform(RTState<NBT> &r, const GridView &g, const double O[3],
-                              const RayGeom &rg, double t0, const BandCtx &bc,
+                              const RayGeom &rg, double t0, const Ctx &bc,
                               const BandRegs<NBT> &br) {
   float Q[3], Dl[3], inv[3];
   int lc[3];
@@ -981,10 +1175,10 @@ __device__ __forceinline__ int brick_of(const GridView &g, int e, const int c[3]
 // is marched, so its latency overlaps the march. Per-launch constants
 // (direction, its inverse and its double-float split) are read from the
 // kernel-parameter bank, not held per thread.
-template <int NBT, int FMT, int K>
+template <int NBT, int FMT, int K, class Ctx>
 __device__ void march_amr(RTState<NBT> &r, const GridView &g, const double O[3], const F2 Of[3],
                           const RayGeom &rg, double t0, int eax, int fp64_level,
-                          const BandCtx &bc, const BandRegs<NBT> &br) {
+                          const Ctx &bc, const BandRegs<NBT> &br) {
   const int B = g.B, lb = g.log2B, Lm = g.Lm;
   int c[3];
 #pragma unroll
@@ -1369,6 +1563,30 @@ __device__ __forceinline__ void trace_ray(RTState<NBT> &st, const GridView &g, c
     if (AMR) march_amr<NBT, FMT, K>(st, g, O, Of, rg, t0, eax, fp64_level, bc, br);
     else march_uniform<NBT, FMT, K>(st, g, O, rg, t0, bc, br);
   }
+}
+
+// An inclined ray in the wide form; its sums are left in wc.sums.
+template <bool AMR, int FMT>
+__device__ __forceinline__ void trace_wide(RTState<0> &st, const GridView &g, const RayGeom &rg, int L,
+                                           int i, int j, int fp64_level, const WideCtx &wc) {
+  wide_init(st, wc);
+  BandRegs<0> br;
+  br.xz = 0xffffffffu;
+  for (int b = 0; b < wc.nbh; ++b) br.xz = min(br.xz, wc.band[b].xz);
+  double O[3], t0;
+  F2 Of[3];
+  int eax;
+  if (!ray_setup(g, rg, L, i, j, O, Of, t0, eax)) return;
+  constexpr int K = DdaChunk<0, -2>::value;
+  if (AMR) march_amr<0, FMT, K>(st, g, O, Of, rg, t0, eax, fp64_level, wc, br);
+  else march_uniform<0, FMT, K>(st, g, O, rg, t0, wc, br);
+  if (st.due)  // the last cells were dark
+    for (int q = 0; q < wc.pairs; ++q) {
+      float4 s = wc.sums[q * blockDim.x];
+      kahan_add(s.x, s.y, 0.f);
+      kahan_add(s.z, s.w, 0.f);
+      wc.sums[q * blockDim.x] = s;
+    }
 }
 
 // World camera -> per-launch ray geometry (FP64, host).

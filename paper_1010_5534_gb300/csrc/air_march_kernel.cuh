@@ -3,6 +3,8 @@
 // of its own (air_march_<width>.cu, air_march_axis.cu), in parallel: one unit
 // with every form took 150 s of a build, the slowest of these takes a quarter.
 #pragma once
+#include <algorithm>
+
 #include "air_march.cuh"
 #include "air_refine.cuh"
 
@@ -14,7 +16,7 @@ struct MarchLaunch {
   const RayGeom &rg;
   const RaySource &src;
   const RayOut &out;
-  int64_t blocks;  // of kMarchBlock rays; with the count on the device, unused
+  int64_t blocks;  // of kMarchBlock / 32 warps, src.rpw rays each; with the count on the device, unused
   int chunks;      // band chunks
   int fp64_level;
   cudaStream_t st;
@@ -108,24 +110,28 @@ __global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
   band_regs<NBT>(br, bc);
 
   if (src.mode == 2) {
-    // new nodes of a sweep counted on the device: block b takes chunk b of
-    // blockDim.x rays, and more from a work counter until the rays run out
+    // new nodes of a sweep counted on the device: warp w of the grid takes rays
+    // [rpw w, + rpw), and more from a work counter until the rays run out
     SweepSlot &s0 = src.sweep->slot[src.q & 3];
     const int64_t first = s0.n, count = src.sweep->slot[(src.q + 1) & 3].n - first;
     if ((src.part == 1 && count > src.few) || (src.part == 2 && count <= src.few)) return;
-    __shared__ long long s_chunk;
-    for (int64_t r0 = (int64_t)blockIdx.x * blockDim.x; r0 < count; r0 = s_chunk * blockDim.x) {
-      const int64_t r = r0 + threadIdx.x;
-      if (r < count) march_one<NBT, AMR, FMT, DIR>(g, rg, src, out, fp64_level, bc, br, chunk, b0,
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (kMarchBlock / 32);
+    const int rpw = DIR == -1 || DIR == -2 ? rays_per_warp(count, gridDim.y, warps) : 32;
+    for (int64_t w = (int64_t)blockIdx.x * (kMarchBlock / 32) + (threadIdx.x >> 5); rpw * w < count;) {
+      const int64_t r = rpw * w + lane;
+      if (lane < rpw && r < count) march_one<NBT, AMR, FMT, DIR>(g, rg, src, out, fp64_level, bc, br, chunk, b0,
                                                    nbh, first + r);
-      if (count <= (int64_t)gridDim.x * blockDim.x) return;
-      __syncthreads();
-      if (threadIdx.x == 0) s_chunk = gridDim.x + (long long)atomicAdd(&s0.ray_ctr[chunk], 1ull);
-      __syncthreads();
+      if (count <= rpw * warps) return;
+      __syncwarp();
+      long long next = 0;
+      if (lane == 0) next = (long long)atomicAdd(&s0.ray_ctr[chunk], 1ull);
+      w = warps + __shfl_sync(0xffffffffu, next, 0);
     }
     return;
   }
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if ((int)(threadIdx.x & 31) >= src.rpw) return;
+  const int64_t r = ((int64_t)blockIdx.x * (kMarchBlock / 32) + (threadIdx.x >> 5)) * src.rpw + (threadIdx.x & 31);
   int L, i, j;
   int64_t k;
   if (src.mode == 0) {
@@ -169,6 +175,137 @@ __global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
   }
 }
 
+// The wide form: bands [blockIdx.y width, + width) in wide_parts() parts. A
+// warp takes rpw rays of a part at a time (a block of four warps at a time waited
+// for its slowest ray: 32-band clumps 8.9 ms, 7.7 by warps).
+// Resident blocks per SM (8 views x 16 bands, batched: 6 blocks 14.95 ms, 5 14.73,
+// 4 13.51, 3 14.01; 32-band clumps: 12.8, 12.2, 9.3, 9.2: the sums of more blocks
+// leave too little L1 for the cells).
+constexpr int kWideBlocks = 4;
+
+template <bool AMR, int FMT>
+__device__ __forceinline__ void wide_one(const GridView &g, const RayGeom &rg, const RaySource &src,
+                                         const RayOut &out, int fp64_level, const WideCtx &wc, int b0,
+                                         bool all, int L, int i, int j, int64_t k) {
+  if (src.use_prop) {  // as in march_one
+    const Proposal &pr = src.prop;
+    const int64_t b = (int64_t)(j >> L) * src.n0 + (i >> L);
+    const int64_t q = prop_index(pr.depth + 4 * b, pr.off[b], L, i, j);
+    if (q >= 0) {
+      if (b0 == 0) {
+        out.N[k] = pr.N[q];
+        out.steps[k] = pr.steps[q];
+      }
+      for (int c = 0; c < wc.nbh; ++c)
+        out.I[(int64_t)(b0 + c) * out.stride + k] = pr.I[(int64_t)(b0 + c) * pr.stride + q];
+      if (out.p && all) out.p[k] = pr.p[q];
+      return;
+    }
+    if (b0 == 0) {
+      if (atomicAdd(&src.sweep->slot[src.q & 3].missed, 1ull) == 0ull) atomicAdd(&src.sweep->fb_waves, 1);
+      atomicAdd(&src.sweep->fb_total, 1ull);
+    }
+  }
+  RTState<0> st;
+  trace_wide<AMR, FMT>(st, g, rg, L, i, j, fp64_level, wc);
+  if (b0 == 0) {
+    out.N[k] = st.N;
+    out.steps[k] = st.steps;
+    if (out.tau0) out.tau0[k] = wc.band[0].kap * st.N;
+    if (out.maxlev) out.maxlev[k] = (uint8_t)st.maxlev;
+  }
+  float p = 0.f;
+  for (int q = 0; q < wc.pairs; ++q) {
+    const float4 s = wc.sums[q * blockDim.x];
+    float *I = out.I + (int64_t)(b0 + 2 * q) * out.stride + (k - out.ioff);
+    I[0] = s.x;
+    p += s.x;
+    if (2 * q + 1 < wc.nbh) {
+      I[out.stride] = s.z;
+      p += s.z;
+    }
+  }
+  if (out.p && all) out.p[k] = p;
+}
+
+template <bool AMR, int FMT>
+__global__ void __launch_bounds__(kMarchBlock, kWideBlocks)
+    k_march_wide(GridView g, RayGeom rg, RaySource src, RayOut out, int fp64_level) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int c0 = blockIdx.y * src.width, nb = min(src.width, g.n_bands - c0);
+  wide_fill<FMT>(smem, g, c0, src.width);
+  float4 *sums = reinterpret_cast<float4 *>(smem + wide_tab_bytes(FMT == kCellXq, g.n_tbins, src.width));
+  wait_prior_grid();
+  __syncthreads();
+  int64_t first = src.first, count = src.count;
+  if (src.mode == 2) {
+    first = src.sweep->slot[src.q & 3].n;
+    count = src.sweep->slot[(src.q + 1) & 3].n - first;
+    if ((src.part == 1 && count > src.few) || (src.part == 2 && count <= src.few)) return;
+  }
+  const int tw = src.tile_w, th = src.mode == 1 ? 32 / tw : 1;
+  const uint32_t tiles_x = src.mode == 1 ? (uint32_t)(src.n0 + tw - 1) / (uint32_t)tw : 1u;
+  if (src.mode == 1) count = 32 * (int64_t)tiles_x * ((src.n0 + th - 1) / th);
+  const int parts = wide_parts(count, nb, src.fill);
+  // items of rpw rays and one part; a warp takes its first by its place in the
+  // grid and, where the count is on the device, more from the work counter
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (kMarchBlock / 32);
+  const int rpw = src.mode == 2 ? rays_per_warp(count, gridDim.y * parts, warps) : src.rpw;
+  const int64_t rounds = (count + rpw - 1) / rpw, items = rounds * parts;
+  for (int64_t it = (int64_t)blockIdx.x * (kMarchBlock / 32) + (threadIdx.x >> 5); it < items;) {
+    const int part = parts == 1 ? 0 : (int)(it / rounds);
+    const int64_t r = (it - part * rounds) * rpw + lane;
+    int b0;
+    const WideCtx wc = wide_ctx<FMT>(smem, sums, src.width, nb, part, parts, &b0);
+    bool mine = lane < rpw && r < count && wc.pairs > 0;
+    int64_t k = first + r;
+    int L = 0, i = 0, j = 0;
+    if (src.mode == 1) {
+      // (32-bit division as in k_march)
+      const uint32_t tile = (uint32_t)(r >> 5), x = (uint32_t)(r & 31), ty = tile / tiles_x;
+      i = (int)((tile - ty * tiles_x) * tw + x % (uint32_t)tw);
+      j = (int)(ty * th + x / (uint32_t)tw);
+      mine = mine && i < src.n0 && j < src.n0;
+      k = (int64_t)j * src.n0 + i;
+    } else if (mine) {
+      if (src.mode == 0 && src.list) k = (int64_t)src.list[r];
+      L = src.lvl[k];
+      i = src.pi[k];
+      j = src.pj[k];
+    }
+    if (mine) wide_one<AMR, FMT>(g, rg, src, out, fp64_level, wc, c0 + b0, gridDim.y == 1 && parts == 1, L, i, j, k);
+    if (items <= warps) return;
+    __syncwarp();
+    long long next = 0;
+    if (lane == 0) next = (long long)atomicAdd(&src.sweep->slot[src.q & 3].ray_ctr[blockIdx.y], 1ull);
+    it = warps + __shfl_sync(0xffffffffu, next, 0);
+  }
+}
+
+template <bool AMR, int FMT>
+static cudaError_t march_wide_form(const MarchLaunch &m, int64_t rays) {
+  const int width = m.src.width;
+  const size_t smem = wide_tab_bytes(FMT == kCellXq, m.g.n_tbins, width) + wide_sum_bytes(width, kMarchBlock);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_march_wide<AMR, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t blocks = m.src.mode == 2 ? (int64_t)sm_count() * kWideBlocks
+                                         : m.blocks * wide_parts(rays, std::min(width, m.g.n_bands), m.src.fill);
+  if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+  return launch_pdl(k_march_wide<AMR, FMT>, dim3((unsigned)blocks, m.chunks), dim3(kMarchBlock), smem, m.st, m.g,
+                    m.rg, m.src, m.out, m.fp64_level);
+}
+
+// Inclined rays in the wide form (m.src.width, m.src.fill set); `rays`: the
+// launch's threads per band chunk where the host knows them.
+static inline cudaError_t march_wide(const MarchLaunch &m, int64_t rays) {
+  const bool amr = m.g.kind == AIR_GRID_AMR;
+  if (m.g.cell_fmt == kCellRho) return amr ? march_wide_form<true, kCellRho>(m, rays) : march_wide_form<false, kCellRho>(m, rays);
+  return amr ? march_wide_form<true, kCellXq>(m, rays) : march_wide_form<false, kCellXq>(m, rays);
+}
+
 // The launch grid of form DIR: blocks over the rays, or, with the count on
 // the device, one wave of the form's resident blocks taking work from the
 // counter.
@@ -189,10 +326,9 @@ static cudaError_t march_any(const MarchLaunch &m) {
   const int moving = (m.rg.Dhi[0] != 0.f) + (m.rg.Dhi[1] != 0.f) + (m.rg.Dhi[2] != 0.f);
   if constexpr (NBT > 1)  // (one band: march_axis_one)
     if (moving == 1) return march_form<NBT, AMR, FMT, -3>(m);
-  // 16 bands per thread leave no registers for the form for few rays
-  if constexpr (NBT <= 8)
-    if (m.few) return march_form<NBT, AMR, FMT, -1>(m);
-  return march_form<NBT, AMR, FMT, -2>(m);
+  // (inclined rays with more bands per thread: march_wide)
+  if constexpr (NBT <= 8) return m.few ? march_form<NBT, AMR, FMT, -1>(m) : march_form<NBT, AMR, FMT, -2>(m);
+  return cudaErrorInvalidValue;
 }
 
 // Rays in any direction, NBT bands per thread.
