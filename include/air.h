@@ -132,8 +132,9 @@ typedef struct {
   int32_t tile_w;                 /* fixed images: a warp traces tile_w x (32 / tile_w)
                                      pixels (1, 2, 4, 8, 16, 32; default 8) */
   int32_t bands_per_thread;       /* single-view renders: bands one thread carries
-                                     along a ray (1, 2, 4, 8, 16; default: all of them up to 8 bands, else 8) */
-  int32_t batch_bands_per_thread; /* batched renders (default 8 for more than 4 bands) */
+                                     along a ray (1, 2, 4, 8, 16; default: all of them up to 8 bands,
+                                     else 8, or all up to 32 where no ray runs along an axis) */
+  int32_t batch_bands_per_thread; /* batched renders (default: see air_batch_opts) */
   int32_t batch_blocks_per_sm;    /* persistent CTAs per SM of batched renders
                                      (default: as many as fit) */
   double best_ms[3];              /* out of air_autotune: fixed, adaptive, batched time */
@@ -167,7 +168,8 @@ AIR_API air_status air_render_adaptive(air_grid *g, const air_view *view, const 
  * NULL for the defaults. */
 typedef struct {
   int32_t bands_per_thread;   /* bands one thread carries along a ray: 1, 2, 4, 8 or 16;
-                                 0 = library default (8 for more than 4 bands) */
+                                 0 = library default (8 for more than 4 bands; for more than
+                                 8, all up to 32 where no view runs along an axis) */
   int32_t use_graph;          /* 1: launch through a CUDA graph captured on first use
                                  (re-captured when the configuration changes) */
   double wait_timeout_ms;     /* time limit of every device-side wait of the persistent

@@ -4,9 +4,9 @@
 //
 // Inside the kernel, per sweep:
 //   march   : a work queue of (ray, band chunk) items over the rays added in
-//             the previous sweep, all views mixed; warps fetch 32 items at a
-//             time with one atomic, so rays of uneven length, level, view and
-//             band balance across the whole GPU;
+//             the previous sweep, all views mixed; warps fetch up to 32 items
+//             (rays_per_warp) at a time with one atomic, so rays of uneven
+//             length, level, view and band balance across the whole GPU;
 //   band sum: p = sum_b I_b when the bands were split over several threads;
 //   scan    : Eq. 2 on every leaf below max_level (all views);
 //   balance : 2:1 closure within each view's tree;

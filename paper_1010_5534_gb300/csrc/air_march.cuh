@@ -3,8 +3,10 @@
 // column density N = sum rho ds and the emergent intensity of the absorbed
 // emission, front to back, I_b = sum_k (j_k/alpha_k)(1 - e^-dtau_k) e^-tau_<k.
 //
-// One thread marches one ray (x a chunk of bands). Warps hold 32 neighbouring
-// pixels, so their cell fetches fall in the same or adjacent cells.
+// One thread marches one ray with a chunk of bands: their sums in registers (up
+// to 8 bands, or 16 along an axis), or in shared memory (the wide form, up to 32
+// bands of an inclined ray). A warp takes up to 32 neighbouring pixels, so their
+// cell fetches fall in the same or adjacent cells.
 //
 // Traversal: the ray's position is kept as an integer finest-level cell
 // coordinate plus a ray parameter t (world length). Inside a block of cells
@@ -15,8 +17,8 @@
 // through the face with the smallest exit parameter and the next brick is the
 // one holding the finest cell across that face, so no cell is skipped or
 // visited twice. A ray along one grid axis crosses every brick whole, and its
-// walk (march_amr_axis) carries no ray parameter. Bricks at level >= fp64_level compute their entry point and
-// exit parameter in FP64. Coarser bricks compute the entry point in
+// walk (march_amr_axis) carries no ray parameter. Bricks at level >= fp64_level
+// compute their entry point and exit parameter in FP64. Coarser bricks compute the entry point in
 // double-float (pairs of FP32 with error-free sums and products), since FP64
 // issues at a small fraction of the FP32 rate on this GPU. Either way the
 // entry point is expressed relative to the entry cell, so FP32 rounding inside
@@ -504,14 +506,6 @@ __device__ __forceinline__ void load_cell(const void *__restrict__ cells, Idx id
     rho = __uint_as_float(c.x);
     aux = c.y;
   }
-}
-
-// Ask L1 for the record of cell idx (a hint: nothing is loaded into registers).
-template <int FMT, typename Idx>
-__device__ __forceinline__ void prefetch_cell(const void *__restrict__ cells, Idx idx) {
-  const void *p = FMT == kCellRho ? (const void *)((const float *)cells + idx)
-                                  : (const void *)((const uint2 *)cells + idx);
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
 // (1 - e^-x) / x for 0 <= x < 1/64 from its Taylor series truncated after
