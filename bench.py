@@ -526,7 +526,9 @@ LARGE = dict(workload="clumps-and-cones block-AMR grid: 512^3 base cells in 32^3
                        "xi_crit 0.5", seed=0, views=16, base_res=1024, max_level=3, xi_crit=0.5,
              fixed_res=8192)
 FP32_OPS_PER_BAND_STEP = 23  # per band and cell: dtau, exponent argument, Taylor (7), both
-                             # cell-term forms (7), select, Kahan sum (4), table lookup (2)
+                             # cell-term forms (7), select, Kahan sum (4), table lookup (2);
+                             # a cell that emits nothing takes none of them, so a
+                             # fraction formed with this count can pass 1
 
 
 def run_large(args):
