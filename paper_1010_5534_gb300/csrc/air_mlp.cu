@@ -140,8 +140,11 @@ constexpr size_t kSmTrain = kSmW + sizeof(uint32_t) * kTile * (kRowIn + 6 * kRow
 // block. Inference: blocks loop over tiles, so the weights are staged once per
 // block and not once per tile.
 //
-// Launched as a dependent of the optimiser step before it: a tile's features
-// are fetched before the wait, the weights after it.
+// A tile's features are fetched before the wait, the weights after it. So only
+// a launch that follows an optimiser step of the same call may be a dependent
+// one: that step has waited for everything before it, and does not write the
+// features. The first launch of a call follows whatever the caller queued,
+// which may be the kernel that writes them (mlp_partials).
 template <bool TRAIN>
 __global__ void __launch_bounds__(kThreads) k_mlp(MlpArgs a) {
   extern __shared__ __align__(16) uint32_t sm[];
@@ -490,8 +493,10 @@ air_status mlp_forward(air_mlp *m, const uint16_t *x, int64_t n, float *logits, 
 }
 
 // Per-block sums of the mean cross-entropy's gradient over x[0..n) and of the
-// loss into m->partial.
-static air_status mlp_partials(air_mlp *m, const uint16_t *x, const int32_t *y, int64_t n) {
+// loss into m->partial. after_step: the launch before this one on the stream
+// is this call's optimiser step (see k_mlp); else an ordinary launch, which
+// everything queued before it is complete for.
+static air_status mlp_partials(air_mlp *m, const uint16_t *x, const int32_t *y, int64_t n, bool after_step) {
   const int64_t blocks = (n + kTile - 1) / kTile;
   CU_TRY(ensure((void **)&m->partial, &m->partial_b, sizeof(float) * (size_t)blocks * (kNP + 1)));
   MlpArgs a{};
@@ -507,13 +512,18 @@ static air_status mlp_partials(air_mlp *m, const uint16_t *x, const int32_t *y, 
     CU_TRY(cudaFuncSetAttribute(k_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmTrain));
     attr = true;
   }
-  CU_TRY(launch_pdl(k_mlp<true>, dim3((unsigned)blocks), dim3(kThreads), kSmTrain, m->stream, a));
+  if (after_step) {
+    CU_TRY(launch_pdl(k_mlp<true>, dim3((unsigned)blocks), dim3(kThreads), kSmTrain, m->stream, a));
+  } else {
+    k_mlp<true><<<(unsigned)blocks, kThreads, kSmTrain, m->stream>>>(a);
+    CU_TRY(cudaGetLastError());
+  }
   return AIR_OK;
 }
 
 // The gradient itself into m->grad (device), the loss to m->d_loss.
 static air_status mlp_grad(air_mlp *m, const uint16_t *x, const int32_t *y, int64_t n) {
-  const air_status s = mlp_partials(m, x, y, n);
+  const air_status s = mlp_partials(m, x, y, n, false);
   if (s) return s;
   const int64_t blocks = (n + kTile - 1) / kTile;
   k_reduce_partials<<<(kNP + 1 + 255) / 256, 256, 0, m->stream>>>(m->partial, blocks, m->grad, m->d_loss);
@@ -521,10 +531,10 @@ static air_status mlp_grad(air_mlp *m, const uint16_t *x, const int32_t *y, int6
   return AIR_OK;
 }
 
-// One minibatch of training; its loss to *loss (device).
+// One minibatch of training (first: of the call); its loss to *loss (device).
 static air_status mlp_step(air_mlp *m, const uint16_t *x, const int32_t *y, int64_t n, float lr,
-                           double *loss) {
-  const air_status s = mlp_partials(m, x, y, n);
+                           double *loss, bool first) {
+  const air_status s = mlp_partials(m, x, y, n, !first);
   if (s) return s;
   m->step += 1;
   const float c1 = 1.0f - powf(0.9f, (float)m->step), c2 = 1.0f - powf(0.999f, (float)m->step);
@@ -646,7 +656,7 @@ air_status air_mlp_train(air_mlp *m, const uint16_t *x, const int32_t *y, int64_
     for (int64_t q = 0; q < nb; ++q) {
       const int64_t bi = (q * stride + (int64_t)e * 7) % nb;
       const int64_t s0 = bi * batch, cnt = std::min<int64_t>(batch, n - s0);
-      const air_status s = mlp_step(m, x + s0 * kIn, y + s0, cnt, lr, m->hist + q);
+      const air_status s = mlp_step(m, x + s0 * kIn, y + s0, cnt, lr, m->hist + q, e == 0 && q == 0);
       if (s) return s;
     }
     if (loss_history) {

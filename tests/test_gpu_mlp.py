@@ -93,3 +93,37 @@ def test_training_learns_a_separable_rule():
     pred = net.forward(_bits(Xq)).cpu().numpy().argmax(axis=1)
     assert (pred == y).mean() > 0.9
     net.close()
+
+
+@pytest.mark.parametrize("n", [300, 40000])
+def test_features_written_by_the_kernel_before(n):
+    """Features (and labels) that a kernel queued just before the call on the
+    same stream writes: the same bits as with features that were there long ago.
+    The kernels before it run long enough for the host to queue the call."""
+    th = scenes.mlp_init(7, scale=0.8)
+    Xq, y = _data(n + 3, n)
+    x, yd = _bits(Xq), torch.from_numpy(y.astype(np.int32)).cuda()
+    busy = torch.zeros(1 << 27, device="cuda")
+    got = []
+    for late in (False, True):
+        net = air.MLP(th)
+        for call in ("loss_grad", "train"):
+            a, b = x, yd
+            if late:
+                a, b = torch.full_like(x, 0x3f80), torch.zeros_like(yd)
+                torch.cuda.synchronize()
+                for _ in range(20):
+                    busy.add_(1.0)
+                a.copy_(x)  # device to device, in stream order
+                b.copy_(yd)
+                a.bitwise_not_().bitwise_not_()
+            if call == "train":
+                h = net.train(a, b, batch=128, epochs=2, lr=1e-3)
+                got.append((np.asarray(h), net.params()))
+            else:
+                loss, g = net.loss_grad(a, b)
+                got.append((np.asarray(loss), g.cpu().numpy()))
+        net.close()
+    for p, q in zip(got[:2], got[2:]):
+        for u, v in zip(p, q):
+            assert (u == v).all()
