@@ -22,7 +22,6 @@
 
 #include <cmath>
 #include <cstring>
-#include <vector>
 
 #include "air_handle.cuh"
 
@@ -651,7 +650,8 @@ air_status air_mlp_train(air_mlp *m, const uint16_t *x, const int32_t *y, int64_
   // the minibatches' losses stay on the device until the epoch ends, so the
   // host queues one minibatch behind the other without waiting
   CU_TRY(ensure((void **)&m->hist, &m->hist_b, sizeof(double) * (size_t)nb));
-  std::vector<double> losses;
+  constexpr int64_t kRead = 512;  // read back at a time: no allocation that could throw
+  double losses[kRead];
   for (int e = 0; e < epochs; ++e) {
     for (int64_t q = 0; q < nb; ++q) {
       const int64_t bi = (q * stride + (int64_t)e * 7) % nb;
@@ -660,12 +660,14 @@ air_status air_mlp_train(air_mlp *m, const uint16_t *x, const int32_t *y, int64_
       if (s) return s;
     }
     if (loss_history) {
-      losses.resize((size_t)nb);
-      CU_TRY(cudaMemcpyAsync(losses.data(), m->hist, sizeof(double) * (size_t)nb, cudaMemcpyDeviceToHost,
-                             m->stream));
-      CU_TRY(cudaStreamSynchronize(m->stream));
       double ep = 0.0;
-      for (const double l : losses) ep += l;
+      for (int64_t q0 = 0; q0 < nb; q0 += kRead) {
+        const int64_t c = std::min(kRead, nb - q0);
+        CU_TRY(cudaMemcpyAsync(losses, m->hist + q0, sizeof(double) * (size_t)c, cudaMemcpyDeviceToHost,
+                               m->stream));
+        CU_TRY(cudaStreamSynchronize(m->stream));
+        for (int64_t q = 0; q < c; ++q) ep += losses[q];
+      }
       loss_history[e] = ep / (double)n;
     }
   }

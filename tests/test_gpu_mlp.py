@@ -127,3 +127,18 @@ def test_features_written_by_the_kernel_before(n):
     for p, q in zip(got[:2], got[2:]):
         for u, v in zip(p, q):
             assert (u == v).all()
+
+
+@pytest.mark.parametrize("n", [511, 512, 513, 1100])
+def test_history_of_many_minibatches(n):
+    """One sample per minibatch: more losses than are read back at a time. With a
+    step that leaves the parameters as they are, an epoch's loss is the mean loss
+    of all samples (sums of FP32 terms, at most 128 of them in FP32)."""
+    th = scenes.mlp_init(8, scale=0.8)
+    Xq, y = _data(n, n)
+    x, yd = _bits(Xq), torch.from_numpy(y.astype(np.int32)).cuda()
+    net = air.MLP(th)
+    loss, _ = net.loss_grad(x, yd)
+    hist = net.train(x, yd, batch=1, epochs=2, lr=1e-14)
+    np.testing.assert_allclose(hist, loss, rtol=128 * 2.0 ** -23)
+    net.close()
