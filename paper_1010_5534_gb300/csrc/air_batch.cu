@@ -128,9 +128,9 @@ __global__ void __launch_bounds__(256) k_vemit(TreeView t, const int16_t *view, 
   block_emit_by_view(LeafPred{t.child, all}, view, e, s0, s1, V, run, wcnt);
 }
 
-// Band flux of every view. A block takes 2048 nodes and kFluxBands bands
-// (blockIdx.y). Nodes of a view lie together, so a warp's strip of 32 nodes
-// mostly belongs to one view: its lanes sum on (flux_add) until the view
+// Band flux of every view, every addition in FP64. A block takes 2048 nodes and
+// kFluxBands bands (blockIdx.y). Nodes of a view lie together, so a warp's strip
+// of 32 nodes mostly belongs to one view: its lanes sum on until the view
 // changes, and the block adds its warps' sums to the view's flux at the end.
 // (An FP64 atomic in shared memory per leaf and band, in the kernel above,
 // took most of the 2 ms that the output of 8 views x 16 bands cost.)
@@ -138,25 +138,15 @@ constexpr int kVfluxRounds = 8;
 __global__ void __launch_bounds__(256) k_vflux(TreeView t, const int16_t *view, int64_t n,
                                                int n_bands, const RayGeom *geoms, double *vflux) {
   __shared__ double sums[kFluxBands][8];
+  __shared__ double red[8][kFluxBands][32];
   __shared__ int views[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b0 = blockIdx.y * kFluxBands, nb = min(kFluxBands, n_bands - b0);
   const int64_t start = (int64_t)blockIdx.x * (256 * kVfluxRounds) + threadIdx.x;
-  float hi[kFluxBands], lo[kFluxBands];
-  double tiny[kFluxBands];
+  double acc[kFluxBands];
   int cur = -1;
 #pragma unroll
-  for (int q = 0; q < kFluxBands; ++q) {
-    hi[q] = lo[q] = 0.f;
-    tiny[q] = 0.0;
-  }
-  // the warp's sum of band q (to every lane), its accumulators emptied
-  auto take = [&](int q) {
-    const double s = flux_warp_sum(hi[q], lo[q], tiny[q]);
-    hi[q] = lo[q] = 0.f;
-    tiny[q] = 0.0;
-    return s;
-  };
+  for (int q = 0; q < kFluxBands; ++q) acc[q] = 0.0;
   auto area = [&](int v) { return geoms[v].pix0 * geoms[v].pix0; };
   for (int r = 0; r < kVfluxRounds; ++r) {
     const int64_t k = start + (int64_t)r * 256;
@@ -168,26 +158,31 @@ __global__ void __launch_bounds__(256) k_vflux(TreeView t, const int16_t *view, 
     if (v0 < 0) break;  // past the end
     if (__all_sync(0xffffffffu, v == v0 || !in)) {
       if (v0 != cur) {
-        if (cur >= 0)
-          for (int q = 0; q < kFluxBands; ++q) {
-            const double s = take(q);
-            if (lane == 0 && q < nb) atomicAdd(&vflux[(int64_t)cur * n_bands + b0 + q], s * area(cur));
-          }
+        if (cur >= 0) {
+          const double s = flux_warp_sum(acc, red[warp]);
+          if ((lane & 7) == 0 && (lane >> 3) < nb) atomicAdd(&vflux[(int64_t)cur * n_bands + b0 + (lane >> 3)], s * area(cur));
+#pragma unroll
+          for (int q = 0; q < kFluxBands; ++q) acc[q] = 0.0;
+        }
         cur = v0;
       }
 #pragma unroll
       for (int q = 0; q < kFluxBands; ++q)
-        if (leaf && q < nb) flux_add(t.I[(int64_t)(b0 + q) * t.cap + k], L, hi[q], lo[q], tiny[q]);
+        if (leaf && q < nb) {
+          const float I = t.I[(int64_t)(b0 + q) * t.cap + k];
+          // (an FP64 conversion costs as much as an addition: normal numbers
+          // are widened by integer operations)
+          const bool normal = fabsf(I) >= 0x1p-126f && fabsf(I) <= FLT_MAX;
+          acc[q] = fma(normal ? widen(I) : (double)I, pow4_neg(L), acc[q]);
+        }
     } else if (leaf) {
       for (int q = 0; q < nb; ++q)
         atomicAdd(&vflux[(int64_t)v * n_bands + b0 + q],
                   (double)t.I[(int64_t)(b0 + q) * t.cap + k] * pow4_neg(L) * area(v));
     }
   }
-  for (int q = 0; q < kFluxBands; ++q) {
-    const double s = take(q);
-    if (lane == 0) sums[q][warp] = s;
-  }
+  const double s4 = flux_warp_sum(acc, red[warp]);
+  if ((lane & 7) == 0) sums[lane >> 3][warp] = s4;
   if (lane == 0) views[warp] = cur;
   __syncthreads();
   if (threadIdx.x < nb) {

@@ -612,6 +612,7 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
   wait_prior_grid();
   __shared__ int32_t chunk_sum[kFluxChunks];
   __shared__ double sh[kFluxBands][8];
+  __shared__ double red[8][kFluxBands][32];
   __shared__ unsigned long long shs[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t start = (int64_t)blockIdx.x * kFluxPerBlock;
@@ -631,11 +632,11 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
     return;
   }
   float hi[kFluxBands], lo[kFluxBands];
-  double tiny[kFluxBands];
+  double rest[kFluxBands];
 #pragma unroll
   for (int q = 0; q < kFluxBands; ++q) {
     hi[q] = lo[q] = 0.f;
-    tiny[q] = 0.0;
+    rest[q] = 0.0;
   }
   // four entries per thread at a time, their loads issued together (a leaf's
   // intensity is not made to wait for its flag)
@@ -671,15 +672,13 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
       if (leaf[r]) {
 #pragma unroll
         for (int q = 0; q < kFluxBands; ++q)
-          if (b0 + q < a.n_bands) flux_add(I[r][q], L[r], hi[q], lo[q], tiny[q]);
+          if (b0 + q < a.n_bands) flux_add(I[r][q], L[r], hi[q], lo[q], rest[q]);
       }
   }
 #pragma unroll
-  for (int q = 0; q < kFluxBands; ++q) {
-    if (b0 + q >= a.n_bands) break;
-    const double s = flux_warp_sum(hi[q], lo[q], tiny[q]);
-    if (lane == 0) sh[q][warp] = s;
-  }
+  for (int q = 0; q < kFluxBands; ++q) rest[q] += (double)hi[q] + (double)lo[q];
+  const double s4 = flux_warp_sum(rest, red[warp]);
+  if ((lane & 7) == 0) sh[lane >> 3][warp] = s4;
   __syncthreads();
   if (count) {
     const int nc = (int)((end - start + kScanItems - 1) / kScanItems);

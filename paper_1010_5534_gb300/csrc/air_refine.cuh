@@ -143,38 +143,37 @@ __device__ __forceinline__ double pow4_neg(int L) {
 }
 
 // A thread's leaves are summed as an unevaluated pair of FP32 numbers
-// (Knuth's two-sum: hi + lo carries the sum to ~2^-44 relative) of I 4^-L, an
-// exact scaling while the product stays a normal number; the rare smaller
-// terms go to an FP64 sum. FP64 work per thread, not per leaf (FP64 issues at
-// 1/64 of the FP32 rate here).
-__device__ __forceinline__ void flux_add(float I, int L, float &hi, float &lo, double &tiny) {
+// (Knuth's two-sum: hi + lo carries the sum of 32 terms to 2^-38 relative or
+// better) of I 4^-L, an exact scaling while the product stays a normal number;
+// the rare smaller terms, and those so large that their sum could leave the
+// FP32 range, go to an FP64 sum. FP64 work per thread, not per leaf (FP64
+// issues at 1/64 of the FP32 rate here); between threads the sums are FP64.
+__device__ __forceinline__ void flux_add(float I, int L, float &hi, float &lo, double &rest) {
   const float x = __fmul_rn(I, __int_as_float((127 - 2 * L) << 23));
-  if (fabsf(x) >= 0x1p-126f || x == 0.f) {
+  const float m = fabsf(x);
+  if ((m >= 0x1p-126f && m <= 0x1p120f) || x == 0.f) {
     const float t = __fadd_rn(hi, x);
     const float bv = __fsub_rn(t, hi);
     lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bv)), __fsub_rn(x, bv)));
     hi = t;
   } else {
-    tiny = fma((double)I, pow4_neg(L), tiny);
+    rest = fma((double)I, pow4_neg(L), rest);
   }
 }
 
-// The warp's sum of such accumulators, in every lane: pairs are added as
-// pairs (two-sum again), and one FP64 value is formed at the end.
-__device__ __forceinline__ double flux_warp_sum(float hi, float lo, double tiny) {
-  for (int off = 16; off > 0; off >>= 1) {
-    const float h2 = __shfl_xor_sync(0xffffffffu, hi, off), l2 = __shfl_xor_sync(0xffffffffu, lo, off);
-    const float t = __fadd_rn(hi, h2);
-    const float bv = __fsub_rn(t, hi);
-    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bv)), __fsub_rn(h2, bv));
-    lo = __fadd_rn(__fadd_rn(lo, l2), e);
-    hi = t;
-  }
-  double s = (double)hi + (double)lo;
-  if (__any_sync(0xffffffffu, tiny != 0.0)) {
-    for (int off = 16; off > 0; off >>= 1) tiny += __shfl_xor_sync(0xffffffffu, tiny, off);
-    s += tiny;
-  }
+// The warp's FP64 sums of v[0 .. kFluxBands), through the warp's rows `red` of
+// shared memory: lane 8 q returns the sum of v[q]. Six FP64 additions per warp
+// for four bands (a butterfly over the lanes takes twenty).
+__device__ __forceinline__ double flux_warp_sum(const double (&v)[kFluxBands], double (*red)[32]) {
+  static_assert(kFluxBands == 4, "eight lanes per band");
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int q = 0; q < kFluxBands; ++q) red[q][lane] = v[q];
+  __syncwarp();
+  const double *r = red[lane >> 3] + (lane & 7);
+  double s = (r[0] + r[8]) + (r[16] + r[24]);
+  for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  __syncwarp();
   return s;
 }
 
