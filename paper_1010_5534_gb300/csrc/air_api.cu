@@ -726,13 +726,13 @@ air_status output_tree(air_grid *g, const Camera &cam, const air_params *pr, air
   fa.host = w.h_flux;
   if (!all) {  // (both arrays hold 3 entries per scan chunk of the whole pyramid)
     fa.chunk_leaves = w.bcount;
-    fa.block_leaves = (int32_t *)w.boff;
+    fa.block_leaves = (int32_t *)w.boff;  // and their prefix sums behind them
   }
   OutView o;
   if ((s = out_view(g, im, n_out, o))) return s;
-  CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, 3));
+  CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, emit_out_scans(all, n) ? 4 : 3));
   CU_TRY(launch_flux_partial(fa, st));
-  CU_TRY(launch_emit_out(t, o, all, n, fa.chunk_leaves, fa.block_leaves, st));
+  CU_TRY(launch_emit_out(t, o, all, n, fa.chunk_leaves, fa.block_leaves, w.boff + flux_blocks(n), w.d_total, st));
   CU_TRY(launch_flux_final(fa, st));
   CU_TRY(prof_close(g));
   s = finish_out(g, im, o, n_out);

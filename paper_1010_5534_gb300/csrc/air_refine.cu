@@ -509,12 +509,15 @@ __global__ void __launch_bounds__(kScanBlock)
 
 // The fields of every round's node are loaded before the ranks are formed,
 // so their latency overlaps the block's ballots and barriers. The leaves in
-// front of the block are added up from the counts of k_flux_partial: those of
-// the flux blocks before, and of the chunks before within its flux block. (A
-// counting and a scanning launch of their own took 25 us for 7.7 M nodes.)
+// front of the block are those of the flux blocks before it and of the chunks
+// before it within its flux block (counts of k_flux_partial). The former are
+// added up here, or, above kFluxDirect flux blocks, read from their prefix sums
+// block_off. (A counting and a scanning launch of their own took 25 us for 7.7 M
+// nodes; but every block adding up all the counts before it is quadratic work.)
 __global__ void __launch_bounds__(kScanBlock) k_emit_out(TreeView t, OutView o, int all, int64_t n,
                                                          const int32_t *__restrict__ chunk_leaves,
-                                                         const int32_t *__restrict__ block_leaves) {
+                                                         const int32_t *__restrict__ block_leaves,
+                                                         const int64_t *__restrict__ block_off) {
   wait_prior_grid();
   __shared__ int32_t wsum[kScanBlock / 32];
   __shared__ uint32_t fsum[kScanBlock / 32];
@@ -523,7 +526,10 @@ __global__ void __launch_bounds__(kScanBlock) k_emit_out(TreeView t, OutView o, 
   uint32_t front = 0;
   if (!all) {
     const int fb = blockIdx.x / kFluxChunks, c0 = fb * kFluxChunks;
-    for (int x = threadIdx.x; x < fb; x += kScanBlock) front += (uint32_t)block_leaves[x];
+    if (!block_off)
+      for (int x = threadIdx.x; x < fb; x += kScanBlock) front += (uint32_t)block_leaves[x];
+    else if (threadIdx.x == kScanBlock - 1)
+      front = (uint32_t)block_off[fb];  // (at most 2^31 nodes)
     if (c0 + (int)threadIdx.x < (int)blockIdx.x) front += (uint32_t)chunk_leaves[c0 + threadIdx.x];
     front = __reduce_add_sync(0xffffffffu, front);
     if (lane == 0) fsum[warp] = front;
@@ -806,12 +812,21 @@ cudaError_t launch_scan_offsets(const int32_t *bcount, int64_t nb, int64_t *boff
 }
 
 
+bool emit_out_scans(int all, int64_t n) { return !all && flux_blocks(n) > kFluxDirect; }
+
 cudaError_t launch_emit_out(const TreeView &t, const OutView &o, int all, int64_t n,
-                            const int32_t *chunk_leaves, const int32_t *block_leaves, cudaStream_t st) {
+                            const int32_t *chunk_leaves, const int32_t *block_leaves, int64_t *block_off,
+                            int64_t *total, cudaStream_t st) {
   const int64_t nb = scan_blocks(n);
   if (nb == 0) return cudaSuccess;
+  const bool scan = emit_out_scans(all, n);
+  if (scan) {
+    k_scan_blocks<<<1, 1024, 0, st>>>(block_leaves, flux_blocks(n), block_off, total);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   return launch_pdl(k_emit_out, dim3((unsigned)nb), dim3(kScanBlock), 0, st, t, o, all, n, chunk_leaves,
-                    block_leaves);
+                    block_leaves, (const int64_t *)(scan ? block_off : nullptr));
 }
 
 // Blocks of the device-count sweep kernels: a few per SM, looping over items.

@@ -64,6 +64,9 @@ struct FluxArgs {
 // of one band.)
 constexpr int64_t kFluxPerBlock = 8192;
 constexpr int kFluxChunks = kFluxPerBlock / kScanItems;
+// Flux blocks whose leaf counts every block of k_emit_out adds up for itself (up
+// to four loads per thread); above, one launch forms their prefix sums first.
+constexpr int64_t kFluxDirect = 1024;
 
 // Device-resident bookkeeping of the sweep loop when the counts stay on the
 // device (render_adaptive without a read-back per sweep). Sweep q starts from
@@ -181,9 +184,13 @@ cudaError_t launch_init_base(const TreeView &t, cudaStream_t st);
 int64_t scan_blocks(int64_t n);
 cudaError_t launch_count_flags(const uint32_t *flag, int64_t n, int32_t *bcount, int64_t *boff,
                                int64_t *total, cudaStream_t st);
-// chunk_leaves, block_leaves: from launch_flux_partial (unused with `all`).
+// chunk_leaves, block_leaves: from launch_flux_partial (unused with `all`);
+// block_off, total: room for the prefix sums of block_leaves and their sum, used
+// where emit_out_scans (a launch of its own).
+bool emit_out_scans(int all, int64_t n);
 cudaError_t launch_emit_out(const TreeView &t, const OutView &o, int all, int64_t n,
-                            const int32_t *chunk_leaves, const int32_t *block_leaves, cudaStream_t st);
+                            const int32_t *chunk_leaves, const int32_t *block_leaves, int64_t *block_off,
+                            int64_t *total, cudaStream_t st);
 // Exclusive scan of nb per-block counts (one block) -> boff, total.
 cudaError_t launch_scan_offsets(const int32_t *bcount, int64_t nb, int64_t *boff, int64_t *total,
                                 cudaStream_t st);
