@@ -8,8 +8,9 @@
 
 namespace air {
 
-// One thread per finest pixel (x, y) of an (n0 2^Lm)^2 raster (for base images
-// and trees without level maps; else k_raster_maps). The covering
+// One thread per finest pixel (x, y) of an (n0 2^Lm)^2 raster (for base images,
+// trees without level maps and rasters of fewer pixels than maps_pixels; else
+// k_raster_maps). The covering
 // leaf is the deepest node containing the pixel. For the bilinear form, with
 // s = Lm - L, the pixel centre on the level-L grid is
 // u = (x + 1/2) 2^-s - 1/2 = (2x + 1 - 2^s) / 2^(s+1): its floor is an
@@ -134,6 +135,15 @@ __global__ void __launch_bounds__(256) k_raster_maps(TreeView t, const int32_t *
   }
 }
 
+// Pixels from which k_raster_maps is the faster one. A raster of fewer pixels is
+// bound by the latency of one thread, which k_raster_maps makes longer, and by
+// the launch. Calls with k_raster and with k_raster_maps, us, one to nine levels:
+// 512^2 pixels 22 to 27 and 23 to 28; 1024^2 nearest 24.4 to 27.1 and 24.6 to
+// 29.4, bilinear 26.3 to 34.9 and 26.2 to 32.1; 1536^2 nearest 29.8 to 31.4 and
+// 29.3 to 33.1, bilinear 38.8 to 51.4 and 33.4 to 39.6; 2048^2 nearest 32.7 to
+// 36.2 and 27.3 to 32.5, bilinear 42.4 to 49.0 and 33.2 to 39.4.
+static int64_t maps_pixels(int mode) { return (int64_t)(mode == AIR_RASTER_NEAREST ? 3 : 2) << 20; }
+
 static bool is_device_ptr(const void *p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -174,7 +184,7 @@ air_status render_raster(air_grid *g, int32_t quantity, int32_t band, int32_t mo
   }
   const int64_t blocks = (n + 255) / 256;
   if (blocks > 0x7fffffff) return set_error(AIR_ERR_ARG, "raster too large");
-  if (Lm == 1 || (Lm > 1 && g->raster.lmap)) {
+  if (n >= maps_pixels(mode) && (Lm == 1 || (Lm > 1 && g->raster.lmap))) {
     const unsigned quads = (unsigned)((n / 4 + 255) / 256);
     if (((uintptr_t)dst & 7) == 0) k_raster_maps<true><<<quads, 256, 0, st>>>(t, g->raster.lmap, Lm, mode, val, dst);
     else k_raster_maps<false><<<quads, 256, 0, st>>>(t, g->raster.lmap, Lm, mode, val, dst);
