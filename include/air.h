@@ -133,7 +133,9 @@ typedef struct {
                                      pixels (1, 2, 4, 8, 16, 32; default 8) */
   int32_t bands_per_thread;       /* single-view renders: bands one thread carries
                                      along a ray (1, 2, 4, 8, 16; default: all of them up to 8 bands,
-                                     else 8, or all up to 32 where no ray runs along an axis) */
+                                     else 8, or all up to 32 where no ray runs along an axis; up to
+                                     8 bands a launch of few inclined rays carries at most 4, also
+                                     where the width that holds all bands is set) */
   int32_t batch_bands_per_thread; /* batched renders (default: see air_batch_opts) */
   int32_t batch_blocks_per_sm;    /* persistent CTAs per SM of batched renders
                                      (default: as many as fit) */

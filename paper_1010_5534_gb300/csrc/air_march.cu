@@ -131,14 +131,16 @@ cudaError_t launch_march(const GridView &g, const Camera &cam, const RaySource &
 
   // A launch of few inclined rays takes as long as its longest ray, and a ray's
   // time is that of one warp working alone, so its bands are spread over more
-  // threads, at most four each (unless the caller has set the bands per thread),
-  // and it takes the form DIR = -1. `few`: the rays that fill that form's threads
+  // threads, at most four each (unless the caller has set a width other than the
+  // default's: setting that one leaves the default as it is, so the autotuner's
+  // widths include it), and it takes the form DIR = -1. `few`: the rays that fill that form's threads
   // twice. Where the count is on the device, both launches are queued and the one
   // that it is not for returns. (Inclined cone, 101^2 base, 4 bands, 30 sweeps,
   // the march: 3.40 ms; with one band per thread 3.75, two 3.71.) Rays along an
   // axis keep the chunks of large launches: their series (column_group) is chosen
   // by the largest opacity of the chunk, so another width gives other last bits.
-  const int narrow = tune.nbt > 0 || moving == 1 ? nbt : std::min(nbt, 4);
+  const bool free_width = tune.nbt <= 0 || (g.n_bands <= 8 && nbt == width_of(g.n_bands));
+  const int narrow = !free_width || moving == 1 ? nbt : std::min(nbt, 4);
   const int nchunks = (g.n_bands + narrow - 1) / narrow;
   if (tune.nbt <= 0 && g.n_bands > 8 && moving > 1) nbt = 16;  // inclined: the wide form
   const bool wide = is_wide(nbt, moving);

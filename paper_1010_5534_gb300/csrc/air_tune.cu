@@ -81,7 +81,9 @@ air_status autotune(air_grid *g, const air_view *view, const air_params *pr, int
   // single-view adaptive image: bands per thread
   {
     double tbest = 1e300;
-    for (int bpt : {1, 2, 4, 8, 16, 0}) {  // 0: the default, another form above 8 bands
+    // 0: the default, a form of its own above 8 bands; up to 8 bands the last
+    // width tried, the one that holds them all, renders as the default does
+    for (int bpt : {1, 2, 4, 8, 16, 0}) {
       if (bpt > 1 && bpt / 2 >= nb) break;
       g->tune.bands_per_thread = bpt;
       air_image im{};
@@ -104,7 +106,7 @@ air_status autotune(air_grid *g, const air_view *view, const air_params *pr, int
     std::vector<air_view> vs(n_views, *view);
     std::vector<air_image> ims(n_views);
     double tbest = 1e300;
-    for (int bpt : {1, 2, 4, 8, 16, 0}) {  // 0: the default, another form above 8 bands
+    for (int bpt : {1, 2, 4, 8, 16, 0}) {  // (0 as above)
       if (bpt > 1 && bpt / 2 >= nb) break;
       for (int per : {0, 1, 2}) {
         g->tune.batch_bands_per_thread = bpt;
