@@ -205,21 +205,21 @@ __global__ void __launch_bounds__(256) k_vflux(TreeView t, const int16_t *view, 
   } while (0)
 
 // Compiled in air_batch_<NBT>.cu.
-extern template bool batch_fns<0>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *);
-extern template bool batch_fns<1>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *);
-extern template bool batch_fns<2>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *);
-extern template bool batch_fns<4>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *);
-extern template bool batch_fns<8>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *);
-extern template bool batch_fns<16>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *);
+extern template bool batch_fns<0>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *, int *);
+extern template bool batch_fns<1>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *, int *);
+extern template bool batch_fns<2>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *, int *);
+extern template bool batch_fns<4>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *, int *);
+extern template bool batch_fns<8>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *, int *);
+extern template bool batch_fns<16>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *, int *);
 
 static bool batch_form(int nbt, const GridView &g, int V, bool inclined, int width, BatchOccFn *occ,
-                       BatchLaunchFn *launch, size_t *smem) {
-  if (width) return batch_fns<0>(g, V, true, width, occ, launch, smem);
-  if (nbt == 1) return batch_fns<1>(g, V, inclined, width, occ, launch, smem);
-  if (nbt == 2) return batch_fns<2>(g, V, inclined, width, occ, launch, smem);
-  if (nbt == 4) return batch_fns<4>(g, V, inclined, width, occ, launch, smem);
-  if (nbt == 8) return batch_fns<8>(g, V, inclined, width, occ, launch, smem);
-  if (nbt == 16) return batch_fns<16>(g, V, inclined, width, occ, launch, smem);
+                       BatchLaunchFn *launch, size_t *smem, int *tabs) {
+  if (width) return batch_fns<0>(g, V, true, width, occ, launch, smem, tabs);
+  if (nbt == 1) return batch_fns<1>(g, V, inclined, width, occ, launch, smem, tabs);
+  if (nbt == 2) return batch_fns<2>(g, V, inclined, width, occ, launch, smem, tabs);
+  if (nbt == 4) return batch_fns<4>(g, V, inclined, width, occ, launch, smem, tabs);
+  if (nbt == 8) return batch_fns<8>(g, V, inclined, width, occ, launch, smem, tabs);
+  if (nbt == 16) return batch_fns<16>(g, V, inclined, width, occ, launch, smem, tabs);
   return false;
 }
 
@@ -291,12 +291,11 @@ air_status render_batch(air_grid *g, const air_view *views, int32_t V, const air
   BatchOccFn occ;
   BatchLaunchFn launch;
   size_t smem = 0;
+  int tabs = 0;
   // inclined views with more than 8 bands (per thread, where the caller has set
-  // that): the wide form, whose chunks hold as many bands as fit, unless its
-  // sums no longer fit beside the tables of every chunk
-  int width = !inclined ? 0 : (set ? (nbt == 16 ? 16 : 0) : (nb > 8 ? wide_width(g->gv, kBatchBlock) : 0));
-  if (width && batch_smem<0>(g->gv, V, width) > kBatchMaxSmem) width = 0;
-  if (!batch_form(nbt, g->gv, V, inclined, width, &occ, &launch, &smem))
+  // that): the wide form, whose chunks hold as many bands as fit
+  const int width = !inclined ? 0 : (set ? (nbt == 16 ? 16 : 0) : (nb > 8 ? wide_width(g->gv, kBatchBlock) : 0));
+  if (!batch_form(nbt, g->gv, V, inclined, width, &occ, &launch, &smem, &tabs))
     return set_error(AIR_ERR_ARG, "bands_per_thread must be 1, 2, 4, 8 or 16");
   g->last.valid = false;  // the batch reuses the single-view workspace
   air_status s = init_scalars(g->ws);
@@ -347,6 +346,7 @@ air_status render_batch(air_grid *g, const air_view *views, int32_t V, const air
     a.geoms = bw.geoms;
     a.V = V;
     a.width = width;
+    a.tabs = tabs;
     a.fill = width && !set ? (int64_t)grid * kBatchBlock * 2 : 0;
     a.chunks = width ? (nb + width - 1) / width : (nb + nbt - 1) / nbt;
     a.fp64_level = pr->fp64_level < 0 ? 3 : pr->fp64_level;

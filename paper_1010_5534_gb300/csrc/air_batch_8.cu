@@ -2,5 +2,5 @@
 #include "air_batch_kernel.cuh"
 
 namespace air {
-template bool batch_fns<8>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *);
+template bool batch_fns<8>(const GridView &, int, bool, int, BatchOccFn *, BatchLaunchFn *, size_t *, int *);
 }  // namespace air

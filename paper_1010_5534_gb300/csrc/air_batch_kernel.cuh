@@ -12,7 +12,6 @@ typedef cudaError_t (*BatchOccFn)(int *, size_t);
 
 constexpr int kBatchBlock = 128;
 constexpr int kBatchMaxViews = 256;
-constexpr size_t kBatchMaxSmem = 227 * 1024;  // shared memory that a block can have
 constexpr uint32_t kErrBalance = 1u, kErrTimeout = 2u, kErrCapacity = 4u;
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -108,15 +107,19 @@ struct EmitChildrenV {
   }
 };
 
-// Shared memory of a block: the emission tables of every band chunk, and the
-// per-view counters.
-// (NBT = 0, the wide form: of every chunk of `width` bands, and the sums.)
+// Table and constants of a band chunk of `width` (the wide form, NBT = 0) or NBT bands.
 template <int NBT>
-static size_t batch_smem(const GridView &g, int V, int width) {
-  const bool table = g.cell_fmt == kCellXq;
-  const size_t tab = NBT == 0 ? ((g.n_bands + width - 1) / width) * wide_tab_bytes(table, g.n_tbins, width) +
-                                    wide_sum_bytes(width, kBatchBlock)
-                              : ((g.n_bands + NBT - 1) / NBT) * chunk_bytes<NBT>(table, g.n_tbins);
+__host__ __device__ __forceinline__ size_t batch_tab_bytes(bool table, int n_tbins, int width) {
+  if constexpr (NBT == 0) return wide_tab_bytes(table, n_tbins, width);
+  else return chunk_bytes<NBT>(table, n_tbins);
+}
+
+// Shared memory of a block: the tables of `tabs` band chunks, the sums of the
+// wide form, and the per-view counters.
+template <int NBT>
+static size_t batch_smem(const GridView &g, int V, int width, int tabs) {
+  const size_t tab = tabs * batch_tab_bytes<NBT>(g.cell_fmt == kCellXq, g.n_tbins, width) +
+                     (NBT == 0 ? wide_sum_bytes(width, kBatchBlock) : 0);
   return tab + 3 * sizeof(int64_t) * V + sizeof(int32_t) * V + sizeof(int32_t) * (kBatchBlock / 32) * V;
 }
 
@@ -129,6 +132,23 @@ template <int NBT, int DIR>
 struct BatchBlocks {
   static constexpr int value = NBT == 0 ? kBatchWideBlocks : NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? (DIR == 0 ? 3 : 4) : (DIR == 0 ? 2 : 3)));
 };
+
+// Band chunks whose tables a block holds. All of them, filled once, where the
+// form's resident blocks then still fit an SM's shared memory; else one at a
+// time, filled again whenever the block's warps go on to the next chunk. (8
+// inclined views, 255 table bins, every chunk held: 32 bands 10.5 ms with two
+// blocks per SM, 64 bands 29.7 with one; one at a time 8.8 and 15.3. Mixed
+// views 16.8 and 46.3, 14.1 and 26.2. 64 bins: 7.8 and 13.0, 13.6 and 25.7.)
+constexpr size_t kSmShared = 228 * 1024, kBlockReserve = 1024;  // of an SM; taken per block
+template <int NBT, int DIR>
+static int batch_tables(const GridView &g, int V, int width) {
+  const int chunks = NBT == 0 ? (g.n_bands + width - 1) / width : (g.n_bands + NBT - 1) / (NBT > 0 ? NBT : 1);
+  auto blocks = [&](int tabs) {
+    return std::min<size_t>(BatchBlocks<NBT, DIR>::value,
+                            kSmShared / (batch_smem<NBT>(g, V, width, tabs) + kBlockReserve));
+  };
+  return blocks(chunks) >= blocks(1) ? chunks : 1;
+}
 
 // Where a traced ray's values go.
 struct BatchOut {
@@ -146,10 +166,10 @@ __device__ __forceinline__ void batch_trace(const BatchArgs &a, unsigned char *s
                                             const BatchOut &o, int64_t k) {
   const GridView &g = a.g;
   if constexpr (NBT == 0) {
-    const size_t tab = wide_tab_bytes(FMT == kCellXq, g.n_tbins, a.width);
+    const size_t tab = batch_tab_bytes<0>(FMT == kCellXq, g.n_tbins, a.width);
     int b0;
-    const int c0 = chunk * a.width;
-    const WideCtx wc = wide_ctx<FMT>(sm + chunk * tab, reinterpret_cast<float4 *>(sm + a.chunks * tab), a.width,
+    const int c0 = chunk * a.width, slot = a.tabs > 1 ? chunk : 0;
+    const WideCtx wc = wide_ctx<FMT>(sm + slot * tab, reinterpret_cast<float4 *>(sm + a.tabs * tab), a.width,
                                      min(a.width, g.n_bands - c0), part, parts, &b0);
     b0 += c0;
     if (wc.pairs <= 0) return;
@@ -174,7 +194,8 @@ __device__ __forceinline__ void batch_trace(const BatchArgs &a, unsigned char *s
     if (all) o.p[k] = p;
   } else {
     const int b0 = chunk * NBT;
-    const BandCtx bc = chunk_ctx<NBT, FMT>(sm + chunk * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g,
+    const int slot = a.tabs > 1 ? chunk : 0;
+    const BandCtx bc = chunk_ctx<NBT, FMT>(sm + slot * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g,
                                            min(NBT, g.n_bands - b0));
     BandRegs<NBT> br;
     band_regs<NBT>(br, bc);
@@ -198,21 +219,50 @@ __device__ __forceinline__ void batch_trace(const BatchArgs &a, unsigned char *s
   }
 }
 
+// Table and constants of chunk `chunk` at `sm`, by the block.
+template <int NBT, int FMT>
+__device__ __forceinline__ void batch_fill(const BatchArgs &a, unsigned char *sm, int chunk) {
+  if constexpr (NBT == 0) wide_fill<FMT>(sm, a.g, chunk * a.width, a.width);
+  else chunk_fill<NBT, FMT>(sm, a.g, chunk * NBT);
+}
+
+// The work of one phase: `items` items (rays x parts) of every band chunk, from
+// the chunks' queues; a warp takes rpw at a time. body(chunk, item), lane by
+// lane. With one table per block, the block goes from chunk to chunk together
+// (and leaves out a chunk whose queue is empty by then); every thread of the
+// block calls this.
+template <int NBT, int FMT, class Body>
+__device__ __forceinline__ void batch_queue(const BatchArgs &a, unsigned char *sm, unsigned long long items,
+                                            int rpw, const Body &body) {
+  const int lane = threadIdx.x & 31;
+  for (int chunk = 0; chunk < a.chunks; ++chunk) {
+    auto take = [&] {
+      unsigned long long b = 0;
+      if (lane == 0) b = atomicAdd(&a.ctl->q_head[chunk], (unsigned long long)rpw);
+      return __shfl_sync(0xffffffffu, b, 0);
+    };
+    unsigned long long b = take();
+    if (a.tabs < a.chunks) {
+      if (!__syncthreads_or(b < items)) continue;
+      batch_fill<NBT, FMT>(a, sm, chunk);
+      __syncthreads();
+    }
+    for (; b < items; b = take()) {
+      const unsigned long long it = lane < rpw ? b + lane : items;
+      if (it < items) body(chunk, it);
+    }
+  }
+}
+
 template <int NBT, bool AMR, int FMT, int DIR>
 __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_air_batch(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const GridView &g = a.g;
   const int V = a.V, nb = g.n_bands;
-  size_t tab_end;
-  if constexpr (NBT == 0) {
-    const size_t tab = wide_tab_bytes(FMT == kCellXq, g.n_tbins, a.width);
-    for (int c = 0; c < a.chunks; ++c) wide_fill<FMT>(smem_raw + c * tab, g, c * a.width, a.width);
-    tab_end = a.chunks * tab + wide_sum_bytes(a.width, kBatchBlock);
-  } else {
-    for (int c = 0; c < a.chunks; ++c)
-      chunk_fill<NBT, FMT>(smem_raw + c * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g, c * NBT);
-    tab_end = a.chunks * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins);
-  }
+  const size_t tab = batch_tab_bytes<NBT>(FMT == kCellXq, g.n_tbins, a.width);
+  if (a.tabs == a.chunks)
+    for (int c = 0; c < a.chunks; ++c) batch_fill<NBT, FMT>(a, smem_raw + c * tab, c);
+  const size_t tab_end = a.tabs * tab + (NBT == 0 ? wide_sum_bytes(a.width, kBatchBlock) : 0);
   int64_t *run = (int64_t *)(smem_raw + tab_end);
   int64_t *tot = run + V;
   int64_t *vbase = tot + V;
@@ -227,7 +277,6 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
   const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
   const unsigned nblk = gridDim.x;
-  const int lane = threadIdx.x & 31;
 
   // step i: the base image of every view, view-major, row-major within a view
   // (mode 2 continues from the base images a mode-1 launch traced)
@@ -248,23 +297,15 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
   int64_t first = a.mode == 2 ? nbase : 0, n = nbase;
   if (a.mode == 2 && a.P > 0) {
     // the proposal wave of every view: (ray, band chunk) items from the queue
-    const int parts = NBT == 0 ? wide_parts(a.P * a.chunks, min(a.width, nb), a.fill) : 1;
-    const unsigned long long items = (unsigned long long)a.P * (unsigned long long)(a.chunks * parts);
+    const int parts = NBT == 0 ? wide_parts(a.P * a.tabs, min(a.width, nb), a.fill) : 1;
     const BatchOut o{a.pN, a.pI, a.pp, a.psteps, nullptr, a.P};
-    const int rpw = rays_per_warp(a.P, a.chunks * parts, (int64_t)nblk * (kBatchBlock / 32));
-    for (;;) {
-      unsigned long long b = 0;
-      if (lane == 0) b = atomicAdd(&a.ctl->q_head, (unsigned long long)rpw);
-      b = __shfl_sync(0xffffffffu, b, 0);
-      if (b >= items) break;
-      const unsigned long long it = lane < rpw ? b + lane : items;
-      if (it < items) {
-        const int cp = (int)(it / (unsigned long long)a.P), chunk = cp / parts;
-        const int64_t q = (int64_t)(it - (unsigned long long)cp * a.P);
-        batch_trace<NBT, AMR, FMT, DIR>(a, smem_raw, a.geoms[a.pview[q]], a.plvl[q], a.ppi[q], a.ppj[q], chunk,
-                                        cp - chunk * parts, parts, a.chunks * parts == 1, o, q);
-      }
-    }
+    const int rpw = rays_per_warp(a.P, a.tabs * parts, (int64_t)nblk * (kBatchBlock / 32));
+    batch_queue<NBT, FMT>(a, smem_raw, (unsigned long long)a.P * parts, rpw, [&](int chunk, unsigned long long it) {
+      const int part = parts == 1 ? 0 : (int)(it / (unsigned long long)a.P);
+      const int64_t q = (int64_t)(it - (unsigned long long)part * a.P);
+      batch_trace<NBT, AMR, FMT, DIR>(a, smem_raw, a.geoms[a.pview[q]], a.plvl[q], a.ppi[q], a.ppj[q], chunk, part,
+                                      parts, a.chunks * parts == 1, o, q);
+    });
     // (the band sums of rays dealt to parts of one chunk: those of several
     // chunks are formed where the pixels take their values)
     if (a.chunks == 1 && parts > 1) {
@@ -276,37 +317,27 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
       }
     }
     if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->q_head = 0ull;
+    if (blockIdx.x == 0 && threadIdx.x < a.chunks) a.ctl->q_head[threadIdx.x] = 0ull;
   }
   int sweep = 0;
   for (;; ++sweep) {
     // step ii: trace the rays added last sweep, all views and band chunks
     const int64_t cnt_r = n - first;
-    const int parts = NBT == 0 ? wide_parts(cnt_r * a.chunks, min(a.width, nb), a.fill) : 1;
+    const int parts = NBT == 0 ? wide_parts(cnt_r * a.tabs, min(a.width, nb), a.fill) : 1;
     const int shares = a.chunks * parts;
-    const unsigned long long items = (unsigned long long)cnt_r * (unsigned long long)shares;
     const BatchOut o{t.N, t.I, t.p, t.steps, a.mode == 1 ? a.maxlev : nullptr, t.cap};
-    const int rpw = rays_per_warp(cnt_r, shares, (int64_t)nblk * (kBatchBlock / 32));
-    for (;;) {
-      unsigned long long b = 0;
-      if (lane == 0) b = atomicAdd(&a.ctl->q_head, (unsigned long long)rpw);
-      b = __shfl_sync(0xffffffffu, b, 0);
-      if (b >= items) break;
-      const unsigned long long it = lane < rpw ? b + lane : items;
-      bool todo = it < items;
-      int cp = 0, v = 0;
-      int64_t k = 0;
-      if (todo) {
-        cp = (int)(it / (unsigned long long)cnt_r);
-        k = first + (int64_t)(it - (unsigned long long)cp * cnt_r);
-        v = a.view[k];
-      }
-      if (todo && a.mode == 2) {
+    const int rpw = rays_per_warp(cnt_r, a.tabs * parts, (int64_t)nblk * (kBatchBlock / 32));
+    batch_queue<NBT, FMT>(a, smem_raw, (unsigned long long)cnt_r * parts, rpw, [&](int chunk, unsigned long long it) {
+      const int part = parts == 1 ? 0 : (int)(it / (unsigned long long)cnt_r);
+      const int64_t k = first + (int64_t)(it - (unsigned long long)part * cnt_r);
+      const int v = a.view[k];
+      if (a.mode == 2) {
         // the pixel's values from its view's proposal wave when the wave
         // traced it (the same trace, so the same bits); else trace it
         const int L = t.lvl[k], i = t.pi[k], j = t.pj[k];
         const int64_t pb = (int64_t)v * nn0 + (int64_t)(j >> L) * n0 + (i >> L);
         const int64_t q = prop_index(a.pdepth + 4 * pb, a.poff[pb], L, i, j);
+        const int cp = chunk * parts + part;
         if (q >= 0) {
           if (cp == 0) {
             t.N[k] = a.pN[q];
@@ -315,19 +346,15 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
           const int b0 = (int)((int64_t)nb * cp / shares), b1 = (int)((int64_t)nb * (cp + 1) / shares);
           for (int c = b0; c < b1; ++c) t.I[(int64_t)c * t.cap + k] = a.pI[(int64_t)c * a.P + q];
           if (a.chunks == 1 && cp == 0) t.p[k] = a.pp[q];
-          todo = false;
-        } else if (cp == 0) {
-          atomicAdd(&a.ctl->fb_rays, 1ull);
+          return;
         }
+        if (cp == 0) atomicAdd(&a.ctl->fb_rays, 1ull);
       }
-      if (todo) {
-        const int chunk = cp / parts;
-        batch_trace<NBT, AMR, FMT, DIR>(a, smem_raw, a.geoms[v], t.lvl[k], t.pi[k], t.pj[k], chunk,
-                                        cp - chunk * parts, parts, shares == 1, o, k);
-      }
-    }
+      batch_trace<NBT, AMR, FMT, DIR>(a, smem_raw, a.geoms[v], t.lvl[k], t.pi[k], t.pj[k], chunk, part, parts,
+                                      shares == 1, o, k);
+    });
     if (!grid_sync(a.ctl, nblk, a.timeout_ns)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->q_head = 0ull;  // next sweep's queue
+    if (blockIdx.x == 0 && threadIdx.x < a.chunks) a.ctl->q_head[threadIdx.x] = 0ull;  // next sweep's queues
     if (shares > 1) {
       for (int64_t k = first + gtid; k < n; k += gstride) {
         float s = 0.f;
@@ -432,24 +459,27 @@ static cudaError_t batch_launch(const BatchArgs &a, int grid, size_t smem, cudaS
 }
 
 template <int NBT, int FMT, int DIR>
-static void batch_pick(bool amr, BatchOccFn *occ, BatchLaunchFn *launch) {
+static void batch_pick(const GridView &g, int V, int width, BatchOccFn *occ, BatchLaunchFn *launch, size_t *smem,
+                       int *tabs) {
+  const bool amr = g.kind == AIR_GRID_AMR;
+  *tabs = batch_tables<NBT, DIR>(g, V, width);
+  *smem = batch_smem<NBT>(g, V, width, *tabs);
   *occ = amr ? batch_occupancy<NBT, true, FMT, DIR> : batch_occupancy<NBT, false, FMT, DIR>;
   *launch = amr ? batch_launch<NBT, true, FMT, DIR> : batch_launch<NBT, false, FMT, DIR>;
 }
 
-// Occupancy and launch functions and shared memory of the kernel for a grid
-// and V views (inclined: all of them are) with NBT bands per thread (0: the
-// wide form, `width` bands per chunk); false where there is no such form.
+// Occupancy and launch functions, shared memory and resident tables of the
+// kernel for a grid and V views (inclined: all of them are) with NBT bands per
+// thread (0: the wide form, `width` bands per chunk); false where there is no
+// such form.
 template <int NBT>
 bool batch_fns(const GridView &g, int V, bool inclined, int width, BatchOccFn *occ, BatchLaunchFn *launch,
-               size_t *smem) {
-  const bool amr = g.kind == AIR_GRID_AMR;
-  *smem = batch_smem<NBT>(g, V, width);
+               size_t *smem, int *tabs) {
   if (g.cell_fmt == kCellLam) {
     // per-cell Lambda exists for one-band grids only
     if constexpr (NBT == 1) {
-      if (inclined) batch_pick<1, kCellLam, -2>(amr, occ, launch);
-      else batch_pick<1, kCellLam, 0>(amr, occ, launch);
+      if (inclined) batch_pick<1, kCellLam, -2>(g, V, width, occ, launch, smem, tabs);
+      else batch_pick<1, kCellLam, 0>(g, V, width, occ, launch, smem, tabs);
       return true;
     }
     return false;
@@ -458,12 +488,12 @@ bool batch_fns(const GridView &g, int V, bool inclined, int width, BatchOccFn *o
   constexpr int DIR = NBT == 0 ? -2 : 0;
   if constexpr (NBT >= 1 && NBT <= 8)
     if (inclined) {
-      if (g.cell_fmt == kCellXq) batch_pick<NBT, kCellXq, -2>(amr, occ, launch);
-      else batch_pick<NBT, kCellRho, -2>(amr, occ, launch);
+      if (g.cell_fmt == kCellXq) batch_pick<NBT, kCellXq, -2>(g, V, width, occ, launch, smem, tabs);
+      else batch_pick<NBT, kCellRho, -2>(g, V, width, occ, launch, smem, tabs);
       return true;
     }
-  if (g.cell_fmt == kCellXq) batch_pick<NBT, kCellXq, DIR>(amr, occ, launch);
-  else batch_pick<NBT, kCellRho, DIR>(amr, occ, launch);
+  if (g.cell_fmt == kCellXq) batch_pick<NBT, kCellXq, DIR>(g, V, width, occ, launch, smem, tabs);
+  else batch_pick<NBT, kCellRho, DIR>(g, V, width, occ, launch, smem, tabs);
   return true;
 }
 

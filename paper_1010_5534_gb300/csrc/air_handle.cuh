@@ -87,18 +87,19 @@ struct RayGeom;
 struct BatchCtl {
   unsigned int bar_count;
   unsigned int bar_gen;
-  unsigned long long q_head;
   long long n_nodes;
   long long need;
   int sweeps;
   unsigned int err;
   unsigned long long fb_rays;  // learned mode: pixels the proposal missed, traced in sweeps
+  unsigned long long q_head[kMaxBands];  // work queue of each band chunk
 };
 
 struct BatchArgs {
   GridView g;
   const RayGeom *geoms;  // [V]
   int V, chunks, fp64_level, xi_norm, refine_on, stall;
+  int tabs;              // band chunks whose tables a block holds: all, or 1 (batch_tables)
   int width;             // the wide march: bands of a chunk, and the threads that a
   int64_t fill;          // chunk's parts should fill (wide_parts)
   double xi_crit;
