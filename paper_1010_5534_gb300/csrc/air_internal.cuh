@@ -15,6 +15,14 @@ constexpr int kMapLevelShift = 27;  // brick map entry: id | level << 27
 constexpr int32_t kMapIdMask = (1 << kMapLevelShift) - 1;
 enum { kCellRho = 0, kCellLam = 1, kCellXq = 2 };
 
+// Whether 32-bit cell indices do for the walk through a uniform grid of these
+// cells. The walk finishes its chunk of K cells after the ray has left the grid
+// (nothing is loaded there), so an index may lie up to K planes of the slowest
+// axis beyond either end.
+__host__ __device__ inline bool walk_index_fits(int n0, int n1, int n2, int K) {
+  return (int64_t)n0 * n1 * ((int64_t)n2 + K) <= 0x7fffffff;
+}
+
 // Per-band constants of the march (one 16-byte load).
 struct __align__(16) BandConst {
   float kap;     // kappa_b

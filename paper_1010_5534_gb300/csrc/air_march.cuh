@@ -1099,9 +1099,7 @@ __device__ void march_uniform(RTState<NBT> &r, const GridView &g, const double O
     inv[a] = rg.invDhi[a];
   }
   // the ray leaves through a face of the grid: no end parameter needed
-  // (indices are 32-bit where every cell has one; a step past the block may
-  // lie one row beyond)
-  if ((int64_t)g.nf[0] * g.nf[1] * ((int64_t)g.nf[2] + 2) <= 0x7fffffff)
+  if (walk_index_fits(g.nf[0], g.nf[1], g.nf[2], K))
     march_block<NBT, FMT, K, int>(r, Q, Dl, inv, FLT_MAX, lc[0], lc[1], lc[2], g.nf[0], g.nf[1], g.nf[2],
                                g.nf[0], g.nf[0] * g.nf[1], g.cells, bc, br);
   else
