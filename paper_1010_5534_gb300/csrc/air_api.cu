@@ -233,6 +233,13 @@ static air_status out_view(air_grid *g, const air_image *im, int64_t n, OutView 
   return AIR_OK;
 }
 
+// Where k_flux_final writes the flux beside its page-locked copy: the caller's
+// device array, unless that is not aligned for FP64 stores (finish_out then
+// copies it there) or not in device memory.
+static double *flux_dest(const air_image *im) {
+  return im->mem == AIR_DEVICE && ((uintptr_t)im->band_flux & 7) == 0 ? im->band_flux : nullptr;
+}
+
 // Staging -> host arrays (host-memory outputs); band flux and step count from
 // the page-locked copy that k_flux_final left.
 static air_status finish_out(air_grid *g, air_image *im, const OutView &o, int64_t n) {
@@ -253,6 +260,10 @@ static air_status finish_out(air_grid *g, air_image *im, const OutView &o, int64
   }
   CU_TRY(cudaStreamSynchronize(st));
   if (im->band_flux && im->mem == AIR_HOST) std::memcpy(im->band_flux, w.h_flux, sizeof(double) * nb);
+  if (im->band_flux && im->mem == AIR_DEVICE && !flux_dest(im)) {
+    CU_TRY(cudaMemcpyAsync(im->band_flux, w.h_flux, sizeof(double) * nb, cudaMemcpyHostToDevice, st));
+    CU_TRY(cudaStreamSynchronize(st));
+  }
   im->n_steps = (int64_t)w.h_flux[nb];
   return AIR_OK;
 }
@@ -304,7 +315,7 @@ air_status render_fixed(air_grid *g, const air_view *view, int32_t res, int32_t 
   FluxArgs fa{};
   fa.n = n; fa.child = nullptr; fa.lvl = nullptr; fa.I = ro.I; fa.stride = ro.stride; fa.steps = w.fsteps;
   fa.n_bands = nb; fa.area0 = (2.0 * cam.H / res) * (2.0 * cam.H / res); fa.partial = w.partial;
-  fa.flux = im->mem == AIR_DEVICE ? im->band_flux : nullptr;
+  fa.flux = flux_dest(im);
   fa.host = w.h_flux;
   const bool list = o.level || o.i || o.j || o.is_leaf;
   CU_TRY(prof_open(g, AIR_PHASE_OUTPUT, list ? 3 : 2));
@@ -722,7 +733,7 @@ air_status output_tree(air_grid *g, const Camera &cam, const air_params *pr, air
   fa.I = spectra_dev ? spectra_dev : t.I;
   fa.stride = spectra_dev ? spectra_cap : t.cap;
   fa.n_bands = nb; fa.area0 = (2.0 * cam.H / n0) * (2.0 * cam.H / n0); fa.partial = w.partial;
-  fa.flux = im->mem == AIR_DEVICE ? im->band_flux : nullptr;
+  fa.flux = flux_dest(im);
   fa.host = w.h_flux;
   if (!all) {  // (both arrays hold 3 entries per scan chunk of the whole pyramid)
     fa.chunk_leaves = w.bcount;
