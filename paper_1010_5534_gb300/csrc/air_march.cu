@@ -19,9 +19,8 @@ __global__ void k_band_sum(const float *__restrict__ I, int n_bands, int64_t str
 
 // Band sums of the new nodes of sweep q, counted on the device, unless they are
 // more than `most` (their threads then held all bands and summed them).
-__global__ void k_band_sum_dev(const float *__restrict__ I, int n_bands, int64_t stride,
-                               const SweepState *__restrict__ S, int q, int64_t most,
-                               float *__restrict__ p) {
+__global__ void k_band_sum_dev(const float *I, int n_bands, int64_t stride, const SweepState *S, int q,
+                               int64_t most, float *__restrict__ p) {
   wait_prior_grid();
   const int64_t first = S->slot[q & 3].n, end = S->slot[(q + 1) & 3].n;
   if (end - first > most) return;

@@ -397,8 +397,7 @@ __global__ void __launch_bounds__(kThreads) k_mlp(MlpArgs a) {
 
 // Sum over blocks of partial[b][j] in FP64, in block order (loads 8 at a
 // time).
-__device__ __forceinline__ double sum_partials(const float *__restrict__ partial, int64_t nblocks,
-                                               int j) {
+__device__ __forceinline__ double sum_partials(const float *partial, int64_t nblocks, int j) {
   double s = 0.0;
   int64_t b = 0;
   for (; b + 8 <= nblocks; b += 8) {
@@ -426,7 +425,7 @@ __global__ void k_reduce_partials(const float *__restrict__ partial, int64_t nbl
 // and the packed BF16 copies of parameter j by one thread; the minibatch's
 // loss to *loss. (Three launches before: reduction, Adam, packing.) Blocks of
 // 64 spread the FP64 sums over 88 SMs.
-__global__ void __launch_bounds__(64) k_step(const float *__restrict__ partial, int64_t nblocks,
+__global__ void __launch_bounds__(64) k_step(const float *partial, int64_t nblocks,
                                              float *__restrict__ th, float *__restrict__ m,
                                              float *__restrict__ v, float *__restrict__ grad,
                                              uint32_t *__restrict__ w, double *__restrict__ loss,

@@ -301,10 +301,9 @@ __global__ void k_open_init(SweepState *S, int64_t n, int32_t *list, uint32_t *f
 // expansion's -- expands it. Every flag is expanded once, and the flags reach
 // the same closure as a scan of every leaf followed by the balance.
 __global__ void __launch_bounds__(kScanBlock)
-    k_scan_balance_dev(TreeView t, const int32_t *__restrict__ open, const SweepState *__restrict__ S,
-                       int q, double xi_crit, int xi_norm, int refine_on, uint32_t *__restrict__ flag,
-                       uint32_t *__restrict__ counts, int64_t nb_cap, uint32_t *__restrict__ err,
-                       const int32_t *lmap) {
+    k_scan_balance_dev(TreeView t, const int32_t *open, const SweepState *S,
+                       int q, double xi_crit, int xi_norm, int refine_on, uint32_t *flag,
+                       uint32_t *counts, int64_t nb_cap, uint32_t *err, const int32_t *lmap) {
   wait_prior_grid();
   const SweepSlot &sl = S->slot[q & 3];
   if (sl.done) return;
@@ -363,9 +362,8 @@ __device__ __forceinline__ void block_sum4(uint32_t (&v)[4], uint32_t (&sh)[4][k
 // then the children below the top level (in order). Block 0 writes the next
 // slot and the host's report.
 __global__ void __launch_bounds__(kScanBlock)
-    k_emit3d(TreeView t, const int32_t *__restrict__ open, int32_t *__restrict__ next,
-             SweepState *__restrict__ S, int q, uint32_t *flag, uint32_t *counts, int64_t nb_cap,
-             const uint32_t *__restrict__ err, SweepReport *rep, uint32_t tag, int32_t *lmap) {
+    k_emit3d(TreeView t, const int32_t *open, int32_t *next, SweepState *S, int q, uint32_t *flag,
+             uint32_t *counts, int64_t nb_cap, const uint32_t *err, SweepReport *rep, uint32_t tag, int32_t *lmap) {
   wait_prior_grid();
   __shared__ uint32_t sums[4][kScanBlock / 32];
   __shared__ int32_t wsum[3][kScanBlock / 32];
@@ -515,9 +513,9 @@ __global__ void __launch_bounds__(kScanBlock)
 // block_off. (A counting and a scanning launch of their own took 25 us for 7.7 M
 // nodes; but every block adding up all the counts before it is quadratic work.)
 __global__ void __launch_bounds__(kScanBlock) k_emit_out(TreeView t, OutView o, int all, int64_t n,
-                                                         const int32_t *__restrict__ chunk_leaves,
-                                                         const int32_t *__restrict__ block_leaves,
-                                                         const int64_t *__restrict__ block_off) {
+                                                         const int32_t *chunk_leaves,
+                                                         const int32_t *block_leaves,
+                                                         const int64_t *block_off) {
   wait_prior_grid();
   __shared__ int32_t wsum[kScanBlock / 32];
   __shared__ uint32_t fsum[kScanBlock / 32];

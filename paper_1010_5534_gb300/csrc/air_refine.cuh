@@ -113,6 +113,10 @@ struct SweepReport {
 // beside this kernel's last ones and wait here in their turn, so a launch
 // costs no gap. (Without the second instruction the next kernel was scheduled
 // only when this one had ended.)
+// So the kernel before may write while this one already runs: what it writes is
+// read by ordinary loads, through pointers without `const __restrict__`. Those
+// make read-only loads, which are defined for data that nothing writes during
+// the kernel and which the wait does not have to order.
 __device__ __forceinline__ void wait_prior_grid() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
