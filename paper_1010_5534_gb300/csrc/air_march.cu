@@ -56,8 +56,9 @@ static int64_t wide_fill_threads() { return (int64_t)sm_count() * kWideBlocks * 
 // Inclined rays with more than 8 bands per thread go to the wide form. (Bands in
 // registers up to 8: the 8-band cone, 1500^2 fixed, 1.09 ms, 1.17 in the wide
 // form; 5 hot bands 300 us, 318. With 32 bands the wide form's one walk wins over
-// four: clumps 11.8 -> 7.9 ms, and 8 views x 16 bands 16.4 -> 13.2.)
-static bool is_wide(int nbt, int moving) { return moving > 1 && nbt > 8; }
+// four: clumps 11.8 -> 7.9 ms, and 8 views x 16 bands 16.4 -> 13.2.) Rays that
+// move along no axis (cells too large, see make_geom) take the same forms.
+static bool is_wide(int nbt, int moving) { return moving != 1 && nbt > 8; }
 
 // The march kernel with NBT bands per thread (the wide form: per chunk, any
 // even number, and `fill` threads to fill).
