@@ -138,7 +138,6 @@ constexpr int kVfluxRounds = 8;
 __global__ void __launch_bounds__(256) k_vflux(TreeView t, const int16_t *view, int64_t n,
                                                int n_bands, const RayGeom *geoms, double *vflux) {
   __shared__ double sums[kFluxBands][8];
-  __shared__ double red[8][kFluxBands][32];
   __shared__ int views[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b0 = blockIdx.y * kFluxBands, nb = min(kFluxBands, n_bands - b0);
@@ -159,7 +158,7 @@ __global__ void __launch_bounds__(256) k_vflux(TreeView t, const int16_t *view, 
     if (__all_sync(0xffffffffu, v == v0 || !in)) {
       if (v0 != cur) {
         if (cur >= 0) {
-          const double s = flux_warp_sum(acc, red[warp]);
+          const double s = flux_warp_sum(acc);
           if ((lane & 7) == 0 && (lane >> 3) < nb) atomicAdd(&vflux[(int64_t)cur * n_bands + b0 + (lane >> 3)], s * area(cur));
 #pragma unroll
           for (int q = 0; q < kFluxBands; ++q) acc[q] = 0.0;
@@ -181,7 +180,7 @@ __global__ void __launch_bounds__(256) k_vflux(TreeView t, const int16_t *view, 
                   (double)t.I[(int64_t)(b0 + q) * t.cap + k] * pow4_neg(L) * area(v));
     }
   }
-  const double s4 = flux_warp_sum(acc, red[warp]);
+  const double s4 = flux_warp_sum(acc);
   if ((lane & 7) == 0) sums[lane >> 3][warp] = s4;
   if (lane == 0) views[warp] = cur;
   __syncthreads();

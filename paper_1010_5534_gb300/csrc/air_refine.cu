@@ -616,7 +616,6 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
   wait_prior_grid();
   __shared__ int32_t chunk_sum[kFluxChunks];
   __shared__ double sh[kFluxBands][8];
-  __shared__ double red[8][kFluxBands][32];
   __shared__ unsigned long long shs[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t start = (int64_t)blockIdx.x * kFluxPerBlock;
@@ -680,8 +679,9 @@ __global__ void __launch_bounds__(256) k_flux_partial(FluxArgs a) {
       }
   }
 #pragma unroll
-  for (int q = 0; q < kFluxBands; ++q) rest[q] += (double)hi[q] + (double)lo[q];
-  const double s4 = flux_warp_sum(rest, red[warp]);
+  for (int q = 0; q < kFluxBands; ++q)
+    if (b0 + q < a.n_bands) rest[q] += (double)hi[q] + (double)lo[q];
+  const double s4 = flux_warp_sum(rest);
   if ((lane & 7) == 0) sh[lane >> 3][warp] = s4;
   __syncthreads();
   if (count) {

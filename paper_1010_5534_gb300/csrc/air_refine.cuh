@@ -168,19 +168,19 @@ __device__ __forceinline__ void flux_add(float I, int L, float &hi, float &lo, d
   }
 }
 
-// The warp's FP64 sums of v[0 .. kFluxBands), through the warp's rows `red` of
-// shared memory: lane 8 q returns the sum of v[q]. Six FP64 additions per warp
-// for four bands (a butterfly over the lanes takes twenty).
-__device__ __forceinline__ double flux_warp_sum(const double (&v)[kFluxBands], double (*red)[32]) {
+// The warp's FP64 sums of v[0 .. kFluxBands): the eight lanes from 8 q on return
+// the sum of v[q]. Lanes first trade away the bands they will not hold, so four
+// bands take six FP64 additions per warp (a butterfly for each takes twenty).
+// No shared memory: with 8 KB of it the flux kernel, launched as a dependent,
+// changed the SMs' split of L1 and shared memory behind the march, and a fixed
+// image of 200^2 pixels took 67 us instead of 52.
+__device__ __forceinline__ double flux_warp_sum(const double (&v)[kFluxBands]) {
   static_assert(kFluxBands == 4, "eight lanes per band");
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int q = 0; q < kFluxBands; ++q) red[q][lane] = v[q];
-  __syncwarp();
-  const double *r = red[lane >> 3] + (lane & 7);
-  double s = (r[0] + r[8]) + (r[16] + r[24]);
+  const bool hi = threadIdx.x & 16, odd = threadIdx.x & 8;
+  const double a = (hi ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
+  const double b = (hi ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 16);
+  double s = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
   for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  __syncwarp();
   return s;
 }
 
