@@ -1404,11 +1404,13 @@ __device__ __forceinline__ void march_amr_axis(RTState<NBT> &r, const GridView &
 // brick's records (and the map entry of the one after) are on their way while
 // a brick is summed. (One kernel with both walks spilled registers; the walk
 // that waits for each column took 26 us a sweep on the ring grid, 8^3 bricks.)
-template <int NBT, int FMT>
+// M: the largest brick edge, 8, or 2 for bricks of one or two cells, where eight
+// cells' instructions per brick are wasted (a fixed image of 500^2 pixels through
+// bricks of one cell 186 us with M = 8, 127 with 2).
+template <int NBT, int FMT, int M>
 __device__ __forceinline__ void march_amr_axis_small(RTState<NBT> &r, const GridView &g, int A,
                                                      int c1, int c2, const RayGeom &rg,
                                                      const BandCtx &bc, const BandRegs<NBT> &br) {
-  constexpr int M = 8;  // largest brick edge
   const int A1 = A == 2 ? 0 : A + 1, A2 = A == 0 ? 2 : A - 1;
   const int B = g.B, lb = g.log2B, Lm = g.Lm;
   const int nfA = A == 0 ? g.nf[0] : (A == 1 ? g.nf[1] : g.nf[2]);
@@ -1515,8 +1517,9 @@ __device__ __forceinline__ void march_axis(RTState<NBT> &st, const GridView &g, 
   if (!axis_ray_setup(g, rg, A, L, i, j, c1, c2)) return;
   if (NBT > 1) band_load<NBT>(br, bc);
   if constexpr (!AMR) march_uniform_axis<NBT, FMT, U>(st, g, A, c1, c2, rg, bc, br);
+  else if constexpr (DIR >= 13) march_amr_axis_small<NBT, FMT, 2>(st, g, A, c1, c2, rg, bc, br);
   else if constexpr (DIR >= 7) march_amr_axis<NBT, FMT, U, false, (DIR < 10 ? 1 : -1), (DIR - 1) % 3>(st, g, A, c1, c2, rg, bc, br);
-  else if constexpr (DIR >= 4) march_amr_axis_small<NBT, FMT>(st, g, A, c1, c2, rg, bc, br);
+  else if constexpr (DIR >= 4) march_amr_axis_small<NBT, FMT, 8>(st, g, A, c1, c2, rg, bc, br);
   else march_amr_axis<NBT, FMT, U, (DIR <= 0)>(st, g, A, c1, c2, rg, bc, br);
 }
 
@@ -1525,8 +1528,8 @@ __device__ __forceinline__ void march_axis(RTState<NBT> &st, const GridView &g, 
 //   0: any direction (the batched kernel);
 //   1 + A: every ray of the launch is parallel to grid axis A, one band (bricks
 //     of 16 cells and more, or a uniform grid); 4 + A: the same with bricks of
-//     at most 8 cells; 7 + A and 10 + A: with 16^3 bricks, towards higher and
-//     lower cells;
+//     4 or 8 cells; 13 + A: of 1 or 2; 7 + A and 10 + A: with 16^3 bricks,
+//     towards higher and lower cells;
 //   -1: inclined rays in launches of few rays (DdaChunk); -2: inclined rays;
 //   -3: rays parallel to some axis, any number of bands.
 template <int NBT, bool AMR, int FMT, int DIR = 0>

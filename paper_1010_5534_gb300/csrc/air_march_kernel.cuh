@@ -343,11 +343,12 @@ cudaError_t march_general(const MarchLaunch &m) {
 }
 
 // One-band grids, every ray parallel to grid axis A: the form DIR = 1 + A, or
-// 4 + A for bricks of at most 8 cells, 7 + A or 10 + A for grids of 16^3 bricks
+// 4 + A for bricks of 4 or 8 cells, 13 + A for 1 or 2, 7 + A or 10 + A for grids of 16^3 bricks
 // with per-cell Lambda (the ordinary one-band grid).
 template <int A, int FMT>
 static cudaError_t march_axis_fmt(const MarchLaunch &m) {
   if (m.g.kind != AIR_GRID_AMR) return march_form<1, false, FMT, 1 + A>(m);
+  if (m.g.B <= 2) return march_form<1, true, FMT, 13 + A>(m);
   if (m.g.B <= 8) return march_form<1, true, FMT, 4 + A>(m);
   if constexpr (FMT == kCellLam)
     if (m.g.B == 16) return m.rg.Dhi[A] > 0.f ? march_form<1, true, FMT, 7 + A>(m) : march_form<1, true, FMT, 10 + A>(m);
