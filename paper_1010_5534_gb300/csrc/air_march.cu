@@ -144,7 +144,9 @@ cudaError_t launch_march(const GridView &g, const Camera &cam, const RaySource &
   const int nchunks = (g.n_bands + narrow - 1) / narrow;
   if (tune.nbt <= 0 && g.n_bands > 8 && moving > 1) nbt = 16;  // inclined: the wide form
   const bool wide = is_wide(nbt, moving);
-  const bool lone = moving > 1 && narrow <= 8;  // there is a form for few rays
+  // there is a form for few rays (its 8 or 16 cells ahead are wasted in bricks of
+  // 1 or 2 cells: 100^2 pixels, one band, 208 and 213 us, 176 and 135 without it)
+  const bool lone = moving > 1 && narrow <= 8 && !(g.kind == AIR_GRID_AMR && g.B <= 2);
   const int64_t few = lone ? few_rays(narrow, nchunks) : 0;
   if (wide && tune.nbt <= 0) nbt = wide_width(g, kMarchBlock);
   const int64_t fill = wide && tune.nbt <= 0 ? wide_fill_threads() : 0;
