@@ -836,6 +836,25 @@ __device__ __forceinline__ void march_block(RTState<NBT> &r, const float Q[3], c
   } while (more);  // until the block is left (through its far face, or by rounding)
 }
 
+// march_block for a block of one cell, at `cells`, one band: a brick of one cell
+// has no walk, and a chunk's other steps are wasted (three inclined views, batched:
+// 1170 us, 972 without them).
+template <int FMT>
+__device__ __forceinline__ void march_cell(RTState<1> &r, const float Q[3], const float Dl[3], const float inv[3],
+                                           float tend, const void *__restrict__ cells, const BandCtx &bc,
+                                           const BandRegs<1> &br) {
+  float rho;
+  uint32_t aux;
+  load_cell<FMT>(cells, 0, rho, aux);
+  float tn = fminf(tend, FLT_MAX);
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    if (Dl[a] != 0.f) tn = fminf(tn, ((Dl[a] > 0.f ? 1.f : 0.f) - Q[a]) * inv[a]);
+  const float ds = fmaxf(tn, 0.f);
+  r.steps += ds > 0.f ? 1u : 0u;
+  rt_term<1, FMT>(r, rho, aux, ds, bc, br);
+}
+
 // Per-launch ray geometry, resolved on the host in FP64: the pixel centre
 // (uc, vc) is the world point C + uc u + vc v (C = image centre - grid origin),
 // its grid coordinate (finest-cell units) that point divided by the cell size
@@ -1308,8 +1327,13 @@ __device__ void march_amr(RTState<NBT> &r, const GridView &g, const double O[3],
     const int64_t boff = (int64_t)code << (3 * lb);
     const void *cb = FMT == kCellRho ? (const void *)((const float *)g.cells + boff)
                                      : (const void *)((const uint2 *)g.cells + boff);
-    march_block<NBT, FMT, K, int>(r, Q, Dl, inv, tend, lc[0], lc[1], lc[2], B, B, B, B, B * B, cb,
-                               bc, br);
+    bool cell = false;
+    if constexpr (NBT == 1) {
+      cell = B == 1;
+      if (cell) march_cell<FMT>(r, Q, Dl, inv, tend, cb, bc, br);
+    }
+    if (!cell)
+      march_block<NBT, FMT, K, int>(r, Q, Dl, inv, tend, lc[0], lc[1], lc[2], B, B, B, B, B * B, cb, bc, br);
     if (out) break;
     // advance to the exit point
     if (deep) t = f2_from(te);
