@@ -125,12 +125,12 @@ static size_t batch_smem(const GridView &g, int V, int width, int tabs) {
 
 // DIR: 0 for any views, -2 when every view is inclined (trace_ray): without the
 // column march of axis rays, which holds a chunk's band constants and partial
-// sums in registers, a block needs 124 registers instead of 168 at 8 bands per
-// thread and 160 instead of 250 at 16.
+// sums in registers, a thread needs 124 registers instead of 168 at 8 bands.
+// (Inclined views with 16 bands per thread take the wide form.)
 constexpr int kBatchWideBlocks = 4;
 template <int NBT, int DIR>
 struct BatchBlocks {
-  static constexpr int value = NBT == 0 ? kBatchWideBlocks : NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? (DIR == 0 ? 3 : 4) : (DIR == 0 ? 2 : 3)));
+  static constexpr int value = NBT == 0 ? kBatchWideBlocks : NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? (DIR == 0 ? 3 : 4) : 2));
 };
 
 // Band chunks whose tables a block holds. All of them, filled once, where the

@@ -31,13 +31,13 @@ struct MarchLaunch {
 // of at most one wave (more registers, deeper load groups) is then the same
 // kernel, so there is one.
 constexpr int kAxisBlocks = 8;
-constexpr int kAxisBlocksSmall = 6;  // bricks of at most 8 cells: two bricks' records in registers
+constexpr int kAxisBlocksSmall = 6;  // bricks of 4 or 8 cells: two bricks' records in registers
 
 // DIR = -1 has the registers of two or three blocks (see DdaChunk).
 template <int NBT, int DIR>
 struct MinBlocks {
   static constexpr int value = DIR == -1 ? (NBT <= 4 ? 3 : 2)
-                               : DIR == -2 ? (NBT <= 1 ? 6 : (NBT <= 2 ? 5 : (NBT <= 8 ? 4 : 3)))
+                               : DIR == -2 ? (NBT <= 1 ? 6 : (NBT <= 2 ? 5 : 4))
                                : DIR >= 4 && DIR <= 6 ? kAxisBlocksSmall
                                : DIR >= 1 ? kAxisBlocks
                                : (NBT <= 1 ? 6 : (NBT <= 2 ? 5 : (NBT <= 4 ? 4 : (NBT <= 8 ? 3 : 2))));
@@ -343,8 +343,9 @@ cudaError_t march_general(const MarchLaunch &m) {
 }
 
 // One-band grids, every ray parallel to grid axis A: the form DIR = 1 + A, or
-// 4 + A for bricks of 4 or 8 cells, 13 + A for 1 or 2, 7 + A or 10 + A for grids of 16^3 bricks
-// with per-cell Lambda (the ordinary one-band grid).
+// 4 + A for bricks of 4 or 8 cells, 13 + A for 1 or 2, 7 + A or 10 + A for grids
+// of 16^3 bricks with per-cell Lambda, the ordinary one-band grid (constant
+// strides would serve 32^3 bricks and several bands too; not tried there).
 template <int A, int FMT>
 static cudaError_t march_axis_fmt(const MarchLaunch &m) {
   if (m.g.kind != AIR_GRID_AMR) return march_form<1, false, FMT, 1 + A>(m);

@@ -252,8 +252,8 @@ __global__ void __launch_bounds__(kScanBlock) k_emit3(TreeView t, const int32_t 
 }
 
 // ---- the sweep with counts on the device ----------------------------------
-// The same steps over open[S->cur] with m = S->m items, in two launches; grids
-// are a few blocks per SM and loop over the items. The first flags and counts,
+// The same steps over the sweep's open list, whose length its slot holds
+// (SweepSlot::m), in two launches; grids are a few blocks per SM and loop over the items. The first flags and counts,
 // the second ranks and emits: each of its blocks adds up the chunk counts in
 // front of its chunk (and in all, to know the totals) from the two count
 // arrays, a few kilobytes that lie in L2. (With a counting and a scanning
@@ -607,7 +607,7 @@ __global__ void k_init_base(TreeView t) {
 // of each band in a fixed order (strided per thread, then a tree), so the
 // result does not depend on scheduling.
 //
-// A block takes per_block entries and kFluxBands bands (blockIdx.y; the last
+// A block takes kFluxPerBlock entries and kFluxBands bands (blockIdx.y; the last
 // row of blocks sums the step counts): leaf flags and levels are read once for
 // the bands of a block, and bands run beside one another. (One block summed
 // every band of 8192 entries, band after band, before: 85 us for 0.8 M leaves
