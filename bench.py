@@ -525,10 +525,6 @@ LARGE = dict(workload="clumps-and-cones block-AMR grid: 512^3 base cells in 32^3
                        "random views; AIR base 1024^2, max level 3 (8192^2 equivalent), "
                        "xi_crit 0.5", seed=0, views=16, base_res=1024, max_level=3, xi_crit=0.5,
              fixed_res=8192)
-FP32_OPS_PER_BAND_STEP = 23  # per band and cell: dtau, exponent argument, Taylor (7), both
-                             # cell-term forms (7), select, Kahan sum (4), table lookup (2);
-                             # a cell that emits nothing takes none of them, so a
-                             # fraction formed with this count can pass 1
 
 
 def run_large(args):
@@ -555,7 +551,7 @@ def run_large(args):
            "grid_upload_s": load_s}
     # batched plain AIR
     batch = {}
-    for bpt in (8, 16):
+    for bpt in (0, 8, 16):  # 0: the library's default
         g.render_batch(vs, n0, Lm, xc, bands_per_thread=bpt, fields=("band_flux",))
         g.profile(True)
         ms, b = _timed(lambda: g.render_batch(vs, n0, Lm, xc, bands_per_thread=bpt,
@@ -646,12 +642,9 @@ def run_large(args):
         fa = fs["band_flux"].double().sum().item()
         out.setdefault("flux_rel_err_vs_fixed", []).append(
             abs(seq[k]["band_flux"].double().sum().item() - fa) / abs(fa))
-    # ALU roofline of the batched kernel: FP32 operations per band-step
-    peak_ops = 152 * 128 * 2.07e9
-    ach = best["band_steps_per_s"] * FP32_OPS_PER_BAND_STEP
-    out["roofline"] = {"bound": "alu", "achieved": ach / 1e12, "peak": peak_ops / 1e12,
-                       "unit": "T FP32 op/s", "frac": ach / peak_ops, "traffic": None,
-                       "kernel": "k_air_batch", "ops_per_band_step": FP32_OPS_PER_BAND_STEP}
+    # (no fraction of the FP32 rate: a band step costs its operations only where
+    # the cell emits, and the emitting ones are not counted)
+    out["band_steps_per_s"] = best["band_steps_per_s"]
     out["total_s"] = time.perf_counter() - t0
     print(json.dumps(out), flush=True)
 
@@ -707,8 +700,6 @@ def large_view_record(air, torch, st, reps=2):
     march_ms = prof["march"][0] / reps
     hbm = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("hbm_gbs", 6800.0) \
         if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else 6800.0
-    peak_ops = 152 * 128 * 2.07e9
-    band_steps_s = sc.n_bands * steps / (march_ms * 1e-3)
     rec = dict(workload=W["workload"] + " -- view 0 of the 16, all 32 bands",
                base_res=n0, max_level=Lm, xi_crit=xc, fixed_res=W["fixed_res"],
                cells=int(sc.n_cells), scene_gen_s=gen_s, grid_upload_s=load_s,
@@ -728,10 +719,7 @@ def large_view_record(air, torch, st, reps=2):
                          "hbm": {"bound": "hbm", "achieved": BYTES_PER_STEP * steps / (march_ms * 1e-3) / 1e9,
                                  "peak": hbm, "unit": "GB/s",
                                  "frac": BYTES_PER_STEP * steps / (march_ms * 1e-3) / 1e9 / hbm},
-                         "alu": {"bound": "alu", "achieved": band_steps_s * FP32_OPS_PER_BAND_STEP / 1e12,
-                                 "peak": peak_ops / 1e12, "unit": "T FP32 op/s",
-                                 "frac": band_steps_s * FP32_OPS_PER_BAND_STEP / peak_ops,
-                                 "ops_per_band_step": FP32_OPS_PER_BAND_STEP}})
+                         "band_steps_per_s": sc.n_bands * steps / (march_ms * 1e-3)})
     g.close()
     del sc, g, flush
     torch.cuda.empty_cache()
@@ -740,10 +728,9 @@ def large_view_record(air, torch, st, reps=2):
 
 def batch_record(air, torch, st):
     """The batched configuration in brief: the cone grid with 16 bands
-    (0.5-10 keV) at 64 random views, one persistent launch (16 bands per
-    thread), against fixed 4096^2 images of two of the views (extrapolated to
-    64) with the band-summed flux error on those two, and the batched march's
-    FP32-issue fraction. Scene generation, upload and one warm-up render are
+    (0.5-10 keV) at 64 random views, one persistent launch, against fixed
+    4096^2 images of two of the views (extrapolated to 64) with the band-summed
+    flux error on those two. Scene generation, upload and one warm-up render are
     outside the timed render."""
     W = WORKLOAD
     t0 = time.perf_counter()
@@ -754,9 +741,9 @@ def batch_record(air, torch, st):
     setup_s = time.perf_counter() - t0
     vs = scenes.random_views(3, 64)
     n0, Lm, xc = W["base_res"], W["max_level"], W["xi_crit"]
-    g.render_batch(vs, n0, Lm, xc, bands_per_thread=8, fields=("band_flux",))
+    g.render_batch(vs, n0, Lm, xc, fields=("band_flux",))
     g.profile(True)
-    ms, b = _timed(lambda: g.render_batch(vs, n0, Lm, xc, bands_per_thread=8, fields=("band_flux",)), st)
+    ms, b = _timed(lambda: g.render_batch(vs, n0, Lm, xc, fields=("band_flux",)), st)
     prof = g.profile_read()
     g.profile(False)
     steps = sum(r["n_steps"] for r in b)
@@ -765,19 +752,13 @@ def batch_record(air, torch, st):
     fixed_view_ms = float(np.mean([x[0] for x in fx]))
     ferr = [abs(float(b[k]["band_flux"].double().sum()) - float(fx[k][1]["band_flux"].double().sum())) /
             abs(float(fx[k][1]["band_flux"].double().sum())) for k in range(2)]
-    band_steps_s = 16 * steps / (prof["batch"][0] * 1e-3)
-    peak_ops = 152 * 128 * 2.07e9
     rec = dict(workload="cone grid, 64 random views x 16 bands (0.5-10 keV), base 256^2, max level 4, "
-                        "xi_crit 0.5, one persistent launch, 16 bands per thread",
+                        "xi_crit 0.5, one persistent launch",
                setup_s=setup_s, batched_ms=ms, rays=int(sum(r["n_rays"] for r in b)), steps=int(steps),
                band_steps_per_s=16 * steps / ms * 1e3, kernel_ms=prof["batch"][0],
                fixed_per_view_ms=fixed_view_ms, fixed_64_views_ms_extrapolated=fixed_view_ms * len(vs),
                batched_speedup_vs_fixed=fixed_view_ms * len(vs) / ms,
-               flux_rel_err_vs_fixed_views_0_1=ferr,
-               roofline={"bound": "alu", "achieved": band_steps_s * FP32_OPS_PER_BAND_STEP / 1e12,
-                         "peak": peak_ops / 1e12, "unit": "T FP32 op/s",
-                         "frac": band_steps_s * FP32_OPS_PER_BAND_STEP / peak_ops,
-                         "ops_per_band_step": FP32_OPS_PER_BAND_STEP, "kernel": "k_air_batch"})
+               flux_rel_err_vs_fixed_views_0_1=ferr)
     g.close()
     del sc, g
     torch.cuda.empty_cache()
