@@ -436,9 +436,13 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
   }
 }
 
+// (One limit of dynamic shared memory for every launch, see kWideShared: the
+// block's tables, constants and sums are below 114 KB by batch_tables, and 256
+// views' counters take 11 KB.)
+constexpr int kBatchShared = 200 * 1024;
 template <int NBT, bool AMR, int FMT, int DIR>
 static cudaError_t batch_occupancy(int *blocks_per_sm, size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(k_air_batch<NBT, AMR, FMT, DIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_air_batch<NBT, AMR, FMT, DIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBatchShared);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_air_batch<NBT, AMR, FMT, DIR>, kBatchBlock, smem);
 }

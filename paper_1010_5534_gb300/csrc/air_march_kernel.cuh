@@ -182,6 +182,10 @@ __global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
 // 4 13.51, 3 14.01; 32-band clumps: 12.8, 12.2, 9.3, 9.2: the sums of more blocks
 // leave too little L1 for the cells).
 constexpr int kWideBlocks = 4;
+// The kernel's limit of dynamic shared memory. It is a property of the function,
+// shared by every thread that launches it, so it is set to one value above what
+// any launch takes (wide_width: 54 KB), not to each launch's own.
+constexpr int kWideShared = 64 * 1024;
 
 template <bool AMR, int FMT>
 __device__ __forceinline__ void wide_one(const GridView &g, const RayGeom &rg, const RaySource &src,
@@ -288,7 +292,7 @@ static cudaError_t march_wide_form(const MarchLaunch &m, int64_t rays) {
   const int width = m.src.width;
   const size_t smem = wide_tab_bytes(FMT == kCellXq, m.g.n_tbins, width) + wide_sum_bytes(width, kMarchBlock);
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_march_wide<AMR, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(k_march_wide<AMR, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideShared);
     if (e != cudaSuccess) return e;
   }
   const int64_t blocks = m.src.mode == 2 ? (int64_t)sm_count() * kWideBlocks
