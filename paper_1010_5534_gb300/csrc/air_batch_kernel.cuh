@@ -198,7 +198,7 @@ __device__ __forceinline__ void batch_trace(const BatchArgs &a, unsigned char *s
     const BandCtx bc = chunk_ctx<NBT, FMT>(sm + slot * chunk_bytes<NBT>(FMT == kCellXq, g.n_tbins), g,
                                            min(NBT, g.n_bands - b0));
     BandRegs<NBT> br;
-    band_regs<NBT>(br, bc);
+    band_regs<NBT, FMT>(br, bc);
     RTState<NBT> st;
     trace_ray<NBT, AMR, FMT, DIR>(st, g, rg, L, i, j, a.fp64_level, bc, br);
     if (chunk == 0) {

@@ -219,9 +219,14 @@ __device__ __forceinline__ BandCtx chunk_ctx(const unsigned char *sm, const Grid
 }
 
 // Per-band constants in registers. One band keeps them for the whole ray; with
-// more, only the column march of axis rays does (band_load), and the cells of
-// inclined rays read their band's constants from shared memory (one 16-byte
-// load that every lane shares, against 24 registers at 8 bands).
+// more, the column march of axis rays does (band_load), and so does every ray of
+// a grid whose emission has no table (kCellRho): there a band's arithmetic is so
+// short that a load per band and cell shows (400^2 inclined pixels, 5 bands: 537 us
+// with the constants in shared memory, 455 in registers). With a table the cells of inclined rays read their band's constants
+// from shared memory (one 16-byte load that every lane shares, against 24
+// registers at 8 bands).
+template <int NBT, int FMT>
+constexpr bool kRegConst = NBT == 1 || (NBT > 1 && FMT == kCellRho);
 template <int NBT>
 struct BandRegs {
   float kap[NBT];  // kappa_b
@@ -253,13 +258,13 @@ __device__ __forceinline__ void band_load(BandRegs<NBT> &br, const BandCtx &bc) 
     br.kmax = fmaxf(br.kmax, c.kap);
   }
 }
-// What a ray starts with: xz, and one band's constants.
-template <int NBT>
+// What a ray starts with: xz, and the constants that stay in registers.
+template <int NBT, int FMT>
 __device__ __forceinline__ void band_regs(BandRegs<NBT> &br, const BandCtx &bc) {
   br.xz = 0xffffffffu;
 #pragma unroll
   for (int b = 0; b < NBT; ++b) br.xz = min(br.xz, bc.band[b].xz);
-  if (NBT == 1) band_load<NBT>(br, bc);
+  if (kRegConst<NBT, FMT>) band_load<NBT>(br, bc);
 }
 
 // Whether a cell emits nothing in any band of the chunk, from its auxiliary
@@ -383,7 +388,7 @@ __device__ __forceinline__ void rt_bands(RTState<NBT> &r, float rho, uint32_t au
 #pragma unroll
       for (int e = 0; e < (NBT == 1 ? 1 : 2); ++e) {
         const int b = 2 * q + e;
-        const BandConst c = NBT == 1 ? BandConst{br.kap[0], br.ik[0], br.nk[0], 0u} : band_const<NBT>(bc, b);
+        const BandConst c = kRegConst<NBT, FMT> ? BandConst{br.kap[b], br.ik[b], br.nk[b], 0u} : band_const<NBT>(bc, b);
         const float dtau = c.kap * rds;
         const float Tn = ex2_approx(c.nk * N);
         // rho Lambda_b

@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kMarchBlock, MinBlocks<NBT, DIR>::value)
   wait_prior_grid();
   __syncthreads();
   BandRegs<NBT> br;
-  band_regs<NBT>(br, bc);
+  band_regs<NBT, FMT>(br, bc);
 
   if (src.mode == 2) {
     // new nodes of a sweep counted on the device: warp w of the grid takes rays
