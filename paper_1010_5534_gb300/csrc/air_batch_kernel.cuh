@@ -137,8 +137,10 @@ struct BatchBlocks {
 // form's resident blocks then still fit an SM's shared memory; else one at a
 // time, filled again whenever the block's warps go on to the next chunk. (8
 // inclined views, 255 table bins, every chunk held: 32 bands 10.5 ms with two
-// blocks per SM, 64 bands 29.7 with one; one at a time 8.8 and 15.3. Mixed
-// views 16.8 and 46.3, 14.1 and 26.2. 64 bins: 7.8 and 13.0, 13.6 and 25.7.)
+// blocks per SM, 64 bands 29.7 with one; one at a time 8.5 and 13.8. Mixed
+// views 16.8 and 46.3, 13.7 and 25.4. 64 bins: 7.7 and 12.9, 13.7 and 25.7.
+// Groups of as many tables as fit, one group at a time: 8.4 and 13.7, but 14.8
+// and 27.7 for mixed views.)
 constexpr size_t kSmShared = 228 * 1024, kBlockReserve = 1024;  // of an SM; taken per block
 template <int NBT, int DIR>
 static int batch_tables(const GridView &g, int V, int width) {
@@ -228,14 +230,17 @@ __device__ __forceinline__ void batch_fill(const BatchArgs &a, unsigned char *sm
 
 // The work of one phase: `items` items (rays x parts) of every band chunk, from
 // the chunks' queues; a warp takes rpw at a time. body(chunk, item), lane by
-// lane. With one table per block, the block goes from chunk to chunk together
-// (and leaves out a chunk whose queue is empty by then); every thread of the
+// lane. With one table per block, the block goes from chunk to chunk together,
+// beginning with the chunk whose table it holds (`held`; another one in every
+// block at first, so the chunks of a phase of few rays are traced side by side)
+// and leaving out chunks whose queues are empty by then. Every thread of the
 // block calls this.
 template <int NBT, int FMT, class Body>
 __device__ __forceinline__ void batch_queue(const BatchArgs &a, unsigned char *sm, unsigned long long items,
-                                            int rpw, const Body &body) {
-  const int lane = threadIdx.x & 31;
-  for (int chunk = 0; chunk < a.chunks; ++chunk) {
+                                            int rpw, int &held, const Body &body) {
+  const int lane = threadIdx.x & 31, from = held;
+  for (int i = 0; i < a.chunks; ++i) {
+    const int chunk = from + i < a.chunks ? from + i : from + i - a.chunks;
     auto take = [&] {
       unsigned long long b = 0;
       if (lane == 0) b = atomicAdd(&a.ctl->q_head[chunk], (unsigned long long)rpw);
@@ -244,8 +249,11 @@ __device__ __forceinline__ void batch_queue(const BatchArgs &a, unsigned char *s
     unsigned long long b = take();
     if (a.tabs < a.chunks) {
       if (!__syncthreads_or(b < items)) continue;
-      batch_fill<NBT, FMT>(a, sm, chunk);
-      __syncthreads();
+      if (chunk != held) {
+        batch_fill<NBT, FMT>(a, sm, chunk);
+        held = chunk;
+        __syncthreads();
+      }
     }
     for (; b < items; b = take()) {
       const unsigned long long it = lane < rpw ? b + lane : items;
@@ -260,8 +268,13 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
   const GridView &g = a.g;
   const int V = a.V, nb = g.n_bands;
   const size_t tab = batch_tab_bytes<NBT>(FMT == kCellXq, g.n_tbins, a.width);
-  if (a.tabs == a.chunks)
+  int held = 0;  // where a block holds one table: its chunk
+  if (a.tabs == a.chunks) {
     for (int c = 0; c < a.chunks; ++c) batch_fill<NBT, FMT>(a, smem_raw + c * tab, c);
+  } else {
+    held = (int)(blockIdx.x % (unsigned)a.chunks);
+    batch_fill<NBT, FMT>(a, smem_raw, held);
+  }
   const size_t tab_end = a.tabs * tab + (NBT == 0 ? wide_sum_bytes(a.width, kBatchBlock) : 0);
   int64_t *run = (int64_t *)(smem_raw + tab_end);
   int64_t *tot = run + V;
@@ -297,10 +310,10 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
   int64_t first = a.mode == 2 ? nbase : 0, n = nbase;
   if (a.mode == 2 && a.P > 0) {
     // the proposal wave of every view: (ray, band chunk) items from the queue
-    const int parts = NBT == 0 ? wide_parts(a.P * a.tabs, min(a.width, nb), a.fill) : 1;
+    const int parts = NBT == 0 ? wide_parts(a.P * a.chunks, min(a.width, nb), a.fill) : 1;
     const BatchOut o{a.pN, a.pI, a.pp, a.psteps, nullptr, a.P};
-    const int rpw = rays_per_warp(a.P, a.tabs * parts, (int64_t)nblk * (kBatchBlock / 32));
-    batch_queue<NBT, FMT>(a, smem_raw, (unsigned long long)a.P * parts, rpw, [&](int chunk, unsigned long long it) {
+    const int rpw = rays_per_warp(a.P, a.chunks * parts, (int64_t)nblk * (kBatchBlock / 32));
+    batch_queue<NBT, FMT>(a, smem_raw, (unsigned long long)a.P * parts, rpw, held, [&](int chunk, unsigned long long it) {
       const int part = parts == 1 ? 0 : (int)(it / (unsigned long long)a.P);
       const int64_t q = (int64_t)(it - (unsigned long long)part * a.P);
       batch_trace<NBT, AMR, FMT, DIR>(a, smem_raw, a.geoms[a.pview[q]], a.plvl[q], a.ppi[q], a.ppj[q], chunk, part,
@@ -323,11 +336,11 @@ __global__ void __launch_bounds__(kBatchBlock, BatchBlocks<NBT, DIR>::value) k_a
   for (;; ++sweep) {
     // step ii: trace the rays added last sweep, all views and band chunks
     const int64_t cnt_r = n - first;
-    const int parts = NBT == 0 ? wide_parts(cnt_r * a.tabs, min(a.width, nb), a.fill) : 1;
+    const int parts = NBT == 0 ? wide_parts(cnt_r * a.chunks, min(a.width, nb), a.fill) : 1;
     const int shares = a.chunks * parts;
     const BatchOut o{t.N, t.I, t.p, t.steps, a.mode == 1 ? a.maxlev : nullptr, t.cap};
-    const int rpw = rays_per_warp(cnt_r, a.tabs * parts, (int64_t)nblk * (kBatchBlock / 32));
-    batch_queue<NBT, FMT>(a, smem_raw, (unsigned long long)cnt_r * parts, rpw, [&](int chunk, unsigned long long it) {
+    const int rpw = rays_per_warp(cnt_r, shares, (int64_t)nblk * (kBatchBlock / 32));
+    batch_queue<NBT, FMT>(a, smem_raw, (unsigned long long)cnt_r * parts, rpw, held, [&](int chunk, unsigned long long it) {
       const int part = parts == 1 ? 0 : (int)(it / (unsigned long long)cnt_r);
       const int64_t k = first + (int64_t)(it - (unsigned long long)part * cnt_r);
       const int v = a.view[k];

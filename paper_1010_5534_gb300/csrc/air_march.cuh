@@ -77,9 +77,12 @@ __host__ __device__ constexpr size_t tab_bytes(int n_tbins) {
   return (sizeof(float) * (size_t)(tab_row<NBT>() * n_tbins) + 15) & ~(size_t)15;
 }
 // Fill the table of bands [b0, b0 + NBT) (zero beyond n_bands) by one block.
+// (Eight entries' loads in flight: a block that goes from chunk to chunk fills
+// its table again and again, see batch_tables.)
 template <int NBT>
 __device__ __forceinline__ void tab_fill(float *tab, const GridView &g, int b0) {
   const int ts = g.n_tbins + 1;
+#pragma unroll 8
   for (int x = threadIdx.x; x < NBT * g.n_tbins; x += blockDim.x) {
     const int k = x / NBT, b = x - k * NBT;
     float v = 0.f, d = 0.f;
@@ -140,15 +143,16 @@ __device__ __forceinline__ void wide_fill(unsigned char *sm, const GridView &g, 
   if (FMT == kCellXq) {
     float *tab = reinterpret_cast<float *>(band + width);
     const int ts = g.n_tbins + 1, row = wide_row(width);
-    for (int k = threadIdx.x >> 5; k < g.n_tbins; k += blockDim.x >> 5)
-      for (int b = threadIdx.x & 31; b < width; b += 32) {
-        float v = 0.f, d = 0.f;
-        if (b0 + b < g.n_bands) {
-          v = g.table[(b0 + b) * ts + k];
-          d = g.table[(b0 + b) * ts + k + 1] - v;
-        }
-        *reinterpret_cast<float2 *>(tab + k * row + 2 * b) = make_float2(v, d);
+#pragma unroll 8
+    for (int x = threadIdx.x; x < width * g.n_tbins; x += blockDim.x) {
+      const int k = x / width, b = x - k * width;
+      float v = 0.f, d = 0.f;
+      if (b0 + b < g.n_bands) {
+        v = g.table[(b0 + b) * ts + k];
+        d = g.table[(b0 + b) * ts + k + 1] - v;
       }
+      *reinterpret_cast<float2 *>(tab + k * row + 2 * b) = make_float2(v, d);
+    }
   }
 }
 // Part `part` of `parts` of the chunk at `sm` (nb of its `width` bands exist);
